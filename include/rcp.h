@@ -295,9 +295,12 @@ typedef struct {
     int64_t nodes, box_tests, tri_tests, sphere_tests;
 } rcp_counters;
 
-/* Rays traced (primary, shadow) by the scene's most recent rcp_render*
- * call, counted on the device during that render. Read it after the render
- * has completed (synchronise its stream first). */
+/* Rays (primary, shadow) of the K passes of the scene's most recent
+ * rcp_render* call, counted on the device during that render. A chained render
+ * stops tracing a pixel whose value repeats an earlier pass's (the later
+ * passes then repeat too); those passes count the rays of the pass they
+ * repeat. Read it after the render has completed (synchronise its stream
+ * first). */
 rcp_status rcp_last_ray_counts(const rcp_scene* scene, int64_t* primary, int64_t* shadow);
 
 /* d_in: previous image (device rgbz, NULL = I_0); d_out: this pass's image

@@ -77,6 +77,16 @@ __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, 
     return out;
 }
 
+// Whether a pixel's values a and b give the next pass the same camera, bit
+// for bit: the lanes of a previous value that camera_ray reads under the
+// mapping (colour; colour and z-depth; the normal's code).
+__device__ __forceinline__ bool same_camera(int mapping, const float4& a, const float4& b) {
+    const uint32_t rgb = (__float_as_uint(a.x) ^ __float_as_uint(b.x)) | (__float_as_uint(a.y) ^ __float_as_uint(b.y)) |
+                         (__float_as_uint(a.z) ^ __float_as_uint(b.z));
+    const uint32_t w = __float_as_uint(a.w) ^ __float_as_uint(b.w);
+    return (mapping == RCP_MAP_NORMAL ? w : mapping == RCP_MAP_DEPTH ? rgb | w : rgb) == 0u;
+}
+
 // A warp counts n finished tiles of view v (with a done counter) at once:
 // every lane's writes for them made visible first, at system scope (the RGB
 // may go straight to host memory, which the host reads once the flag is set),
@@ -208,8 +218,44 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                 float4 out = FUSED && v.in ? __ldg(v.in + p) : make_float4(0.5f, 0.5f, 0.5f, 0.f);
                 uint32_t code;
                 int32_t prim;
-                for (int n = 0; n < (CHAIN ? v.passes : 1); ++n) {
-                    prefetch_record(S, hint.x);  // its lines arrive while the camera ray is made
+                if (CHAIN) {
+                    float4 prev = out;  // I_{n-2} where out is I_{n-1}
+                    int32_t prev_prim = -1;
+                    uint32_t prev_shadow = 0;
+                    const int K = v.passes;
+                    for (int n = 1; n <= K; ++n) {
+                        prefetch_record(S, hint.x);  // its lines arrive while the camera ray is made
+                        const RayF r = camera_ray(v, (float)x + 0.5f, (float)y + 0.5f, out, S.tmin);
+                        const uint32_t before = n_shadow;
+                        int32_t id;
+                        float4 cur = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code,
+                                                        id, s_order, hint);
+                        ++n_primary;
+                        if (v.mapping == RCP_MAP_NORMAL) cur.w = __uint_as_float(code);
+                        const uint32_t shadow = n_shadow - before;
+                        const uint32_t left = (uint32_t)(K - n);
+                        const bool fixed = same_camera(v.mapping, cur, out);
+                        if (fixed || (n > 1 && same_camera(v.mapping, cur, prev))) {
+                            // the orbit has closed: I_{n+1} is I_n, or I_{n+1}, I_{n+2}, ... alternate
+                            // between I_{n-1} and I_n
+                            const uint32_t odd = fixed ? 0u : (left + 1) / 2;
+                            n_primary += left;
+                            n_shadow += odd * prev_shadow + (left - odd) * shadow;
+                            if (fixed || !(left & 1u)) {
+                                out = cur;
+                                prim = id;
+                            } else {
+                                prim = prev_prim;  // out already holds I_{n-1}
+                            }
+                            break;
+                        }
+                        prev = out;
+                        out = cur;
+                        prim = prev_prim = id;
+                        prev_shadow = shadow;
+                    }
+                } else {
+                    prefetch_record(S, hint.x);
                     RayF r;
                     if (FUSED) {
                         r = camera_ray(v, (float)x + 0.5f, (float)y + 0.5f, out, S.tmin);
