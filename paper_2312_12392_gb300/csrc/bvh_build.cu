@@ -50,10 +50,10 @@ rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
 namespace {
 
 constexpr int BUILD_BLOCK = 256;
-// Most primitives in one leaf slot. A leaf's meta byte holds count << 5 |
-// offset with bit 7 clear (bit 7 marks an internal child), so count <= 3.
+// Most primitives in one leaf slot: a node's header has 3 bits per slot for
+// the count in unary.
 constexpr int LEAF_MAX = 3;
-static_assert(LEAF_MAX >= 1 && LEAF_MAX <= 3, "a leaf's count must leave the meta byte's top bit clear");
+static_assert(LEAF_MAX >= 1 && LEAF_MAX <= 3, "a leaf's count must fit the 3 unary bits of its slot");
 
 __device__ __forceinline__ uint32_t f2ord(float f) {
     const uint32_t u = __float_as_uint(f);
@@ -1018,7 +1018,7 @@ __global__ void k_collapse(BinTree bt, const int2* __restrict__ frontier, int n_
     WNode nd;
     nd.child_base = child_base;
     nd.prim_base = prim_base;
-    uint32_t meta[2] = {0, 0};
+    uint32_t leaf_bits = 0;
     uint32_t imask = 0;
     for (int c = 0; c < m; ++c)
         if (is_int[c]) imask |= 1u << slot_of[c];
@@ -1029,15 +1029,13 @@ __global__ void k_collapse(BinTree bt, const int2* __restrict__ frontier, int n_
         for (int q = 0; q < m; ++q)
             if (slot_of[q] == s) c = q;
         if (c < 0) continue;
-        uint32_t mb;
         if (is_int[c]) {
-            const uint32_t rank = __popc(imask & ((1u << s) - 1u));
-            mb = 0x80u | rank;
+            const uint32_t rank = __popc(imask & bits_below(s));
             const uint32_t slot_idx = atomicAdd(&counters[2], 1u);
             next_front[slot_idx] = make_int2(cref[c], (int)(child_base + rank));
         } else {
             const int cnt = clast[c] - cfirst[c] + 1;
-            mb = ((uint32_t)cnt << 5) | (uint32_t)poff;
+            leaf_bits |= bits_below(cnt) << (3 * s);
             for (int q = 0; q < cnt; ++q) {
                 const uint32_t ref = bt.sorted_ids[cfirst[c] + q];
                 const int64_t rec = (int64_t)(prim_base + poff + q);
@@ -1050,10 +1048,9 @@ __global__ void k_collapse(BinTree bt, const int2* __restrict__ frontier, int n_
             poff += cnt;
             leaf_max = max(leaf_max, cnt);
         }
-        meta[s >> 2] |= mb << (8 * (s & 3));
     }
-    nd.meta_lo = meta[0];
-    nd.meta_hi = meta[1];
+    nd.slots = imask | leaf_bits << 8;
+    nd.pad = 0;
     float3 ulo, uhi;
     write_child_boxes(nd, clo, chi, slot_of, m, ulo, uhi);
     nodes[w] = nd;
@@ -1144,14 +1141,14 @@ __global__ void __launch_bounds__(REFIT_BLOCK) k_refit_wide(WNode* __restrict__ 
     if (live) {
         float* nf = reinterpret_cast<float*>(nodes + w);
         const uint4 hd = *reinterpret_cast<const uint4*>(nf + 48);
-        const uint32_t mb = ((s < 4 ? hd.z : hd.w) >> (8 * (s & 3))) & 0xffu;
-        if (mb & 0x80u) {
-            const int64_t c = hd.x + __popc(internal_mask(hd.z, hd.w) & ((1u << s) - 1u));
+        const uint32_t leaf_bits = hd.z >> 8;
+        if (hd.z & (1u << s)) {
+            const int64_t c = hd.x + __popc(hd.z & bits_below(s));
             const float4 l = nbox[2 * c], h = nbox[2 * c + 1];
             lo = make_float3(l.x, l.y, l.z);
             hi = make_float3(h.x, h.y, h.z);
-        } else if (mb) {
-            const int cnt = mb >> 5, off = mb & 31;
+        } else {
+            const int cnt = __popc((leaf_bits >> (3 * s)) & 7u), off = __popc(leaf_bits & bits_below(3 * s));
             const float2* b = rbox + 3 * ((int64_t)hd.y + off);
             for (int q = 0; q < cnt; ++q) {
                 const float2 a = b[3 * q], m = b[3 * q + 1], z = b[3 * q + 2];
@@ -1204,18 +1201,17 @@ __global__ void k_validate(const WNode* __restrict__ nodes, int64_t n_nodes, con
     const int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (w >= n_nodes) return;
     const WNode nd = nodes[w];
-    const uint32_t imask = internal_mask(nd.meta_lo, nd.meta_hi);
+    const uint32_t imask = nd.slots & 0xffu, leaf_bits = nd.slots >> 8;
     for (int s = 0; s < 8; ++s) {
-        const uint32_t mb = ((s < 4 ? nd.meta_lo : nd.meta_hi) >> (8 * (s & 3))) & 0xffu;
-        if (!mb) {
-            if (imask & (1u << s)) atomicAdd(&errors[0], 1);
-            continue;
-        }
+        const uint32_t lb = (leaf_bits >> (3 * s)) & 7u;
+        const bool internal = imask & (1u << s);
+        if (lb & (lb + 1u)) atomicAdd(&errors[0], 1);  // a count in unary
+        if (!internal && !lb) continue;  // empty
         double lo[3], hi[3];
         slot_box(nd, s, lo, hi);
-        if (mb & 0x80u) {
-            if (!(imask & (1u << s)) || (mb & 0x7fu) != (uint32_t)__popc(imask & ((1u << s) - 1u))) atomicAdd(&errors[0], 1);
-            const int64_t c = nd.child_base + (mb & 7u);
+        if (internal) {
+            if (lb) atomicAdd(&errors[0], 1);  // a slot is a child or a leaf
+            const int64_t c = (int64_t)nd.child_base + __popc(imask & bits_below(s));
             if (c <= w || c >= n_nodes) {
                 atomicAdd(&errors[1], 1);
                 continue;
@@ -1225,8 +1221,7 @@ __global__ void k_validate(const WNode* __restrict__ nodes, int64_t n_nodes, con
             if (l.x < lo[0] || l.y < lo[1] || l.z < lo[2] || h.x > hi[0] || h.y > hi[1] || h.z > hi[2])
                 atomicAdd(&errors[2], 1);
         } else {
-            if (imask & (1u << s)) atomicAdd(&errors[0], 1);
-            const int cnt = mb >> 5, off = mb & 31;
+            const int cnt = __popc(lb), off = __popc(leaf_bits & bits_below(3 * s));
             for (int q = 0; q < cnt; ++q) {
                 const int64_t r = (int64_t)nd.prim_base + off + q;
                 if (r >= n_records) {

@@ -23,28 +23,25 @@ constexpr uint32_t SPHERE_BIT = 0x80000000u;
 constexpr int MAX_STACK = 64;  // traversal stack entries (>= BVH depth)
 
 // One 8-wide node, 13 rows of 16 bytes. Child slot s (0..7) has the float
-// box lo_a[s]..hi_a[s] per axis a (an empty slot: lo = +inf, hi = -inf), and
-// meta[s]: 0 = empty, 0x80 | rank = internal child (node child_base + rank,
-// ranks counted in slot order), (count << 5) | offset = leaf of `count` (1..3)
-// primitive records at prim_base + offset. Rows 0-1 lo_x, 2-3 hi_x, 4-5 lo_y,
-// 6-7 hi_y, 8-9 lo_z, 10-11 hi_z, 12 the header.
+// box lo_a[s]..hi_a[s] per axis a (an empty slot: lo = +inf, hi = -inf).
+// slots: bit s set = slot s holds an internal child, node child_base + the
+// number of internal slots below s; bits 8 + 3 s .. 10 + 3 s hold a leaf
+// slot's record count (1..3) in unary, and the records of a node's leaves lie
+// from prim_base on in slot order, so the record of leaf bit j is prim_base +
+// the number of leaf bits below j. Rows 0-1 lo_x, 2-3 hi_x, 4-5 lo_y, 6-7
+// hi_y, 8-9 lo_z, 10-11 hi_z, 12 the header.
 struct __align__(16) WNode {
     float lo_x[8], hi_x[8], lo_y[8], hi_y[8], lo_z[8], hi_z[8];
     uint32_t child_base;
     uint32_t prim_base;
-    uint32_t meta_lo, meta_hi;  // meta[0..3], meta[4..7]
+    uint32_t slots;  // internal mask | leaf record bits << 8
+    uint32_t pad;
 };
 constexpr int NODE_ROWS = 13;
 static_assert(sizeof(WNode) == 16 * NODE_ROWS, "WNode must be 13 rows of 16 bytes");
 
-// Slots holding internal children: bit s set when meta byte s has its top bit.
-// Each half gathers bits 7, 15, 23, 31 into bits 28..31 with one multiply
-// (the partial products below bit 28 never carry into it).
-__host__ __device__ __forceinline__ uint32_t internal_mask(uint32_t meta_lo, uint32_t meta_hi) {
-    const uint32_t a = ((meta_lo & 0x80808080u) * 0x00204081u) >> 28;
-    const uint32_t b = ((meta_hi & 0x80808080u) * 0x00204081u) >> 28;
-    return a | (b << 4);
-}
+// Bits below bit b of a mask's slot or leaf bit b (b <= 24).
+__host__ __device__ __forceinline__ uint32_t bits_below(uint32_t b) { return (1u << b) - 1u; }
 
 struct LightDev {
     int type;

@@ -58,8 +58,8 @@ template <bool COUNT>
 __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, const float* Fw, uint2* stack,
                                               int stride, const StackCfg& stk, bool& overflow, WorkCount& wc,
                                               uint32_t& n_shadow, uint32_t& code, int32_t& prim,
-                                              const uint8_t* order_lut, int2& hint) {
-    const Hit h = traverse<false, COUNT>(S, r, stack, stride, stk, overflow, wc, order_lut, hint.x);
+                                              const uint8_t* walk_lut, int2& hint) {
+    const Hit h = traverse<false, COUNT>(S, r, stack, stride, stk, overflow, wc, walk_lut, hint.x);
     prefetch_record(S, hint.y);  // the previous occluder, ahead of the shadow walk
     const ShadeInfo si = shade_primary(S, r, h);
     float4 out = si.c_shadow;
@@ -67,7 +67,7 @@ __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, 
     if (si.need_shadow) {
         ++n_shadow;
         const Hit hs =
-            traverse<true, COUNT>(S, si.shadow, stack, stride, stk, overflow, wc, order_lut, hint.y);
+            traverse<true, COUNT>(S, si.shadow, stack, stride, stk, overflow, wc, walk_lut, hint.y);
         if (hs.rec < 0) out = si.c_lit;
         hint.y = hs.rec;
     }
@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                                                  unsigned long long* ray_counts, unsigned long long* counters) {
     static_assert(!CHAIN || (FUSED && !MS), "a chained launch makes its rays itself, one per pixel");
     extern __shared__ uint2 s_stack[];
-    __shared__ uint8_t s_order[ORDER_LUT_BYTES];
+    __shared__ __align__(16) uint8_t s_lut[WALK_LUT_BYTES];
     __shared__ SceneDev s_scene[MULTI ? BLOCK / 32 : 1];  // MULTI: the scene of each warp's current tile
     // per warp: the view (with a done counter) whose tiles it finished last,
     // and how many of them it has not yet counted. Done counters come with
@@ -128,7 +128,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
     constexpr bool SIGNAL = MULTI;
     __shared__ const ViewDev* s_done_v[BLOCK / 32];
     __shared__ int s_done_n[BLOCK / 32];
-    fill_order_lut<BLOCK>(s_order);
+    fill_walk_lut<BLOCK>(s_lut);
     if ((threadIdx.x & 31) == 0) {
         s_done_v[threadIdx.x >> 5] = nullptr;
         s_done_n[threadIdx.x >> 5] = 0;
@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                         uint32_t code;
                         int32_t prim;
                         const float4 o = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc,
-                                                            n_shadow, code, prim, s_order, hint);
+                                                            n_shadow, code, prim, s_lut, hint);
                         ++n_primary;
                         acc.x = __fadd_rn(acc.x, o.x);
                         acc.y = __fadd_rn(acc.y, o.y);
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                         const uint32_t before = n_shadow;
                         int32_t id;
                         float4 cur = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code,
-                                                        id, s_order, hint);
+                                                        id, s_lut, hint);
                         ++n_primary;
                         if (v.mapping == RCP_MAP_NORMAL) cur.w = __uint_as_float(code);
                         const uint32_t shadow = n_shadow - before;
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                         r.tmax = b.w;
                     }
                     out = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code, prim,
-                                             s_order, hint);
+                                             s_lut, hint);
                     ++n_primary;
                     if (v.mapping == RCP_MAP_NORMAL) out.w = __uint_as_float(code);
                 }
@@ -334,8 +334,8 @@ __global__ void __launch_bounds__(BLOCK) k_debug_trace(SceneDev S, int64_t n, co
                                                        float* __restrict__ t_out, int32_t* __restrict__ prim_out,
                                                        int stack_entries, int* status) {
     extern __shared__ uint2 s_stack[];
-    __shared__ uint8_t s_order[ORDER_LUT_BYTES];
-    fill_order_lut<BLOCK>(s_order);
+    __shared__ __align__(16) uint8_t s_lut[WALK_LUT_BYTES];
+    fill_walk_lut<BLOCK>(s_lut);
     __syncthreads();
     uint2* stack = s_stack + threadIdx.x;
     const StackCfg stk{stack_entries, 0, nullptr, 0};
@@ -346,8 +346,8 @@ __global__ void __launch_bounds__(BLOCK) k_debug_trace(SceneDev S, int64_t n, co
         RayF r{a.x, a.y, a.z, b.x, b.y, b.z, a.w, b.w};
         Hit h;
         if (brute) h = any ? traverse_brute<true>(S, r) : traverse_brute<false>(S, r);
-        else h = any ? traverse<true, false>(S, r, stack, BLOCK, stk, overflow, wc, s_order)
-                     : traverse<false, false>(S, r, stack, BLOCK, stk, overflow, wc, s_order);
+        else h = any ? traverse<true, false>(S, r, stack, BLOCK, stk, overflow, wc, s_lut)
+                     : traverse<false, false>(S, r, stack, BLOCK, stk, overflow, wc, s_lut);
         if (any) {
             prim_out[i] = h.rec >= 0 ? 1 : 0;
             t_out[i] = 0.f;
