@@ -52,16 +52,17 @@ __global__ void __launch_bounds__(256) k_camera(const ViewDev* __restrict__ view
 
 // Trace, shadow and shade one camera ray; returns the pixel value: RGB and
 // the hit's z-depth t (d . F) along the view axis F (0 on a miss).
+// code: the hit normal's code when want_code.
 // hint: the records of this pixel's previous primary hit and shadow occluder
 // (-1 none), tested first; updated to this ray's.
 template <bool COUNT>
 __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, const float* Fw, uint2* stack,
                                               int stride, const StackCfg& stk, bool& overflow, WorkCount& wc,
                                               uint32_t& n_shadow, uint32_t& code, int32_t& prim,
-                                              const uint8_t* walk_lut, int2& hint) {
+                                              const uint8_t* walk_lut, int2& hint, bool want_code) {
     const Hit h = traverse<false, COUNT>(S, r, stack, stride, stk, overflow, wc, walk_lut, hint.x);
     prefetch_record(S, hint.y);  // the previous occluder, ahead of the shadow walk
-    const ShadeInfo si = shade_primary(S, r, h);
+    const ShadeInfo si = shade_primary(S, r, h, want_code);
     float4 out = si.c_shadow;
     hint.x = h.rec;
     if (si.need_shadow) {
@@ -112,8 +113,12 @@ __device__ __forceinline__ void tiles_done(const ViewDev* v, int n, int lane) {
 // pass's outputs. At one sample per pixel with a camera that reads only the
 // pixel's own previous value (every mapping but the image-space one), this
 // computes exactly what one launch per pass computes.
+// CHAIN: 24 warps per SM (80 registers; what spills is the pixel's state
+// between passes, outside the walk). 20, 28 and 32 warps: 1.575, 1.574 and
+// 1.773 against 1.559 ms for a mid 1080p K = 6 frame, forest 1.810, 1.820 and
+// 1.983 against 1.785 ms.
 template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN>
-__global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 warps per SM, as the one-pass kernel
+__global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
     k_trace(SceneDev S0, const ViewDev* __restrict__ views, int n_views,
                                                  int64_t total_chunks, int chunk_tiles,
                                                  const float4* __restrict__ rays, unsigned* work, StackCfg stk,
@@ -163,6 +168,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                 const int x = tx * 8 + (lane & 7), y = ty * 4 + (lane >> 3);
                 if (x >= v.W || y >= v.H) continue;
                 const int64_t p = (int64_t)y * v.W + x;
+                const bool want_code = v.mapping == RCP_MAP_NORMAL;
                 if (MS) {
                     // jittered samples (§2): each reads I_{n-1} at its own position
                     const int ns = v.spp > 0 ? v.spp : 1;
@@ -182,7 +188,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                         uint32_t code;
                         int32_t prim;
                         const float4 o = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc,
-                                                            n_shadow, code, prim, s_lut, hint);
+                                                            n_shadow, code, prim, s_lut, hint, want_code);
                         ++n_primary;
                         acc.x = __fadd_rn(acc.x, o.x);
                         acc.y = __fadd_rn(acc.y, o.y);
@@ -229,7 +235,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                         const uint32_t before = n_shadow;
                         int32_t id;
                         float4 cur = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code,
-                                                        id, s_lut, hint);
+                                                        id, s_lut, hint, want_code);
                         ++n_primary;
                         if (v.mapping == RCP_MAP_NORMAL) cur.w = __uint_as_float(code);
                         const uint32_t shadow = n_shadow - before;
@@ -272,7 +278,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 640 / BLOCK : 0)  // CHAIN: 20 
                         r.tmax = b.w;
                     }
                     out = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code, prim,
-                                             s_lut, hint);
+                                             s_lut, hint, want_code);
                     ++n_primary;
                     if (v.mapping == RCP_MAP_NORMAL) out.w = __uint_as_float(code);
                 }

@@ -290,11 +290,15 @@ __device__ __forceinline__ void fill_walk_lut(uint8_t* lut) {
 // o * (1/d) up and the FMA down, far planes the reverse, so each computed
 // entry is <= and each exit >= the exact (p - o) * (1/d) of the rounded
 // reciprocal. The reciprocal's own relative error (<= 2^-24, different per
-// axis) is covered by scaling the far planes' reciprocal by RCP_FAR_SCALE =
-// 1 + 2^-21 away from zero. RCP_BOX_SLACK = 1 + 2^-17 widens the current
-// closest hit, so that boxes holding an equal-t hit (ties go to the lower
-// id) are still entered. The box test therefore never misses a primitive hit.
-#define RCP_FAR_SCALE 1.000000476837158203125f
+// axis) is covered by scaling the entry by RCP_ENTRY_SCALE = 1 - 2^-21 where
+// it is compared with the exit (entries are >= t_min >= 0): entry <= exit of a
+// box the ray meets then holds with a margin of 2^-21 against 2^-23. Near and
+// far planes share one reciprocal per axis; a second, magnified one for the
+// far planes gave the same margin for 3 more live values, 6 as broadcast
+// pairs. RCP_BOX_SLACK = 1 + 2^-17 widens the current closest hit, so that
+// boxes holding an equal-t hit (ties go to the lower id) are still entered.
+// The box test therefore never misses a primitive hit.
+#define RCP_ENTRY_SCALE 0.999999523162841796875f
 #define RCP_BOX_SLACK 1.0000076f
 
 // The traversal stack of one thread: `entries` groups in shared memory at
@@ -374,13 +378,9 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
     const uint32_t oct = (dx < 0.f ? 1u : 0u) | (dy < 0.f ? 2u : 0u) | (dz < 0.f ? 4u : 0u);
     const uint8_t* ord = walk_lut + (oct << 8);
     const uint32_t* leaf_lut = reinterpret_cast<const uint32_t*>(walk_lut + ORDER_LUT_BYTES);
-    // far-plane reciprocals, magnified away from zero
-    const float fdx = dx > 0.f ? __fmul_ru(idx, RCP_FAR_SCALE) : __fmul_rd(idx, RCP_FAR_SCALE);
-    const float fdy = dy > 0.f ? __fmul_ru(idy, RCP_FAR_SCALE) : __fmul_rd(idy, RCP_FAR_SCALE);
-    const float fdz = dz > 0.f ? __fmul_ru(idz, RCP_FAR_SCALE) : __fmul_rd(idz, RCP_FAR_SCALE);
     // -o * (1/d): rounded down for near planes, up for far planes
     const float nox = -__fmul_ru(r.ox, idx), noy = -__fmul_ru(r.oy, idy), noz = -__fmul_ru(r.oz, idz);
-    const float fox = -__fmul_rd(r.ox, fdx), foy = -__fmul_rd(r.oy, fdy), foz = -__fmul_rd(r.oz, fdz);
+    const float fox = -__fmul_rd(r.ox, idx), foy = -__fmul_rd(r.oy, idy), foz = -__fmul_rd(r.oz, idz);
     // node rows of the near and far planes per axis (lo rows first, then hi)
     const int rxn = (oct & 1u) ? 2 : 0, rxf = 2 - rxn;
     const int ryn = (oct & 2u) ? 6 : 4, ryf = 10 - ryn;
@@ -429,9 +429,9 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
             const uint4 hd = __ldg(reinterpret_cast<const uint4*>(np + 12));
             if (COUNT) wc.nodes++;
             // Missed slots, bit s for slot s. A slot is missed when its exit is
-            // before its entry, the sign of exit - entry (exact in sign: the
-            // difference of two floats never rounds across zero, and neither
-            // is NaN; inf - inf is a positive NaN, a hit). Shifting the sign
+            // before its entry, the sign of exit - entry (one rounding, which
+            // never crosses zero, and neither is NaN; inf - inf is a positive
+            // NaN, a hit). Shifting the sign
             // bits in from slot 7 down to slot 0 takes one funnel shift a slot
             // and the subtraction two slots at once, where a comparison and a
             // select took two instructions a slot on the ALU pipe.
@@ -454,22 +454,24 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
                     float t0x[2], t1x[2], t0y[2], t1y[2], t0z[2], t1z[2], tn[2], tf[2], d[2];
                     f2_unpack(f2_fma_rd(f2_pack(nxs[k], nxs[k + 1]), f2_pack(idx, idx), f2_pack(nox, nox)), t0x[0],
                               t0x[1]);
-                    f2_unpack(f2_fma_ru(f2_pack(fxs[k], fxs[k + 1]), f2_pack(fdx, fdx), f2_pack(fox, fox)), t1x[0],
+                    f2_unpack(f2_fma_ru(f2_pack(fxs[k], fxs[k + 1]), f2_pack(idx, idx), f2_pack(fox, fox)), t1x[0],
                               t1x[1]);
                     f2_unpack(f2_fma_rd(f2_pack(nys[k], nys[k + 1]), f2_pack(idy, idy), f2_pack(noy, noy)), t0y[0],
                               t0y[1]);
-                    f2_unpack(f2_fma_ru(f2_pack(fys[k], fys[k + 1]), f2_pack(fdy, fdy), f2_pack(foy, foy)), t1y[0],
+                    f2_unpack(f2_fma_ru(f2_pack(fys[k], fys[k + 1]), f2_pack(idy, idy), f2_pack(foy, foy)), t1y[0],
                               t1y[1]);
                     f2_unpack(f2_fma_rd(f2_pack(nzs[k], nzs[k + 1]), f2_pack(idz, idz), f2_pack(noz, noz)), t0z[0],
                               t0z[1]);
-                    f2_unpack(f2_fma_ru(f2_pack(fzs[k], fzs[k + 1]), f2_pack(fdz, fdz), f2_pack(foz, foz)), t1z[0],
+                    f2_unpack(f2_fma_ru(f2_pack(fzs[k], fzs[k + 1]), f2_pack(idz, idz), f2_pack(foz, foz)), t1z[0],
                               t1z[1]);
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
                         tn[j] = fmax3(t0x[j], t0y[j], fmaxf(t0z[j], r.tmin));
                         tf[j] = fmin3(t1x[j], t1y[j], fminf(t1z[j], tfar_lim));
                     }
-                    f2_unpack(f2_fma_rn(f2_pack(tn[0], tn[1]), f2_pack(-1.f, -1.f), f2_pack(tf[0], tf[1])), d[0], d[1]);
+                    f2_unpack(f2_fma_rn(f2_pack(tn[0], tn[1]), f2_pack(-RCP_ENTRY_SCALE, -RCP_ENTRY_SCALE),
+                                        f2_pack(tf[0], tf[1])),
+                              d[0], d[1]);
                     missed = __funnelshift_l(__float_as_uint(d[1]), missed, 1);
                     missed = __funnelshift_l(__float_as_uint(d[0]), missed, 1);
                 }
@@ -541,7 +543,7 @@ struct ShadeInfo {
     float4 c_lit;     // colour if the light is visible
     RayF shadow;      // the shadow ray (valid when need_shadow)
     bool need_shadow;
-    uint32_t normal_code;  // octahedral code of the facing hit normal, 0 on a miss
+    uint32_t normal_code;  // octahedral code of the facing hit normal (when wanted), 0 on a miss
 };
 
 __device__ __forceinline__ float clamp01(float x) { return fminf(fmaxf(x, 0.f), 1.f); }
@@ -549,7 +551,9 @@ __device__ __forceinline__ float clamp01(float x) { return fminf(fmaxf(x, 0.f), 
 // Shading of §2 stage 2 (reading: the paper gives no shading model):
 // hit -> albedo * (a + (1 - a) V max(0, N.L)), N facing the ray; miss -> sky
 // (1 - s)(1,1,1) + s (0.5, 0.7, 1), s = (d_y + 1)/2; clamped to [0, 1].
-__device__ __forceinline__ ShadeInfo shade_primary(const SceneDev& S, const RayF& r, const Hit& h) {
+// want_code: also the normal's code (the normal mapping reads it; its two
+// divisions are left out otherwise).
+__device__ __forceinline__ ShadeInfo shade_primary(const SceneDev& S, const RayF& r, const Hit& h, bool want_code) {
     ShadeInfo si;
     si.need_shadow = false;
     si.normal_code = 0u;
@@ -599,7 +603,7 @@ __device__ __forceinline__ ShadeInfo shade_primary(const SceneDev& S, const RayF
         ly = S.light.y;
         lz = S.light.z;
     }
-    si.normal_code = normal_encode(nx, ny, nz);
+    if (want_code) si.normal_code = normal_encode(nx, ny, nz);
     const float ndl = fdot(nx, ny, nz, lx, ly, lz);
     const float a = S.light.ambient;
     const float4 alb = __ldg(S.albedo + h.id);
