@@ -122,7 +122,7 @@ typedef struct rcp_scene rcp_scene;
 /* Scene statistics (sizes, BVH shape, build time). */
 typedef struct {
     int64_t n_tris, n_spheres;
-    int64_t n_nodes;      /* 8-wide BVH nodes (208 bytes each) */
+    int64_t n_nodes;      /* 8-wide BVH nodes (304 bytes each) */
     int32_t depth;        /* levels of the 8-wide BVH */
     int32_t max_leaf;     /* largest leaf (primitives) */
     int64_t device_bytes; /* device memory held by the scene */

@@ -431,8 +431,7 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     const SceneDev S = sc.dev();
     RCP_CUDA(record(ctx.pass_ev[0]));
     if (ctx.chained) {  // one descriptor per view, all K passes
-        rcp_status r = launch_chain(S, cfg, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays,
-                                    counters, st);
+        rcp_status r = launch_chain(S, cfg, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays, st);
         if (r != RCP_OK) return r;
         RCP_CUDA(record(ctx.pass_ev[1]));
         ctx.launches = 1;

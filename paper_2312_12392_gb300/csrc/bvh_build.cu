@@ -843,20 +843,21 @@ __device__ __forceinline__ void ref_box(const BinTree& bt, int ref, float3& lo, 
 // union of the children.
 __device__ void write_child_boxes(WNode& nd, const float3* clo, const float3* chi, const int* slot_of, int m,
                                   float3& ulo, float3& uhi) {
-    for (int s = 0; s < 8; ++s) {
-        nd.lo_x[s] = nd.lo_y[s] = nd.lo_z[s] = INFINITY;
-        nd.hi_x[s] = nd.hi_y[s] = nd.hi_z[s] = -INFINITY;
-    }
+    for (int a = 0; a < 3; ++a)
+        for (int s = 0; s < 8; ++s) {
+            nd.box[a][0][s] = nd.box[a][2][s] = INFINITY;
+            nd.box[a][1][s] = -INFINITY;
+        }
     ulo = make_float3(INFINITY, INFINITY, INFINITY);
     uhi = make_float3(-INFINITY, -INFINITY, -INFINITY);
     for (int c = 0; c < m; ++c) {
         const int sl = slot_of[c];
-        nd.lo_x[sl] = clo[c].x;
-        nd.lo_y[sl] = clo[c].y;
-        nd.lo_z[sl] = clo[c].z;
-        nd.hi_x[sl] = chi[c].x;
-        nd.hi_y[sl] = chi[c].y;
-        nd.hi_z[sl] = chi[c].z;
+        nd.box[0][0][sl] = nd.box[0][2][sl] = clo[c].x;
+        nd.box[1][0][sl] = nd.box[1][2][sl] = clo[c].y;
+        nd.box[2][0][sl] = nd.box[2][2][sl] = clo[c].z;
+        nd.box[0][1][sl] = chi[c].x;
+        nd.box[1][1][sl] = chi[c].y;
+        nd.box[2][1][sl] = chi[c].z;
         ulo = make_float3(fminf(ulo.x, clo[c].x), fminf(ulo.y, clo[c].y), fminf(ulo.z, clo[c].z));
         uhi = make_float3(fmaxf(uhi.x, chi[c].x), fmaxf(uhi.y, chi[c].y), fmaxf(uhi.z, chi[c].z));
     }
@@ -1123,7 +1124,7 @@ __global__ void k_refit_records(float4* __restrict__ prims, int64_t n, Parts par
 // Recompute the child boxes of the nodes in [begin, end) (one level, deepest
 // first). Eight lanes per node, lane s for slot s: the slot's box is the union
 // of its leaf records' boxes (rbox) or its internal child's box, and each of
-// the node's six box rows (8 floats, one 32-byte sector) is written by its
+// the node's nine box rows (8 floats, one 32-byte sector) is written by its
 // eight lanes together. Empty slots get the empty box (+inf, -inf) that the
 // collapse gave them. Only the node's header is read. The node's union box
 // (nbox) is reduced over its eight lanes, which share a warp.
@@ -1139,8 +1140,8 @@ __global__ void __launch_bounds__(REFIT_BLOCK) k_refit_wide(WNode* __restrict__ 
     const bool live = w < end;
     float3 lo = make_float3(INFINITY, INFINITY, INFINITY), hi = make_float3(-INFINITY, -INFINITY, -INFINITY);
     if (live) {
-        float* nf = reinterpret_cast<float*>(nodes + w);
-        const uint4 hd = *reinterpret_cast<const uint4*>(nf + 48);
+        WNode& nd = nodes[w];
+        const uint4 hd = *reinterpret_cast<const uint4*>(&nd.child_base);
         const uint32_t leaf_bits = hd.z >> 8;
         if (hd.z & (1u << s)) {
             const int64_t c = hd.x + __popc(hd.z & bits_below(s));
@@ -1156,12 +1157,12 @@ __global__ void __launch_bounds__(REFIT_BLOCK) k_refit_wide(WNode* __restrict__ 
                 hi = make_float3(fmaxf(hi.x, m.y), fmaxf(hi.y, z.x), fmaxf(hi.z, z.y));
             }
         }
-        nf[s] = lo.x;
-        nf[8 + s] = hi.x;
-        nf[16 + s] = lo.y;
-        nf[24 + s] = hi.y;
-        nf[32 + s] = lo.z;
-        nf[40 + s] = hi.z;
+        nd.box[0][0][s] = nd.box[0][2][s] = lo.x;
+        nd.box[0][1][s] = hi.x;
+        nd.box[1][0][s] = nd.box[1][2][s] = lo.y;
+        nd.box[1][1][s] = hi.y;
+        nd.box[2][0][s] = nd.box[2][2][s] = lo.z;
+        nd.box[2][1][s] = hi.z;
     }
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
@@ -1181,12 +1182,10 @@ __global__ void __launch_bounds__(REFIT_BLOCK) k_refit_wide(WNode* __restrict__ 
 // ---------------------------------------------------------------- validation
 
 __device__ __forceinline__ void slot_box(const WNode& nd, int s, double lo[3], double hi[3]) {
-    lo[0] = nd.lo_x[s];
-    lo[1] = nd.lo_y[s];
-    lo[2] = nd.lo_z[s];
-    hi[0] = nd.hi_x[s];
-    hi[1] = nd.hi_y[s];
-    hi[2] = nd.hi_z[s];
+    for (int a = 0; a < 3; ++a) {
+        lo[a] = nd.box[a][0][s];
+        hi[a] = nd.box[a][1][s];
+    }
 }
 
 // n_records leaf records over n_prims primitives; rec_box (nullable): each
@@ -1209,6 +1208,8 @@ __global__ void k_validate(const WNode* __restrict__ nodes, int64_t n_nodes, con
         if (!internal && !lb) continue;  // empty
         double lo[3], hi[3];
         slot_box(nd, s, lo, hi);
+        for (int a = 0; a < 3; ++a)
+            if (nd.box[a][2][s] != nd.box[a][0][s]) atomicAdd(&errors[2], 1);
         if (internal) {
             if (lb) atomicAdd(&errors[0], 1);  // a slot is a child or a leaf
             const int64_t c = (int64_t)nd.child_base + __popc(imask & bits_below(s));

@@ -1,7 +1,7 @@
 // rcp_internal.cuh -- shared device types of the renderer (not part of the ABI).
 //
 // Layout in device memory (all 16-byte aligned):
-//  * WNode: one 8-wide BVH node with float child boxes, 208 bytes = 13 x float4.
+//  * WNode: one 8-wide BVH node with float child boxes, 304 bytes = 19 x float4.
 //  * Prim records: 3 x float4 = 48 bytes per primitive, in leaf order:
 //      triangle  w0 = (v0.xyz, e1.x)  w1 = (e1.yz, e2.xy)  w2 = (e2.z, id, 0, 0)
 //      sphere    w0 = (centre, r)     w1 = 0               w2 = (0, id | SPHERE_BIT, 0, 0)
@@ -22,23 +22,27 @@ namespace rcp {
 constexpr uint32_t SPHERE_BIT = 0x80000000u;
 constexpr int MAX_STACK = 64;  // traversal stack entries (>= BVH depth)
 
-// One 8-wide node, 13 rows of 16 bytes. Child slot s (0..7) has the float
-// box lo_a[s]..hi_a[s] per axis a (an empty slot: lo = +inf, hi = -inf).
+// One 8-wide node, 19 rows of 16 bytes. Child slot s (0..7) has the float
+// box box[a][0][s]..box[a][1][s] per axis a (an empty slot: lo = +inf, hi =
+// -inf); box[a][2] repeats the low planes behind the high ones, so that a ray
+// finds its near planes at box[a][n] and its far planes right behind them, n =
+// 0 or 1 by the sign of its direction: one address per axis instead of two
+// (rows 6a + 2n .. 6a + 2n + 3). A ray reads 13 of the rows, whichever its
+// octant: the copies cost memory (304 bytes against 208), not traffic.
 // slots: bit s set = slot s holds an internal child, node child_base + the
 // number of internal slots below s; bits 8 + 3 s .. 10 + 3 s hold a leaf
 // slot's record count (1..3) in unary, and the records of a node's leaves lie
 // from prim_base on in slot order, so the record of leaf bit j is prim_base +
-// the number of leaf bits below j. Rows 0-1 lo_x, 2-3 hi_x, 4-5 lo_y, 6-7
-// hi_y, 8-9 lo_z, 10-11 hi_z, 12 the header.
+// the number of leaf bits below j. The header is row 18.
 struct __align__(16) WNode {
-    float lo_x[8], hi_x[8], lo_y[8], hi_y[8], lo_z[8], hi_z[8];
+    float box[3][3][8];
     uint32_t child_base;
     uint32_t prim_base;
     uint32_t slots;  // internal mask | leaf record bits << 8
     uint32_t pad;
 };
-constexpr int NODE_ROWS = 13;
-static_assert(sizeof(WNode) == 16 * NODE_ROWS, "WNode must be 13 rows of 16 bytes");
+constexpr int NODE_ROWS = 19;
+static_assert(sizeof(WNode) == 16 * NODE_ROWS, "WNode must be 19 rows of 16 bytes");
 
 // Bits below bit b of a mask's slot or leaf bit b (b <= 24).
 __host__ __device__ __forceinline__ uint32_t bits_below(uint32_t b) { return (1u << b) - 1u; }

@@ -119,8 +119,7 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
 // camera (cfg.fused is not read), and a mapping that reads only the pixel's
 // own previous value; cfg.multi: the views name their scenes.
 rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
-                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays,
-                        unsigned long long* d_counters, cudaStream_t st);
+                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays, cudaStream_t st);
 rcp_status launch_debug_trace(const SceneDev& S, int64_t n, const float* orig_tmin, const float* dir_tmax, int any,
                               int brute, float* t_out, int32_t* prim_out, int stack_entries, int* d_status,
                               cudaStream_t st);

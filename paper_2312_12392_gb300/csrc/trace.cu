@@ -55,12 +55,12 @@ __global__ void __launch_bounds__(256) k_camera(const ViewDev* __restrict__ view
 // code: the hit normal's code when want_code.
 // hint: the records of this pixel's previous primary hit and shadow occluder
 // (-1 none), tested first; updated to this ray's.
-template <bool COUNT>
+template <bool COUNT, bool SPILL>
 __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, const float* Fw, uint2* stack,
                                               int stride, const StackCfg& stk, bool& overflow, WorkCount& wc,
                                               uint32_t& n_shadow, uint32_t& code, int32_t& prim,
                                               const uint8_t* walk_lut, int2& hint, bool want_code) {
-    const Hit h = traverse<false, COUNT>(S, r, stack, stride, stk, overflow, wc, walk_lut, hint.x);
+    const Hit h = traverse<false, COUNT, SPILL>(S, r, stack, stride, stk, overflow, wc, walk_lut, hint.x);
     prefetch_record(S, hint.y);  // the previous occluder, ahead of the shadow walk
     const ShadeInfo si = shade_primary(S, r, h, want_code);
     float4 out = si.c_shadow;
@@ -68,7 +68,7 @@ __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, 
     if (si.need_shadow) {
         ++n_shadow;
         const Hit hs =
-            traverse<true, COUNT>(S, si.shadow, stack, stride, stk, overflow, wc, walk_lut, hint.y);
+            traverse<true, COUNT, SPILL>(S, si.shadow, stack, stride, stk, overflow, wc, walk_lut, hint.y);
         if (hs.rec < 0) out = si.c_lit;
         hint.y = hs.rec;
     }
@@ -117,7 +117,7 @@ __device__ __forceinline__ void tiles_done(const ViewDev* v, int n, int lane) {
 // between passes, outside the walk). 20, 28 and 32 warps: 1.575, 1.574 and
 // 1.773 against 1.559 ms for a mid 1080p K = 6 frame, forest 1.810, 1.820 and
 // 1.983 against 1.785 ms.
-template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN>
+template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
 __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
     k_trace(SceneDev S0, const ViewDev* __restrict__ views, int n_views,
                                                  int64_t total_chunks, int chunk_tiles,
@@ -168,7 +168,6 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                 const int x = tx * 8 + (lane & 7), y = ty * 4 + (lane >> 3);
                 if (x >= v.W || y >= v.H) continue;
                 const int64_t p = (int64_t)y * v.W + x;
-                const bool want_code = v.mapping == RCP_MAP_NORMAL;
                 if (MS) {
                     // jittered samples (§2): each reads I_{n-1} at its own position
                     const int ns = v.spp > 0 ? v.spp : 1;
@@ -187,8 +186,11 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                         const RayF r = camera_ray(v, px, py, c, S.tmin);
                         uint32_t code;
                         int32_t prim;
-                        const float4 o = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc,
-                                                            n_shadow, code, prim, s_lut, hint, want_code);
+                        // the mapping is compared here: kept live across the walk it takes the kernel
+                        // from 96 to 128 registers (4 samples at 720p 3.17 against 3.44 ms)
+                        const float4 o = trace_shade<COUNT, SPILL>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc,
+                                                            n_shadow, code, prim, s_lut, hint,
+                                                            v.mapping == RCP_MAP_NORMAL);
                         ++n_primary;
                         acc.x = __fadd_rn(acc.x, o.x);
                         acc.y = __fadd_rn(acc.y, o.y);
@@ -220,6 +222,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                 int2 hint = v.hint && stk.hints ? v.hint[p] : make_int2(-1, -1);
                 if (!(stk.hints & 1)) hint.x = -1;
                 if (!(stk.hints & 2)) hint.y = -1;
+                const bool want_code = v.mapping == RCP_MAP_NORMAL;
                 // CHAIN: passes 1..K, the camera reading this pixel's own previous value
                 float4 out = FUSED && v.in ? __ldg(v.in + p) : make_float4(0.5f, 0.5f, 0.5f, 0.f);
                 uint32_t code;
@@ -234,7 +237,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                         const RayF r = camera_ray(v, (float)x + 0.5f, (float)y + 0.5f, out, S.tmin);
                         const uint32_t before = n_shadow;
                         int32_t id;
-                        float4 cur = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code,
+                        float4 cur = trace_shade<COUNT, SPILL>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code,
                                                         id, s_lut, hint, want_code);
                         ++n_primary;
                         if (v.mapping == RCP_MAP_NORMAL) cur.w = __uint_as_float(code);
@@ -277,7 +280,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                         r.dz = b.z;
                         r.tmax = b.w;
                     }
-                    out = trace_shade<COUNT>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code, prim,
+                    out = trace_shade<COUNT, SPILL>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc, n_shadow, code, prim,
                                              s_lut, hint, want_code);
                     ++n_primary;
                     if (v.mapping == RCP_MAP_NORMAL) out.w = __uint_as_float(code);
@@ -352,8 +355,8 @@ __global__ void __launch_bounds__(BLOCK) k_debug_trace(SceneDev S, int64_t n, co
         RayF r{a.x, a.y, a.z, b.x, b.y, b.z, a.w, b.w};
         Hit h;
         if (brute) h = any ? traverse_brute<true>(S, r) : traverse_brute<false>(S, r);
-        else h = any ? traverse<true, false>(S, r, stack, BLOCK, stk, overflow, wc, s_lut)
-                     : traverse<false, false>(S, r, stack, BLOCK, stk, overflow, wc, s_lut);
+        else h = any ? traverse<true, false, true>(S, r, stack, BLOCK, stk, overflow, wc, s_lut)
+                     : traverse<false, false, true>(S, r, stack, BLOCK, stk, overflow, wc, s_lut);
         if (any) {
             prim_out[i] = h.rec >= 0 ? 1 : 0;
             t_out[i] = 0.f;
@@ -455,11 +458,11 @@ int sm_count() {
     return sms;
 }
 
-template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN>
+template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
 rcp_status launch_trace_t(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                           int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
                           unsigned long long* d_counters, cudaStream_t st) {
-    auto kern = k_trace<BLOCK, FUSED, COUNT, MS, MULTI, CHAIN>;
+    auto kern = k_trace<BLOCK, FUSED, COUNT, MS, MULTI, CHAIN, SPILL>;
     const size_t smem = sizeof(uint2) * (size_t)cfg.stack * BLOCK;
     if (smem > 48 * 1024) RCP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int per_sm = cfg.blocks_per_sm;
@@ -481,21 +484,43 @@ rcp_status launch_trace_t(const SceneDev& S, const LaunchCfg& cfg, const ViewDev
     return RCP_OK;
 }
 
-template <bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN = false>
-rcp_status launch_trace_b(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
+// SPILL: the walk checks its shared stack's end. Launches whose stack holds one
+// group per level of their trees (the default, and every server launch) take
+// the walk without the checks (together with the adjacent near and far rows of
+// a node: a mid 1080p K = 6 frame 1.548 -> 1.469 ms, of which 3 % are the
+// checks; forest 1.774 -> 1.699 ms). The counting and separate-camera kernels,
+// which no frame is timed on, always check.
+template <bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
+rcp_status launch_trace_s(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                           int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
                           unsigned long long* d_counters, cudaStream_t st) {
     switch (cfg.block) {
         case 64:
-            return launch_trace_t<64, FUSED, COUNT, MS, MULTI, CHAIN>(S, cfg, d_views, n_views, total_chunks, rays,
+            return launch_trace_t<64, FUSED, COUNT, MS, MULTI, CHAIN, SPILL>(S, cfg, d_views, n_views, total_chunks, rays,
                                                                       d_work, d_rays, d_counters, st);
         case 256:
-            return launch_trace_t<256, FUSED, COUNT, MS, MULTI, CHAIN>(S, cfg, d_views, n_views, total_chunks, rays,
+            return launch_trace_t<256, FUSED, COUNT, MS, MULTI, CHAIN, SPILL>(S, cfg, d_views, n_views, total_chunks, rays,
                                                                        d_work, d_rays, d_counters, st);
         default:
-            return launch_trace_t<128, FUSED, COUNT, MS, MULTI, CHAIN>(S, cfg, d_views, n_views, total_chunks, rays,
+            return launch_trace_t<128, FUSED, COUNT, MS, MULTI, CHAIN, SPILL>(S, cfg, d_views, n_views, total_chunks, rays,
                                                                        d_work, d_rays, d_counters, st);
     }
+}
+
+template <bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN = false>
+rcp_status launch_trace_b(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
+                          int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
+                          unsigned long long* d_counters, cudaStream_t st) {
+    if (MULTI || (FUSED && !COUNT && cfg.spill_entries == 0)) {
+        if (MULTI && cfg.spill_entries != 0) {
+            set_error("launch over several scenes: the shared stack must hold one group per tree level");
+            return RCP_ERR_STATE;
+        }
+        return launch_trace_s<FUSED, COUNT, MS, MULTI, CHAIN, COUNT || !FUSED>(
+            S, cfg, d_views, n_views, total_chunks, rays, d_work, d_rays, d_counters, st);
+    }
+    return launch_trace_s<FUSED, COUNT, MS, false, CHAIN, true>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                d_rays, d_counters, st);
 }
 
 }  // namespace
@@ -534,19 +559,16 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
 }
 
 rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
-                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays,
-                        unsigned long long* d_counters, cudaStream_t st) {
-    if (cfg.ms) {
-        set_error("launch_chain: a chained launch is single-sample");
+                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays, cudaStream_t st) {
+    if (cfg.ms || cfg.count) {
+        set_error("launch_chain: a chained launch is single-sample and keeps no work counters");
         return RCP_ERR_STATE;
     }
     if (cfg.multi)  // views of several scenes: no counters
         return launch_trace_b<true, false, false, true, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
                                                               d_rays, nullptr, st);
-    return cfg.count ? launch_trace_b<true, true, false, false, true>(S, cfg, d_views, n_views, total_chunks,
-                                                                      nullptr, d_work, d_rays, d_counters, st)
-                     : launch_trace_b<true, false, false, false, true>(S, cfg, d_views, n_views, total_chunks,
-                                                                       nullptr, d_work, d_rays, d_counters, st);
+    return launch_trace_b<true, false, false, false, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
+                                                           d_rays, nullptr, st);
 }
 
 rcp_status launch_debug_trace(const SceneDev& S, int64_t n, const float* orig_tmin, const float* dir_tmax, int any,

@@ -1,7 +1,7 @@
 // trace.cuh -- device functions of one recursive-camera-painting pass.
 //
 //  * camera_ray: the per-pixel camera of §2 (Eq. 2-4) and §3 (Eq. 5);
-//  * traverse<ANY>: closest-hit (ANY = false) or any-hit (ANY = true) walk of
+//  * traverse<ANY, ...>: closest-hit (ANY = false) or any-hit (ANY = true) walk of
 //    the 8-wide BVH (float child boxes) with a per-thread stack and the
 //    block's traversal-order table in shared memory;
 //  * hit_triangle / hit_sphere: Moller-Trumbore and the analytic sphere test;
@@ -308,7 +308,9 @@ __device__ __forceinline__ void fill_walk_lut(uint8_t* lut) {
 // register). A stack as deep as the tree (one group per level) never
 // reaches the spill region; a shorter shared stack trades the spill traffic of
 // deep walks for less shared memory per block. Pushing past both sets
-// `overflow` and drops the group, which ends the walk early.
+// `overflow` and drops the group, which ends the walk early. The walk of a
+// stack that holds one group per level (SPILL = false) has neither branch: the
+// groups on the stack lie on one path from the root, at most depth - 1 of them.
 struct StackCfg {
     int entries;        // shared-memory entries per thread
     int spill_entries;  // global-memory entries per thread above those
@@ -336,7 +338,7 @@ __device__ __forceinline__ uint2* spill_slot(const StackCfg& sc, int i) {
 // an any-hit walk at once. The result does not depend on it: the walk still
 // keeps the least (t, id) over every record in a box the ray enters up to
 // t (1 + 2^-17), and an any-hit answer is a yes/no.
-template <bool ANY, bool COUNT>
+template <bool ANY, bool COUNT, bool SPILL>
 __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2* stack, int stride,
                                         const StackCfg& stk, bool& overflow, WorkCount& wc, const uint8_t* walk_lut,
                                         int32_t first_rec = -1) {
@@ -381,10 +383,8 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
     // -o * (1/d): rounded down for near planes, up for far planes
     const float nox = -__fmul_ru(r.ox, idx), noy = -__fmul_ru(r.oy, idy), noz = -__fmul_ru(r.oz, idz);
     const float fox = -__fmul_rd(r.ox, idx), foy = -__fmul_rd(r.oy, idy), foz = -__fmul_rd(r.oz, idz);
-    // node rows of the near and far planes per axis (lo rows first, then hi)
-    const int rxn = (oct & 1u) ? 2 : 0, rxf = 2 - rxn;
-    const int ryn = (oct & 2u) ? 6 : 4, ryf = 10 - ryn;
-    const int rzn = (oct & 4u) ? 10 : 8, rzf = 18 - rzn;
+    // node rows of the near planes per axis; the far planes' rows follow them
+    const int rx = (oct & 1u) ? 2 : 0, ry = (oct & 2u) ? 8 : 6, rz = (oct & 4u) ? 14 : 12;
     float tfar_lim = __fmul_rn(h.t, RCP_BOX_SLACK);  // +inf without a first hit
 
     // node group: x = first child node index, y = imask | (slots still to visit) << 8;
@@ -408,14 +408,14 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
         if (group.y <= 0xffu) {
             if (sp == 0) break;
             --sp;
-            group = sp < stk.entries ? stack[sp * stride] : *spill_slot(stk, sp);
+            group = !SPILL || sp < stk.entries ? stack[sp * stride] : *spill_slot(stk, sp);
         }
         {
             const uint32_t slot = ord[group.y >> 8];
             group.y &= ~(1u << (slot + 8));
             const uint32_t node = group.x + __popc(group.y & bits_below(slot));
             if (group.y > 0xffu) {
-                if (sp < stk.entries) {
+                if (!SPILL || sp < stk.entries) {
                     stack[sp * stride] = group;
                     ++sp;
                 } else if (sp < stk.entries + stk.spill_entries) {
@@ -426,7 +426,8 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
                 }
             }
             const float4* np = S.nodes + NODE_ROWS * (size_t)node;
-            const uint4 hd = __ldg(reinterpret_cast<const uint4*>(np + 12));
+            const uint4 hd = __ldg(reinterpret_cast<const uint4*>(np + NODE_ROWS - 1));
+            const float4 *px = np + rx, *py = np + ry, *pz = np + rz;
             if (COUNT) wc.nodes++;
             // Missed slots, bit s for slot s. A slot is missed when its exit is
             // before its entry, the sign of exit - entry (one rounding, which
@@ -441,9 +442,9 @@ __device__ __forceinline__ Hit traverse(const SceneDev& S, const RayF& r, uint2*
             // form that tests one half at a time)
 #pragma unroll
             for (int half = 1; half >= 0; --half) {
-                const float4 nx = __ldg(np + rxn + half), fx = __ldg(np + rxf + half);
-                const float4 ny = __ldg(np + ryn + half), fy = __ldg(np + ryf + half);
-                const float4 nz = __ldg(np + rzn + half), fz = __ldg(np + rzf + half);
+                const float4 nx = __ldg(px + half), fx = __ldg(px + 2 + half);
+                const float4 ny = __ldg(py + half), fy = __ldg(py + 2 + half);
+                const float4 nz = __ldg(pz + half), fz = __ldg(pz + 2 + half);
                 // two slots per instruction: the planes of slots (0,1) and (2,3)
                 // of this half against the ray's terms, each broadcast to a pair
                 const float nxs[4] = {nx.x, nx.y, nx.z, nx.w}, fxs[4] = {fx.x, fx.y, fx.z, fx.w};
