@@ -261,8 +261,9 @@ rcp_status rcp_render_batch_device(const rcp_scene* scene, int n_views, const rc
  * previous pass (a closer far limit from the start), bit 1 = its shadow walk
  * first tests its previous occluder; chain_passes: 1 = one launch runs all K
  * passes, each warp carrying the pixels of its tile from pass to pass in
- * registers (renders of K >= 2 at one sample per pixel with the fused camera
- * and any mapping but RCP_MAP_IMAGE; others run one launch per pass). A new
+ * registers (renders at one sample per pixel; jittered samples run one launch
+ * per pass), and an RCP_MAP_IMAGE render's gathers in one launch after its
+ * traced pass. A new
  * scene starts at {128, 0, 32, 1, 0, 3, 1}. No choice changes any result. */
 typedef struct {
     int32_t block;
@@ -311,14 +312,16 @@ rcp_status rcp_count_pass(const rcp_scene* scene, const rcp_camera* cam, int wid
 /* Device time (ms) of each launch of the scene's most recent render, from CUDA
  * events recorded on the render's stream between the launches (inside the
  * captured graph): one per pass, or one for all K passes when they ran
- * chained. Read after the render has completed. */
+ * chained (an RCP_MAP_IMAGE render of K >= 2: the traced pass, then all
+ * gathers). Read after the render has completed. */
 rcp_status rcp_last_pass_times(const rcp_scene* scene, float* ms, int max_passes, int* n_passes);
 
 /* Bytes that one rcp_render call of K passes over n_views views copies from
  * host to device: the views' per-pass descriptors (camera terms, image
  * pointers), uploaded once per call. The library's own bookkeeping, not part of
  * the method. A render whose passes run chained uploads one descriptor per
- * view: rcp_render_h2d_bytes(n_views, 1). Returns -1 when K or n_views is out
+ * view, rcp_render_h2d_bytes(n_views, 1), or two (RCP_MAP_IMAGE, K >= 2).
+ * Returns -1 when K or n_views is out
  * of range. */
 int64_t rcp_render_h2d_bytes(int n_views, int K);
 

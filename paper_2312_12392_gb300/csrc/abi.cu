@@ -430,11 +430,21 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     RCP_CUDA(cudaMemsetAsync(ctx.d_rays, 0, sizeof(unsigned long long) * 2, st));
     const SceneDev S = sc.dev();
     RCP_CUDA(record(ctx.pass_ev[0]));
-    if (ctx.chained) {  // one descriptor per view, all K passes
-        rcp_status r = launch_chain(S, cfg, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays, st);
+    if (ctx.chained) {  // one descriptor per view, all K passes (image mode: pass 1, then the gathers' descriptors)
+        rcp_status r = ctx.image_mode
+                           ? launch_pass(S, cfg, ctx.d_views, ctx.n_views, ctx.total_pix, ctx.total_chunks, nullptr,
+                                         ctx.d_work, ctx.d_rays, nullptr, st)
+                           : launch_chain(S, cfg, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays,
+                                          st);
         if (r != RCP_OK) return r;
         RCP_CUDA(record(ctx.pass_ev[1]));
         ctx.launches = 1;
+        if (ctx.image_mode) {
+            r = launch_imagespace_chain(ctx.d_views + ctx.n_views, ctx.n_views, ctx.total_chunks, st);
+            if (r != RCP_OK) return r;
+            RCP_CUDA(record(ctx.pass_ev[2]));
+            ctx.launches = 2;
+        }
         return RCP_OK;
     }
     ctx.launches = ctx.K;
@@ -452,7 +462,7 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
 // Run the K passes through the context's CUDA graph (captured on first use or
 // when the launch configuration changes).
 rcp_status run_graph(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cudaStream_t st) {
-    const std::string key = cfg_key(cfg) + (ctx.image_mode ? "/image" : (ctx.chained ? "/chain" : "/trace"));
+    const std::string key = cfg_key(cfg) + (ctx.image_mode ? "/image" : "/trace") + (ctx.chained ? "/chain" : "");
     if (!ctx.graph || ctx.graph_key != key) {
         if (ctx.graph) {
             cudaGraphExecDestroy(ctx.graph);
@@ -480,14 +490,20 @@ rcp_status run_graph(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cuda
 
 // Stage the view descriptors of one render (n_views views, K passes): one per
 // view and pass, or, when the passes run chained (chain: the tuning asks for
-// it and the render allows it), one per view that runs all K passes.
+// it and the render allows it), one per view that runs all K passes (an
+// image-space render: one per view that traces pass 1, then one per view that
+// gathers passes 2..K).
 rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const float4* const* ins,
                        float4* const* outs, int32_t* const* prims, float* const* rgbs, cudaStream_t st,
                        bool chain = false) {
     RCP_CUDA(cudaEventSynchronize(ctx.staged));  // previous copy out of the staging buffer is done
     const int K = ctx.K, nv = ctx.n_views;
     ctx.image_mode = base[0].mapping == RCP_MAP_IMAGE && K > 1;
-    ctx.chained = chain && base[0].mapping != RCP_MAP_IMAGE && base[0].spp == 0;
+    // a single traced pass takes the one-pass kernel, which keeps no state
+    // between passes (90 registers, nothing spilled in the walk): mid 1080p
+    // K = 1 0.335 against 0.316 ms chained
+    ctx.chained = chain && base[0].spp == 0 && K > 1;
+    if (ctx.image_mode && !ctx.base_img) RCP_CUDA(cudaMalloc((void**)&ctx.base_img, sizeof(float4) * ctx.total_pix));
     if (ctx.chained) {
         for (int i = 0; i < nv; ++i) {
             ViewDev v = base[i];
@@ -498,13 +514,23 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
             v.prim = prims ? prims[i] : nullptr;
             v.rgb = rgbs ? rgbs[i] : nullptr;
             v.passes = K;
+            if (ctx.image_mode) {
+                ViewDev& w = ctx.h_views[nv + i];
+                w = v;
+                w.base = ctx.base_img + base[i].pix_begin;
+                w.passes = K - 1;
+                v.out = ctx.base_img + base[i].pix_begin;
+                v.prim = nullptr;
+                v.rgb = nullptr;
+                v.passes = 1;
+            }
             ctx.h_views[i] = v;
         }
-        RCP_CUDA(cudaMemcpyAsync(ctx.d_views, ctx.h_views, sizeof(ViewDev) * (size_t)nv, cudaMemcpyHostToDevice, st));
+        RCP_CUDA(cudaMemcpyAsync(ctx.d_views, ctx.h_views, sizeof(ViewDev) * (size_t)nv * (ctx.image_mode ? 2 : 1),
+                                 cudaMemcpyHostToDevice, st));
         RCP_CUDA(cudaEventRecord(ctx.staged, st));
         return RCP_OK;
     }
-    if (ctx.image_mode && !ctx.base_img) RCP_CUDA(cudaMalloc((void**)&ctx.base_img, sizeof(float4) * ctx.total_pix));
     for (int n = 0; n < K; ++n) {
         for (int i = 0; i < nv; ++i) {
             ViewDev v = base[i];

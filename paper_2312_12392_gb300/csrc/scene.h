@@ -33,12 +33,13 @@ struct RenderCtx {
     float4* io = nullptr;        // host-API input / final image
     float4* base_img = nullptr;  // image-space mapping: the traced pass-1 image
     bool image_mode = false;     // passes 2..K are image-space gathers
-    bool chained = false;        // one launch runs all K passes (one descriptor per view)
+    bool chained = false;        // one launch runs all K passes (one descriptor per view), or, in image mode, one
+                                 // launch traces pass 1 and one gathers passes 2..K (two descriptors per view)
     int32_t* io_prim = nullptr;  // host-API hit ids
     int2* hints = nullptr;       // per pixel: latest primary-hit and shadow-occluder records (-1 none)
     cudaEvent_t staged = nullptr;
     cudaEvent_t pass_ev[17] = {};  // timing events around every launch (recorded inside the graph)
-    int launches = 0;              // launches of the latest enqueue: K, or 1 when the passes are chained
+    int launches = 0;              // launches of the latest enqueue: K, or 1 (image mode: 2) when chained
     cudaGraphExec_t graph = nullptr;
     std::string graph_key;
     cudaEvent_t done = nullptr;  // recorded after the context's latest launch
@@ -135,6 +136,9 @@ bool use_direct_output(const void* p, size_t bytes);
 void touch_pages(void* p, size_t bytes);
 // Image-space pass over every view (views' base/in/out set).
 rcp_status launch_imagespace(const ViewDev* d_views, int n_views, int64_t total_pix, cudaStream_t st);
+// All of each view's image-space passes in one launch (views' base, out and
+// passes set).
+rcp_status launch_imagespace_chain(const ViewDev* d_views, int n_views, int64_t total_chunks, cudaStream_t st);
 rcp_status launch_imagespace_single(const float4* base, const float4* prev, float4* out, int W, int H, float kpx,
                                     cudaStream_t st);
 
