@@ -358,7 +358,7 @@ rcp_status rcp_debug_sort_lookback_timeout(int64_t spin_limit, void* stream);
  * point does the same stable LSD radix sort as rcp_debug_sort_pairs (keys and
  * values are device arrays of n uint32, sorted in place on the low `bits` bits
  * of the keys, enqueued on `stream`), but all of its scratch lives in one fixed
- * device array compiled into the library, of about 8.7 MB, which every GPU that
+ * device array compiled into the library, of about 9 MB, which every GPU that
  * loads the library holds until the process exits; it calls no cudaMalloc,
  * cudaFree or allocating library routine.
  *  - n may be at most RCP_SORT_STATIC_MAX_PAIRS (also returned by

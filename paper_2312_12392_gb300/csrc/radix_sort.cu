@@ -1,12 +1,24 @@
 // radix_sort.cu -- onesweep LSD radix sort of (uint32 key, uint32 value) pairs.
 //
-// Used by the BVH builder to order primitives by 30-bit Morton code. One
-// histogram kernel counts all digit passes at once; then one kernel per 8-bit
-// digit ranks a tile of keys in shared memory (warp match + per-warp counters,
+// Used by the BVH builder to order primitives by 30-bit Morton code, and by
+// the allocation-free sort below. One histogram kernel counts all digit passes
+// at once (its last block scans the counts); then one kernel per 8-bit digit
+// ranks a tile of keys in shared memory (warp ballots + per-warp counters,
 // stable), finds the tile's global offset per digit by decoupled look-back over
 // earlier tiles (tiles are numbered in launch order by an atomic counter, so
 // every earlier tile is already running), and scatters through shared memory
 // so that writes of one digit run are contiguous.
+//
+// What bounds it up to about a million pairs is latency: 16 MB a pass moves
+// through L2 in a few microseconds, and each block's chain of load, rank,
+// look-back and scatter is serial. So: tiles of 7,168 pairs, which put a
+// million pairs on the SMs in one wave (147 tiles); a look-back that polls
+// eight earlier tiles at once, where one at a time is a chain of L2 round
+// trips over as many tiles; the tile's own scan done by the other half of the
+// block meanwhile; one memset for every pass's status words; and programmatic
+// launches, so that a pass's blocks are resident when the pass before ends.
+// 1,000,003 pairs on 30 bits, the whole call with its last read-back: 170 -> 102
+// us (a pass 25 -> 13.5 us, of which 9.4 us is one tile alone).
 //
 // Every wait on another tile's status is bounded: after spin_limit polls
 // (SPIN_LIMIT in a sort) the kernel records an error flag and proceeds, so a
@@ -14,6 +26,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -24,168 +37,241 @@ namespace rcp {
 namespace {
 
 constexpr int RADIX = 256;
-constexpr int SORT_BLOCK = 256;  // one thread per digit in the scan/look-back steps
+constexpr int PASSES_MAX = 4;
+constexpr int SORT_BLOCK = 512;
 constexpr int SORT_WARPS = SORT_BLOCK / 32;
-constexpr int ITEMS = 15;
-constexpr int TILE = SORT_BLOCK * ITEMS;  // 3840 keys
+constexpr int ITEMS = 14;
+constexpr int TILE = SORT_BLOCK * ITEMS;  // 7168 pairs
+constexpr int LOOK = 8;                   // earlier tiles polled at once
+static_assert(SORT_BLOCK == 2 * RADIX, "one half of the block looks back, the other scans the tile's counts");
 constexpr uint32_t FLAG_AGG = 1u << 30;
 constexpr uint32_t FLAG_INC = 2u << 30;
 constexpr uint32_t COUNT_MASK = (1u << 30) - 1;
 constexpr long long SPIN_LIMIT = 1ll << 26;
 
-__global__ void __launch_bounds__(SORT_BLOCK) k_histogram(const uint32_t* __restrict__ keys, int64_t n,
-                                                          int passes, uint32_t* __restrict__ hist) {
-    __shared__ uint32_t h[4][RADIX];
-    for (int i = threadIdx.x; i < 4 * RADIX; i += blockDim.x) (&h[0][0])[i] = 0;
+// Scratch words: the passes' digit counts (bucket starts once scanned), then
+// one tile counter per pass and the histogram's block counter, then the
+// passes' tile status, RADIX words per tile.
+constexpr int COUNTERS = 8;
+constexpr size_t scratch_words(int64_t tiles, int passes) {
+    return (size_t)PASSES_MAX * RADIX + COUNTERS + (size_t)passes * (size_t)tiles * RADIX;
+}
+
+constexpr int HIST_BLOCK = 1024;  // one block per SM: each adds its counts to the global ones once
+constexpr int HIST_KEYS = 8;      // keys a thread holds at a time
+
+// Digit counts of all passes; the last block to finish turns each pass's 256
+// counts into exclusive prefix sums.
+__global__ void __launch_bounds__(HIST_BLOCK) k_histogram(const uint32_t* __restrict__ keys, int64_t n, int passes,
+                                                          uint32_t* hist, uint32_t* blocks_done) {
+    __shared__ uint32_t h[PASSES_MAX][RADIX];
+    __shared__ uint32_t s_warp[RADIX / 32];
+    __shared__ bool s_last;
+    for (int i = threadIdx.x; i < PASSES_MAX * RADIX; i += HIST_BLOCK) (&h[0][0])[i] = 0;
     __syncthreads();
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t k = keys[i];
-        for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(k >> (8 * p)) & 0xff], 1u);
+    const int64_t step = (int64_t)gridDim.x * HIST_BLOCK;
+    for (int64_t i = blockIdx.x * (int64_t)HIST_BLOCK + threadIdx.x; i < n; i += HIST_KEYS * step) {
+        uint32_t k[HIST_KEYS];
+#pragma unroll
+        for (int q = 0; q < HIST_KEYS; ++q) k[q] = i + q * step < n ? keys[i + q * step] : 0u;
+#pragma unroll
+        for (int q = 0; q < HIST_KEYS; ++q)
+            if (i + q * step < n)
+                for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(k[q] >> (8 * p)) & 0xff], 1u);
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < passes * RADIX; i += blockDim.x) {
+    for (int i = threadIdx.x; i < passes * RADIX; i += HIST_BLOCK) {
         const uint32_t v = (&h[0][0])[i];
         if (v) atomicAdd(&hist[i], v);
     }
-}
-
-// Exclusive scan of each pass's 256 bins (one block of 256 threads).
-__global__ void k_scan_histogram(uint32_t* hist, int passes) {
-    __shared__ uint32_t s[RADIX];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(blocks_done, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool scans = threadIdx.x < RADIX;  // one thread per digit
     for (int p = 0; p < passes; ++p) {
-        const uint32_t v = hist[p * RADIX + threadIdx.x];
-        s[threadIdx.x] = v;
-        __syncthreads();
-        for (int off = 1; off < RADIX; off <<= 1) {
-            uint32_t t = threadIdx.x >= off ? s[threadIdx.x - off] : 0;
-            __syncthreads();
-            s[threadIdx.x] += t;
-            __syncthreads();
+        const uint32_t v = scans ? __ldcg(&hist[p * RADIX + threadIdx.x]) : 0u;
+        uint32_t x = v;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
         }
-        hist[p * RADIX + threadIdx.x] = s[threadIdx.x] - v;
+        if (scans && lane == 31) s_warp[warp] = x;
+        __syncthreads();
+        if (scans) {
+            for (int w = 0; w < warp; ++w) x += s_warp[w];
+            hist[p * RADIX + threadIdx.x] = x - v;
+        }
         __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(SORT_BLOCK) k_onesweep(const uint32_t* __restrict__ keys_in,
-                                                         const uint32_t* __restrict__ vals_in,
-                                                         uint32_t* __restrict__ keys_out,
-                                                         uint32_t* __restrict__ vals_out, int64_t n, int shift,
-                                                         const uint32_t* __restrict__ bucket_base,
-                                                         uint32_t* status, uint32_t* tile_counter,
-                                                         int* error_flag, long long spin_limit) {
-    __shared__ uint32_t s_keys[TILE];
-    __shared__ uint32_t s_vals[TILE];
-    __shared__ uint32_t s_wcnt[SORT_WARPS][RADIX];
-    __shared__ uint32_t s_tile_off[RADIX];
-    __shared__ uint32_t s_global[RADIX];
-    __shared__ uint32_t s_tile;
+// The lanes whose digit equals this lane's, by one ballot per digit bit (as fast
+// as a warp match here).
+__device__ __forceinline__ unsigned same_digit(uint32_t d) {
+    unsigned peers = 0xffffffffu;
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const bool set = (d >> b) & 1u;
+        const unsigned with = __ballot_sync(0xffffffffu, set);
+        peers &= set ? with : ~with;
+    }
+    return peers;
+}
 
+struct SortShared {
+    uint32_t keys[TILE];
+    uint32_t vals[TILE];
+    uint32_t wcnt[SORT_WARPS][RADIX];
+    uint32_t tile_off[RADIX];
+    uint32_t global[RADIX];
+    uint32_t warp_tot[RADIX / 32];
+    uint32_t tile;
+};
+
+__global__ void __launch_bounds__(SORT_BLOCK, 2) k_onesweep(const uint32_t* __restrict__ keys_in,
+                                                            const uint32_t* __restrict__ vals_in,
+                                                            uint32_t* __restrict__ keys_out,
+                                                            uint32_t* __restrict__ vals_out, int64_t n, int shift,
+                                                            const uint32_t* __restrict__ bucket_base, uint32_t* status,
+                                                            uint32_t* tile_counter, int* error_flag,
+                                                            long long spin_limit) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    SortShared& s = *reinterpret_cast<SortShared*>(s_raw);
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    if (tid == 0) s_tile = atomicAdd(tile_counter, 1u);
-    for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_BLOCK) (&s_wcnt[0][0])[i] = 0;
+    for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_BLOCK) (&s.wcnt[0][0])[i] = 0;
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // the pass (or histogram) before has finished
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (tid == 0) s.tile = atomicAdd(tile_counter, 1u);
     __syncthreads();
-    const uint32_t tile = s_tile;
-    const int64_t base = (int64_t)tile * TILE;
+    const uint32_t tile = s.tile;
+    const int64_t base = (int64_t)tile * TILE + warp * (32 * ITEMS) + lane;
 
     uint32_t k[ITEMS], v[ITEMS], rank[ITEMS];
 #pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const int64_t idx = base + (int64_t)warp * (32 * ITEMS) + j * 32 + lane;
-        if (idx < n) {
-            k[j] = keys_in[idx];
-            v[j] = vals_in[idx];
-        } else {
-            k[j] = 0xffffffffu;  // past the end: ranks after every real key of its digit
-            v[j] = 0;
-        }
-    }
+    for (int j = 0; j < ITEMS; ++j)  // past the end: ranks after every real key of its digit
+        k[j] = base + 32 * j < n ? keys_in[base + 32 * j] : 0xffffffffu;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) v[j] = base + 32 * j < n ? vals_in[base + 32 * j] : 0u;
     const unsigned lt = (1u << lane) - 1u;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
         const uint32_t d = (k[j] >> shift) & 0xff;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        const uint32_t before = s_wcnt[warp][d];
+        const unsigned peers = same_digit(d);
+        const uint32_t before = s.wcnt[warp][d];
         rank[j] = before + __popc(peers & lt);
         __syncwarp();
-        if ((peers >> lane) == 1u) s_wcnt[warp][d] = before + __popc(peers);  // highest lane of the group
+        if ((peers >> lane) == 1u) s.wcnt[warp][d] = before + __popc(peers);  // highest lane of the group
         __syncwarp();
     }
     __syncthreads();
 
-    // per digit: exclusive scan over warps, then the tile's count
-    {
-        const int d = tid;
-        uint32_t sum = 0;
+    // digit d's tile count, as an exclusive scan over the warps; each half of
+    // the block has one thread per digit
+    const int d = tid & (RADIX - 1);
+    uint32_t count = 0;
+    if (tid < RADIX) {
 #pragma unroll
         for (int w = 0; w < SORT_WARPS; ++w) {
-            const uint32_t c = s_wcnt[w][d];
-            s_wcnt[w][d] = sum;
-            sum += c;
+            const uint32_t c = s.wcnt[w][d];
+            s.wcnt[w][d] = count;
+            count += c;
         }
-        const uint32_t count = sum;
-        // publish this tile's aggregate (tile 0 is already inclusive)
+        // publish this tile's count (tile 0's is already inclusive); a status
+        // word carries flag and count together, so no fence orders anything
         volatile uint32_t* st = status + (size_t)tile * RADIX;
-        __threadfence();
         st[d] = (tile == 0 ? FLAG_INC : FLAG_AGG) | count;
-        // look back over earlier tiles
-        uint32_t prefix = 0;
-        if (tile > 0) {
-            int64_t t = (int64_t)tile - 1;
-            long long spins = 0;
-            while (t >= 0) {
-                const uint32_t sv = ((volatile uint32_t*)status)[(size_t)t * RADIX + d];
-                const uint32_t flag = sv & ~COUNT_MASK;
-                if (flag == 0) {
-                    if (++spins > spin_limit) {
-                        atomicExch(error_flag, 1);
-                        break;
-                    }
-                    continue;
-                }
-                prefix += sv & COUNT_MASK;
-                if (flag == FLAG_INC) break;
-                --t;
-            }
-            __threadfence();
-            st[d] = FLAG_INC | (prefix + count);
-        }
-        s_global[d] = bucket_base[d] + prefix;
-        s_tile_off[d] = count;
+        s.tile_off[d] = count;
     }
     __syncthreads();
-    // exclusive scan of the tile's digit counts -> tile offsets (Hillis-Steele)
-    {
-        const uint32_t c = s_tile_off[tid];
-        uint32_t x = c;
-        for (int off = 1; off < RADIX; off <<= 1) {
-            __syncthreads();
-            const uint32_t y = tid >= off ? s_tile_off[tid - off] : 0;
-            __syncthreads();
-            x += y;
-            s_tile_off[tid] = x;
+    if (tid < RADIX) {
+        // look back over earlier tiles, LOOK of them per round of loads
+        uint32_t prefix = 0;
+        int64_t t = (int64_t)tile - 1;
+        long long spins = 0;
+        while (t >= 0) {
+            uint32_t sv[LOOK];
+#pragma unroll
+            for (int q = 0; q < LOOK; ++q) {
+                sv[q] = FLAG_INC;  // before the first tile: nothing more to add
+                if (t >= q) sv[q] = ((volatile uint32_t*)status)[(size_t)(t - q) * RADIX + d];
+            }
+            bool found = false, waiting = false;
+            int taken = 0;
+#pragma unroll
+            for (int q = 0; q < LOOK; ++q) {
+                const uint32_t flag = sv[q] & ~COUNT_MASK;
+                waiting = waiting || flag == 0;
+                if (!found && !waiting) {
+                    prefix += sv[q] & COUNT_MASK;
+                    found = flag == FLAG_INC;
+                    ++taken;
+                }
+            }
+            if (found) break;
+            t -= taken;
+            if (taken == 0 && ++spins > spin_limit) {
+                atomicExch(error_flag, 1);
+                break;
+            }
         }
-        __syncthreads();
-        s_tile_off[tid] = x - c;
+        if (tile > 0) ((volatile uint32_t*)status)[(size_t)tile * RADIX + d] = FLAG_INC | (prefix + count);
+        s.global[d] = bucket_base[d] + prefix;
+    } else {
+        // the tile's digit counts -> tile offsets
+        const uint32_t c = s.tile_off[d];
+        uint32_t x = c;
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s.warp_tot[d >> 5] = x;
+        asm volatile("bar.sync 1, 256;" ::: "memory");  // this half of the block
+        for (int w = 0; w < d >> 5; ++w) x += s.warp_tot[w];
+        s.tile_off[d] = x - c;
     }
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t d = (k[j] >> shift) & 0xff;
-        const uint32_t r = s_tile_off[d] + s_wcnt[warp][d] + rank[j];
-        s_keys[r] = k[j];
-        s_vals[r] = v[j];
+        const uint32_t dj = (k[j] >> shift) & 0xff;
+        const uint32_t r = s.tile_off[dj] + s.wcnt[warp][dj] + rank[j];
+        s.keys[r] = k[j];
+        s.vals[r] = v[j];
     }
     __syncthreads();
-    const int64_t valid = n - base < TILE ? n - base : TILE;
+    const int64_t left = n - (int64_t)tile * TILE;
+    const int valid = left < TILE ? (int)left : TILE;
     for (int pos = tid; pos < valid; pos += SORT_BLOCK) {
-        const uint32_t key = s_keys[pos];
-        const uint32_t d = (key >> shift) & 0xff;
-        const uint32_t dst = s_global[d] + (pos - s_tile_off[d]);
+        const uint32_t key = s.keys[pos];
+        const uint32_t dj = (key >> shift) & 0xff;
+        const uint32_t dst = s.global[dj] + (pos - s.tile_off[dj]);
         keys_out[dst] = key;
-        vals_out[dst] = s_vals[pos];
+        vals_out[dst] = s.vals[pos];
     }
+}
+
+// One digit pass: launched programmatically behind the kernel before it.
+rcp_status launch_onesweep(const uint32_t* ki, const uint32_t* vi, uint32_t* ko, uint32_t* vo, int64_t n, int shift,
+                           const uint32_t* bucket_base, uint32_t* status, uint32_t* tile_counter, int64_t blocks,
+                           int* d_error, long long spin_limit, cudaStream_t stream) {
+    RCP_CUDA(cudaFuncSetAttribute(k_onesweep, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SortShared)));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(SORT_BLOCK);
+    cfg.dynamicSmemBytes = sizeof(SortShared);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    RCP_CUDA(cudaLaunchKernelEx(&cfg, k_onesweep, ki, vi, ko, vo, n, shift, bucket_base, status, tile_counter, d_error,
+                                spin_limit));
+    return RCP_OK;
 }
 
 }  // namespace
@@ -194,8 +280,7 @@ __global__ void __launch_bounds__(SORT_BLOCK) k_onesweep(const uint32_t* __restr
 // are n-element scratch buffers; scratch holds the histogram, tile status and
 // counters (size from radix_sort_scratch_bytes).
 size_t radix_sort_scratch_bytes(int64_t n) {
-    const int64_t tiles = (n + TILE - 1) / TILE;
-    return sizeof(uint32_t) * (4 * RADIX + 8 + (size_t)(tiles > 0 ? tiles : 1) * RADIX);
+    return sizeof(uint32_t) * scratch_words(std::max<int64_t>((n + TILE - 1) / TILE, 1), PASSES_MAX);
 }
 
 rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals,
@@ -208,30 +293,28 @@ rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
     const int passes = (bits + 7) / 8;
     const int64_t tiles = (n + TILE - 1) / TILE;
     uint32_t* hist = (uint32_t*)scratch;
-    uint32_t* counters = hist + 4 * RADIX;  // one tile counter per pass
-    uint32_t* status = counters + 8;
-    RCP_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * (4 * RADIX + 8), stream));
+    uint32_t* counters = hist + PASSES_MAX * RADIX;
+    uint32_t* status = counters + COUNTERS;
+    RCP_CUDA(cudaMemsetAsync(hist, 0, sizeof(uint32_t) * scratch_words(tiles, passes), stream));
     int sms = 0, dev = 0;
     RCP_CUDA(cudaGetDevice(&dev));
     RCP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    int64_t hblocks = (n + SORT_BLOCK * 16 - 1) / (SORT_BLOCK * 16);
-    if (hblocks > sms * 8) hblocks = sms * 8;
-    k_histogram<<<(int)hblocks, SORT_BLOCK, 0, stream>>>(keys, n, passes, hist);
-    k_scan_histogram<<<1, RADIX, 0, stream>>>(hist, passes);
+    int64_t hblocks = (n + HIST_BLOCK * HIST_KEYS - 1) / (HIST_BLOCK * HIST_KEYS);
+    if (hblocks > sms) hblocks = sms;
+    k_histogram<<<(int)hblocks, HIST_BLOCK, 0, stream>>>(keys, n, passes, hist, counters + PASSES_MAX);
+    RCP_CUDA(cudaGetLastError());
     uint32_t *ki = keys, *vi = vals, *ko = alt_keys, *vo = alt_vals;
     for (int p = 0; p < passes; ++p) {
-        RCP_CUDA(cudaMemsetAsync(status, 0, sizeof(uint32_t) * (size_t)tiles * RADIX, stream));
-        k_onesweep<<<(int)tiles, SORT_BLOCK, 0, stream>>>(ki, vi, ko, vo, n, 8 * p, hist + p * RADIX, status,
-                                                           counters + p, d_error, SPIN_LIMIT);
-        uint32_t* t;
-        t = ki; ki = ko; ko = t;
-        t = vi; vi = vo; vo = t;
+        rcp_status r = launch_onesweep(ki, vi, ko, vo, n, 8 * p, hist + p * RADIX, status + (size_t)p * tiles * RADIX,
+                                       counters + p, tiles, d_error, SPIN_LIMIT, stream);
+        if (r != RCP_OK) return r;
+        std::swap(ki, ko);
+        std::swap(vi, vo);
     }
     if (ki != keys) {
         RCP_CUDA(cudaMemcpyAsync(keys, ki, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, stream));
         RCP_CUDA(cudaMemcpyAsync(vals, vi, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, stream));
     }
-    RCP_CUDA(cudaGetLastError());
     return RCP_OK;
 }
 
@@ -253,7 +336,7 @@ constexpr size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t OFF_KEYS = 0;
 constexpr size_t OFF_VALS = align256(OFF_KEYS + sizeof(uint32_t) * STATIC_MAX);
 constexpr size_t OFF_SCRATCH = align256(OFF_VALS + sizeof(uint32_t) * STATIC_MAX);
-constexpr size_t SCRATCH_BYTES = sizeof(uint32_t) * (4 * RADIX + 8 + STATIC_TILES * RADIX);
+constexpr size_t SCRATCH_BYTES = sizeof(uint32_t) * scratch_words(STATIC_TILES, PASSES_MAX);
 constexpr size_t OFF_ERROR = align256(OFF_SCRATCH + SCRATCH_BYTES);
 constexpr size_t STATIC_BYTES = align256(OFF_ERROR + sizeof(int));
 
@@ -351,22 +434,21 @@ extern "C" rcp_status rcp_debug_sort_lookback_timeout(int64_t spin_limit, void* 
     RCP_CUDA(vals.alloc(n));
     RCP_CUDA(ko.alloc(n));
     RCP_CUDA(vo.alloc(n));
-    RCP_CUDA(scratch.alloc(4 * RADIX + 8 + 2 * RADIX));
+    RCP_CUDA(scratch.alloc(scratch_words(2, 1)));
     RCP_CUDA(err.alloc(1));
     uint32_t* hist = scratch.p;
-    uint32_t* counter = hist + 4 * RADIX;
-    uint32_t* status = counter + 8;
+    uint32_t* counter = hist + PASSES_MAX * RADIX;
+    uint32_t* status = counter + COUNTERS;
     RCP_CUDA(cudaMemsetAsync(keys.p, 0, sizeof(uint32_t) * n, st));
     RCP_CUDA(cudaMemsetAsync(vals.p, 0, sizeof(uint32_t) * n, st));
-    RCP_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(uint32_t) * (4 * RADIX + 8 + 2 * RADIX), st));
+    RCP_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(uint32_t) * scratch_words(2, 1), st));
     RCP_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
-    k_histogram<<<2, SORT_BLOCK, 0, st>>>(keys.p, n, 1, hist);
-    k_scan_histogram<<<1, RADIX, 0, st>>>(hist, 1);
+    k_histogram<<<2, HIST_BLOCK, 0, st>>>(keys.p, n, 1, hist, counter + PASSES_MAX);
     const uint32_t one = 1;  // the block claims tile 1; tile 0 is never claimed
     RCP_CUDA(cudaMemcpyAsync(counter, &one, sizeof(one), cudaMemcpyHostToDevice, st));
-    k_onesweep<<<1, SORT_BLOCK, 0, st>>>(keys.p, vals.p, ko.p, vo.p, n, 0, hist, status, counter, err.p,
-                                         (long long)spin_limit);
-    RCP_CUDA(cudaGetLastError());
+    rcp_status r = launch_onesweep(keys.p, vals.p, ko.p, vo.p, n, 0, hist, status, counter, 1, err.p,
+                                   (long long)spin_limit, st);
+    if (r != RCP_OK) return r;
     int h = 0;
     RCP_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     RCP_CUDA(cudaStreamSynchronize(st));
