@@ -63,6 +63,27 @@ __device__ __forceinline__ float ord2f(uint32_t u) {
     return __uint_as_float((u & 0x80000000u) ? (u & 0x7fffffffu) : ~u);
 }
 
+// *bad = 1 when any of v[0..n) (16-byte aligned) is infinite or NaN: its
+// exponent bits are all set. Bound by reading v once.
+__global__ void __launch_bounds__(BUILD_BLOCK) k_any_non_finite(const float* __restrict__ v, int64_t n, int* bad) {
+    const uint4* v4 = reinterpret_cast<const uint4*>(v);
+    bool found = false;
+    const auto non_finite = [](uint32_t u) { return (u & 0x7f800000u) == 0x7f800000u; };
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = t; i < n / 4; i += step) {
+        const uint4 u = v4[i];
+        found = found || non_finite(u.x) || non_finite(u.y) || non_finite(u.z) || non_finite(u.w);
+    }
+    for (int64_t i = n / 4 * 4 + t; i < n; i += step) found = found || non_finite(__float_as_uint(v[i]));
+    if (found) *bad = 1;
+}
+
+__global__ void __launch_bounds__(BUILD_BLOCK) k_widen_albedo(const float* __restrict__ a, int64_t n,
+                                                              float4* __restrict__ out) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = make_float4(a[3 * i], a[3 * i + 1], a[3 * i + 2], 0.f);
+}
+
 // bounds layout: [0..2] centroid min, [3..5] centroid max, [6..8] box min, [9..11] box max
 __global__ void k_init_bounds(uint32_t* b) {
     const int i = threadIdx.x;
@@ -1360,6 +1381,28 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
 }
 
 }  // namespace
+
+rcp_status ingest_scene(Scene& sc, const float* albedo3, bool* bad_tri, bool* bad_sph, cudaStream_t st) {
+    const int64_t N = sc.T + sc.S;
+    *bad_tri = *bad_sph = false;
+    if (N == 0) return RCP_OK;
+    DevBuf<int> bad;
+    RCP_CUDA(bad.alloc(2));
+    RCP_CUDA(cudaMemsetAsync(bad.p, 0, 2 * sizeof(int), st));
+    int sms = 148, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    k_any_non_finite<<<grid_for(9 * sc.T / 4 + 1, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(sc.d_tri, 9 * sc.T,
+                                                                                                bad.p);
+    k_any_non_finite<<<grid_for(sc.S + 1, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(sc.d_sph, 4 * sc.S, bad.p + 1);
+    k_widen_albedo<<<grid_for(N, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(albedo3, N, sc.d_albedo);
+    int h[2];
+    RCP_CUDA(cudaMemcpyAsync(h, bad.p, sizeof(h), cudaMemcpyDeviceToHost, st));
+    RCP_CUDA(cudaStreamSynchronize(st));
+    *bad_tri = h[0] != 0;
+    *bad_sph = h[1] != 0;
+    return RCP_OK;
+}
 
 rcp_status build_bvh(Scene& sc, cudaStream_t st) {
     const int64_t T = sc.T, N = sc.T + sc.S;

@@ -83,6 +83,10 @@ struct Scene {
     int64_t device_bytes() const;
 };
 
+// The scene's arrays as uploaded: whether every vertex and sphere is finite,
+// and d_albedo (a float4 per primitive) from 3 floats per primitive. Waits for
+// the stream.
+rcp_status ingest_scene(Scene& sc, const float* albedo3, bool* bad_tri, bool* bad_sph, cudaStream_t st);
 rcp_status build_bvh(Scene& sc, cudaStream_t st);
 rcp_status refit_bvh(Scene& sc, cudaStream_t st);
 rcp_status validate_bvh(const Scene& sc, cudaStream_t st);
