@@ -486,6 +486,11 @@ __global__ void k_record_parts(const float4* __restrict__ prims, int64_t R, cons
 // globally smallest pair is always mutual: every iteration merges at least
 // one pair, and a run of equal boxes pairs up (0,1), (2,3), ... at once.
 // Node indices count down: the last merge creates the root, node 0.
+// What bounds a round is launches more than work: 29 rounds of a million
+// triangles took 3.4 ms in 4 to 6 launches and a host wait each, 0.75 ms of it
+// in kernels. A round is now two launches without the host, and the rounds of
+// PLOC_LAST clusters or fewer run in one block: 1.8 ms with its allocations,
+// 0.87 ms of it in kernels.
 constexpr int PLOC_R = 16;
 constexpr int PLOC_BLOCK = 256;
 
@@ -493,14 +498,58 @@ __device__ __forceinline__ float union_area(float4 alo, float4 ahi, float4 blo, 
     const float dx = fmaxf(ahi.x, bhi.x) - fminf(alo.x, blo.x);
     const float dy = fmaxf(ahi.y, bhi.y) - fminf(alo.y, blo.y);
     const float dz = fmaxf(ahi.z, bhi.z) - fminf(alo.z, blo.z);
-    const float a = dx * dy + dy * dz + dz * dx;
+    // explicit operations: every kernel that compares areas computes the same bits
+    const float a = __fmaf_rn(dz, dx, __fmaf_rn(dy, dz, __fmul_rn(dx, dy)));
     return a == a ? a : INFINITY;
 }
 
+// The best partner of cluster i of n: the one within PLOC_R positions that
+// comes first by (union area, index gap, parity of the lower index, lower
+// index). Gaps are taken in increasing order, so only the two clusters at one
+// gap, of lower indices i - g and i, need the tie's rules. box(j, lo, hi)
+// reads cluster j's box. -1 when i is alone.
+template <class Box>
+__device__ __forceinline__ int ploc_partner(int i, int n, Box box) {
+    float4 alo, ahi;
+    box(i, alo, ahi);
+    float best = INFINITY;
+    int partner = -1;
+#pragma unroll 4
+    for (int g = 1; g <= PLOC_R; ++g) {
+        const bool has_l = i - g >= 0, has_r = i + g < n;
+        float4 l, h;
+        float al = INFINITY, ar = INFINITY;
+        if (has_l) {
+            box(i - g, l, h);
+            al = union_area(alo, ahi, l, h);
+        }
+        if (has_r) {
+            box(i + g, l, h);
+            ar = union_area(alo, ahi, l, h);
+        }
+        const bool left_first = !(g & 1) || !((i - g) & 1);
+        const bool left = has_l && (!has_r || al < ar || (al == ar && left_first));
+        const float a = left ? al : ar;
+        if ((has_l || has_r) && (partner < 0 || a < best)) {
+            best = a;
+            partner = left ? i - g : i + g;
+        }
+    }
+    return partner;
+}
+
+// A round's state: n clusters, `created` nodes so far; round r reads
+// state[r] and its merge writes state[r + 1].
+struct PlocState {
+    int n, created, stalled, pad;  // stalled: a round of two clusters or more merged none
+};
+
 __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_nn(const float4* __restrict__ clo, const float4* __restrict__ chi,
-                                                        int64_t n, int* __restrict__ nn) {
+                                                        const PlocState* __restrict__ state, int* __restrict__ nn) {
     __shared__ float4 slo[PLOC_BLOCK + 2 * PLOC_R], shi[PLOC_BLOCK + 2 * PLOC_R];
+    const int n = state->n;
     const int64_t first = (int64_t)blockIdx.x * PLOC_BLOCK;
+    if (first >= n) return;  // the grid covers an earlier round's count
     for (int t = threadIdx.x; t < PLOC_BLOCK + 2 * PLOC_R; t += PLOC_BLOCK) {
         const int64_t g = first - PLOC_R + t;
         if (g >= 0 && g < n) {
@@ -509,83 +558,253 @@ __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_nn(const float4* __restrict
         }
     }
     __syncthreads();
-    const int64_t i = first + threadIdx.x;
+    const int i = (int)first + threadIdx.x;
     if (i >= n) return;
-    const int li = threadIdx.x + PLOC_R;
-    const float4 alo = slo[li], ahi = shi[li];
-    float ba = 0.f;
-    int64_t bj = -1, bgap = 0, blo = 0;
-    for (int o = -PLOC_R; o <= PLOC_R; ++o) {
-        const int64_t j = i + o;
-        if (o == 0 || j < 0 || j >= n) continue;
-        const float a = union_area(alo, ahi, slo[li + o], shi[li + o]);
-        const int64_t gap = o < 0 ? -o : o, lo = o < 0 ? j : i;
-        bool better = bj < 0 || a < ba;
-        if (!better && a == ba) {
-            if (gap != bgap) better = gap < bgap;
-            else if ((lo & 1) != (blo & 1)) better = (lo & 1) < (blo & 1);
-            else better = lo < blo;
-        }
-        if (better) {
-            ba = a;
-            bj = j;
-            bgap = gap;
-            blo = lo;
-        }
-    }
-    nn[i] = (int)bj;
-}
-
-// flag word per cluster: merges here (lower end of a mutual pair) << 32 | stays
-__global__ void k_ploc_flags(const int* __restrict__ nn, int64_t n, unsigned long long* __restrict__ flags) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int j = nn[i];
-        const bool mutual = j >= 0 && nn[j] == (int)i;
-        const unsigned long long merge = (mutual && i < j) ? 1ull : 0ull;
-        const unsigned long long keep = (mutual && i > j) ? 0ull : 1ull;
-        flags[i] = (merge << 32) | keep;
-    }
+    const int shift = PLOC_R - (int)first;  // cluster j is at slo[j + shift]
+    nn[i] = ploc_partner(i, n, [&](int j, float4& l, float4& h) {
+        l = slo[j + shift];
+        h = shi[j + shift];
+    });
 }
 
 __device__ __forceinline__ int leaf_count(const int* cnt, int ref) { return ref >= 0 ? cnt[ref] : 1; }
 
-// Merge mutual pairs into new nodes and compact the cluster array;
-// scan[i] = exclusive prefix of the flag words.
-__global__ void k_ploc_merge(const int* __restrict__ nn, int64_t n, const unsigned long long* __restrict__ scan,
-                             const int* __restrict__ ref, const float4* __restrict__ clo,
-                             const float4* __restrict__ chi, int node_base, int* __restrict__ ref_out,
-                             float4* __restrict__ lo_out, float4* __restrict__ hi_out, int2* __restrict__ child,
-                             float4* __restrict__ blo, float4* __restrict__ bhi, int* __restrict__ cnt,
-                             int* __restrict__ parent_int, int* __restrict__ parent_leaf) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int j = nn[i];
-        const bool mutual = j >= 0 && nn[j] == (int)i;
-        if (mutual && i > j) continue;
-        const unsigned long long s = scan[i];
-        const int64_t pos = (int64_t)(s & 0xffffffffull);
-        if (mutual) {
-            const int node = node_base + (int)(s >> 32);
-            const int ra = ref[i], rb = ref[j];
-            const float4 la = clo[i], ha = chi[i], lb = clo[j], hb = chi[j];
-            const float4 l = make_float4(fminf(la.x, lb.x), fminf(la.y, lb.y), fminf(la.z, lb.z), 0.f);
-            const float4 h = make_float4(fmaxf(ha.x, hb.x), fmaxf(ha.y, hb.y), fmaxf(ha.z, hb.z), 0.f);
-            child[node] = make_int2(ra, rb);
-            blo[node] = l;
-            bhi[node] = h;
-            cnt[node] = leaf_count(cnt, ra) + leaf_count(cnt, rb);
-            if (ra >= 0) parent_int[ra] = node;
-            else parent_leaf[-ra - 1] = node;
-            if (rb >= 0) parent_int[rb] = node;
-            else parent_leaf[-rb - 1] = node;
-            ref_out[pos] = node;
-            lo_out[pos] = l;
-            hi_out[pos] = h;
-        } else {
-            ref_out[pos] = ref[i];
-            lo_out[pos] = clo[i];
-            hi_out[pos] = chi[i];
+// Where the clustering writes its tree.
+struct PlocTree {
+    int2* child;
+    float4* blo;
+    float4* bhi;
+    int* cnt;
+    int* parent_int;
+    int* parent_leaf;
+};
+
+__device__ __forceinline__ void ploc_new_node(const PlocTree& t, int node, int ra, int rb, float4 l, float4 h) {
+    t.child[node] = make_int2(ra, rb);
+    t.blo[node] = l;
+    t.bhi[node] = h;
+    t.cnt[node] = leaf_count(t.cnt, ra) + leaf_count(t.cnt, rb);
+    if (ra >= 0) t.parent_int[ra] = node;
+    else t.parent_leaf[-ra - 1] = node;
+    if (rb >= 0) t.parent_int[rb] = node;
+    else t.parent_leaf[-rb - 1] = node;
+}
+
+__device__ __forceinline__ void box_union(float4 la, float4 ha, float4 lb, float4 hb, float4& l, float4& h) {
+    l = make_float4(fminf(la.x, lb.x), fminf(la.y, lb.y), fminf(la.z, lb.z), 0.f);
+    h = make_float4(fmaxf(ha.x, hb.x), fmaxf(ha.y, hb.y), fmaxf(ha.z, hb.z), 0.f);
+}
+
+// Merge mutual pairs into new nodes and compact the cluster array, in one
+// pass: each tile of PLOC_TILE clusters counts its merges and the clusters it
+// keeps, finds the counts before it by decoupled look-back (tiles numbered by
+// an atomic counter, so every earlier tile is already running; each wait is
+// bounded), and writes its nodes and its part of the next array. The merge
+// with m merges before it, over all rounds, becomes node N - 2 - m: the last
+// one is the root, node 0. A status word carries both counts, 31 bits each,
+// and its flag.
+constexpr int PLOC_ITEMS = 4;
+constexpr int PLOC_TILE = PLOC_BLOCK * PLOC_ITEMS;
+constexpr unsigned long long PLOC_AGG = 1ull << 62, PLOC_INC = 2ull << 62, PLOC_COUNTS = (1ull << 62) - 1;
+constexpr int PLOC_SPINS = 1 << 26;
+
+__global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_merge(const int* __restrict__ nn, PlocState* __restrict__ state,
+                                                           unsigned* ticket, unsigned long long* status, int64_t N,
+                                                           const int* __restrict__ ref, const float4* __restrict__ clo,
+                                                           const float4* __restrict__ chi, int* __restrict__ ref_out,
+                                                           float4* __restrict__ lo_out, float4* __restrict__ hi_out,
+                                                           PlocTree tree, int* err) {
+    __shared__ unsigned long long s_warp[PLOC_BLOCK / 32];
+    __shared__ unsigned long long s_before;
+    __shared__ unsigned s_tile;
+    if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const int64_t n = state->n, tile = s_tile, base = tile * PLOC_TILE + threadIdx.x * PLOC_ITEMS;
+    if (tile * PLOC_TILE >= n) return;
+    // per cluster: merges here (the lower end of a mutual pair) << 31 | stays
+    int partner[PLOC_ITEMS];
+    unsigned long long flag[PLOC_ITEMS], mine = 0;
+#pragma unroll
+    for (int q = 0; q < PLOC_ITEMS; ++q) {
+        const int64_t i = base + q;
+        partner[q] = -1;
+        flag[q] = 0;
+        if (i < n) {
+            const int j = nn[i];
+            if (j >= 0 && nn[j] == (int)i) partner[q] = j;
+            const bool gone = partner[q] >= 0 && i > j;
+            flag[q] = gone ? 0ull : (partner[q] >= 0 ? 1ull << 31 : 0ull) | 1ull;
+        }
+        mine += flag[q];
+    }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long x = mine;
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) s_warp[warp] = x;
+    __syncthreads();
+    unsigned long long total = 0, run = x - mine;
+    for (int w = 0; w < PLOC_BLOCK / 32; ++w) {
+        if (w < warp) run += s_warp[w];
+        total += s_warp[w];
+    }
+    if (warp == 0) {  // 32 earlier tiles per round of the look-back
+        volatile unsigned long long* st = status;
+        if (lane == 0) st[tile] = (tile == 0 ? PLOC_INC : PLOC_AGG) | total;
+        unsigned long long before = 0;
+        int64_t t = tile - 1;
+        for (int spins = 0; t >= 0;) {
+            unsigned long long w = PLOC_INC;  // before the first tile: nothing more to add
+            if (t >= lane) w = st[t - lane];
+            const unsigned waiting = __ballot_sync(0xffffffffu, (w >> 62) == 0);
+            const unsigned inclusive = __ballot_sync(0xffffffffu, (w >> 62) == 2);
+            // the nearest tiles up to the first inclusive one, if none of them still counts
+            const int last = inclusive ? __ffs(inclusive) - 1 : 31;
+            const unsigned use = 0xffffffffu >> (31 - last);
+            if (waiting & use) {
+                if (++spins > PLOC_SPINS) {
+                    if (lane == 0) atomicAdd(err, 1);
+                    break;
+                }
+                continue;
+            }
+            unsigned long long v = (use >> lane) & 1u ? w & PLOC_COUNTS : 0ull;
+            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            before += v;
+            if (inclusive) break;
+            t -= 32;
+        }
+        if (lane == 0) {
+            if (tile > 0) st[tile] = PLOC_INC | (before + total);
+            s_before = before;
         }
     }
+    __syncthreads();
+    run += s_before;
+    const int created = state->created;
+#pragma unroll
+    for (int q = 0; q < PLOC_ITEMS; ++q) {
+        const int64_t i = base + q;
+        if (flag[q]) {
+            const int64_t pos = (int64_t)(run & 0x7fffffffull);
+            float4 l = clo[i], h = chi[i];
+            int r = ref[i];
+            if (partner[q] >= 0) {
+                const int j = partner[q];
+                const int node = (int)(N - 2 - created - (int64_t)(run >> 31));
+                const float4 la = l, ha = h;
+                box_union(la, ha, clo[j], chi[j], l, h);
+                ploc_new_node(tree, node, r, ref[j], l, h);
+                r = node;
+            }
+            ref_out[pos] = r;
+            lo_out[pos] = l;
+            hi_out[pos] = h;
+        }
+        run += flag[q];
+    }
+    if ((tile + 1) * PLOC_TILE >= n && threadIdx.x == PLOC_BLOCK - 1) {  // the last tile: run is the round's total
+        const int merges = (int)(run >> 31);
+        state[1] = PlocState{(int)(run & 0x7fffffffull), created + merges, state->stalled | (n > 1 && merges == 0), 0};
+    }
+}
+
+// The last rounds in one block: PLOC_LAST clusters or fewer, the boxes of this
+// round's array and the next one in shared memory, until one cluster is left.
+// A round of separate launches costs about 10 us however few clusters it has,
+// and more than half of a build's rounds are below this size.
+constexpr int PLOC_LAST = 2048;
+constexpr int PLOC_LAST_BLOCK = 1024;
+constexpr int PLOC_LAST_ITEMS = PLOC_LAST / PLOC_LAST_BLOCK;
+struct PlocLastShared {
+    float4 lo[2][PLOC_LAST], hi[2][PLOC_LAST];
+    int ref[2][PLOC_LAST];
+    int nn[PLOC_LAST];
+    unsigned warp_tot[PLOC_LAST_BLOCK / 32];
+};
+
+__global__ void __launch_bounds__(PLOC_LAST_BLOCK) k_ploc_last(PlocState* state, int64_t N, const int* __restrict__ ref,
+                                                               const float4* __restrict__ clo,
+                                                               const float4* __restrict__ chi, PlocTree tree) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    PlocLastShared& s = *reinterpret_cast<PlocLastShared*>(s_raw);
+    int n = state->n, created = state->created, cur = 0;
+    bool stalled = false;
+    for (int i = threadIdx.x; i < n; i += PLOC_LAST_BLOCK) {
+        s.lo[0][i] = clo[i];
+        s.hi[0][i] = chi[i];
+        s.ref[0][i] = ref[i];
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    while (n > 1 && !stalled) {
+        for (int i = threadIdx.x; i < n; i += PLOC_LAST_BLOCK) {
+            s.nn[i] = ploc_partner(i, n, [&](int j, float4& l, float4& h) {
+                l = s.lo[cur][j];
+                h = s.hi[cur][j];
+            });
+        }
+        __syncthreads();
+        // consecutive clusters per thread, so that the scan keeps the array's
+        // order; merges << 16 | stays (both at most PLOC_LAST)
+        const int base = threadIdx.x * PLOC_LAST_ITEMS;
+        int partner[PLOC_LAST_ITEMS];
+        unsigned flag[PLOC_LAST_ITEMS], mine = 0;
+#pragma unroll
+        for (int q = 0; q < PLOC_LAST_ITEMS; ++q) {
+            const int i = base + q;
+            partner[q] = -1;
+            flag[q] = 0;
+            if (i < n) {
+                const int j = s.nn[i];
+                if (j >= 0 && s.nn[j] == i) partner[q] = j;
+                flag[q] = partner[q] >= 0 && i > j ? 0u : (partner[q] >= 0 ? 1u << 16 : 0u) | 1u;
+            }
+            mine += flag[q];
+        }
+        unsigned x = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) s.warp_tot[warp] = x;
+        __syncthreads();
+        unsigned run = x - mine, total = 0;
+        for (int w = 0; w < PLOC_LAST_BLOCK / 32; ++w) {
+            const unsigned t = s.warp_tot[w];
+            if (w < warp) run += t;
+            total += t;
+        }
+#pragma unroll
+        for (int q = 0; q < PLOC_LAST_ITEMS; ++q) {
+            const int i = base + q;
+            if (flag[q]) {
+                const int pos = (int)(run & 0xffffu);
+                float4 l = s.lo[cur][i], h = s.hi[cur][i];
+                int r = s.ref[cur][i];
+                if (partner[q] >= 0) {
+                    const int j = partner[q], node = (int)(N - 2 - created - (int)(run >> 16));
+                    const float4 la = l, ha = h;
+                    box_union(la, ha, s.lo[cur][j], s.hi[cur][j], l, h);
+                    ploc_new_node(tree, node, r, s.ref[cur][j], l, h);
+                    r = node;
+                }
+                s.lo[cur ^ 1][pos] = l;
+                s.hi[cur ^ 1][pos] = h;
+                s.ref[cur ^ 1][pos] = r;
+            }
+            run += flag[q];
+        }
+        const int merges = (int)(total >> 16);
+        created += merges;
+        stalled = merges == 0;
+        n = (int)(total & 0xffffu);
+        cur ^= 1;
+        __syncthreads();  // the next array (and, in global memory, the new nodes' counts) before the next round
+    }
+    if (threadIdx.x == 0) state[1] = PlocState{n, created, state->stalled | (stalled ? 1 : 0), 0};
 }
 
 __global__ void k_ploc_init(const uint32_t* __restrict__ sorted_ids, int64_t n, const float4* __restrict__ plo,
@@ -1324,10 +1543,11 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
                       int* d_err, int cap, cudaStream_t st) {
     DevBuf<int> ref_a, ref_b, nn, cnt, pos;
     DevBuf<float4> lo_a, hi_a, lo_b, hi_b;
-    DevBuf<unsigned long long> flags, aux, total;
-    const std::vector<int64_t> lv = scan_levels(N);
-    int64_t aux_n = 0;
-    for (int64_t t : lv) aux_n += t;
+    // per batch of PLOC_BATCH rounds: the rounds' states, tile counters and tile status
+    constexpr int PLOC_BATCH = 4;
+    DevBuf<PlocState> state;
+    DevBuf<unsigned long long> marks;
+    const int64_t tiles_max = (N + PLOC_TILE - 1) / PLOC_TILE;
     RCP_CUDA(ref_a.alloc(N));
     RCP_CUDA(ref_b.alloc(N));
     RCP_CUDA(nn.alloc(N));
@@ -1337,39 +1557,52 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
     RCP_CUDA(hi_a.alloc(N));
     RCP_CUDA(lo_b.alloc(N));
     RCP_CUDA(hi_b.alloc(N));
-    RCP_CUDA(flags.alloc(N));
-    RCP_CUDA(aux.alloc(aux_n));
-    RCP_CUDA(total.alloc(1));
+    RCP_CUDA(state.alloc(PLOC_BATCH + 2));
+    RCP_CUDA(marks.alloc(PLOC_BATCH * (1 + tiles_max)));
     RCP_CUDA(cudaMemsetAsync(parent_int, 0xff, sizeof(int) * N, st));
     RCP_CUDA(cudaMemsetAsync(parent_leaf, 0xff, sizeof(int) * N, st));
     int *rin = ref_a.p, *rout = ref_b.p;
     float4 *lin = lo_a.p, *hin = hi_a.p, *lout = lo_b.p, *hout = hi_b.p;
     k_ploc_init<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(ids_in, N, plo, phi, rin, lin, hin);
-    int64_t n = N, created = 0;
-    while (n > 1) {
-        k_ploc_nn<<<(unsigned)((n + PLOC_BLOCK - 1) / PLOC_BLOCK), PLOC_BLOCK, 0, st>>>(lin, hin, n, nn.p);
-        k_ploc_flags<<<grid_for(n, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(nn.p, n, flags.p);
-        scan_u64(flags.p, n, aux.p, lv, 0, total.p, st);
-        unsigned long long ht = 0;
-        RCP_CUDA(cudaMemcpyAsync(&ht, total.p, sizeof(ht), cudaMemcpyDeviceToHost, st));
+    const PlocTree tree{child, blo, bhi, cnt.p, parent_int, parent_leaf};
+    PlocState h{(int)N, 0, 0, 0};
+    RCP_CUDA(cudaMemcpyAsync(state.p, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+    // The rounds run without the host between them: each reads its count from
+    // the device, under a grid sized for the count at the batch's start, which
+    // only shrinks. The host reads the count once per batch.
+    while (h.n > PLOC_LAST) {
+        const int64_t n0 = h.n, tiles = (n0 + PLOC_TILE - 1) / PLOC_TILE;
+        RCP_CUDA(cudaMemsetAsync(marks.p, 0, sizeof(unsigned long long) * PLOC_BATCH * (1 + tiles), st));
+        for (int r = 0; r < PLOC_BATCH; ++r) {
+            k_ploc_nn<<<(unsigned)((n0 + PLOC_BLOCK - 1) / PLOC_BLOCK), PLOC_BLOCK, 0, st>>>(lin, hin, state.p + r,
+                                                                                              nn.p);
+            k_ploc_merge<<<(unsigned)tiles, PLOC_BLOCK, 0, st>>>(
+                nn.p, state.p + r, (unsigned*)(marks.p + r), marks.p + PLOC_BATCH + r * tiles, N, rin, lin, hin, rout,
+                lout, hout, tree, d_err);
+            std::swap(rin, rout);
+            std::swap(lin, lout);
+            std::swap(hin, hout);
+        }
+        RCP_CUDA(cudaGetLastError());
+        RCP_CUDA(cudaMemcpyAsync(state.p, state.p + PLOC_BATCH, sizeof(h), cudaMemcpyDeviceToDevice, st));
+        RCP_CUDA(cudaMemcpyAsync(&h, state.p, sizeof(h), cudaMemcpyDeviceToHost, st));
         RCP_CUDA(cudaStreamSynchronize(st));
-        const int64_t merges = (int64_t)(ht >> 32), keeps = (int64_t)(ht & 0xffffffffull);
-        // the smallest pair is always mutual, so an iteration without a merge
-        // means the device state is corrupt
-        if (merges < 1 || keeps != n - merges || created + merges > N - 1) {
+        // the smallest pair is always mutual, so a round without a merge means
+        // the device state is corrupt
+        if (h.stalled || h.n < 1 || h.n >= n0 || h.n + h.created != N) {
             set_error("BVH build: clustering made no progress");
             return RCP_ERR_STATE;
         }
-        const int node_base = (int)(N - 1 - created - merges);
-        k_ploc_merge<<<grid_for(n, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(nn.p, n, flags.p, rin, lin, hin,
-                                                                             node_base, rout, lout, hout, child,
-                                                                             blo, bhi, cnt.p, parent_int,
-                                                                             parent_leaf);
-        created += merges;
-        n = keeps;
-        std::swap(rin, rout);
-        std::swap(lin, lout);
-        std::swap(hin, hout);
+    }
+    RCP_CUDA(cudaFuncSetAttribute(k_ploc_last, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(PlocLastShared)));
+    k_ploc_last<<<1, PLOC_LAST_BLOCK, sizeof(PlocLastShared), st>>>(state.p, N, rin, lin, hin, tree);
+    RCP_CUDA(cudaGetLastError());
+    RCP_CUDA(cudaMemcpyAsync(&h, state.p + 1, sizeof(h), cudaMemcpyDeviceToHost, st));
+    RCP_CUDA(cudaStreamSynchronize(st));
+    if (h.stalled || h.n != 1 || h.created != N - 1) {
+        set_error("BVH build: clustering made no progress");
+        return RCP_ERR_STATE;
     }
     k_dfs_offsets<<<grid_for(2 * N - 1, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(child, parent_int, parent_leaf,
                                                                                  cnt.p, N, range, pos.p, d_err);
