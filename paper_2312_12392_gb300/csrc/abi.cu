@@ -108,19 +108,14 @@ rcp_status cuda_fail(cudaError_t e, const char* what) {
 
 RenderCtx::~RenderCtx() {
     if (graph) cudaGraphExecDestroy(graph);
-    for (auto* p : img)
-        if (p) cudaFree(p);
+    if (img[0]) cudaFree(img[0]);
     if (rays) cudaFree(rays);
-    if (d_views) cudaFree(d_views);
+    if (block) cudaFree(block);
     if (h_views) cudaFreeHost(h_views);
-    if (d_work) cudaFree(d_work);
-    if (d_status) cudaFree(d_status);
     if (d_rgb) cudaFree(d_rgb);
-    if (d_rays) cudaFree(d_rays);
     if (io) cudaFree(io);
     if (io_prim) cudaFree(io_prim);
     if (base_img) cudaFree(base_img);
-    if (hints) cudaFree(hints);
     if (done) {
         cudaEventSynchronize(done);
         cudaEventDestroy(done);
@@ -132,8 +127,7 @@ RenderCtx::~RenderCtx() {
 
 Scene::~Scene() {
     ctx.clear();
-    for (void* p : {(void*)d_tri, (void*)d_sph, (void*)d_albedo, d_nodes, (void*)d_nbox, (void*)d_prims,
-                    (void*)d_refbox, (void*)d_part_uv, (void*)d_rec_id, (void*)d_rbox, (void*)d_dev,
+    for (void* p : {(void*)d_store, d_nodes, (void*)d_prims, (void*)d_refbox, (void*)d_part_uv, (void*)d_rbox,
                     (void*)d_spill})
         if (p) cudaFree(p);
 }
@@ -380,8 +374,7 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
         *out = it->second.get();
         return RCP_OK;
     }
-    const int64_t need =
-        total_pix * (int64_t)(sizeof(float4) * 2 + sizeof(int2)) + (int64_t)sizeof(ViewDev) * K * n_views;
+    const int64_t need = total_pix * (int64_t)sizeof(int2) + (int64_t)sizeof(ViewDev) * K * n_views;
     for (;;) {
         int64_t held = 0;
         for (auto& kv : sc.ctx) held += kv.second->bytes;
@@ -399,17 +392,17 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
     c->total_chunks = total_chunks;
     c->bytes = need;
     c->last_use = ++sc.use_clock;
-    RCP_CUDA(cudaMalloc((void**)&c->img[0], sizeof(float4) * total_pix));
-    RCP_CUDA(cudaMalloc((void**)&c->img[1], sizeof(float4) * total_pix));
-    RCP_CUDA(cudaMalloc((void**)&c->hints, sizeof(int2) * total_pix));
+    // one allocation: counters and status, view descriptors, hints
+    const size_t head = 256, views = (sizeof(ViewDev) * (size_t)K * n_views + 255) & ~(size_t)255;
+    RCP_CUDA(cudaMalloc((void**)&c->block, head + views + sizeof(int2) * total_pix));
+    c->d_rays = (unsigned long long*)c->block;
+    c->d_work = (unsigned*)(c->d_rays + 2);  // K + 1 <= 17 counters
+    c->d_status = (int*)(c->block + head) - 4;
+    c->d_views = (ViewDev*)(c->block + head);
+    c->hints = (int2*)(c->block + head + views);
+    RCP_CUDA(cudaMemset(c->block, 0, head));
     RCP_CUDA(cudaMemset(c->hints, 0xff, sizeof(int2) * total_pix));  // -1: no earlier hit
-    RCP_CUDA(cudaMalloc((void**)&c->d_views, sizeof(ViewDev) * (size_t)K * n_views));
     RCP_CUDA(cudaMallocHost((void**)&c->h_views, sizeof(ViewDev) * (size_t)K * n_views));
-    RCP_CUDA(cudaMalloc((void**)&c->d_work, sizeof(unsigned) * (K + 1)));
-    RCP_CUDA(cudaMalloc((void**)&c->d_status, sizeof(int) * 4));
-    RCP_CUDA(cudaMemset(c->d_status, 0, sizeof(int) * 4));
-    RCP_CUDA(cudaMalloc((void**)&c->d_rays, sizeof(unsigned long long) * 2));
-    RCP_CUDA(cudaMemset(c->d_rays, 0, sizeof(unsigned long long) * 2));
     RCP_CUDA(cudaEventCreateWithFlags(&c->staged, cudaEventDisableTiming));
     RCP_CUDA(cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming));
     for (int n = 0; n <= K; ++n) RCP_CUDA(cudaEventCreate(&c->pass_ev[n]));
@@ -426,8 +419,7 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     auto record = [&](cudaEvent_t e) {
         return capturing ? cudaEventRecordWithFlags(e, st, cudaEventRecordExternal) : cudaEventRecord(e, st);
     };
-    RCP_CUDA(cudaMemsetAsync(ctx.d_work, 0, sizeof(unsigned) * (ctx.K + 1), st));
-    RCP_CUDA(cudaMemsetAsync(ctx.d_rays, 0, sizeof(unsigned long long) * 2, st));
+    RCP_CUDA(cudaMemsetAsync(ctx.d_rays, 0, sizeof(unsigned long long) * 2 + sizeof(unsigned) * (ctx.K + 1), st));
     const SceneDev S = sc.dev();
     RCP_CUDA(record(ctx.pass_ev[0]));
     if (ctx.chained) {  // one descriptor per view, all K passes (image mode: pass 1, then the gathers' descriptors)
@@ -459,11 +451,23 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     return RCP_OK;
 }
 
-// Run the K passes through the context's CUDA graph (captured on first use or
-// when the launch configuration changes).
+// Run the K passes through the context's CUDA graph, captured when a launch
+// configuration comes a second time: the first time its launches are enqueued
+// directly, since capturing and instantiating a graph takes longer than the
+// few launches of a frame that may be the only one of its shape. On a stream
+// that is itself being captured the graph is used from the start.
 rcp_status run_graph(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cudaStream_t st) {
     const std::string key = cfg_key(cfg) + (ctx.image_mode ? "/image" : "/trace") + (ctx.chained ? "/chain" : "");
     if (!ctx.graph || ctx.graph_key != key) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+        if (capture == cudaStreamCaptureStatusNone && ctx.seen_key != key) {
+            ctx.seen_key = key;
+            rcp_status r = enqueue_passes(sc, ctx, cfg, nullptr, st, false);
+            if (r != RCP_OK) return r;
+            RCP_CUDA(cudaEventRecord(ctx.done, st));
+            return RCP_OK;
+        }
         if (ctx.graph) {
             cudaGraphExecDestroy(ctx.graph);
             ctx.graph = nullptr;
@@ -485,6 +489,16 @@ rcp_status run_graph(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cuda
     }
     RCP_CUDA(cudaGraphLaunch(ctx.graph, st));
     RCP_CUDA(cudaEventRecord(ctx.done, st));
+    return RCP_OK;
+}
+
+// The context's ping-pong images: renders of several launches, and inputs and
+// outputs that the caller leaves to the library. A chained render has none.
+rcp_status ensure_img(RenderCtx& ctx) {
+    if (ctx.img[0]) return RCP_OK;
+    RCP_CUDA(cudaMalloc((void**)&ctx.img[0], sizeof(float4) * 2 * ctx.total_pix));
+    ctx.img[1] = ctx.img[0] + ctx.total_pix;
+    ctx.bytes += (int64_t)sizeof(float4) * 2 * ctx.total_pix;
     return RCP_OK;
 }
 
@@ -530,6 +544,10 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
                                  cudaMemcpyHostToDevice, st));
         RCP_CUDA(cudaEventRecord(ctx.staged, st));
         return RCP_OK;
+    }
+    if (K > 1) {
+        rcp_status r = ensure_img(ctx);
+        if (r != RCP_OK) return r;
     }
     for (int n = 0; n < K; ++n) {
         for (int i = 0; i < nv; ++i) {
@@ -676,19 +694,21 @@ rcp_status rcp_scene_create_ex(const float* tri, int64_t T, const float* sph, in
     sc->S = S;
     const int64_t N = T + S;
     cudaStream_t st = lib_stream();
-    RCP_CUDA(cudaMalloc((void**)&sc->d_tri, sizeof(float) * 9 * (T ? T : 1)));
-    RCP_CUDA(cudaMalloc((void**)&sc->d_sph, sizeof(float) * 4 * (S ? S : 1)));
-    RCP_CUDA(cudaMalloc((void**)&sc->d_albedo, sizeof(float4) * (N ? N : 1)));
+    // one allocation, each part on a 256-byte boundary
+    const auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t tri_b = pad(sizeof(float) * 9 * T), sph_b = pad(sizeof(float) * 4 * S), alb_b = pad(sizeof(float4) * N);
+    RCP_CUDA(cudaMalloc((void**)&sc->d_store, tri_b + sph_b + alb_b + sizeof(SceneDev)));
+    sc->d_tri = (float*)sc->d_store;
+    sc->d_sph = (float*)(sc->d_store + tri_b);
+    sc->d_albedo = (float4*)(sc->d_store + tri_b + sph_b);
+    sc->d_dev = (SceneDev*)(sc->d_store + tri_b + sph_b + alb_b);
     if (T) RCP_CUDA(cudaMemcpyAsync(sc->d_tri, tri, sizeof(float) * 9 * T, cudaMemcpyHostToDevice, st));
     if (S) RCP_CUDA(cudaMemcpyAsync(sc->d_sph, sph, sizeof(float) * 4 * S, cudaMemcpyHostToDevice, st));
     // finite coordinates are checked, and the albedo widened to a float4 per
     // primitive, on the device: one host thread took 4.4 ms over a million
     // triangles for the two, these kernels and the 12 MB upload 0.2 ms
-    DevBuf<float> alb;
-    RCP_CUDA(alb.alloc(3 * N));
-    if (N) RCP_CUDA(cudaMemcpyAsync(alb.p, albedo, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, st));
     bool bad_tri = false, bad_sph = false;
-    rcp_status r = ingest_scene(*sc, alb.p, &bad_tri, &bad_sph, st);
+    rcp_status r = ingest_scene(*sc, albedo, &bad_tri, &bad_sph, st);
     if (r != RCP_OK) return r;
     if (bad_tri || bad_sph) {
         set_error(bad_tri ? "rcp_scene_create: non-finite vertex" : "rcp_scene_create: non-finite sphere");
@@ -715,7 +735,6 @@ rcp_status rcp_scene_create_ex(const float* tri, int64_t T, const float* sph, in
     r = validate_bvh(*sc, st);
     if (r != RCP_OK) return r;
     const SceneDev dv = sc->dev();
-    RCP_CUDA(cudaMalloc((void**)&sc->d_dev, sizeof(SceneDev)));
     RCP_CUDA(cudaMemcpy(sc->d_dev, &dv, sizeof(SceneDev), cudaMemcpyHostToDevice));
     *out = sc.release();
     return RCP_OK;
@@ -889,6 +908,10 @@ rcp_status rcp_render_pass(const rcp_scene* csc, const rcp_camera* cam, int W, i
     if (r != RCP_OK) return r;
     // I_{n-1} goes to ctx->img[1] (unused by a one-pass render) and I_n to
     // ctx->io: separate buffers, since jittered samples read neighbouring pixels
+    if (in_rgbz) {
+        r = ensure_img(*ctx);
+        if (r != RCP_OK) return r;
+    }
     if (in_rgbz) RCP_CUDA(cudaMemcpyAsync(ctx->img[1], in_rgbz, sizeof(float4) * P, cudaMemcpyHostToDevice, st));
     const float4* ins[1] = {in_rgbz ? ctx->img[1] : nullptr};
     float4* outs[1] = {ctx->io};
@@ -967,6 +990,10 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     int64_t tp, tc;
     layout_views(base, tp, tc);
     const float4* ins[1] = {(const float4*)d_in};
+    if (!d_out) {
+        r = ensure_img(*ctx);
+        if (r != RCP_OK) return r;
+    }
     float4* outs[1] = {d_out ? (float4*)d_out : ctx->img[0]};
     r = stage_views(*ctx, base, ins, outs, nullptr, nullptr, st);
     if (r != RCP_OK) return r;

@@ -1540,25 +1540,25 @@ void scan_u64(unsigned long long* d, int64_t n, unsigned long long* aux, const s
 // leaves renumbered depth-first: ids_out[j] is the primitive of leaf j.
 rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, const float4* plo, const float4* phi,
                       int2* child, int2* range, float4* blo, float4* bhi, int* parent_int, int* parent_leaf,
-                      int* d_err, int cap, cudaStream_t st) {
-    DevBuf<int> ref_a, ref_b, nn, cnt, pos;
-    DevBuf<float4> lo_a, hi_a, lo_b, hi_b;
+                      int* d_err, int cap, Arena& arena, cudaStream_t st) {
+    Carved<int> ref_a, ref_b, nn, cnt, pos;
+    Carved<float4> lo_a, hi_a, lo_b, hi_b;
     // per batch of PLOC_BATCH rounds: the rounds' states, tile counters and tile status
     constexpr int PLOC_BATCH = 4;
-    DevBuf<PlocState> state;
-    DevBuf<unsigned long long> marks;
+    Carved<PlocState> state;
+    Carved<unsigned long long> marks;
     const int64_t tiles_max = (N + PLOC_TILE - 1) / PLOC_TILE;
-    RCP_CUDA(ref_a.alloc(N));
-    RCP_CUDA(ref_b.alloc(N));
-    RCP_CUDA(nn.alloc(N));
-    RCP_CUDA(cnt.alloc(N));
-    RCP_CUDA(pos.alloc(N));
-    RCP_CUDA(lo_a.alloc(N));
-    RCP_CUDA(hi_a.alloc(N));
-    RCP_CUDA(lo_b.alloc(N));
-    RCP_CUDA(hi_b.alloc(N));
-    RCP_CUDA(state.alloc(PLOC_BATCH + 2));
-    RCP_CUDA(marks.alloc(PLOC_BATCH * (1 + tiles_max)));
+    RCP_CUDA(ref_a.alloc(arena, N));
+    RCP_CUDA(ref_b.alloc(arena, N));
+    RCP_CUDA(nn.alloc(arena, N));
+    RCP_CUDA(cnt.alloc(arena, N));
+    RCP_CUDA(pos.alloc(arena, N));
+    RCP_CUDA(lo_a.alloc(arena, N));
+    RCP_CUDA(hi_a.alloc(arena, N));
+    RCP_CUDA(lo_b.alloc(arena, N));
+    RCP_CUDA(hi_b.alloc(arena, N));
+    RCP_CUDA(state.alloc(arena, PLOC_BATCH + 2));
+    RCP_CUDA(marks.alloc(arena, PLOC_BATCH * (1 + tiles_max)));
     RCP_CUDA(cudaMemsetAsync(parent_int, 0xff, sizeof(int) * N, st));
     RCP_CUDA(cudaMemsetAsync(parent_leaf, 0xff, sizeof(int) * N, st));
     int *rin = ref_a.p, *rout = ref_b.p;
@@ -1608,7 +1608,7 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
                                                                                  cnt.p, N, range, pos.p, d_err);
     k_dfs_apply<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(pos.p, ids_in, N, ids_out, child, d_err);
     RCP_CUDA(cudaGetLastError());
-    // the scratch above is freed on return: finish using it first
+    // the scratch above is given back by the caller: finish using it first
     RCP_CUDA(cudaStreamSynchronize(st));
     return RCP_OK;
 }
@@ -1619,8 +1619,13 @@ rcp_status ingest_scene(Scene& sc, const float* albedo3, bool* bad_tri, bool* ba
     const int64_t N = sc.T + sc.S;
     *bad_tri = *bad_sph = false;
     if (N == 0) return RCP_OK;
-    DevBuf<int> bad;
-    RCP_CUDA(bad.alloc(2));
+    Arena arena;
+    Carved<float> raw;
+    Carved<int> bad;
+    RCP_CUDA(arena.reserve(sizeof(float) * 3 * N + 1024));
+    RCP_CUDA(raw.alloc(arena, 3 * N));
+    RCP_CUDA(bad.alloc(arena, 2));
+    RCP_CUDA(cudaMemcpyAsync(raw.p, albedo3, sizeof(float) * 3 * N, cudaMemcpyHostToDevice, st));
     RCP_CUDA(cudaMemsetAsync(bad.p, 0, 2 * sizeof(int), st));
     int sms = 148, dev = 0;
     cudaGetDevice(&dev);
@@ -1628,7 +1633,7 @@ rcp_status ingest_scene(Scene& sc, const float* albedo3, bool* bad_tri, bool* ba
     k_any_non_finite<<<grid_for(9 * sc.T / 4 + 1, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(sc.d_tri, 9 * sc.T,
                                                                                                 bad.p);
     k_any_non_finite<<<grid_for(sc.S + 1, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(sc.d_sph, 4 * sc.S, bad.p + 1);
-    k_widen_albedo<<<grid_for(N, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(albedo3, N, sc.d_albedo);
+    k_widen_albedo<<<grid_for(N, BUILD_BLOCK, sms * 8), BUILD_BLOCK, 0, st>>>(raw.p, N, sc.d_albedo);
     int h[2];
     RCP_CUDA(cudaMemcpyAsync(h, bad.p, sizeof(h), cudaMemcpyDeviceToHost, st));
     RCP_CUDA(cudaStreamSynchronize(st));
@@ -1649,29 +1654,39 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
     const int cap = sms * 16;
-    DevBuf<float4> plo, phi;
-    DevBuf<uint32_t> bounds;
-    RCP_CUDA(plo.alloc(N));
-    RCP_CUDA(phi.alloc(N));
-    RCP_CUDA(bounds.alloc(12));
+    const bool split = sc.split_max > 1 && T > 0, sah = sah;
+    // Temporaries in one allocation: 32 bytes per primitive (48 when split),
+    // and per reference 72 that live through the build, then the clustering's
+    // 84 or what follows it (the slot costs' 40 under the surface-area policy,
+    // arrivals and frontiers 8, and the nodes' first estimate, one per five
+    // references at 336 bytes), whichever is more.
+    const auto per_reference = [&](int64_t refs) {
+        return (size_t)refs * (72 + std::max(84, 8 + (sah ? 40 : 0) + 68)) + radix_sort_scratch_bytes(refs) + (1 << 20);
+    };
+    Arena arena;
+    RCP_CUDA(arena.reserve(split ? (size_t)N * 48 + (1 << 20) : (size_t)N * 32 + per_reference(N)));
+    Carved<float4> plo, phi;
+    Carved<uint32_t> bounds;
+    RCP_CUDA(plo.alloc(arena, N));
+    RCP_CUDA(phi.alloc(arena, N));
+    RCP_CUDA(bounds.alloc(arena, 12));
     k_init_bounds<<<1, 32, 0, st>>>(bounds.p);
     k_prim_bounds<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(sc.d_tri, sc.d_sph, T, N, plo.p, phi.p,
                                                                           bounds.p);
     // references: the primitives themselves, or split triangles (R >= N)
     int64_t R = N;
-    DevBuf<float4> rlo, rhi;
-    DevBuf<uint32_t> rprim;
+    Carved<float4> rlo, rhi;
+    Carved<uint32_t> rprim;
     const float4* ref_lo = plo.p;
     const float4* ref_hi = phi.p;
-    const bool split = sc.split_max > 1 && T > 0;
     if (split) {
-        DevBuf<unsigned long long> counts, aux, total;
+        Carved<unsigned long long> counts, aux, total;
         const std::vector<int64_t> lv = scan_levels(N);
         int64_t aux_n = 0;
         for (int64_t t : lv) aux_n += t;
-        RCP_CUDA(counts.alloc(N));
-        RCP_CUDA(aux.alloc(aux_n));
-        RCP_CUDA(total.alloc(1));
+        RCP_CUDA(counts.alloc(arena, N));
+        RCP_CUDA(aux.alloc(arena, aux_n));
+        RCP_CUDA(total.alloc(arena, 1));
         k_split_count<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(sc.d_tri, T, N, sc.split_max,
                                                                               counts.p);
         scan_u64(counts.p, N, aux.p, lv, 0, total.p, st);
@@ -1683,17 +1698,18 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
             set_error("BVH build: split references out of range (at most 2^30 - 1)");
             return RCP_ERR_ARG;
         }
-        RCP_CUDA(rlo.alloc(R));
-        RCP_CUDA(rhi.alloc(R));
-        RCP_CUDA(rprim.alloc(R));
-        DevBuf<int> split_err;
-        RCP_CUDA(split_err.alloc(1));
+        RCP_CUDA(arena.reserve((size_t)R * 36 + per_reference(R)));
+        RCP_CUDA(rlo.alloc(arena, R));
+        RCP_CUDA(rhi.alloc(arena, R));
+        RCP_CUDA(rprim.alloc(arena, R));
+        Carved<int> split_err;
+        RCP_CUDA(split_err.alloc(arena, 1));
         RCP_CUDA(cudaMemsetAsync(split_err.p, 0, sizeof(int), st));
         k_split_write<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(
             sc.d_tri, T, N, sc.split_max, counts.p, R, plo.p, phi.p, rlo.p, rhi.p, rprim.p, split_err.p);
         int h_err = 0;
         RCP_CUDA(cudaMemcpyAsync(&h_err, split_err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-        RCP_CUDA(cudaStreamSynchronize(st));  // counts and aux are freed on leaving this block
+        RCP_CUDA(cudaStreamSynchronize(st));
         if (h_err) {
             set_error("BVH build: split references counted and written differently");
             return RCP_ERR_STATE;
@@ -1701,32 +1717,25 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
         ref_lo = rlo.p;
         ref_hi = rhi.p;
     }
-    const int64_t n_nodes_cap = R > 1 ? R : 1;
-    DevBuf<float4> blo, bhi;
-    DevBuf<uint32_t> keys, vals, akeys, avals, counters;
-    DevBuf<int2> child, range, fa, fb;
-    DevBuf<int> parent_int, parent_leaf, err;
-    DevBuf<char> scratch;
-    RCP_CUDA(keys.alloc(R));
-    RCP_CUDA(vals.alloc(R));
-    RCP_CUDA(akeys.alloc(R));
-    RCP_CUDA(avals.alloc(R));
-    RCP_CUDA(counters.alloc(4));
-    RCP_CUDA(err.alloc(2));
-    RCP_CUDA(child.alloc(R));
-    RCP_CUDA(range.alloc(R));
-    RCP_CUDA(blo.alloc(R));
-    RCP_CUDA(bhi.alloc(R));
-    RCP_CUDA(parent_int.alloc(R));
-    RCP_CUDA(parent_leaf.alloc(R));
-    RCP_CUDA(fa.alloc(n_nodes_cap));
-    RCP_CUDA(fb.alloc(n_nodes_cap));
-    RCP_CUDA(scratch.alloc(radix_sort_scratch_bytes(R)));
-    // outputs sized for the worst case, trimmed at the end
-    DevBuf<WNode> nodes_full;
-    DevBuf<float4> nbox_full, prims, rec_box;
-    RCP_CUDA(nodes_full.alloc(n_nodes_cap));
-    RCP_CUDA(nbox_full.alloc(2 * n_nodes_cap));
+    Carved<float4> blo, bhi;
+    Carved<uint32_t> keys, vals, akeys, avals, counters;
+    Carved<int2> child, range, fa, fb;
+    Carved<int> parent_int, parent_leaf, err;
+    Carved<char> scratch;
+    RCP_CUDA(keys.alloc(arena, R));
+    RCP_CUDA(vals.alloc(arena, R));
+    RCP_CUDA(akeys.alloc(arena, R));
+    RCP_CUDA(avals.alloc(arena, R));
+    RCP_CUDA(counters.alloc(arena, 4));
+    RCP_CUDA(err.alloc(arena, 2));
+    RCP_CUDA(child.alloc(arena, R));
+    RCP_CUDA(range.alloc(arena, R));
+    RCP_CUDA(blo.alloc(arena, R));
+    RCP_CUDA(bhi.alloc(arena, R));
+    RCP_CUDA(parent_int.alloc(arena, R));
+    RCP_CUDA(parent_leaf.alloc(arena, R));
+    RCP_CUDA(scratch.alloc(arena, radix_sort_scratch_bytes(R)));
+    DevBuf<float4> prims, rec_box;  // the scene's own
     RCP_CUDA(prims.alloc(3 * R));
     if (split) RCP_CUDA(rec_box.alloc(2 * R));
     RCP_CUDA(cudaMemsetAsync(err.p, 0, 2 * sizeof(int), st));
@@ -1735,9 +1744,9 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
     rcp_status rs = radix_sort_pairs(keys.p, vals.p, akeys.p, avals.p, R, 30, scratch.p, err.p, st);
     if (rs != RCP_OK) return rs;
     uint32_t* ids = vals.p;  // reference indices in leaf order (Morton order, then depth-first)
-    DevBuf<float4> dp;
-    DevBuf<uint2> slot_split;
-    DevBuf<int> arrivals;
+    Carved<float4> dp;
+    Carved<uint2> slot_split;
+    Carved<int> arrivals;
     if (R >= 2) {
         // a sort whose look-back wait ran out leaves no valid permutation to cluster
         int sort_flag = 0;
@@ -1747,8 +1756,10 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
             set_error("radix sort: look-back wait ran out");
             return RCP_ERR_TIMEOUT;
         }
+        const Arena::Mark before = arena.mark();
         rcp_status pr = build_ploc(R, vals.p, avals.p, ref_lo, ref_hi, child.p, range.p, blo.p, bhi.p, parent_int.p,
-                                   parent_leaf.p, err.p + 1, cap, st);
+                                   parent_leaf.p, err.p + 1, cap, arena, st);
+        arena.release(before);
         if (pr != RCP_OK) {
             return pr;
         }
@@ -1756,15 +1767,15 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
     }
     if (R >= 2) {
         // node boxes from the padded leaves (the clustering used exact boxes)
-        RCP_CUDA(arrivals.alloc(R - 1));
+        RCP_CUDA(arrivals.alloc(arena, R - 1));
         RCP_CUDA(cudaMemsetAsync(arrivals.p, 0, sizeof(int) * (R - 1), st));
         k_refit_padded<<<grid_for(R, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(
             child.p, parent_int.p, parent_leaf.p, ids, ref_lo, ref_hi, split ? rprim.p : nullptr, sc.d_tri,
             sc.d_sph, T, R, blo.p, bhi.p, arrivals.p, err.p + 1);
     }
-    if (R >= 2 && sc.collapse == RCP_COLLAPSE_SAH) {
-        RCP_CUDA(dp.alloc(2 * (R - 1)));
-        RCP_CUDA(slot_split.alloc(R - 1));
+    if (R >= 2 && sah) {
+        RCP_CUDA(dp.alloc(arena, 2 * (R - 1)));
+        RCP_CUDA(slot_split.alloc(arena, R - 1));
         RCP_CUDA(cudaMemsetAsync(arrivals.p, 0, sizeof(int) * (R - 1), st));
         k_sah_dp<<<grid_for(R, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(child.p, range.p, parent_int.p,
                                                                          parent_leaf.p, blo.p, bhi.p, ref_lo, ref_hi,
@@ -1796,6 +1807,17 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
     std::vector<int64_t> level_begin;
     int depth = 0;
     int64_t n_nodes = 0;
+    // Nodes (and their boxes) as the collapse numbers them. A level's launch
+    // writes the nodes numbered before it, so there is room for those by then.
+    // An internal child holds LEAF_MAX + 1 references or more, which bounds a
+    // frontier.
+    Carved<WNode> nodes_full;
+    Carved<float4> nbox_full;
+    int64_t node_cap = R / 5 + 64;
+    RCP_CUDA(fa.alloc(arena, R / (LEAF_MAX + 1) + 1));
+    RCP_CUDA(fb.alloc(arena, R / (LEAF_MAX + 1) + 1));
+    RCP_CUDA(nodes_full.alloc(arena, node_cap));
+    RCP_CUDA(nbox_full.alloc(arena, 2 * node_cap));
     if (N > 0) {
         int2 root = make_int2(R >= 2 ? 0 : -1, 0);
         RCP_CUDA(cudaMemcpyAsync(fa.p, &root, sizeof(int2), cudaMemcpyHostToDevice, st));
@@ -1815,7 +1837,7 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
         }
         RCP_CUDA(cudaMemsetAsync(d_max_leaf, 0, sizeof(int), st));
         BinTree bt{child.p, range.p, blo.p, bhi.p, ref_lo, ref_hi, ids,
-                   sc.collapse == RCP_COLLAPSE_SAH ? slot_split.p : nullptr, split ? rprim.p : nullptr, sc.d_tri,
+                   sah ? slot_split.p : nullptr, split ? rprim.p : nullptr, sc.d_tri,
                    sc.d_sph, T};
         int n_front = 1;
         int64_t begin = 0;
@@ -1839,35 +1861,32 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
             n_front = (int)hc[2];
             n_nodes = hc[0];
             std::swap(cur, nxt);
+            if (n_nodes > node_cap) {  // the written nodes move to a larger array
+                node_cap = std::max(2 * node_cap, n_nodes);
+                Carved<WNode> more;
+                Carved<float4> more_box;
+                RCP_CUDA(more.alloc(arena, node_cap));
+                RCP_CUDA(more_box.alloc(arena, 2 * node_cap));
+                RCP_CUDA(cudaMemcpyAsync(more.p, nodes_full.p, sizeof(WNode) * begin, cudaMemcpyDeviceToDevice, st));
+                RCP_CUDA(cudaMemcpyAsync(more_box.p, nbox_full.p, sizeof(float4) * 2 * begin, cudaMemcpyDeviceToDevice,
+                                         st));
+                nodes_full = more;
+                nbox_full = more_box;
+            }
         }
         level_begin.push_back(begin);
         RCP_CUDA(cudaMemcpyAsync(&sc.max_leaf, d_max_leaf, sizeof(int), cudaMemcpyDeviceToHost, st));
     }
     // the parts of split references, for refits
-    DevBuf<uint32_t> part_uv, rec_id;
+    DevBuf<uint32_t> parts;  // PART_MAX words per record, then the records' ids
     if (split) {
-        RCP_CUDA(part_uv.alloc(PART_MAX * R));
-        RCP_CUDA(rec_id.alloc(R));
+        RCP_CUDA(parts.alloc((PART_MAX + 1) * R));
         k_record_parts<<<grid_for(R, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(prims.p, R, rec_box.p, sc.d_tri, T,
-                                                                               part_uv.p, rec_id.p);
+                                                                               parts.p, parts.p + PART_MAX * R);
     }
     // trim the node arrays to size
-    if (sc.d_nodes) cudaFree(sc.d_nodes);
-    if (sc.d_nbox) cudaFree(sc.d_nbox);
-    if (sc.d_prims) cudaFree(sc.d_prims);
-    if (sc.d_refbox) cudaFree(sc.d_refbox);
-    if (sc.d_part_uv) cudaFree(sc.d_part_uv);
-    if (sc.d_rec_id) cudaFree(sc.d_rec_id);
-    if (sc.d_rbox) cudaFree(sc.d_rbox);
-    sc.d_rbox = nullptr;
-    sc.d_part_uv = nullptr;
-    sc.d_rec_id = nullptr;
-    sc.d_nodes = nullptr;
-    sc.d_nbox = nullptr;
-    sc.d_prims = nullptr;
-    sc.d_refbox = nullptr;
-    RCP_CUDA(cudaMalloc((void**)&sc.d_nodes, sizeof(WNode) * (n_nodes ? n_nodes : 1)));
-    RCP_CUDA(cudaMalloc((void**)&sc.d_nbox, sizeof(float4) * 2 * (n_nodes ? n_nodes : 1)));
+    RCP_CUDA(cudaMalloc((void**)&sc.d_nodes, (sizeof(WNode) + sizeof(float4) * 2) * (n_nodes ? n_nodes : 1)));
+    sc.d_nbox = (float4*)((WNode*)sc.d_nodes + n_nodes);
     if (n_nodes) {
         RCP_CUDA(cudaMemcpyAsync(sc.d_nodes, nodes_full.p, sizeof(WNode) * n_nodes, cudaMemcpyDeviceToDevice, st));
         RCP_CUDA(cudaMemcpyAsync(sc.d_nbox, nbox_full.p, sizeof(float4) * 2 * n_nodes, cudaMemcpyDeviceToDevice,
@@ -1877,8 +1896,8 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
     RCP_CUDA(cudaStreamSynchronize(st));
     sc.d_prims = prims.release();
     sc.d_refbox = rec_box.release();
-    sc.d_part_uv = part_uv.release();
-    sc.d_rec_id = rec_id.release();
+    sc.d_part_uv = parts.release();
+    sc.d_rec_id = sc.d_part_uv ? sc.d_part_uv + PART_MAX * R : nullptr;
     sc.n_records = R;
     sc.n_nodes = n_nodes;
     sc.depth = depth;
@@ -1927,24 +1946,19 @@ rcp_status refit_bvh(Scene& sc, cudaStream_t st) {
 rcp_status validate_bvh(const Scene& sc, cudaStream_t st) {
     const int64_t N = sc.T + sc.S, R = sc.n_records;
     if (N == 0) return RCP_OK;
-    DevBuf<unsigned> seen_rec, seen_id, node_refs;
-    DevBuf<int> errors;
-    RCP_CUDA(seen_rec.alloc(R));
-    RCP_CUDA(seen_id.alloc(N));
-    RCP_CUDA(node_refs.alloc(sc.n_nodes));
-    RCP_CUDA(errors.alloc(8));
-    RCP_CUDA(cudaMemsetAsync(seen_rec.p, 0, sizeof(unsigned) * R, st));
-    RCP_CUDA(cudaMemsetAsync(seen_id.p, 0, sizeof(unsigned) * N, st));
-    RCP_CUDA(cudaMemsetAsync(node_refs.p, 0, sizeof(unsigned) * sc.n_nodes, st));
-    RCP_CUDA(cudaMemsetAsync(errors.p, 0, sizeof(int) * 8, st));
+    DevBuf<unsigned> words;  // per record, per primitive and per node its references counted, then the errors
+    RCP_CUDA(words.alloc(R + N + sc.n_nodes + 8));
+    RCP_CUDA(cudaMemsetAsync(words.p, 0, sizeof(unsigned) * (R + N + sc.n_nodes + 8), st));
+    unsigned *seen_rec = words.p, *seen_id = seen_rec + R, *node_refs = seen_id + N;
+    int* errors = (int*)(node_refs + sc.n_nodes);
     k_validate<<<(int)((sc.n_nodes + 127) / 128), 128, 0, st>>>((const WNode*)sc.d_nodes, sc.n_nodes, sc.d_nbox,
                                                                  sc.d_prims, R, N, sc.d_refbox,
                                                                  Parts{sc.d_part_uv, sc.d_rec_id}, sc.d_tri, sc.d_sph,
-                                                                 sc.T, seen_rec.p, seen_id.p, node_refs.p, errors.p);
+                                                                 sc.T, seen_rec, seen_id, node_refs, errors);
     k_check_counts<<<grid_for(std::max<int64_t>(std::max(R, N), sc.n_nodes), 256, 4096), 256, 0, st>>>(
-        seen_rec.p, R, seen_id.p, N, sc.split_max > 1, node_refs.p, sc.n_nodes, errors.p);
+        seen_rec, R, seen_id, N, sc.split_max > 1, node_refs, sc.n_nodes, errors);
     int h[8];
-    RCP_CUDA(cudaMemcpyAsync(h, errors.p, sizeof(h), cudaMemcpyDeviceToHost, st));
+    RCP_CUDA(cudaMemcpyAsync(h, errors, sizeof(h), cudaMemcpyDeviceToHost, st));
     RCP_CUDA(cudaStreamSynchronize(st));
     static const char* what[8] = {"slot masks",       "child index order", "child box outside slot",
                                   "leaf record range", "primitive outside leaf slot",

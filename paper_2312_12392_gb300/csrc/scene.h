@@ -22,13 +22,14 @@ struct RenderCtx {
     int K = 0;
     int64_t total_pix = 0;
     int64_t total_chunks = 0;
-    float4* img[2] = {nullptr, nullptr};
+    float4* img[2] = {nullptr, nullptr};  // from the first render that needs them (ensure_img), one allocation
+    char* block = nullptr;  // one allocation: d_views, d_work, d_rays, d_status and hints
     float4* rays = nullptr;
     ViewDev* d_views = nullptr;  // K * n_views
     ViewDev* h_views = nullptr;  // pinned staging
     unsigned* d_work = nullptr;  // one work counter per launch
     int* d_status = nullptr;     // [0] stack overflow
-    unsigned long long* d_rays = nullptr;  // rays traced by the last render: primary, shadow
+    unsigned long long* d_rays = nullptr;  // rays of the last render: primary, shadow (right before d_work)
     float* d_rgb = nullptr;      // packed RGB for host output
     float4* io = nullptr;        // host-API input / final image
     float4* base_img = nullptr;  // image-space mapping: the traced pass-1 image
@@ -41,7 +42,7 @@ struct RenderCtx {
     cudaEvent_t pass_ev[17] = {};  // timing events around every launch (recorded inside the graph)
     int launches = 0;              // launches of the latest enqueue: K, or 1 (image mode: 2) when chained
     cudaGraphExec_t graph = nullptr;
-    std::string graph_key;
+    std::string graph_key, seen_key;  // the captured configuration; the one last enqueued directly
     cudaEvent_t done = nullptr;  // recorded after the context's latest launch
     uint64_t last_use = 0;
     int64_t bytes = 0;
@@ -50,14 +51,16 @@ struct RenderCtx {
 
 struct Scene {
     int64_t T = 0, S = 0;
+    char* d_store = nullptr;  // one allocation: triangles, spheres, albedo and the device copy of dev()
     float* d_tri = nullptr;
     float* d_sph = nullptr;
     float4* d_albedo = nullptr;
-    void* d_nodes = nullptr;  // WNode[n_nodes]
-    float4* d_nbox = nullptr;  // 2 per node: union box of the node's children
+    void* d_nodes = nullptr;  // WNode[n_nodes], then nbox
+    float4* d_nbox = nullptr;  // 2 per node: union box of the node's children (in d_nodes' allocation)
     float4* d_prims = nullptr;  // 3 per leaf record (n_records)
     float4* d_refbox = nullptr;  // 2 per record: its exact clipped box in a split build (else null)
-    uint32_t* d_part_uv = nullptr;  // split build: 9 per record, its part of its triangle as 16-bit (u, v) pairs
+    uint32_t* d_part_uv = nullptr;  // split build: 9 per record, its part of its triangle as 16-bit (u, v) pairs,
+                                    // then rec_id
     uint32_t* d_rec_id = nullptr;   // split build: each record's primitive id (with the sphere flag)
     float2* d_rbox = nullptr;       // 3 per record: padded record boxes of the latest refit (from the first refit)
     int64_t n_records = 0;       // leaf records: T + S, more when triangles are split
@@ -84,8 +87,8 @@ struct Scene {
 };
 
 // The scene's arrays as uploaded: whether every vertex and sphere is finite,
-// and d_albedo (a float4 per primitive) from 3 floats per primitive. Waits for
-// the stream.
+// and d_albedo (a float4 per primitive) from 3 floats per primitive (host).
+// Waits for the stream.
 rcp_status ingest_scene(Scene& sc, const float* albedo3, bool* bad_tri, bool* bad_sph, cudaStream_t st);
 rcp_status build_bvh(Scene& sc, cudaStream_t st);
 rcp_status refit_bvh(Scene& sc, cudaStream_t st);
