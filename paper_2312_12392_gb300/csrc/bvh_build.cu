@@ -1654,7 +1654,7 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     }
     const int cap = sms * 16;
-    const bool split = sc.split_max > 1 && T > 0, sah = sah;
+    const bool split = sc.split_max > 1 && T > 0, sah = sc.collapse == RCP_COLLAPSE_SAH;
     // Temporaries in one allocation: 32 bytes per primitive (48 when split),
     // and per reference 72 that live through the build, then the clustering's
     // 84 or what follows it (the slot costs' 40 under the surface-area policy,
