@@ -116,6 +116,7 @@ RenderCtx::~RenderCtx() {
     if (io) cudaFree(io);
     if (io_prim) cudaFree(io_prim);
     if (base_img) cudaFree(base_img);
+    if (repeat) cudaFree(repeat);
     if (done) {
         cudaEventSynchronize(done);
         cudaEventDestroy(done);
@@ -196,6 +197,7 @@ void make_view(ViewDev& v, const rcp_camera& cam, int W, int H, const rcp_params
     v.hint = nullptr;
     v.scene = nullptr;
     v.status = nullptr;
+    v.repeat = MsRepeat{};
     v.done_count = nullptr;
     v.done_flag = nullptr;
     v.tiles_x = (W + 7) / 8;
@@ -502,6 +504,35 @@ rcp_status ensure_img(RenderCtx& ctx) {
     return RCP_OK;
 }
 
+// The state of a multi-sample render that leaves out repeated tiles: two
+// passes' tile flags and shadow counts and (ids) hit ids. One allocation.
+struct RepeatLayout {
+    size_t shadow, ids, total;  // the flags come first
+};
+RepeatLayout repeat_layout(const RenderCtx& ctx, bool ids) {
+    const auto pad = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    RepeatLayout l;
+    l.shadow = pad(2 * (size_t)ctx.total_chunks);
+    l.ids = l.shadow + pad(sizeof(unsigned) * 2 * (size_t)ctx.total_chunks);
+    l.total = l.ids + (ids ? pad(sizeof(int32_t) * 2 * (size_t)ctx.total_pix) : 0);
+    return l;
+}
+
+rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
+    if (ctx.repeat && (ctx.repeat_ids || !ids)) return RCP_OK;
+    if (ctx.repeat) {
+        RCP_CUDA(cudaEventSynchronize(ctx.done));  // no launch may still use the smaller one
+        cudaFree(ctx.repeat);
+        ctx.bytes -= (int64_t)repeat_layout(ctx, ctx.repeat_ids).total;
+        ctx.repeat = nullptr;
+    }
+    const RepeatLayout l = repeat_layout(ctx, ids);
+    RCP_CUDA(cudaMalloc((void**)&ctx.repeat, l.total));
+    ctx.repeat_ids = ids;
+    ctx.bytes += (int64_t)l.total;
+    return RCP_OK;
+}
+
 // Stage the view descriptors of one render (n_views views, K passes): one per
 // view and pass, or, when the passes run chained (chain: the tuning asks for
 // it and the render allows it), one per view that runs all K passes (an
@@ -549,6 +580,15 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
         rcp_status r = ensure_img(ctx);
         if (r != RCP_OK) return r;
     }
+    bool want_ids = false;
+    for (int i = 0; prims && i < nv; ++i) want_ids = want_ids || prims[i];
+    const bool repeats = base[0].spp > 0 && K > 2;
+    RepeatLayout lay{};
+    if (repeats) {
+        rcp_status r = ensure_repeat(ctx, want_ids);
+        if (r != RCP_OK) return r;
+        lay = repeat_layout(ctx, ctx.repeat_ids);
+    }
     for (int n = 0; n < K; ++n) {
         for (int i = 0; i < nv; ++i) {
             ViewDev v = base[i];
@@ -567,6 +607,23 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
             v.status = ctx.d_status;
             v.prim = (n == K - 1 && prims && !ctx.image_mode) ? prims[i] : nullptr;
             v.rgb = (n == K - 1 && rgbs && !ctx.image_mode) ? rgbs[i] : nullptr;
+            if (repeats) {  // pass n + 1 writes its flags, counts and ids at parity n & 1
+                const int64_t tile = base[i].chunk_begin;
+                uint8_t* flags = (uint8_t*)ctx.repeat + tile;
+                unsigned* shadow = (unsigned*)(ctx.repeat + lay.shadow) + tile;
+                int32_t* ids = want_ids && prims[i] ? (int32_t*)(ctx.repeat + lay.ids) + off : nullptr;
+                const int64_t odd = n & 1, even = odd ^ 1;
+                MsRepeat& m = v.repeat;
+                m.flags_in = n > 0 ? flags + even * ctx.total_chunks : nullptr;
+                m.flags_out = flags + odd * ctx.total_chunks;
+                m.two_ago = n > 1 ? ctx.img[odd] + off : nullptr;
+                m.has_two_ago = n > 1 && n < K - 1;
+                m.ids_two_ago = ids ? ids + odd * ctx.total_pix : nullptr;
+                m.ids_before = ids ? ids + even * ctx.total_pix : nullptr;
+                m.shadow_before = shadow + even * ctx.total_chunks;
+                m.shadow = shadow + odd * ctx.total_chunks;
+                if (ids && n < K - 1) v.prim = ids + odd * ctx.total_pix;
+            }
             ctx.h_views[(size_t)n * nv + i] = v;
         }
     }

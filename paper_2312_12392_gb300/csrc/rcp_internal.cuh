@@ -67,6 +67,21 @@ struct SceneDev {
     float eps;   // 1e-4 * diameter (shadow-ray offset)
 };
 
+// Pass n of a multi-sample render of several passes: what it needs to leave
+// out the tiles whose values repeat (flags_out null: it traces every tile). A tile's flags of a pass: bit 0 = every
+// pixel equals the pass before, bit 1 = every pixel equals the pass before that
+// (all four lanes, bit for bit).
+struct MsRepeat {
+    const uint8_t* flags_in;  // pass n-1's flags per tile, nullptr in pass 1
+    uint8_t* flags_out;       // pass n's
+    int has_two_ago;          // out held I_{n-2} before this pass (n >= 3, not the last pass)
+    const float4* two_ago;    // I_{n-2} (n >= 3); the pass's own out unless it is the last pass
+    const int32_t* ids_two_ago;  // hit ids of passes n-2 and n-1 (null unless the render returns ids)
+    const int32_t* ids_before;
+    const unsigned* shadow_before;  // per tile, shadow rays of pass n-1
+    unsigned* shadow;               // per tile, of pass n-2 on entry, of pass n afterwards
+};
+
 // One view (camera + image) of a batched pass. The camera terms are
 // precomputed on the host in double and rounded once:
 //   g(x, y) = fF + (2x + 1 - W) fR + (H - 2y - 1) fU  (eye -> focal-plane point)
@@ -96,6 +111,7 @@ struct ViewDev {
     int tiles_x;
     int spp;              // samples per pixel, 0 = one at the centre
     float jit[2 * RCP_MAX_SPP];
+    MsRepeat repeat;
     int* done_count;  // nullable: tiles of this view still to finish in the launch (device)
     int* done_flag;   // set to 1 (host-visible) once they have all finished
 };

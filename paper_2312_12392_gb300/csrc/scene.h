@@ -37,6 +37,8 @@ struct RenderCtx {
     bool chained = false;        // one launch runs all K passes (one descriptor per view), or, in image mode, one
                                  // launch traces pass 1 and one gathers passes 2..K (two descriptors per view)
     int32_t* io_prim = nullptr;  // host-API hit ids
+    char* repeat = nullptr;      // multi-sample renders of 3 passes or more (ensure_repeat)
+    bool repeat_ids = false;     // with two passes' hit ids
     int2* hints = nullptr;       // per pixel: latest primary-hit and shadow-occluder records (-1 none)
     cudaEvent_t staged = nullptr;
     cudaEvent_t pass_ev[17] = {};  // timing events around every launch (recorded inside the graph)

@@ -88,6 +88,62 @@ __device__ __forceinline__ bool same_camera(int mapping, const float4& a, const 
     return (mapping == RCP_MAP_NORMAL ? w : mapping == RCP_MAP_DEPTH ? rgb | w : rgb) == 0u;
 }
 
+__device__ __forceinline__ bool same_bits(const float4& a, const float4& b) {
+    return ((__float_as_uint(a.x) ^ __float_as_uint(b.x)) | (__float_as_uint(a.y) ^ __float_as_uint(b.y)) |
+            (__float_as_uint(a.z) ^ __float_as_uint(b.z)) | (__float_as_uint(a.w) ^ __float_as_uint(b.w))) == 0u;
+}
+
+// Whether pass n of a multi-sample render repeats an earlier pass on this
+// tile, and if so its outputs. A tile's samples read the previous image within
+// one pixel of the tile, so its values are a function of the tile and its
+// eight neighbours: where all nine of them had I_{n-1} = I_{n-3}, the tile's
+// I_n is I_{n-2}, which its ping-pong buffer still holds; where all nine had
+// I_{n-1} = I_{n-2}, it is I_{n-1}, the same bits again. The last pass copies
+// them to its output. Called by the whole warp. Ray counts are those of the
+// pass repeated. On the mid terrain (720p, 4 samples, K = 6, TARGET) about a
+// quarter of all tile passes repeat, the cheaper ones, whose rays stay within a
+// triangle: a frame 3.17 -> 2.96 ms with the 24 warps per SM above.
+__device__ __forceinline__ bool repeat_tile(const ViewDev& v, int tile, int lane, uint32_t& n_primary,
+                                            uint32_t& n_shadow) {
+    const MsRepeat& m = v.repeat;
+    if (!m.flags_in) return false;
+    const int tx = tile % v.tiles_x, ty = tile / v.tiles_x, tiles_y = (v.H + 3) / 4;
+    unsigned f = 3u;  // outside the image: no constraint
+    if (lane < 9) {
+        const int x = tx + lane % 3 - 1, y = ty + lane / 3 - 1;
+        if (x >= 0 && x < v.tiles_x && y >= 0 && y < tiles_y) f = m.flags_in[(int64_t)y * v.tiles_x + x];
+    }
+    const bool two = __all_sync(0xffffffffu, f & 2u), one = __all_sync(0xffffffffu, f & 1u);
+    if (!two && !one) return false;
+    const int x = tx * 8 + (lane & 7), y = ty * 4 + (lane >> 3);
+    if (x < v.W && y < v.H) {
+        const int64_t p = (int64_t)y * v.W + x;
+        if (v.out != m.two_ago) {  // the last pass
+            const float4 c = two ? m.two_ago[p] : v.in[p];
+            v.out[p] = c;
+            if (v.rgb) {
+                v.rgb[3 * p] = c.x;
+                v.rgb[3 * p + 1] = c.y;
+                v.rgb[3 * p + 2] = c.z;
+            }
+        }
+        if (v.prim) {
+            const int32_t* ids = two ? m.ids_two_ago : m.ids_before;
+            if (v.prim != ids) v.prim[p] = ids[p];
+        }
+        n_primary += v.spp > 0 ? v.spp : 1;
+    }
+    __syncwarp();
+    if (lane == 0) {
+        const unsigned own = m.flags_in[tile];
+        m.flags_out[tile] = (uint8_t)(2u | (two ? own & 1u : 1u));
+        const unsigned sh = two ? m.shadow[tile] : m.shadow_before[tile];
+        m.shadow[tile] = sh;
+        n_shadow += sh;
+    }
+    return true;
+}
+
 // A warp counts n finished tiles of view v (with a done counter) at once:
 // every lane's writes for them made visible first, at system scope (the RGB
 // may go straight to host memory, which the host reads once the flag is set),
@@ -113,12 +169,13 @@ __device__ __forceinline__ void tiles_done(const ViewDev* v, int n, int lane) {
 // pass's outputs. At one sample per pixel with a camera that reads only the
 // pixel's own previous value (every mapping but the image-space one), this
 // computes exactly what one launch per pass computes.
-// CHAIN: 24 warps per SM (80 registers; what spills is the pixel's state
+// CHAIN and MS: 24 warps per SM (80 registers; what spills is the pixel's state
 // between passes, outside the walk). 20, 28 and 32 warps: 1.575, 1.574 and
 // 1.773 against 1.559 ms for a mid 1080p K = 6 frame, forest 1.810, 1.820 and
-// 1.983 against 1.785 ms.
+// 1.983 against 1.785 ms; 4 samples at 720p K = 6 with 16, 20, 24 and 28 warps:
+// 3.069, 3.033, 2.964 and 3.002 ms.
 template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
-__global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
+__global__ void __launch_bounds__(BLOCK, CHAIN || MS ? 768 / BLOCK : 0)
     k_trace(SceneDev S0, const ViewDev* __restrict__ views, int n_views,
                                                  int64_t total_chunks, int chunk_tiles,
                                                  const float4* __restrict__ rays, unsigned* work, StackCfg stk,
@@ -162,6 +219,10 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                 __syncwarp();
             }
             const SceneDev& S = MULTI ? s_scene[threadIdx.x >> 5] : S0;
+            if (MS && !MULTI && v.repeat.flags_out && repeat_tile(v, (int)(chunk - v.chunk_begin), lane, n_primary, n_shadow))
+                continue;
+            bool same1 = true, same2 = true;  // MS: this pixel equals the pass before, and the one before that
+            const uint32_t shadow_before = n_shadow;
             do {  // the tile's pixel of this lane ("continue" leaves the block)
                 const int64_t tile = chunk - v.chunk_begin;
                 const int tx = (int)(tile % v.tiles_x), ty = (int)(tile / v.tiles_x);
@@ -186,8 +247,6 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                         const RayF r = camera_ray(v, px, py, c, S.tmin);
                         uint32_t code;
                         int32_t prim;
-                        // the mapping is compared here: kept live across the walk it takes the kernel
-                        // from 96 to 128 registers (4 samples at 720p 3.17 against 3.44 ms)
                         const float4 o = trace_shade<COUNT, SPILL>(S, r, v.Fw, stack, BLOCK, stk, overflow, wc,
                                                             n_shadow, code, prim, s_lut, hint,
                                                             v.mapping == RCP_MAP_NORMAL);
@@ -205,6 +264,10 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                     float4 out = make_float4(__fdiv_rn(acc.x, fn), __fdiv_rn(acc.y, fn), __fdiv_rn(acc.z, fn),
                                              __fdiv_rn(acc.w, fn));
                     if (v.mapping == RCP_MAP_NORMAL) out.w = __uint_as_float(code0);
+                    if (!MULTI && v.repeat.flags_out) {
+                        same1 = v.in && same_bits(out, __ldg(v.in + p));
+                        same2 = v.repeat.has_two_ago && same_bits(out, v.out[p]);
+                    }
                     v.out[p] = out;
                     if (v.hint) v.hint[p] = hint;
                     if (v.prim) v.prim[p] = prim0;
@@ -298,6 +361,15 @@ __global__ void __launch_bounds__(BLOCK, CHAIN ? 768 / BLOCK : 0)
                     overflow = false;
                 }
             } while (0);
+            if (MS && !MULTI && v.repeat.flags_out) {
+                const bool all1 = __all_sync(0xffffffffu, same1), all2 = __all_sync(0xffffffffu, same2);
+                const unsigned sh = __reduce_add_sync(0xffffffffu, n_shadow - shadow_before);
+                if (lane == 0) {
+                    const int64_t tile = chunk - v.chunk_begin;
+                    v.repeat.flags_out[tile] = (uint8_t)((all1 ? 1 : 0) | (all2 ? 2 : 0));
+                    v.repeat.shadow[tile] = sh;
+                }
+            }
             if (SIGNAL && v.done_count) {  // counted when the warp leaves the view
                 const int w = threadIdx.x >> 5;
                 __syncwarp();
