@@ -220,9 +220,9 @@ rcp_status rcp_render_pass(const rcp_scene* scene, const rcp_camera* cam, int wi
  * except for a one-pass (K = 1) render with spp > 0, whose samples read
  * neighbouring pixels of d_in),
  * last pass's hit ids to d_prim (device, nullable). Enqueued on `stream`
- * (cudaStream_t, NULL = legacy default); the call returns once enqueued. The
- * K-pass sequence is captured once per (scene, shape, K) in a CUDA graph and
- * replayed. Intermediate images live in library-owned device memory. */
+ * (cudaStream_t, NULL = legacy default); the call returns once enqueued. A
+ * K-pass sequence of several launches is captured per (scene, shape, K) in a
+ * CUDA graph and replayed. Intermediate images live in library-owned device memory. */
 rcp_status rcp_render_device(const rcp_scene* scene, const rcp_camera* cam, int width, int height,
                              int K, const rcp_params* params, const float* d_in, float* d_out,
                              int32_t* d_prim, void* stream);

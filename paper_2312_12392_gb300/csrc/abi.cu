@@ -421,31 +421,36 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     auto record = [&](cudaEvent_t e) {
         return capturing ? cudaEventRecordWithFlags(e, st, cudaEventRecordExternal) : cudaEventRecord(e, st);
     };
-    RCP_CUDA(cudaMemsetAsync(ctx.d_rays, 0, sizeof(unsigned long long) * 2 + sizeof(unsigned) * (ctx.K + 1), st));
     const SceneDev S = sc.dev();
-    RCP_CUDA(record(ctx.pass_ev[0]));
+    LaunchCfg first = cfg;
+    if (ctx.direct) {
+        RCP_CUDA(record(ctx.pass_ev[0]));
+        rcp_status r = launch_stage_views(ctx.h_views, ctx.n_desc, ctx.d_views, (unsigned*)ctx.d_rays, 4 + ctx.K + 1, st);
+        if (r != RCP_OK) return r;
+        first.behind_stage = true;
+    } else {
+        RCP_CUDA(cudaMemsetAsync(ctx.d_rays, 0, sizeof(unsigned long long) * 2 + sizeof(unsigned) * (ctx.K + 1), st));
+        RCP_CUDA(record(ctx.pass_ev[0]));
+    }
     if (ctx.chained) {  // one descriptor per view, all K passes (image mode: pass 1, then the gathers' descriptors)
         rcp_status r = ctx.image_mode
-                           ? launch_pass(S, cfg, ctx.d_views, ctx.n_views, ctx.total_pix, ctx.total_chunks, nullptr,
+                           ? launch_pass(S, first, ctx.d_views, ctx.n_views, ctx.total_pix, ctx.total_chunks, nullptr,
                                          ctx.d_work, ctx.d_rays, nullptr, st)
-                           : launch_chain(S, cfg, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays,
+                           : launch_chain(S, first, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays,
                                           st);
         if (r != RCP_OK) return r;
         RCP_CUDA(record(ctx.pass_ev[1]));
-        ctx.launches = 1;
         if (ctx.image_mode) {
             r = launch_imagespace_chain(ctx.d_views + ctx.n_views, ctx.n_views, ctx.total_chunks, st);
             if (r != RCP_OK) return r;
             RCP_CUDA(record(ctx.pass_ev[2]));
-            ctx.launches = 2;
         }
         return RCP_OK;
     }
-    ctx.launches = ctx.K;
     for (int n = 0; n < ctx.K; ++n) {
         rcp_status r = (ctx.image_mode && n > 0)
                            ? launch_imagespace(ctx.d_views + (size_t)n * ctx.n_views, ctx.n_views, ctx.total_pix, st)
-                           : launch_pass(S, cfg, ctx.d_views + (size_t)n * ctx.n_views, ctx.n_views, ctx.total_pix,
+                           : launch_pass(S, n == 0 ? first : cfg, ctx.d_views + (size_t)n * ctx.n_views, ctx.n_views, ctx.total_pix,
                                          ctx.total_chunks, ctx.rays, ctx.d_work + n, ctx.d_rays, counters, st);
         if (r != RCP_OK) return r;
         RCP_CUDA(record(ctx.pass_ev[n + 1]));
@@ -453,12 +458,22 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     return RCP_OK;
 }
 
-// Run the K passes through the context's CUDA graph, captured when a launch
+// Enqueue a frame. One of few descriptors and launches (ctx.direct) goes
+// straight onto the stream: k_stage_views and the launch or two behind it take
+// less of the device's time between kernels than a copy and a graph (a 128x128
+// K = 6 frame of five primitives 45.9 -> 34.5 us, 32 us of it one warp's
+// chain of twelve rays). Others run through the context's CUDA graph, captured when a launch
 // configuration comes a second time: the first time its launches are enqueued
 // directly, since capturing and instantiating a graph takes longer than the
 // few launches of a frame that may be the only one of its shape. On a stream
 // that is itself being captured the graph is used from the start.
-rcp_status run_graph(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cudaStream_t st) {
+rcp_status run_frame(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cudaStream_t st) {
+    if (ctx.direct) {
+        rcp_status r = enqueue_passes(sc, ctx, cfg, nullptr, st, false);
+        if (r != RCP_OK) return r;
+        RCP_CUDA(cudaEventRecord(ctx.done, st));
+        return RCP_OK;
+    }
     const std::string key = cfg_key(cfg) + (ctx.image_mode ? "/image" : "/trace") + (ctx.chained ? "/chain" : "");
     if (!ctx.graph || ctx.graph_key != key) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
@@ -533,6 +548,15 @@ rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
     return RCP_OK;
 }
 
+// The staged descriptors to the device (a direct frame's go with its launch).
+rcp_status upload_views(RenderCtx& ctx, cudaStream_t st) {
+    if (ctx.direct) return RCP_OK;
+    RCP_CUDA(cudaMemcpyAsync(ctx.d_views, ctx.h_views, sizeof(ViewDev) * (size_t)ctx.n_desc, cudaMemcpyHostToDevice,
+                             st));
+    RCP_CUDA(cudaEventRecord(ctx.staged, st));
+    return RCP_OK;
+}
+
 // Stage the view descriptors of one render (n_views views, K passes): one per
 // view and pass, or, when the passes run chained (chain: the tuning asks for
 // it and the render allows it), one per view that runs all K passes (an
@@ -540,7 +564,7 @@ rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
 // gathers passes 2..K).
 rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const float4* const* ins,
                        float4* const* outs, int32_t* const* prims, float* const* rgbs, cudaStream_t st,
-                       bool chain = false) {
+                       bool chain = false, bool allow_direct = false) {
     RCP_CUDA(cudaEventSynchronize(ctx.staged));  // previous copy out of the staging buffer is done
     const int K = ctx.K, nv = ctx.n_views;
     ctx.image_mode = base[0].mapping == RCP_MAP_IMAGE && K > 1;
@@ -548,6 +572,13 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
     // between passes (90 registers, nothing spilled in the walk): mid 1080p
     // K = 1 0.335 against 0.316 ms chained
     ctx.chained = chain && base[0].spp == 0 && K > 1;
+    ctx.launches = ctx.chained ? (ctx.image_mode ? 2 : 1) : K;
+    ctx.n_desc = ctx.chained ? nv * (ctx.image_mode ? 2 : 1) : nv * K;
+    // a stream that is being captured takes the copy and the graph
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+    ctx.direct = allow_direct && (ctx.chained || K == 1) && ctx.n_desc <= STAGE_VIEWS &&
+                 capture == cudaStreamCaptureStatusNone;
     if (ctx.image_mode && !ctx.base_img) RCP_CUDA(cudaMalloc((void**)&ctx.base_img, sizeof(float4) * ctx.total_pix));
     if (ctx.chained) {
         for (int i = 0; i < nv; ++i) {
@@ -571,10 +602,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
             }
             ctx.h_views[i] = v;
         }
-        RCP_CUDA(cudaMemcpyAsync(ctx.d_views, ctx.h_views, sizeof(ViewDev) * (size_t)nv * (ctx.image_mode ? 2 : 1),
-                                 cudaMemcpyHostToDevice, st));
-        RCP_CUDA(cudaEventRecord(ctx.staged, st));
-        return RCP_OK;
+        return upload_views(ctx, st);
     }
     if (K > 1) {
         rcp_status r = ensure_img(ctx);
@@ -627,9 +655,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
             ctx.h_views[(size_t)n * nv + i] = v;
         }
     }
-    RCP_CUDA(cudaMemcpyAsync(ctx.d_views, ctx.h_views, sizeof(ViewDev) * (size_t)K * nv, cudaMemcpyHostToDevice, st));
-    RCP_CUDA(cudaEventRecord(ctx.staged, st));
-    return RCP_OK;
+    return upload_views(ctx, st);
 }
 
 rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const int* Ws, const int* Hs, int K,
@@ -673,14 +699,14 @@ rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const in
     if (r != RCP_OK) return r;
     LaunchCfg cfg = cfg_override ? *cfg_override : cfg_of(sc);
     cfg.ms = p->spp > 0;
-    r = stage_views(*ctx, base, ins, outs, prims, rgbs, st, cfg.chain);
+    r = stage_views(*ctx, base, ins, outs, prims, rgbs, st, cfg.chain, true);
     if (r != RCP_OK) return r;
     if (ctx->chained) cfg.fused = true;  // a chained launch makes its rays itself
     r = ensure_spill(sc, cfg);
     if (r != RCP_OK) return r;
     r = ensure_rays(*ctx, cfg);
     if (r != RCP_OK) return r;
-    r = run_graph(sc, *ctx, cfg, st);
+    r = run_frame(sc, *ctx, cfg, st);
     sc.last = ctx;
     if (ctx_out) *ctx_out = ctx;
     return r;

@@ -33,6 +33,7 @@ struct RenderCtx {
     float* d_rgb = nullptr;      // packed RGB for host output
     float4* io = nullptr;        // host-API input / final image
     float4* base_img = nullptr;  // image-space mapping: the traced pass-1 image
+    bool direct = false;         // descriptors staged by a launch, the frame's launches enqueued directly
     bool image_mode = false;     // passes 2..K are image-space gathers
     bool chained = false;        // one launch runs all K passes (one descriptor per view), or, in image mode, one
                                  // launch traces pass 1 and one gathers passes 2..K (two descriptors per view)
@@ -42,7 +43,8 @@ struct RenderCtx {
     int2* hints = nullptr;       // per pixel: latest primary-hit and shadow-occluder records (-1 none)
     cudaEvent_t staged = nullptr;
     cudaEvent_t pass_ev[17] = {};  // timing events around every launch (recorded inside the graph)
-    int launches = 0;              // launches of the latest enqueue: K, or 1 (image mode: 2) when chained
+    int n_desc = 0;                // descriptors of the latest render
+    int launches = 0;              // launches of the latest render: K, or 1 (image mode: 2) when chained
     cudaGraphExec_t graph = nullptr;
     std::string graph_key, seen_key;  // the captured configuration; the one last enqueued directly
     cudaEvent_t done = nullptr;  // recorded after the context's latest launch
@@ -115,6 +117,7 @@ struct LaunchCfg {
     bool ms = false;  // jittered multi-sample kernel
     bool multi = false;  // each view names its scene (views of several scenes; the server's launches)
     int hints = 3;    // previous-hit hints: bit 0 primary, bit 1 shadow
+    bool behind_stage = false;  // the launch before is launch_stage_views: launched programmatically behind it
     bool chain = false;  // all K passes in one launch where the render allows it
 };
 
@@ -130,6 +133,11 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
 // own previous value; cfg.multi: the views name their scenes.
 rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                         int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays, cudaStream_t st);
+// n descriptors (at most STAGE_VIEWS) to d_views, and n_zero words at `zero`
+// to 0, in one launch.
+constexpr int STAGE_VIEWS = 4;
+rcp_status launch_stage_views(const ViewDev* views, int n, ViewDev* d_views, unsigned* zero, int n_zero,
+                              cudaStream_t st);
 rcp_status launch_debug_trace(const SceneDev& S, int64_t n, const float* orig_tmin, const float* dir_tmax, int any,
                               int brute, float* t_out, int32_t* prim_out, int stack_entries, int* d_status,
                               cudaStream_t st);

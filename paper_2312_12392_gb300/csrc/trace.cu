@@ -78,6 +78,23 @@ __device__ __forceinline__ float4 trace_shade(const SceneDev& S, const RayF& r, 
     return out;
 }
 
+// A frame's descriptors, from the launch's parameters, and its counters
+// zeroed. One launch in the place of a copy and a memset, behind which the
+// trace kernel is launched programmatically: its blocks are resident and their
+// tables filled when the descriptors are there.
+struct StageArgs {
+    ViewDev v[STAGE_VIEWS];
+};
+__global__ void k_stage_views(const __grid_constant__ StageArgs a, int n, ViewDev* __restrict__ views,
+                              uint32_t* __restrict__ zero, int n_zero) {
+    asm volatile("griddepcontrol.launch_dependents;");
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(&a);
+    uint32_t* dst = reinterpret_cast<uint32_t*>(views);
+    for (int i = threadIdx.x; i < n * (int)(sizeof(ViewDev) / 4); i += blockDim.x) dst[i] = src[i];
+    for (int i = threadIdx.x; i < n_zero; i += blockDim.x) zero[i] = 0u;
+}
+static_assert(sizeof(StageArgs) <= 4000, "the staged descriptors fit a launch's parameters");
+
 // Whether a pixel's values a and b give the next pass the same camera, bit
 // for bit: the lanes of a previous value that camera_ray reads under the
 // mapping (colour; colour and z-depth; the normal's code).
@@ -196,6 +213,7 @@ __global__ void __launch_bounds__(BLOCK, CHAIN || MS ? 768 / BLOCK : 0)
         s_done_n[threadIdx.x >> 5] = 0;
     }
     __syncthreads();
+    asm volatile("griddepcontrol.wait;" ::: "memory");  // launched behind k_stage_views: its descriptors and counters
     uint2* stack = s_stack + threadIdx.x;
     const int lane = threadIdx.x & 31;
     bool overflow = false;
@@ -587,9 +605,18 @@ rcp_status launch_trace_t(const SceneDev& S, const LaunchCfg& cfg, const ViewDev
         set_error("traversal spill region too small for the launch");
         return RCP_ERR_STATE;
     }
-    kern<<<(int)grid, BLOCK, smem, st>>>(S, d_views, n_views, total_chunks, cfg.chunk / 32, rays, d_work, stk, d_rays,
-                                         d_counters);
-    RCP_CUDA(cudaGetLastError());
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)grid);
+    lc.blockDim = dim3(BLOCK);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    lc.attrs = &attr;
+    lc.numAttrs = cfg.behind_stage ? 1 : 0;
+    RCP_CUDA(cudaLaunchKernelEx(&lc, kern, S, d_views, n_views, total_chunks, cfg.chunk / 32, rays, d_work, stk, d_rays,
+                                d_counters));
     return RCP_OK;
 }
 
@@ -632,6 +659,16 @@ rcp_status launch_trace_b(const SceneDev& S, const LaunchCfg& cfg, const ViewDev
                                                                 d_rays, d_counters, st);
 }
 
+// The trace kernel over rays that the camera kernel made.
+rcp_status launch_separate(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
+                           int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
+                           unsigned long long* d_counters, cudaStream_t st) {
+    return cfg.count ? launch_trace_b<false, true, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                 d_rays, d_counters, st)
+                     : launch_trace_b<false, false, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                  d_rays, d_counters, st);
+}
+
 }  // namespace
 
 rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
@@ -649,6 +686,9 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
         if (g < 1) g = 1;
         k_camera<<<(int)g, 256, 0, st>>>(d_views, n_views, total_pix, S.tmin, rays);
         RCP_CUDA(cudaGetLastError());
+        LaunchCfg behind_camera = cfg;  // the trace kernel waits for the rays as a stream does
+        behind_camera.behind_stage = false;
+        return launch_separate(S, behind_camera, d_views, n_views, total_chunks, rays, d_work, d_rays, d_counters, st);
     }
     if (cfg.ms) {  // jittered samples: camera inside the trace kernel
         return cfg.count ? launch_trace_b<true, true, true, false>(S, cfg, d_views, n_views, total_chunks, rays,
@@ -656,15 +696,10 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
                          : launch_trace_b<true, false, true, false>(S, cfg, d_views, n_views, total_chunks, rays,
                                                                     d_work, d_rays, d_counters, st);
     }
-    if (cfg.count)
-        return cfg.fused ? launch_trace_b<true, true, false, false>(S, cfg, d_views, n_views, total_chunks, rays,
-                                                                    d_work, d_rays, d_counters, st)
-                         : launch_trace_b<false, true, false, false>(S, cfg, d_views, n_views, total_chunks, rays,
-                                                                     d_work, d_rays, d_counters, st);
-    return cfg.fused ? launch_trace_b<true, false, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
-                                                                 d_rays, d_counters, st)
-                     : launch_trace_b<false, false, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
-                                                                  d_rays, d_counters, st);
+    return cfg.count ? launch_trace_b<true, true, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                d_rays, d_counters, st)
+                     : launch_trace_b<true, false, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                 d_rays, d_counters, st);
 }
 
 rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
@@ -678,6 +713,15 @@ rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* 
                                                               d_rays, nullptr, st);
     return launch_trace_b<true, false, false, false, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
                                                            d_rays, nullptr, st);
+}
+
+rcp_status launch_stage_views(const ViewDev* views, int n, ViewDev* d_views, unsigned* zero, int n_zero,
+                              cudaStream_t st) {
+    StageArgs a;
+    for (int i = 0; i < n; ++i) a.v[i] = views[i];
+    k_stage_views<<<1, 256, 0, st>>>(a, n, d_views, zero, n_zero);
+    RCP_CUDA(cudaGetLastError());
+    return RCP_OK;
 }
 
 rcp_status launch_debug_trace(const SceneDev& S, int64_t n, const float* orig_tmin, const float* dir_tmax, int any,
