@@ -1,24 +1,29 @@
-// radix_sort.cu -- onesweep LSD radix sort of (uint32 key, uint32 value) pairs.
+// radix_sort.cu -- LSD radix sort of (uint32 key, uint32 value) pairs, 8 bits a pass.
 //
 // Used by the BVH builder to order primitives by 30-bit Morton code, and by
-// the allocation-free sort below. One histogram kernel counts all digit passes
-// at once (its last block scans the counts); then one kernel per 8-bit digit
-// ranks a tile of keys in shared memory (warp ballots + per-warp counters,
-// stable), finds the tile's global offset per digit by decoupled look-back over
-// earlier tiles (tiles are numbered in launch order by an atomic counter, so
-// every earlier tile is already running), and scatters through shared memory
-// so that writes of one digit run are contiguous.
+// the allocation-free sort below. A pass ranks a tile of keys in shared memory
+// (warp ballots + per-warp counters, stable), finds the tile's place per digit
+// among all tiles, and scatters through shared memory so that writes of one
+// digit run are contiguous.
+//  * While the tiles fit the GPU at once (one per SM, 1.09 million pairs on
+//    152 SMs), one cooperative launch runs every pass (k_sort_resident).
+//  * Beyond that, onesweep: one histogram kernel counts all digit passes at
+//    once (its last block scans the counts), then one launch per digit finds a
+//    tile's place by decoupled look-back over earlier tiles (numbered in launch
+//    order by an atomic counter, so every earlier tile is already running).
 //
 // What bounds it up to about a million pairs is latency: 16 MB a pass moves
 // through L2 in a few microseconds, and each block's chain of load, rank,
-// look-back and scatter is serial. So: tiles of 7,168 pairs, which put a
-// million pairs on the SMs in one wave (147 tiles); a look-back that polls
-// eight earlier tiles at once, where one at a time is a chain of L2 round
-// trips over as many tiles; the tile's own scan done by the other half of the
-// block meanwhile; one memset for every pass's status words; and programmatic
-// launches, so that a pass's blocks are resident when the pass before ends.
-// 1,000,003 pairs on 30 bits, the whole call with its last read-back: 170 -> 102
-// us (a pass 25 -> 13.5 us, of which 9.4 us is one tile alone).
+// place and scatter is serial (9 us a pass for a single tile, of which about
+// 3.5 us are shared-memory bank conflicts of random digits and 3 us the two
+// barriers). So: tiles of 7,168 pairs over 1,024 threads, which put a million
+// pairs on the SMs in one wave; in onesweep a look-back that polls eight
+// earlier tiles at once, where one at a time is a chain of L2 round trips, the
+// tile's own scan done by other warps meanwhile, one memset for every pass's
+// status words, and programmatic launches, so that a pass's blocks are
+// resident when the pass before ends. 1,000,003 pairs on 30 bits, the whole
+// call with its last read-back: 170 us (four passes of 25 us and a histogram),
+// onesweep as here 102 us, resident 96 us (53 us in the kernel).
 //
 // Every wait on another tile's status is bounded: after spin_limit polls
 // (SPIN_LIMIT in a sort) the kernel records an error flag and proceeds, so a
@@ -38,12 +43,13 @@ namespace {
 
 constexpr int RADIX = 256;
 constexpr int PASSES_MAX = 4;
-constexpr int SORT_BLOCK = 512;
+constexpr int SORT_BLOCK = 1024;
 constexpr int SORT_WARPS = SORT_BLOCK / 32;
-constexpr int ITEMS = 14;
+constexpr int ITEMS = 7;
 constexpr int TILE = SORT_BLOCK * ITEMS;  // 7168 pairs
 constexpr int LOOK = 8;                   // earlier tiles polled at once
-static_assert(SORT_BLOCK == 2 * RADIX, "one half of the block looks back, the other scans the tile's counts");
+constexpr int GROUPS = SORT_BLOCK / RADIX;  // of one thread per digit each
+static_assert(SORT_BLOCK % RADIX == 0 && GROUPS >= 2, "one group looks back while another scans the tile's counts");
 constexpr uint32_t FLAG_AGG = 1u << 30;
 constexpr uint32_t FLAG_INC = 2u << 30;
 constexpr uint32_t COUNT_MASK = (1u << 30) - 1;
@@ -128,11 +134,78 @@ struct SortShared {
     uint32_t wcnt[SORT_WARPS][RADIX];
     uint32_t tile_off[RADIX];
     uint32_t global[RADIX];
-    uint32_t warp_tot[RADIX / 32];
+    uint32_t warp_tot[2][RADIX / 32];
     uint32_t tile;
 };
 
-__global__ void __launch_bounds__(SORT_BLOCK, 2) k_onesweep(const uint32_t* __restrict__ keys_in,
+// Rank a tile's keys by digit: rank[j] is key j's place among its warp's keys
+// of the digit, s.wcnt[w][d] the warps' counts (zeroed before).
+__device__ __forceinline__ void rank_keys(SortShared& s, const uint32_t (&k)[ITEMS], uint32_t (&rank)[ITEMS],
+                                          int shift) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t d = (k[j] >> shift) & 0xff;
+        const unsigned peers = same_digit(d);
+        const uint32_t before = s.wcnt[warp][d];
+        rank[j] = before + __popc(peers & lt);
+        __syncwarp();
+        if ((peers >> lane) == 1u) s.wcnt[warp][d] = before + __popc(peers);  // highest lane of the group
+        __syncwarp();
+    }
+}
+
+// Digit d's count in the tile; s.wcnt becomes its exclusive scan over the warps.
+__device__ __forceinline__ uint32_t scan_warp_counts(SortShared& s, int d) {
+    uint32_t count = 0;
+#pragma unroll
+    for (int w = 0; w < SORT_WARPS; ++w) {
+        const uint32_t c = s.wcnt[w][d];
+        s.wcnt[w][d] = count;
+        count += c;
+    }
+    return count;
+}
+
+// Exclusive scan of one value per digit over 256 threads of the block (d: the
+// thread's digit), which meet at named barrier `bar`.
+__device__ __forceinline__ uint32_t scan_digits(uint32_t (&warp_tot)[RADIX / 32], uint32_t c, int d, int bar) {
+    const int lane = threadIdx.x & 31;
+    uint32_t x = c;
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) warp_tot[d >> 5] = x;
+    asm volatile("bar.sync %0, 256;" ::"r"(bar) : "memory");
+    for (int w = 0; w < d >> 5; ++w) x += warp_tot[w];
+    return x - c;
+}
+
+// The tile's pairs into shared memory in digit order, then to their places.
+__device__ __forceinline__ void scatter_tile(SortShared& s, const uint32_t (&k)[ITEMS], const uint32_t (&v)[ITEMS],
+                                             const uint32_t (&rank)[ITEMS], int shift, int valid,
+                                             uint32_t* __restrict__ keys_out, uint32_t* __restrict__ vals_out) {
+    const int warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+        const uint32_t d = (k[j] >> shift) & 0xff;
+        const uint32_t r = s.tile_off[d] + s.wcnt[warp][d] + rank[j];
+        s.keys[r] = k[j];
+        s.vals[r] = v[j];
+    }
+    __syncthreads();
+    for (int pos = threadIdx.x; pos < valid; pos += SORT_BLOCK) {
+        const uint32_t key = s.keys[pos];
+        const uint32_t d = (key >> shift) & 0xff;
+        const uint32_t dst = s.global[d] + (pos - s.tile_off[d]);
+        keys_out[dst] = key;
+        vals_out[dst] = s.vals[pos];
+    }
+}
+
+__global__ void __launch_bounds__(SORT_BLOCK, 1) k_onesweep(const uint32_t* __restrict__ keys_in,
                                                             const uint32_t* __restrict__ vals_in,
                                                             uint32_t* __restrict__ keys_out,
                                                             uint32_t* __restrict__ vals_out, int64_t n, int shift,
@@ -157,30 +230,13 @@ __global__ void __launch_bounds__(SORT_BLOCK, 2) k_onesweep(const uint32_t* __re
         k[j] = base + 32 * j < n ? keys_in[base + 32 * j] : 0xffffffffu;
 #pragma unroll
     for (int j = 0; j < ITEMS; ++j) v[j] = base + 32 * j < n ? vals_in[base + 32 * j] : 0u;
-    const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t d = (k[j] >> shift) & 0xff;
-        const unsigned peers = same_digit(d);
-        const uint32_t before = s.wcnt[warp][d];
-        rank[j] = before + __popc(peers & lt);
-        __syncwarp();
-        if ((peers >> lane) == 1u) s.wcnt[warp][d] = before + __popc(peers);  // highest lane of the group
-        __syncwarp();
-    }
+    rank_keys(s, k, rank, shift);
     __syncthreads();
 
-    // digit d's tile count, as an exclusive scan over the warps; each half of
-    // the block has one thread per digit
     const int d = tid & (RADIX - 1);
     uint32_t count = 0;
     if (tid < RADIX) {
-#pragma unroll
-        for (int w = 0; w < SORT_WARPS; ++w) {
-            const uint32_t c = s.wcnt[w][d];
-            s.wcnt[w][d] = count;
-            count += c;
-        }
+        count = scan_warp_counts(s, d);
         // publish this tile's count (tile 0's is already inclusive); a status
         // word carries flag and count together, so no fence orders anything
         volatile uint32_t* st = status + (size_t)tile * RADIX;
@@ -221,36 +277,103 @@ __global__ void __launch_bounds__(SORT_BLOCK, 2) k_onesweep(const uint32_t* __re
         }
         if (tile > 0) ((volatile uint32_t*)status)[(size_t)tile * RADIX + d] = FLAG_INC | (prefix + count);
         s.global[d] = bucket_base[d] + prefix;
-    } else {
-        // the tile's digit counts -> tile offsets
-        const uint32_t c = s.tile_off[d];
-        uint32_t x = c;
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s.warp_tot[d >> 5] = x;
-        asm volatile("bar.sync 1, 256;" ::: "memory");  // this half of the block
-        for (int w = 0; w < d >> 5; ++w) x += s.warp_tot[w];
-        s.tile_off[d] = x - c;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int j = 0; j < ITEMS; ++j) {
-        const uint32_t dj = (k[j] >> shift) & 0xff;
-        const uint32_t r = s.tile_off[dj] + s.wcnt[warp][dj] + rank[j];
-        s.keys[r] = k[j];
-        s.vals[r] = v[j];
+    } else if (tid < 2 * RADIX) {
+        s.tile_off[d] = scan_digits(s.warp_tot[0], s.tile_off[d], d, 1);
     }
     __syncthreads();
     const int64_t left = n - (int64_t)tile * TILE;
+    scatter_tile(s, k, v, rank, shift, left < TILE ? (int)left : TILE, keys_out, vals_out);
+}
+
+// ---- all passes in one launch, while the tiles fit the GPU at once ----
+// Up to one tile per SM, a block keeps its tile's place through every pass: it
+// ranks its keys, publishes its 256 digit counts, and after a grid-wide barrier
+// adds up every tile's counts itself (all tiles' and the earlier tiles'), where
+// separate passes need a histogram beforehand and look back tile by tile; the
+// pairs go to the other buffer and a second barrier ends the pass. The launch is cooperative, so that every block
+// that a barrier waits for runs; each wait is bounded all the same.
+struct ResidentShared {
+    SortShared t;
+    uint32_t part[GROUPS][2][RADIX];  // per group: all tiles' counts, earlier tiles' counts
+};
+
+__device__ __forceinline__ void grid_barrier(uint32_t* arrived, uint32_t target, int* error_flag,
+                                             long long spin_limit) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(arrived, 1u);
+        long long spins = 0;
+        while (*(volatile uint32_t*)arrived < target)
+            if (++spins > spin_limit) {
+                atomicExch(error_flag, 1);
+                break;
+            }
+        __threadfence();
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(SORT_BLOCK, 1) k_sort_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys,
+                                                                 uint32_t* alt_vals, int64_t n, int passes,
+                                                                 uint32_t* counts, uint32_t* arrived, int* error_flag,
+                                                                 long long spin_limit) {
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    ResidentShared& rs = *reinterpret_cast<ResidentShared*>(s_raw);
+    SortShared& s = rs.t;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tiles = gridDim.x, tile = blockIdx.x;
+    const int64_t base = (int64_t)tile * TILE + warp * (32 * ITEMS) + lane;
+    const int64_t left = n - (int64_t)tile * TILE;
     const int valid = left < TILE ? (int)left : TILE;
-    for (int pos = tid; pos < valid; pos += SORT_BLOCK) {
-        const uint32_t key = s.keys[pos];
-        const uint32_t dj = (key >> shift) & 0xff;
-        const uint32_t dst = s.global[dj] + (pos - s.tile_off[dj]);
-        keys_out[dst] = key;
-        vals_out[dst] = s.vals[pos];
+    const int d = tid & (RADIX - 1), group = tid / RADIX;
+    uint32_t barriers = 0;
+    for (int p = 0; p < passes; ++p) {
+        const uint32_t *ki = p & 1 ? alt_keys : keys, *vi = p & 1 ? alt_vals : vals;
+        const int shift = 8 * p;
+        for (int i = tid; i < SORT_WARPS * RADIX; i += SORT_BLOCK) (&s.wcnt[0][0])[i] = 0;
+        uint32_t k[ITEMS], v[ITEMS], rank[ITEMS];
+        // other blocks wrote these in the pass before: past this SM's L1
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j)  // past the end: ranks after every real key of its digit
+            k[j] = base + 32 * j < n ? __ldcg(ki + base + 32 * j) : 0xffffffffu;
+#pragma unroll
+        for (int j = 0; j < ITEMS; ++j) v[j] = base + 32 * j < n ? __ldcg(vi + base + 32 * j) : 0u;
+        __syncthreads();
+        rank_keys(s, k, rank, shift);
+        __syncthreads();
+        uint32_t* cnt = counts + (size_t)p * tiles * RADIX;
+        if (tid < RADIX) {
+            const uint32_t c = scan_warp_counts(s, d);
+            s.tile_off[d] = c;
+            __stcg(cnt + (size_t)tile * RADIX + d, c);
+        }
+        grid_barrier(arrived, ++barriers * tiles, error_flag, spin_limit);
+        // each group adds up its share of the tiles
+        uint32_t all = 0, earlier = 0;
+        const int t0 = group * tiles / GROUPS, t1 = (group + 1) * tiles / GROUPS;
+#pragma unroll 8
+        for (int t = t0; t < t1; ++t) {
+            const uint32_t c = __ldcg(cnt + (size_t)t * RADIX + d);
+            all += c;
+            if (t < tile) earlier += c;
+        }
+        rs.part[group][0][d] = all;
+        rs.part[group][1][d] = earlier;
+        __syncthreads();
+        if (group == 0) {
+            all = earlier = 0;
+            for (int g = 0; g < GROUPS; ++g) {
+                all += rs.part[g][0][d];
+                earlier += rs.part[g][1][d];
+            }
+            s.global[d] = scan_digits(s.warp_tot[1], all, d, 1) + earlier;
+        } else if (group == 1) {
+            s.tile_off[d] = scan_digits(s.warp_tot[0], s.tile_off[d], d, 2);
+        }
+        __syncthreads();
+        scatter_tile(s, k, v, rank, shift, valid, p & 1 ? keys : alt_keys, p & 1 ? vals : alt_vals);
+        if (p + 1 < passes) grid_barrier(arrived, ++barriers * tiles, error_flag, spin_limit);
     }
 }
 
@@ -271,6 +394,34 @@ rcp_status launch_onesweep(const uint32_t* ki, const uint32_t* vi, uint32_t* ko,
     cfg.numAttrs = 1;
     RCP_CUDA(cudaLaunchKernelEx(&cfg, k_onesweep, ki, vi, ko, vo, n, shift, bucket_base, status, tile_counter, d_error,
                                 spin_limit));
+    return RCP_OK;
+}
+
+rcp_status launch_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n, int passes,
+                           uint32_t* counts, uint32_t* arrived, int64_t tiles, int* d_error, cudaStream_t stream) {
+    RCP_CUDA(cudaFuncSetAttribute(k_sort_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)sizeof(ResidentShared)));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)tiles);
+    cfg.blockDim = dim3(SORT_BLOCK);
+    cfg.dynamicSmemBytes = sizeof(ResidentShared);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeCooperative;
+    attr.val.cooperative = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    RCP_CUDA(cudaLaunchKernelEx(&cfg, k_sort_resident, keys, vals, alt_keys, alt_vals, n, passes, counts, arrived,
+                                d_error, SPIN_LIMIT));
+    return RCP_OK;
+}
+
+// The sorted pairs, if they lie elsewhere, back to the caller's arrays.
+rcp_status copy_back(uint32_t* keys, uint32_t* vals, const uint32_t* ki, const uint32_t* vi, int64_t n,
+                     cudaStream_t stream) {
+    if (ki == keys) return RCP_OK;
+    RCP_CUDA(cudaMemcpyAsync(keys, ki, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, stream));
+    RCP_CUDA(cudaMemcpyAsync(vals, vi, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, stream));
     return RCP_OK;
 }
 
@@ -299,11 +450,22 @@ rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
     int sms = 0, dev = 0;
     RCP_CUDA(cudaGetDevice(&dev));
     RCP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    uint32_t *ki = keys, *vi = vals, *ko = alt_keys, *vo = alt_vals;
+    // One tile per SM at most: one launch for all passes (1,000,003 pairs 96 us, onesweep 102 us)
+    if (tiles <= sms) {
+        rcp_status r = launch_resident(keys, vals, alt_keys, alt_vals, n, passes, status, counters, tiles, d_error,
+                                       stream);
+        if (r != RCP_OK) return r;
+        if (passes & 1) {
+            std::swap(ki, ko);
+            std::swap(vi, vo);
+        }
+        return copy_back(keys, vals, ki, vi, n, stream);
+    }
     int64_t hblocks = (n + HIST_BLOCK * HIST_KEYS - 1) / (HIST_BLOCK * HIST_KEYS);
     if (hblocks > sms) hblocks = sms;
     k_histogram<<<(int)hblocks, HIST_BLOCK, 0, stream>>>(keys, n, passes, hist, counters + PASSES_MAX);
     RCP_CUDA(cudaGetLastError());
-    uint32_t *ki = keys, *vi = vals, *ko = alt_keys, *vo = alt_vals;
     for (int p = 0; p < passes; ++p) {
         rcp_status r = launch_onesweep(ki, vi, ko, vo, n, 8 * p, hist + p * RADIX, status + (size_t)p * tiles * RADIX,
                                        counters + p, tiles, d_error, SPIN_LIMIT, stream);
@@ -311,11 +473,7 @@ rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
         std::swap(ki, ko);
         std::swap(vi, vo);
     }
-    if (ki != keys) {
-        RCP_CUDA(cudaMemcpyAsync(keys, ki, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, stream));
-        RCP_CUDA(cudaMemcpyAsync(vals, vi, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, stream));
-    }
-    return RCP_OK;
+    return copy_back(keys, vals, ki, vi, n, stream);
 }
 
 }  // namespace rcp
