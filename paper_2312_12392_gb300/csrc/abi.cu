@@ -404,7 +404,7 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
     c->hints = (int2*)(c->block + head + views);
     RCP_CUDA(cudaMemset(c->block, 0, head));
     RCP_CUDA(cudaMemset(c->hints, 0xff, sizeof(int2) * total_pix));  // -1: no earlier hit
-    RCP_CUDA(cudaMallocHost((void**)&c->h_views, sizeof(ViewDev) * (size_t)K * n_views));
+    c->views.resize((size_t)K * n_views);
     RCP_CUDA(cudaEventCreateWithFlags(&c->staged, cudaEventDisableTiming));
     RCP_CUDA(cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming));
     for (int n = 0; n <= K; ++n) RCP_CUDA(cudaEventCreate(&c->pass_ev[n]));
@@ -425,7 +425,7 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     LaunchCfg first = cfg;
     if (ctx.direct) {
         RCP_CUDA(record(ctx.pass_ev[0]));
-        rcp_status r = launch_stage_views(ctx.h_views, ctx.n_desc, ctx.d_views, (unsigned*)ctx.d_rays, 4 + ctx.K + 1, st);
+        rcp_status r = launch_stage_views(ctx.views.data(), ctx.n_desc, ctx.d_views, (unsigned*)ctx.d_rays, 4 + ctx.K + 1, st);
         if (r != RCP_OK) return r;
         first.behind_stage = true;
     } else {
@@ -551,6 +551,9 @@ rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
 // The staged descriptors to the device (a direct frame's go with its launch).
 rcp_status upload_views(RenderCtx& ctx, cudaStream_t st) {
     if (ctx.direct) return RCP_OK;
+    if (!ctx.h_views) RCP_CUDA(cudaMallocHost((void**)&ctx.h_views, sizeof(ViewDev) * ctx.views.size()));
+    RCP_CUDA(cudaEventSynchronize(ctx.staged));  // the previous copy out of the staging buffer is done
+    std::copy(ctx.views.begin(), ctx.views.begin() + ctx.n_desc, ctx.h_views);
     RCP_CUDA(cudaMemcpyAsync(ctx.d_views, ctx.h_views, sizeof(ViewDev) * (size_t)ctx.n_desc, cudaMemcpyHostToDevice,
                              st));
     RCP_CUDA(cudaEventRecord(ctx.staged, st));
@@ -565,7 +568,6 @@ rcp_status upload_views(RenderCtx& ctx, cudaStream_t st) {
 rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const float4* const* ins,
                        float4* const* outs, int32_t* const* prims, float* const* rgbs, cudaStream_t st,
                        bool chain = false, bool allow_direct = false) {
-    RCP_CUDA(cudaEventSynchronize(ctx.staged));  // previous copy out of the staging buffer is done
     const int K = ctx.K, nv = ctx.n_views;
     ctx.image_mode = base[0].mapping == RCP_MAP_IMAGE && K > 1;
     // a single traced pass takes the one-pass kernel, which keeps no state
@@ -591,7 +593,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
             v.rgb = rgbs ? rgbs[i] : nullptr;
             v.passes = K;
             if (ctx.image_mode) {
-                ViewDev& w = ctx.h_views[nv + i];
+                ViewDev& w = ctx.views[nv + i];
                 w = v;
                 w.base = ctx.base_img + base[i].pix_begin;
                 w.passes = K - 1;
@@ -600,7 +602,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
                 v.rgb = nullptr;
                 v.passes = 1;
             }
-            ctx.h_views[i] = v;
+            ctx.views[i] = v;
         }
         return upload_views(ctx, st);
     }
@@ -652,7 +654,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
                 m.shadow = shadow + odd * ctx.total_chunks;
                 if (ids && n < K - 1) v.prim = ids + odd * ctx.total_pix;
             }
-            ctx.h_views[(size_t)n * nv + i] = v;
+            ctx.views[(size_t)n * nv + i] = v;
         }
     }
     return upload_views(ctx, st);

@@ -1078,31 +1078,6 @@ __device__ __forceinline__ void ref_box(const BinTree& bt, int ref, float3& lo, 
 
 }  // namespace
 
-// Child boxes of up to 8 children into their slots, exactly as computed
-// (empty slots get lo = +inf, hi = -inf, which no ray enters); returns the
-// union of the children.
-__device__ void write_child_boxes(WNode& nd, const float3* clo, const float3* chi, const int* slot_of, int m,
-                                  float3& ulo, float3& uhi) {
-    for (int a = 0; a < 3; ++a)
-        for (int s = 0; s < 8; ++s) {
-            nd.box[a][0][s] = nd.box[a][2][s] = INFINITY;
-            nd.box[a][1][s] = -INFINITY;
-        }
-    ulo = make_float3(INFINITY, INFINITY, INFINITY);
-    uhi = make_float3(-INFINITY, -INFINITY, -INFINITY);
-    for (int c = 0; c < m; ++c) {
-        const int sl = slot_of[c];
-        nd.box[0][0][sl] = nd.box[0][2][sl] = clo[c].x;
-        nd.box[1][0][sl] = nd.box[1][2][sl] = clo[c].y;
-        nd.box[2][0][sl] = nd.box[2][2][sl] = clo[c].z;
-        nd.box[0][1][sl] = chi[c].x;
-        nd.box[1][1][sl] = chi[c].y;
-        nd.box[2][1][sl] = chi[c].z;
-        ulo = make_float3(fminf(ulo.x, clo[c].x), fminf(ulo.y, clo[c].y), fminf(ulo.z, clo[c].z));
-        uhi = make_float3(fmaxf(uhi.x, chi[c].x), fmaxf(uhi.y, chi[c].y), fmaxf(uhi.z, chi[c].z));
-    }
-}
-
 __device__ __forceinline__ void write_prim_record(float4* __restrict__ rec, const float* __restrict__ tri,
                                                   const float* __restrict__ sph, int64_t T, uint32_t id) {
     if (id < T) {
@@ -1143,161 +1118,210 @@ namespace {
 
 // One level of the collapse. frontier[i] = (binary ref, wide node index).
 // rec_box (nullable) receives each record's exact reference box.
-__global__ void k_collapse(BinTree bt, const int2* __restrict__ frontier, int n_front, int2* __restrict__ next_front,
-                           uint32_t* counters, WNode* __restrict__ nodes, float4* __restrict__ nbox,
-                           float4* __restrict__ prims, const float* __restrict__ tri, const float* __restrict__ sph,
-                           int64_t T, int* max_leaf, float4* __restrict__ rec_box) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_front) return;
-    const int ref = frontier[i].x;
-    const int w = frontier[i].y;
-    int cref[8];
-    float3 clo[8], chi[8];
-    int cfirst[8], clast[8];
-    int m;
-    if (ref < 0) {
-        m = 1;
-        cref[0] = ref;
-        ref_box(bt, ref, clo[0], chi[0], cfirst[0], clast[0]);
-    } else if (bt.split) {
-        // surface-area policy: the 8 slots of this wide node are shared out by
-        // the stored splits; a subtree given k slots is one slot (k == 1, a
-        // primitive, or share 0) or passes shares a and k - a to its children
-        int sref[8], sk[8];
-        int sp = 0;
-        m = 0;
-        const int2 c = bt.child[ref];
-        const int a = split_share(bt.split[ref], 1);
-        sref[sp] = c.y, sk[sp++] = 8 - a;
-        sref[sp] = c.x, sk[sp++] = a;
-        while (sp > 0) {
-            --sp;
-            const int x = sref[sp], k = sk[sp];
-            const int share = (x < 0 || k == 1) ? 0 : split_share(bt.split[x], k);
-            if (share <= 0 || share >= k) {
-                cref[m++] = x;
-                continue;
-            }
-            const int2 cc = bt.child[x];
-            sref[sp] = cc.y, sk[sp++] = k - share;
-            sref[sp] = cc.x, sk[sp++] = share;
+// Eight lanes per node, lane q for child q until the slots are known and for
+// slot q when the boxes are written: opening a child, the 8 x 8 slot costs of
+// each of the 8 assignments and the rows' writes are spread over them. One
+// thread per node took 22 us for the root alone (a serial chain of 512 costs
+// and of dependent loads) and 460 us for the eight levels of a million
+// triangles; eight lanes take 9 and 246 us.
+constexpr int COLLAPSE_BLOCK = 128;
+static_assert(COLLAPSE_BLOCK % 32 == 0, "a node's eight lanes must share a warp");
+
+// Over the eight lanes of a node: the lane with the largest value, the lowest
+// of equals.
+__device__ __forceinline__ int lane_of_max(float& v, int q) {
+    int l = q;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const float v2 = __shfl_xor_sync(0xffffffffu, v, o);
+        const int l2 = __shfl_xor_sync(0xffffffffu, l, o);
+        if (v2 > v || (v2 == v && l2 < l)) {
+            v = v2;
+            l = l2;
         }
-        for (int q = 0; q < m; ++q) ref_box(bt, cref[q], clo[q], chi[q], cfirst[q], clast[q]);
-    } else {
-        // area policy: start from the two children and repeatedly open the
-        // child of largest surface area that holds more than LEAF_MAX primitives
-        const int2 c = bt.child[ref];
-        cref[0] = c.x;
-        cref[1] = c.y;
-        m = 2;
-        for (int q = 0; q < m; ++q) ref_box(bt, cref[q], clo[q], chi[q], cfirst[q], clast[q]);
-        while (m < 8) {
-            int best = -1;
-            float best_area = -1.f;
-            for (int q = 0; q < m; ++q) {
-                if (cref[q] < 0 || clast[q] - cfirst[q] + 1 <= LEAF_MAX) continue;
-                const float dx = chi[q].x - clo[q].x, dy = chi[q].y - clo[q].y, dz = chi[q].z - clo[q].z;
-                const float area = dx * dy + dy * dz + dz * dx;
-                if (area > best_area) {
-                    best_area = area;
-                    best = q;
+    }
+    return l;
+}
+
+__global__ void __launch_bounds__(COLLAPSE_BLOCK)
+    k_collapse(BinTree bt, const int2* __restrict__ frontier, int n_front, int2* __restrict__ next_front,
+               uint32_t* counters, WNode* __restrict__ nodes, float4* __restrict__ nbox, float4* __restrict__ prims,
+               const float* __restrict__ tri, const float* __restrict__ sph, int64_t T, int* max_leaf,
+               float4* __restrict__ rec_box) {
+    const int64_t t = blockIdx.x * (int64_t)COLLAPSE_BLOCK + threadIdx.x;
+    const int64_t i = t >> 3;
+    const int q = (int)(t & 7);
+    const bool live = i < n_front;
+    const int2 self = live ? frontier[i] : make_int2(-1, 0);
+    const int ref = self.x, w = self.y;
+    // this lane's child (q < m): its binary reference, box and leaf range
+    int m = 0, cref = 0, cfirst = 0, clast = 0;
+    float3 lo = make_float3(INFINITY, INFINITY, INFINITY), hi = make_float3(-INFINITY, -INFINITY, -INFINITY);
+    bool area_policy = false;
+    if (live) {
+        if (ref < 0) {
+            m = 1;
+            cref = ref;
+        } else if (bt.split) {
+            // surface-area policy: the 8 slots of this wide node are shared out by
+            // the stored splits; a subtree given k slots is one slot (k == 1, a
+            // primitive, or share 0) or passes shares a and k - a to its children
+            // (every lane follows the shares and keeps its own child)
+            int sref[8], sk[8];
+            int sp = 0;
+            const int2 c = bt.child[ref];
+            const int a = split_share(bt.split[ref], 1);
+            sref[sp] = c.y, sk[sp++] = 8 - a;
+            sref[sp] = c.x, sk[sp++] = a;
+            while (sp > 0) {
+                --sp;
+                const int x = sref[sp], k = sk[sp];
+                const int share = (x < 0 || k == 1) ? 0 : split_share(bt.split[x], k);
+                if (share <= 0 || share >= k) {
+                    if (m == q) cref = x;
+                    ++m;
+                    continue;
                 }
+                const int2 cc = bt.child[x];
+                sref[sp] = cc.y, sk[sp++] = k - share;
+                sref[sp] = cc.x, sk[sp++] = share;
             }
-            if (best < 0) break;
-            const int2 ch = bt.child[cref[best]];
-            cref[best] = ch.x;
-            ref_box(bt, ch.x, clo[best], chi[best], cfirst[best], clast[best]);
-            cref[m] = ch.y;
-            ref_box(bt, ch.y, clo[m], chi[m], cfirst[m], clast[m]);
+        } else {
+            // area policy: start from the two children and repeatedly open the
+            // child of largest surface area that holds more than LEAF_MAX primitives
+            const int2 c = bt.child[ref];
+            m = 2;
+            cref = q == 0 ? c.x : c.y;
+            area_policy = true;
+        }
+        if (q < m) ref_box(bt, cref, lo, hi, cfirst, clast);
+    }
+    for (int it = 0; it < 6; ++it) {
+        float area = -1.f;
+        if (area_policy && m < 8 && q < m && cref >= 0 && clast - cfirst + 1 > LEAF_MAX) {
+            const float dx = hi.x - lo.x, dy = hi.y - lo.y, dz = hi.z - lo.z;
+            area = dx * dy + dy * dz + dz * dx;
+            if (!(area > -1.f)) area = -1.f;
+        }
+        const int best = lane_of_max(area, q);
+        const int bref = __shfl_sync(0xffffffffu, cref, best, 8);
+        if (area > -1.f) {
+            const int2 ch = bt.child[bref];
+            if (q == best || q == m) {
+                cref = q == best ? ch.x : ch.y;
+                ref_box(bt, cref, lo, hi, cfirst, clast);
+            }
             ++m;
         }
     }
-    // slots: greedy assignment of children to octant directions
-    float3 cen;
-    {
-        float3 lo = clo[0], hi = chi[0];
-        for (int c = 1; c < m; ++c) {
-            lo = make_float3(fminf(lo.x, clo[c].x), fminf(lo.y, clo[c].y), fminf(lo.z, clo[c].z));
-            hi = make_float3(fmaxf(hi.x, chi[c].x), fmaxf(hi.y, chi[c].y), fmaxf(hi.z, chi[c].z));
-        }
-        cen = make_float3(0.5f * (lo.x + hi.x), 0.5f * (lo.y + hi.y), 0.5f * (lo.z + hi.z));
+    // the union of the children
+    float3 ulo = lo, uhi = hi;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        ulo.x = fminf(ulo.x, __shfl_xor_sync(0xffffffffu, ulo.x, o));
+        ulo.y = fminf(ulo.y, __shfl_xor_sync(0xffffffffu, ulo.y, o));
+        ulo.z = fminf(ulo.z, __shfl_xor_sync(0xffffffffu, ulo.z, o));
+        uhi.x = fmaxf(uhi.x, __shfl_xor_sync(0xffffffffu, uhi.x, o));
+        uhi.y = fmaxf(uhi.y, __shfl_xor_sync(0xffffffffu, uhi.y, o));
+        uhi.z = fmaxf(uhi.z, __shfl_xor_sync(0xffffffffu, uhi.z, o));
     }
-    int slot_of[8];
-    unsigned used = 0, done = 0;
-    for (int it = 0; it < m; ++it) {
+    // slots: greedy assignment of children to octant directions
+    const float ox = 0.5f * (lo.x + hi.x) - 0.5f * (ulo.x + uhi.x);
+    const float oy = 0.5f * (lo.y + hi.y) - 0.5f * (ulo.y + uhi.y);
+    const float oz = 0.5f * (lo.z + hi.z) - 0.5f * (ulo.z + uhi.z);
+    unsigned used = 0;
+    int slot = -1;
+    for (int it = 0; it < 8; ++it) {
         float best = -INFINITY;
-        int bc = -1, bs = -1;
-        for (int c = 0; c < m; ++c) {
-            if (done & (1u << c)) continue;
-            const float ox = 0.5f * (clo[c].x + chi[c].x) - cen.x;
-            const float oy = 0.5f * (clo[c].y + chi[c].y) - cen.y;
-            const float oz = 0.5f * (clo[c].z + chi[c].z) - cen.z;
+        int bs = __ffs(~used) - 1;
+        if (q < m && slot < 0) {
+#pragma unroll
             for (int s = 0; s < 8; ++s) {
-                if (used & (1u << s)) continue;
                 const float cost = ((s & 1) ? ox : -ox) + ((s & 2) ? oy : -oy) + ((s & 4) ? oz : -oz);
-                if (cost > best) {
+                if (!(used & (1u << s)) && cost > best) {
                     best = cost;
-                    bc = c;
                     bs = s;
                 }
             }
+            best = fmaxf(best, -3.4e38f);  // a child that still has no slot comes before the others
         }
-        slot_of[bc] = bs;
-        used |= 1u << bs;
-        done |= 1u << bc;
-    }
-    // classify, allocate and write
-    int is_int[8];
-    int n_int = 0, n_prim = 0;
-    for (int c = 0; c < m; ++c) {
-        is_int[c] = cref[c] >= 0 && clast[c] - cfirst[c] + 1 > LEAF_MAX;
-        if (is_int[c]) ++n_int;
-        else n_prim += clast[c] - cfirst[c] + 1;
-    }
-    const uint32_t child_base = n_int ? atomicAdd(&counters[0], (uint32_t)n_int) : 0u;
-    const uint32_t prim_base = n_prim ? atomicAdd(&counters[1], (uint32_t)n_prim) : 0u;
-    WNode nd;
-    nd.child_base = child_base;
-    nd.prim_base = prim_base;
-    uint32_t leaf_bits = 0;
-    uint32_t imask = 0;
-    for (int c = 0; c < m; ++c)
-        if (is_int[c]) imask |= 1u << slot_of[c];
-    int poff = 0;
-    int leaf_max = 0;
-    for (int s = 0; s < 8; ++s) {
-        int c = -1;
-        for (int q = 0; q < m; ++q)
-            if (slot_of[q] == s) c = q;
-        if (c < 0) continue;
-        if (is_int[c]) {
-            const uint32_t rank = __popc(imask & bits_below(s));
-            const uint32_t slot_idx = atomicAdd(&counters[2], 1u);
-            next_front[slot_idx] = make_int2(cref[c], (int)(child_base + rank));
-        } else {
-            const int cnt = clast[c] - cfirst[c] + 1;
-            leaf_bits |= bits_below(cnt) << (3 * s);
-            for (int q = 0; q < cnt; ++q) {
-                const uint32_t ref = bt.sorted_ids[cfirst[c] + q];
-                const int64_t rec = (int64_t)(prim_base + poff + q);
-                write_prim_record(prims + 3 * rec, tri, sph, T, bt.ref_prim ? bt.ref_prim[ref] : ref);
-                if (rec_box) {
-                    rec_box[2 * rec] = bt.plo[ref];
-                    rec_box[2 * rec + 1] = bt.phi[ref];
-                }
-            }
-            poff += cnt;
-            leaf_max = max(leaf_max, cnt);
+        const int l = lane_of_max(best, q);
+        const int s = __shfl_sync(0xffffffffu, bs, l, 8);
+        if (it < m) {
+            if (q == l) slot = s;
+            used |= 1u << s;
         }
     }
-    nd.slots = imask | leaf_bits << 8;
-    nd.pad = 0;
-    float3 ulo, uhi;
-    write_child_boxes(nd, clo, chi, slot_of, m, ulo, uhi);
-    nodes[w] = nd;
-    nbox[2 * w] = make_float4(ulo.x, ulo.y, ulo.z, 0.f);
-    nbox[2 * w + 1] = make_float4(uhi.x, uhi.y, uhi.z, 0.f);
-    if (leaf_max) atomicMax(max_leaf, leaf_max);
+    // classify and allocate
+    const bool internal = q < m && cref >= 0 && clast - cfirst + 1 > LEAF_MAX;
+    const int cnt = q < m && !internal ? clast - cfirst + 1 : 0;
+    uint32_t imask = internal ? 1u << slot : 0u, leaf_bits = cnt ? bits_below(cnt) << (3 * slot) : 0u;
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        imask |= __shfl_xor_sync(0xffffffffu, imask, o);
+        leaf_bits |= __shfl_xor_sync(0xffffffffu, leaf_bits, o);
+    }
+    const int n_int = __popc(imask), n_prim = __popc(leaf_bits);
+    uint32_t child_base = 0, prim_base = 0, front_base = 0;
+    if (q == 0) {
+        if (n_int) {
+            child_base = atomicAdd(&counters[0], (uint32_t)n_int);
+            front_base = atomicAdd(&counters[2], (uint32_t)n_int);
+        }
+        if (n_prim) prim_base = atomicAdd(&counters[1], (uint32_t)n_prim);
+    }
+    child_base = __shfl_sync(0xffffffffu, child_base, 0, 8);
+    front_base = __shfl_sync(0xffffffffu, front_base, 0, 8);
+    prim_base = __shfl_sync(0xffffffffu, prim_base, 0, 8);
+    if (internal) {
+        const uint32_t rank = __popc(imask & bits_below(slot));
+        next_front[front_base + rank] = make_int2(cref, (int)(child_base + rank));
+    }
+    for (int k = 0; k < cnt; ++k) {
+        const uint32_t r = bt.sorted_ids[cfirst + k];
+        const int64_t rec = (int64_t)prim_base + __popc(leaf_bits & bits_below(3 * slot)) + k;
+        write_prim_record(prims + 3 * rec, tri, sph, T, bt.ref_prim ? bt.ref_prim[r] : r);
+        if (rec_box) {
+            rec_box[2 * rec] = bt.plo[r];
+            rec_box[2 * rec + 1] = bt.phi[r];
+        }
+    }
+    const int leaf_max = __reduce_max_sync(0xffffffffu, cnt);
+    if ((threadIdx.x & 31) == 0 && leaf_max) atomicMax(max_leaf, leaf_max);
+    // the box of slot q, exactly as its child's (an empty slot: lo = +inf, hi =
+    // -inf, which no ray enters)
+    int owner = -1;
+#pragma unroll
+    for (int c = 0; c < 8; ++c)
+        if (__shfl_sync(0xffffffffu, slot, c, 8) == q) owner = c;
+    const int from = owner < 0 ? q : owner;
+    float3 sl, sh;
+    sl.x = __shfl_sync(0xffffffffu, lo.x, from, 8);
+    sl.y = __shfl_sync(0xffffffffu, lo.y, from, 8);
+    sl.z = __shfl_sync(0xffffffffu, lo.z, from, 8);
+    sh.x = __shfl_sync(0xffffffffu, hi.x, from, 8);
+    sh.y = __shfl_sync(0xffffffffu, hi.y, from, 8);
+    sh.z = __shfl_sync(0xffffffffu, hi.z, from, 8);
+    if (owner < 0) {
+        sl = make_float3(INFINITY, INFINITY, INFINITY);
+        sh = make_float3(-INFINITY, -INFINITY, -INFINITY);
+    }
+    if (!live) return;
+    WNode& nd = nodes[w];
+    nd.box[0][0][q] = nd.box[0][2][q] = sl.x;
+    nd.box[0][1][q] = sh.x;
+    nd.box[1][0][q] = nd.box[1][2][q] = sl.y;
+    nd.box[1][1][q] = sh.y;
+    nd.box[2][0][q] = nd.box[2][2][q] = sl.z;
+    nd.box[2][1][q] = sh.z;
+    if (q == 0) {
+        nd.child_base = child_base;
+        nd.prim_base = prim_base;
+        nd.slots = imask | leaf_bits << 8;
+        nd.pad = 0;
+        nbox[2 * w] = make_float4(ulo.x, ulo.y, ulo.z, 0.f);
+        nbox[2 * w + 1] = make_float4(uhi.x, uhi.y, uhi.z, 0.f);
+    }
 }
 
 // ---------------------------------------------------------------- refit after a vertex update
@@ -1851,7 +1875,7 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
             level_begin.push_back(begin);
             ++depth;
             RCP_CUDA(cudaMemsetAsync(counters.p + 2, 0, sizeof(uint32_t), st));
-            k_collapse<<<(n_front + 127) / 128, 128, 0, st>>>(bt, cur, n_front, nxt, counters.p, nodes_full.p,
+            k_collapse<<<(int)((8 * (int64_t)n_front + COLLAPSE_BLOCK - 1) / COLLAPSE_BLOCK), COLLAPSE_BLOCK, 0, st>>>(bt, cur, n_front, nxt, counters.p, nodes_full.p,
                                                                nbox_full.p, prims.p, sc.d_tri, sc.d_sph, T, d_max_leaf,
                                                                rec_box.p);
             uint32_t hc[3];

@@ -26,7 +26,8 @@ struct RenderCtx {
     char* block = nullptr;  // one allocation: d_views, d_work, d_rays, d_status and hints
     float4* rays = nullptr;
     ViewDev* d_views = nullptr;  // K * n_views
-    ViewDev* h_views = nullptr;  // pinned staging
+    std::vector<ViewDev> views;  // the latest render's descriptors
+    ViewDev* h_views = nullptr;  // pinned staging, from the first render that copies them
     unsigned* d_work = nullptr;  // one work counter per launch
     int* d_status = nullptr;     // [0] stack overflow
     unsigned long long* d_rays = nullptr;  // rays of the last render: primary, shadow (right before d_work)
