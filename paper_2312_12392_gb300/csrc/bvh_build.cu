@@ -35,6 +35,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <cmath>
 #include <string>
 #include <vector>
 
@@ -608,106 +609,123 @@ constexpr int PLOC_TILE = PLOC_BLOCK * PLOC_ITEMS;
 constexpr unsigned long long PLOC_AGG = 1ull << 62, PLOC_INC = 2ull << 62, PLOC_COUNTS = (1ull << 62) - 1;
 constexpr int PLOC_SPINS = 1 << 26;
 
+// Called by one whole warp of a block: publishes the tile's counts and returns
+// the sum of the earlier tiles', 32 of them per round of loads. Past
+// PLOC_SPINS polls it records an error and goes on.
+__device__ __forceinline__ unsigned long long counts_before(unsigned long long* status, int64_t tile,
+                                                            unsigned long long total, int* err) {
+    const int lane = threadIdx.x & 31;
+    volatile unsigned long long* st = status;
+    if (lane == 0) st[tile] = (tile == 0 ? PLOC_INC : PLOC_AGG) | total;
+    unsigned long long before = 0;
+    int64_t t = tile - 1;
+    for (int spins = 0; t >= 0;) {
+        unsigned long long w = PLOC_INC;  // before the first tile: nothing more to add
+        if (t >= lane) w = st[t - lane];
+        const unsigned waiting = __ballot_sync(0xffffffffu, (w >> 62) == 0);
+        const unsigned inclusive = __ballot_sync(0xffffffffu, (w >> 62) == 2);
+        // the nearest tiles up to the first inclusive one, if none of them still counts
+        const int last = inclusive ? __ffs(inclusive) - 1 : 31;
+        const unsigned use = 0xffffffffu >> (31 - last);
+        if (waiting & use) {
+            if (++spins > PLOC_SPINS) {
+                if (lane == 0) atomicAdd(err, 1);
+                break;
+            }
+            continue;
+        }
+        unsigned long long v = (use >> lane) & 1u ? w & PLOC_COUNTS : 0ull;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        before += v;
+        if (inclusive) break;
+        t -= 32;
+    }
+    if (lane == 0 && tile > 0) st[tile] = PLOC_INC | (before + total);
+    return before;
+}
+
 __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_merge(const int* __restrict__ nn, PlocState* __restrict__ state,
                                                            unsigned* ticket, unsigned long long* status, int64_t N,
                                                            const int* __restrict__ ref, const float4* __restrict__ clo,
                                                            const float4* __restrict__ chi, int* __restrict__ ref_out,
                                                            float4* __restrict__ lo_out, float4* __restrict__ hi_out,
                                                            PlocTree tree, int* err) {
-    __shared__ unsigned long long s_warp[PLOC_BLOCK / 32];
+    constexpr int WARPS = PLOC_BLOCK / 32, ROWS = PLOC_ITEMS * WARPS;
+    static_assert(ROWS == 32, "one warp scans the rows' counts");
+    __shared__ unsigned long long s_row[ROWS];  // per 32 clusters: counts before them in the tile
     __shared__ unsigned long long s_before;
     __shared__ unsigned s_tile;
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
-    const int64_t n = state->n, tile = s_tile, base = tile * PLOC_TILE + threadIdx.x * PLOC_ITEMS;
+    const int64_t n = state->n, tile = s_tile;
     if (tile * PLOC_TILE >= n) return;
-    // per cluster: merges here (the lower end of a mutual pair) << 31 | stays
-    int partner[PLOC_ITEMS];
-    unsigned long long flag[PLOC_ITEMS], mine = 0;
-#pragma unroll
-    for (int q = 0; q < PLOC_ITEMS; ++q) {
-        const int64_t i = base + q;
-        partner[q] = -1;
-        flag[q] = 0;
-        if (i < n) {
-            const int j = nn[i];
-            if (j >= 0 && nn[j] == (int)i) partner[q] = j;
-            const bool gone = partner[q] >= 0 && i > j;
-            flag[q] = gone ? 0ull : (partner[q] >= 0 ? 1ull << 31 : 0ull) | 1ull;
-        }
-        mine += flag[q];
-    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long x = mine;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) s_warp[warp] = x;
-    __syncthreads();
-    unsigned long long total = 0, run = x - mine;
-    for (int w = 0; w < PLOC_BLOCK / 32; ++w) {
-        if (w < warp) run += s_warp[w];
-        total += s_warp[w];
-    }
-    if (warp == 0) {  // 32 earlier tiles per round of the look-back
-        volatile unsigned long long* st = status;
-        if (lane == 0) st[tile] = (tile == 0 ? PLOC_INC : PLOC_AGG) | total;
-        unsigned long long before = 0;
-        int64_t t = tile - 1;
-        for (int spins = 0; t >= 0;) {
-            unsigned long long w = PLOC_INC;  // before the first tile: nothing more to add
-            if (t >= lane) w = st[t - lane];
-            const unsigned waiting = __ballot_sync(0xffffffffu, (w >> 62) == 0);
-            const unsigned inclusive = __ballot_sync(0xffffffffu, (w >> 62) == 2);
-            // the nearest tiles up to the first inclusive one, if none of them still counts
-            const int last = inclusive ? __ffs(inclusive) - 1 : 31;
-            const unsigned use = 0xffffffffu >> (31 - last);
-            if (waiting & use) {
-                if (++spins > PLOC_SPINS) {
-                    if (lane == 0) atomicAdd(err, 1);
-                    break;
-                }
-                continue;
-            }
-            unsigned long long v = (use >> lane) & 1u ? w & PLOC_COUNTS : 0ull;
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            before += v;
-            if (inclusive) break;
-            t -= 32;
-        }
-        if (lane == 0) {
-            if (tile > 0) st[tile] = PLOC_INC | (before + total);
-            s_before = before;
-        }
-    }
-    __syncthreads();
-    run += s_before;
-    const int created = state->created;
+    // cluster q PLOC_BLOCK + threadIdx.x of the tile: per row of 32, ballots
+    // give the counts and each lane's place. Merges (the lower end of a mutual
+    // pair) << 31 | stays.
+    int partner[PLOC_ITEMS];
+    unsigned merges[PLOC_ITEMS], stays[PLOC_ITEMS];
 #pragma unroll
     for (int q = 0; q < PLOC_ITEMS; ++q) {
-        const int64_t i = base + q;
-        if (flag[q]) {
-            const int64_t pos = (int64_t)(run & 0x7fffffffull);
-            float4 l = clo[i], h = chi[i];
-            int r = ref[i];
-            if (partner[q] >= 0) {
-                const int j = partner[q];
-                const int node = (int)(N - 2 - created - (int64_t)(run >> 31));
-                const float4 la = l, ha = h;
-                box_union(la, ha, clo[j], chi[j], l, h);
-                ploc_new_node(tree, node, r, ref[j], l, h);
-                r = node;
-            }
-            ref_out[pos] = r;
-            lo_out[pos] = l;
-            hi_out[pos] = h;
-        }
-        run += flag[q];
+        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
+        partner[q] = i < n ? nn[i] : -1;
     }
-    if ((tile + 1) * PLOC_TILE >= n && threadIdx.x == PLOC_BLOCK - 1) {  // the last tile: run is the round's total
-        const int merges = (int)(run >> 31);
-        state[1] = PlocState{(int)(run & 0x7fffffffull), created + merges, state->stalled | (n > 1 && merges == 0), 0};
+#pragma unroll
+    for (int q = 0; q < PLOC_ITEMS; ++q) {
+        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
+        if (partner[q] >= 0 && nn[partner[q]] != (int)i) partner[q] = -1;
+    }
+#pragma unroll
+    for (int q = 0; q < PLOC_ITEMS; ++q) {
+        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
+        const bool merge = partner[q] > i, gone = partner[q] >= 0 && partner[q] < i;
+        merges[q] = __ballot_sync(0xffffffffu, merge);
+        stays[q] = __ballot_sync(0xffffffffu, i < n && !gone);
+        if (lane == 0)
+            s_row[q * WARPS + warp] = (unsigned long long)__popc(merges[q]) << 31 | (unsigned)__popc(stays[q]);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        const unsigned long long mine = s_row[lane];
+        unsigned long long x = mine;
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += y;
+        }
+        s_row[lane] = x - mine;
+        const unsigned long long total = __shfl_sync(0xffffffffu, x, 31);
+        const unsigned long long before = counts_before(status, tile, total, err);
+        if (lane == 0) s_before = before;
+        // the last tile's counts and those before it are the round's
+        if (lane == 0 && (tile + 1) * PLOC_TILE >= n) {
+            const unsigned long long all = before + total;
+            const int merged = (int)(all >> 31);
+            state[1] = PlocState{(int)(all & 0x7fffffffull), state->created + merged,
+                                 state->stalled | (n > 1 && merged == 0), 0};
+        }
+    }
+    __syncthreads();
+    const int created = state->created;
+    const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+    for (int q = 0; q < PLOC_ITEMS; ++q) {
+        if (!((stays[q] >> lane) & 1u)) continue;
+        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
+        const unsigned long long run = s_before + s_row[q * WARPS + warp];
+        const int64_t pos = (int64_t)(run & 0x7fffffffull) + __popc(stays[q] & lt);
+        float4 l = clo[i], h = chi[i];
+        int r = ref[i];
+        if (partner[q] >= 0) {
+            const int j = partner[q];
+            const int node = (int)(N - 2 - created - (int64_t)(run >> 31) - __popc(merges[q] & lt));
+            const float4 la = l, ha = h;
+            box_union(la, ha, clo[j], chi[j], l, h);
+            ploc_new_node(tree, node, r, ref[j], l, h);
+            r = node;
+        }
+        ref_out[pos] = r;
+        lo_out[pos] = l;
+        hi_out[pos] = h;
     }
 }
 
@@ -1567,8 +1585,8 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
                       int* d_err, int cap, Arena& arena, cudaStream_t st) {
     Carved<int> ref_a, ref_b, nn, cnt, pos;
     Carved<float4> lo_a, hi_a, lo_b, hi_b;
-    // per batch of PLOC_BATCH rounds: the rounds' states, tile counters and tile status
-    constexpr int PLOC_BATCH = 4;
+    // per batch of up to PLOC_BATCH rounds: the rounds' states, tile counters and tile status
+    constexpr int PLOC_BATCH = 16;
     Carved<PlocState> state;
     Carved<unsigned long long> marks;
     const int64_t tiles_max = (N + PLOC_TILE - 1) / PLOC_TILE;
@@ -1596,8 +1614,12 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
     // only shrinks. The host reads the count once per batch.
     while (h.n > PLOC_LAST) {
         const int64_t n0 = h.n, tiles = (n0 + PLOC_TILE - 1) / PLOC_TILE;
+        // a round leaves three clusters of four or a little more: as many
+        // rounds as that ratio needs, an even number of array swaps
+        const int need = (int)std::ceil(std::log((double)n0 / PLOC_LAST) / std::log(4.0 / 3.0));
+        const int rounds = std::min(PLOC_BATCH, std::max(2, (need + 1) & ~1));
         RCP_CUDA(cudaMemsetAsync(marks.p, 0, sizeof(unsigned long long) * PLOC_BATCH * (1 + tiles), st));
-        for (int r = 0; r < PLOC_BATCH; ++r) {
+        for (int r = 0; r < rounds; ++r) {
             k_ploc_nn<<<(unsigned)((n0 + PLOC_BLOCK - 1) / PLOC_BLOCK), PLOC_BLOCK, 0, st>>>(lin, hin, state.p + r,
                                                                                               nn.p);
             k_ploc_merge<<<(unsigned)tiles, PLOC_BLOCK, 0, st>>>(
@@ -1608,7 +1630,7 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
             std::swap(hin, hout);
         }
         RCP_CUDA(cudaGetLastError());
-        RCP_CUDA(cudaMemcpyAsync(state.p, state.p + PLOC_BATCH, sizeof(h), cudaMemcpyDeviceToDevice, st));
+        RCP_CUDA(cudaMemcpyAsync(state.p, state.p + rounds, sizeof(h), cudaMemcpyDeviceToDevice, st));
         RCP_CUDA(cudaMemcpyAsync(&h, state.p, sizeof(h), cudaMemcpyDeviceToHost, st));
         RCP_CUDA(cudaStreamSynchronize(st));
         // the smallest pair is always mutual, so a round without a merge means
