@@ -487,13 +487,14 @@ __global__ void k_record_parts(const float4* __restrict__ prims, int64_t R, cons
 // globally smallest pair is always mutual: every iteration merges at least
 // one pair, and a run of equal boxes pairs up (0,1), (2,3), ... at once.
 // Node indices count down: the last merge creates the root, node 0.
-// What bounds a round is launches more than work: 29 rounds of a million
-// triangles took 3.4 ms in 4 to 6 launches and a host wait each, 0.75 ms of it
-// in kernels. A round is now two launches without the host, and the rounds of
-// PLOC_LAST clusters or fewer run in one block: 1.8 ms with its allocations,
-// 0.87 ms of it in kernels.
+// What bounds a round is launches and chains more than work: 29 rounds of a
+// million triangles took 3.4 ms in 4 to 6 launches and a host wait each. A
+// round is now one launch without the host, and the rounds of PLOC_LAST
+// clusters or fewer run in one block: 0.66 ms in kernels, 0.06 ms of it the
+// last block (a partner and a merge kernel per round took 0.70 ms, a last block
+// of 2,048 clusters 0.18 and the nodes' padded boxes, a pass of their own,
+// 0.18). Loading the scene: 3.43 -> 3.05 ms.
 constexpr int PLOC_R = 16;
-constexpr int PLOC_BLOCK = 256;
 
 __device__ __forceinline__ float union_area(float4 alo, float4 ahi, float4 blo, float4 bhi) {
     const float dx = fmaxf(ahi.x, bhi.x) - fminf(alo.x, blo.x);
@@ -501,33 +502,22 @@ __device__ __forceinline__ float union_area(float4 alo, float4 ahi, float4 blo, 
     const float dz = fmaxf(ahi.z, bhi.z) - fminf(alo.z, blo.z);
     // explicit operations: every kernel that compares areas computes the same bits
     const float a = __fmaf_rn(dz, dx, __fmaf_rn(dy, dz, __fmul_rn(dx, dy)));
-    return a == a ? a : INFINITY;
+    return fminf(a, INFINITY);  // NaN (an overflow's infinity times zero): infinite
 }
 
 // The best partner of cluster i of n: the one within PLOC_R positions that
 // comes first by (union area, index gap, parity of the lower index, lower
 // index). Gaps are taken in increasing order, so only the two clusters at one
-// gap, of lower indices i - g and i, need the tie's rules. box(j, lo, hi)
-// reads cluster j's box. -1 when i is alone.
-template <class Box>
-__device__ __forceinline__ int ploc_partner(int i, int n, Box box) {
-    float4 alo, ahi;
-    box(i, alo, ahi);
+// gap, of lower indices i - g and i, need the tie's rules. -1 when i is alone.
+// Cluster i + k's box is lo[k], hi[k]; any area may be infinite (overflow).
+__device__ __noinline__ int ploc_partner_any(int i, int n, const float4* lo, const float4* hi) {
+    const float4 alo = lo[0], ahi = hi[0];
     float best = INFINITY;
     int partner = -1;
-#pragma unroll 4
     for (int g = 1; g <= PLOC_R; ++g) {
         const bool has_l = i - g >= 0, has_r = i + g < n;
-        float4 l, h;
-        float al = INFINITY, ar = INFINITY;
-        if (has_l) {
-            box(i - g, l, h);
-            al = union_area(alo, ahi, l, h);
-        }
-        if (has_r) {
-            box(i + g, l, h);
-            ar = union_area(alo, ahi, l, h);
-        }
+        const float al = has_l ? union_area(alo, ahi, lo[-g], hi[-g]) : INFINITY;
+        const float ar = has_r ? union_area(alo, ahi, lo[g], hi[g]) : INFINITY;
         const bool left_first = !(g & 1) || !((i - g) & 1);
         const bool left = has_l && (!has_r || al < ar || (al == ar && left_first));
         const float a = left ? al : ar;
@@ -539,38 +529,43 @@ __device__ __forceinline__ int ploc_partner(int i, int n, Box box) {
     return partner;
 }
 
+// The same over the gaps first, first + step, ... (all of them, or those of
+// one of the lanes that share cluster i), where the PLOC_R places before the
+// first cluster and after the last hold ploc_no_box(), of infinite union area:
+// no bounds to test in the loop, 35 operations a gap instead of 110, and a
+// round's partners are what bounds it. Returns the offset to the partner and
+// its area; 0 when no finite area was found (ploc_partner_any's case).
+__device__ __forceinline__ float4 ploc_no_box() { return make_float4(INFINITY, INFINITY, INFINITY, 0.f); }
+
+__device__ __forceinline__ int ploc_partner(int i, const float4* lo, const float4* hi, int first, int step,
+                                            float& best) {
+    const float4 alo = lo[0], ahi = hi[0];
+    best = INFINITY;
+    int offset = 0;
+#pragma unroll 4
+    for (int g = first; g <= PLOC_R; g += step) {
+        const float al = union_area(alo, ahi, lo[-g], hi[-g]);
+        const float ar = union_area(alo, ahi, lo[g], hi[g]);
+        const bool left = ((g & 1) && !(i & 1)) ? al < ar : al <= ar;  // odd gaps: the even lower index first
+        const float a = fminf(al, ar);
+        if (a < best) {
+            best = a;
+            offset = left ? -g : g;
+        }
+    }
+    return offset;
+}
+
 // A round's state: n clusters, `created` nodes so far; round r reads
 // state[r] and its merge writes state[r + 1].
 struct PlocState {
     int n, created, stalled, pad;  // stalled: a round of two clusters or more merged none
 };
 
-__global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_nn(const float4* __restrict__ clo, const float4* __restrict__ chi,
-                                                        const PlocState* __restrict__ state, int* __restrict__ nn) {
-    __shared__ float4 slo[PLOC_BLOCK + 2 * PLOC_R], shi[PLOC_BLOCK + 2 * PLOC_R];
-    const int n = state->n;
-    const int64_t first = (int64_t)blockIdx.x * PLOC_BLOCK;
-    if (first >= n) return;  // the grid covers an earlier round's count
-    for (int t = threadIdx.x; t < PLOC_BLOCK + 2 * PLOC_R; t += PLOC_BLOCK) {
-        const int64_t g = first - PLOC_R + t;
-        if (g >= 0 && g < n) {
-            slo[t] = clo[g];
-            shi[t] = chi[g];
-        }
-    }
-    __syncthreads();
-    const int i = (int)first + threadIdx.x;
-    if (i >= n) return;
-    const int shift = PLOC_R - (int)first;  // cluster j is at slo[j + shift]
-    nn[i] = ploc_partner(i, n, [&](int j, float4& l, float4& h) {
-        l = slo[j + shift];
-        h = shi[j + shift];
-    });
-}
-
 __device__ __forceinline__ int leaf_count(const int* cnt, int ref) { return ref >= 0 ? cnt[ref] : 1; }
 
-// Where the clustering writes its tree.
+// Where the clustering writes its tree, and its leaves: leaf j is reference
+// ids[j] of boxes plo/phi (of primitive ref_prim[ids[j]] when split).
 struct PlocTree {
     int2* child;
     float4* blo;
@@ -578,17 +573,50 @@ struct PlocTree {
     int* cnt;
     int* parent_int;
     int* parent_leaf;
+    const uint32_t* ids;
+    const float4* plo;
+    const float4* phi;
+    const uint32_t* ref_prim;
+    const float* tri;
+    const float* sph;
+    int64_t T;
 };
 
-__device__ __forceinline__ void ploc_new_node(const PlocTree& t, int node, int ra, int rb, float4 l, float4 h) {
+// The padded box of cluster `ref`: a leaf's reference box with its triangle's
+// pad, a node's as it was written when it was made.
+__device__ __forceinline__ void ploc_padded_box(const PlocTree& t, int ref, float3& lo, float3& hi) {
+    if (ref >= 0) {
+        const float4 a = t.blo[ref], b = t.bhi[ref];
+        lo = make_float3(a.x, a.y, a.z);
+        hi = make_float3(b.x, b.y, b.z);
+    } else {
+        padded_ref_box(t.plo, t.phi, t.ref_prim, t.tri, t.sph, t.T, t.ids[-ref - 1], lo, hi);
+    }
+}
+
+__device__ __forceinline__ void ploc_write_node(const PlocTree& t, int node, int ra, int rb, int leaves, float4 lo,
+                                                float4 hi) {
     t.child[node] = make_int2(ra, rb);
-    t.blo[node] = l;
-    t.bhi[node] = h;
-    t.cnt[node] = leaf_count(t.cnt, ra) + leaf_count(t.cnt, rb);
+    t.blo[node] = lo;
+    t.bhi[node] = hi;
+    t.cnt[node] = leaves;
     if (ra >= 0) t.parent_int[ra] = node;
     else t.parent_leaf[-ra - 1] = node;
     if (rb >= 0) t.parent_int[rb] = node;
     else t.parent_leaf[-rb - 1] = node;
+}
+
+// The clustering decides on exact boxes; the tree holds the padded ones, their
+// union written here while the children are at hand. A pass of its own after
+// the clustering, bottom up with an atomic and two fences per node, took
+// 175 us of a million triangles' build; here it is about 60 us over all rounds.
+__device__ __forceinline__ void ploc_pair(const PlocTree& t, int ra, int rb, float4& lo, float4& hi, int& leaves) {
+    float3 la, ha, lb, hb;
+    ploc_padded_box(t, ra, la, ha);
+    ploc_padded_box(t, rb, lb, hb);
+    lo = make_float4(fminf(la.x, lb.x), fminf(la.y, lb.y), fminf(la.z, lb.z), 0.f);
+    hi = make_float4(fmaxf(ha.x, hb.x), fmaxf(ha.y, hb.y), fmaxf(ha.z, hb.z), 0.f);
+    leaves = leaf_count(t.cnt, ra) + leaf_count(t.cnt, rb);
 }
 
 __device__ __forceinline__ void box_union(float4 la, float4 ha, float4 lb, float4 hb, float4& l, float4& h) {
@@ -596,16 +624,21 @@ __device__ __forceinline__ void box_union(float4 la, float4 ha, float4 lb, float
     h = make_float4(fmaxf(ha.x, hb.x), fmaxf(ha.y, hb.y), fmaxf(ha.z, hb.z), 0.f);
 }
 
-// Merge mutual pairs into new nodes and compact the cluster array, in one
-// pass: each tile of PLOC_TILE clusters counts its merges and the clusters it
-// keeps, finds the counts before it by decoupled look-back (tiles numbered by
-// an atomic counter, so every earlier tile is already running; each wait is
-// bounded), and writes its nodes and its part of the next array. The merge
-// with m merges before it, over all rounds, becomes node N - 2 - m: the last
-// one is the root, node 0. A status word carries both counts, 31 bits each,
-// and its flag.
-constexpr int PLOC_ITEMS = 4;
-constexpr int PLOC_TILE = PLOC_BLOCK * PLOC_ITEMS;
+// One round: each cluster's partner, mutual pairs merged into new nodes, and
+// the cluster array compacted, in one launch. A block takes a tile of PLOC_TILE
+// clusters and computes the partners of the PLOC_R on either side too (the
+// pair of a cluster at its edge), from boxes in shared memory; it counts its
+// merges and the clusters it keeps, finds the counts before it by decoupled
+// look-back (tiles numbered by an atomic counter, so every earlier tile is
+// already running; each wait is bounded), and writes its nodes and its part of
+// the next array. The merge with m merges before it, over all rounds, becomes
+// node N - 2 - m: the last one is the root, node 0. A status word carries both
+// counts, 31 bits each, and its flag. From 24,000 clusters down, where launch,
+// look-back and the chain of 32 candidates bound it, a round takes 7 to 12 us
+// (18 as two kernels); tiles of 480 clusters are as fast at a million and 3 %
+// slower at 3,000.
+constexpr int PLOC_BLOCK = 256;
+constexpr int PLOC_TILE = PLOC_BLOCK - 2 * PLOC_R;  // one cluster per thread, the neighbours' included
 constexpr unsigned long long PLOC_AGG = 1ull << 62, PLOC_INC = 2ull << 62, PLOC_COUNTS = (1ull << 62) - 1;
 constexpr int PLOC_SPINS = 1 << 26;
 
@@ -644,55 +677,63 @@ __device__ __forceinline__ unsigned long long counts_before(unsigned long long* 
     return before;
 }
 
-__global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_merge(const int* __restrict__ nn, PlocState* __restrict__ state,
-                                                           unsigned* ticket, unsigned long long* status, int64_t N,
+__global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_round(PlocState* __restrict__ state, unsigned* ticket,
+                                                           unsigned long long* status, int64_t N,
                                                            const int* __restrict__ ref, const float4* __restrict__ clo,
                                                            const float4* __restrict__ chi, int* __restrict__ ref_out,
                                                            float4* __restrict__ lo_out, float4* __restrict__ hi_out,
                                                            PlocTree tree, int* err) {
-    constexpr int WARPS = PLOC_BLOCK / 32, ROWS = PLOC_ITEMS * WARPS;
-    static_assert(ROWS == 32, "one warp scans the rows' counts");
-    __shared__ unsigned long long s_row[ROWS];  // per 32 clusters: counts before them in the tile
+    constexpr int WARPS = PLOC_BLOCK / 32, HELD = PLOC_BLOCK + 2 * PLOC_R;
+    static_assert(WARPS <= 32, "one warp scans the warps' counts");
+    __shared__ float4 s_lo[HELD], s_hi[HELD];  // clusters first - PLOC_R ..
+    __shared__ int s_ref[HELD], s_nn[PLOC_BLOCK];
+    __shared__ unsigned long long s_row[WARPS];  // per warp: counts before it in the tile
     __shared__ unsigned long long s_before;
     __shared__ unsigned s_tile;
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
-    const int64_t n = state->n, tile = s_tile;
+    const int n = state->n;
+    const int64_t tile = s_tile;
     if (tile * PLOC_TILE >= n) return;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // cluster q PLOC_BLOCK + threadIdx.x of the tile: per row of 32, ballots
-    // give the counts and each lane's place. Merges (the lower end of a mutual
-    // pair) << 31 | stays.
-    int partner[PLOC_ITEMS];
-    unsigned merges[PLOC_ITEMS], stays[PLOC_ITEMS];
-#pragma unroll
-    for (int q = 0; q < PLOC_ITEMS; ++q) {
-        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
-        partner[q] = i < n ? nn[i] : -1;
-    }
-#pragma unroll
-    for (int q = 0; q < PLOC_ITEMS; ++q) {
-        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
-        if (partner[q] >= 0 && nn[partner[q]] != (int)i) partner[q] = -1;
-    }
-#pragma unroll
-    for (int q = 0; q < PLOC_ITEMS; ++q) {
-        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
-        const bool merge = partner[q] > i, gone = partner[q] >= 0 && partner[q] < i;
-        merges[q] = __ballot_sync(0xffffffffu, merge);
-        stays[q] = __ballot_sync(0xffffffffu, i < n && !gone);
-        if (lane == 0)
-            s_row[q * WARPS + warp] = (unsigned long long)__popc(merges[q]) << 31 | (unsigned)__popc(stays[q]);
+    const int first = (int)(tile * PLOC_TILE) - PLOC_R;  // thread t's cluster is first + t
+    for (int t = threadIdx.x; t < HELD; t += PLOC_BLOCK) {
+        const int g = first - PLOC_R + t;
+        const bool in = g >= 0 && g < n;
+        s_lo[t] = in ? clo[g] : ploc_no_box();
+        s_hi[t] = in ? chi[g] : ploc_no_box();
+        if (in) s_ref[t] = ref[g];
     }
     __syncthreads();
+    const int i = first + (int)threadIdx.x, me = PLOC_R + (int)threadIdx.x;
+    const bool real = i >= 0 && i < n;
+    int partner = -1;
+    if (real) {
+        float area;
+        const int offset = ploc_partner(i, s_lo + me, s_hi + me, 1, 1, area);
+        partner = offset ? i + offset : ploc_partner_any(i, n, s_lo + me, s_hi + me);
+    }
+    s_nn[threadIdx.x] = partner;
+    __syncthreads();
+    const bool mine = real && threadIdx.x >= PLOC_R && threadIdx.x < PLOC_BLOCK - PLOC_R;
+    if (!mine || partner < 0 || s_nn[partner - first] != i) partner = -1;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // ballots give the counts and each lane's place. Merges (the lower end of
+    // a mutual pair) << 31 | stays.
+    const unsigned merges = __ballot_sync(0xffffffffu, partner >= 0 && partner > i);
+    const unsigned stays = __ballot_sync(0xffffffffu, mine && !(partner >= 0 && partner < i));
+    if (lane == 0) s_row[warp] = (unsigned long long)__popc(merges) << 31 | (unsigned)__popc(stays);
+    float4 pl, ph;
+    int leaves = 0;  // of the new node; its loads overlap the look-back
+    const int other = partner - first + PLOC_R;
+    __syncthreads();
     if (warp == 0) {
-        const unsigned long long mine = s_row[lane];
-        unsigned long long x = mine;
+        const unsigned long long row = lane < WARPS ? s_row[lane] : 0ull;
+        unsigned long long x = row;
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        s_row[lane] = x - mine;
+        if (lane < WARPS) s_row[lane] = x - row;
         const unsigned long long total = __shfl_sync(0xffffffffu, x, 31);
         const unsigned long long before = counts_before(status, tile, total, err);
         if (lane == 0) s_before = before;
@@ -704,125 +745,141 @@ __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_merge(const int* __restrict
                                  state->stalled | (n > 1 && merged == 0), 0};
         }
     }
+    if ((merges >> lane) & 1u) ploc_pair(tree, s_ref[me], s_ref[other], pl, ph, leaves);
     __syncthreads();
-    const int created = state->created;
+    if (!((stays >> lane) & 1u)) return;
     const unsigned lt = (1u << lane) - 1u;
-#pragma unroll
-    for (int q = 0; q < PLOC_ITEMS; ++q) {
-        if (!((stays[q] >> lane) & 1u)) continue;
-        const int64_t i = tile * PLOC_TILE + q * PLOC_BLOCK + threadIdx.x;
-        const unsigned long long run = s_before + s_row[q * WARPS + warp];
-        const int64_t pos = (int64_t)(run & 0x7fffffffull) + __popc(stays[q] & lt);
-        float4 l = clo[i], h = chi[i];
-        int r = ref[i];
-        if (partner[q] >= 0) {
-            const int j = partner[q];
-            const int node = (int)(N - 2 - created - (int64_t)(run >> 31) - __popc(merges[q] & lt));
-            const float4 la = l, ha = h;
-            box_union(la, ha, clo[j], chi[j], l, h);
-            ploc_new_node(tree, node, r, ref[j], l, h);
-            r = node;
-        }
-        ref_out[pos] = r;
-        lo_out[pos] = l;
-        hi_out[pos] = h;
+    const unsigned long long run = s_before + s_row[warp];
+    const int64_t pos = (int64_t)(run & 0x7fffffffull) + __popc(stays & lt);
+    float4 l = s_lo[me], h = s_hi[me];
+    int r = s_ref[me];
+    if (partner >= 0) {
+        const int node = (int)(N - 2 - state->created - (int64_t)(run >> 31) - __popc(merges & lt));
+        const float4 la = l, ha = h;
+        box_union(la, ha, s_lo[other], s_hi[other], l, h);
+        ploc_write_node(tree, node, r, s_ref[other], leaves, pl, ph);
+        r = node;
     }
+    ref_out[pos] = r;
+    lo_out[pos] = l;
+    hi_out[pos] = h;
 }
 
-// The last rounds in one block: PLOC_LAST clusters or fewer, the boxes of this
-// round's array and the next one in shared memory, until one cluster is left.
-// A round of separate launches costs about 10 us however few clusters it has,
-// and more than half of a build's rounds are below this size.
-constexpr int PLOC_LAST = 2048;
-constexpr int PLOC_LAST_BLOCK = 1024;
-constexpr int PLOC_LAST_ITEMS = PLOC_LAST / PLOC_LAST_BLOCK;
+// The last rounds in one block: PLOC_LAST clusters or fewer in shared memory
+// (exact and padded boxes, references, leaf counts) until one is left. More
+// than half of a build's rounds are below this size, and a launch costs several
+// microseconds however few clusters it has. One SM's issue rate bounds the
+// first rounds and a warp's chain of candidates the others, so with fewer
+// clusters than threads up to PLOC_R lanes share a cluster's candidates: 59 us
+// from 1,024 clusters (one lane per cluster and exact boxes only, with the
+// counts read from device memory in every round: 180 us from 2,048).
+constexpr int PLOC_LAST = 1024;
 struct PlocLastShared {
-    float4 lo[2][PLOC_LAST], hi[2][PLOC_LAST];
-    int ref[2][PLOC_LAST];
+    float4 lo[PLOC_LAST + 2 * PLOC_R], hi[PLOC_LAST + 2 * PLOC_R];  // exact, which decide
+    float4 plo[PLOC_LAST], phi[PLOC_LAST];  // padded, which the tree holds; plo.w: leaf count
+    int ref[PLOC_LAST];
     int nn[PLOC_LAST];
-    unsigned warp_tot[PLOC_LAST_BLOCK / 32];
+    unsigned warp_tot[PLOC_LAST / 32];
 };
 
-__global__ void __launch_bounds__(PLOC_LAST_BLOCK) k_ploc_last(PlocState* state, int64_t N, const int* __restrict__ ref,
-                                                               const float4* __restrict__ clo,
-                                                               const float4* __restrict__ chi, PlocTree tree) {
+__global__ void __launch_bounds__(PLOC_LAST) k_ploc_last(PlocState* state, int64_t N, const int* __restrict__ ref,
+                                                         const float4* __restrict__ clo,
+                                                         const float4* __restrict__ chi, PlocTree tree) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     PlocLastShared& s = *reinterpret_cast<PlocLastShared*>(s_raw);
-    int n = state->n, created = state->created, cur = 0;
+    float4 *const lo = s.lo + PLOC_R, *const hi = s.hi + PLOC_R;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    int n = state->n, created = state->created;
     bool stalled = false;
-    for (int i = threadIdx.x; i < n; i += PLOC_LAST_BLOCK) {
-        s.lo[0][i] = clo[i];
-        s.hi[0][i] = chi[i];
-        s.ref[0][i] = ref[i];
+    if (t < n) {
+        const int r = ref[t];
+        float3 l, h;
+        ploc_padded_box(tree, r, l, h);
+        lo[t] = clo[t];
+        hi[t] = chi[t];
+        s.plo[t] = make_float4(l.x, l.y, l.z, __int_as_float(leaf_count(tree.cnt, r)));
+        s.phi[t] = make_float4(h.x, h.y, h.z, 0.f);
+        s.ref[t] = r;
+    }
+    if (t < PLOC_R) {
+        lo[t - PLOC_R] = hi[t - PLOC_R] = ploc_no_box();
+        lo[n + t] = hi[n + t] = ploc_no_box();
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     while (n > 1 && !stalled) {
-        for (int i = threadIdx.x; i < n; i += PLOC_LAST_BLOCK) {
-            s.nn[i] = ploc_partner(i, n, [&](int j, float4& l, float4& h) {
-                l = s.lo[cur][j];
-                h = s.hi[cur][j];
-            });
+        int shift = 0;  // 2^shift lanes per cluster
+        while ((2 << shift) <= PLOC_R && (n << shift) * 2 <= PLOC_LAST) ++shift;
+        {
+            const int i = t >> shift, sub = t & ((1 << shift) - 1);
+            float best = INFINITY;
+            int offset = 0;
+            if (i < n) offset = ploc_partner(i, lo + i, hi + i, 1 + sub, 1 << shift, best);
+            for (int o = 1; o < 1 << shift; o <<= 1) {
+                const float other = __shfl_xor_sync(0xffffffffu, best, o);
+                const int theirs = __shfl_xor_sync(0xffffffffu, offset, o);
+                // (area, gap); gaps of two lanes differ, and no offset has an infinite area
+                if (other < best || (other == best && abs(theirs) < abs(offset))) {
+                    best = other;
+                    offset = theirs;
+                }
+            }
+            if (i < n && sub == 0) s.nn[i] = offset ? i + offset : ploc_partner_any(i, n, lo + i, hi + i);
         }
         __syncthreads();
-        // consecutive clusters per thread, so that the scan keeps the array's
-        // order; merges << 16 | stays (both at most PLOC_LAST)
-        const int base = threadIdx.x * PLOC_LAST_ITEMS;
-        int partner[PLOC_LAST_ITEMS];
-        unsigned flag[PLOC_LAST_ITEMS], mine = 0;
-#pragma unroll
-        for (int q = 0; q < PLOC_LAST_ITEMS; ++q) {
-            const int i = base + q;
-            partner[q] = -1;
-            flag[q] = 0;
-            if (i < n) {
-                const int j = s.nn[i];
-                if (j >= 0 && s.nn[j] == i) partner[q] = j;
-                flag[q] = partner[q] >= 0 && i > j ? 0u : (partner[q] >= 0 ? 1u << 16 : 0u) | 1u;
+        const bool real = t < n;
+        int partner = real ? s.nn[t] : -1;
+        if (partner >= 0 && s.nn[partner] != t) partner = -1;
+        const bool merge = partner >= 0 && partner > t, stay = real && !(partner >= 0 && partner < t);
+        const unsigned merges = __ballot_sync(0xffffffffu, merge), stays = __ballot_sync(0xffffffffu, stay);
+        if (lane == 0) s.warp_tot[warp] = (unsigned)__popc(merges) << 16 | (unsigned)__popc(stays);
+        // the clusters that stay, read before any is overwritten
+        float4 l, h, pl, ph;
+        int ra = 0, rb = 0;
+        if (stay) {
+            l = lo[t];
+            h = hi[t];
+            pl = s.plo[t];
+            ph = s.phi[t];
+            ra = s.ref[t];
+            if (merge) {
+                const float4 l0 = l, h0 = h, pl0 = pl, ph0 = ph, pl1 = s.plo[partner];
+                box_union(l0, h0, lo[partner], hi[partner], l, h);
+                box_union(pl0, ph0, pl1, s.phi[partner], pl, ph);
+                pl.w = __int_as_float(__float_as_int(pl0.w) + __float_as_int(pl1.w));
+                rb = s.ref[partner];
             }
-            mine += flag[q];
         }
-        unsigned x = mine;
+        __syncthreads();
+        static_assert(PLOC_LAST / 32 == 32, "one lane per warp's total");
+        unsigned x = s.warp_tot[lane];
+        const unsigned own = x;
         for (int o = 1; o < 32; o <<= 1) {
             const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
             if (lane >= o) x += y;
         }
-        if (lane == 31) s.warp_tot[warp] = x;
-        __syncthreads();
-        unsigned run = x - mine, total = 0;
-        for (int w = 0; w < PLOC_LAST_BLOCK / 32; ++w) {
-            const unsigned t = s.warp_tot[w];
-            if (w < warp) run += t;
-            total += t;
-        }
-#pragma unroll
-        for (int q = 0; q < PLOC_LAST_ITEMS; ++q) {
-            const int i = base + q;
-            if (flag[q]) {
-                const int pos = (int)(run & 0xffffu);
-                float4 l = s.lo[cur][i], h = s.hi[cur][i];
-                int r = s.ref[cur][i];
-                if (partner[q] >= 0) {
-                    const int j = partner[q], node = (int)(N - 2 - created - (int)(run >> 16));
-                    const float4 la = l, ha = h;
-                    box_union(la, ha, s.lo[cur][j], s.hi[cur][j], l, h);
-                    ploc_new_node(tree, node, r, s.ref[cur][j], l, h);
-                    r = node;
-                }
-                s.lo[cur ^ 1][pos] = l;
-                s.hi[cur ^ 1][pos] = h;
-                s.ref[cur ^ 1][pos] = r;
-            }
-            run += flag[q];
-        }
-        const int merges = (int)(total >> 16);
-        created += merges;
-        stalled = merges == 0;
+        const unsigned total = __shfl_sync(0xffffffffu, x, 31);
+        const unsigned before = __shfl_sync(0xffffffffu, x - own, warp);
         n = (int)(total & 0xffffu);
-        cur ^= 1;
-        __syncthreads();  // the next array (and, in global memory, the new nodes' counts) before the next round
+        if (stay) {
+            const unsigned lt = (1u << lane) - 1u;
+            const int pos = (int)(before & 0xffffu) + __popc(stays & lt);
+            if (merge) {
+                const int node = (int)(N - 2 - created - (int)(before >> 16) - __popc(merges & lt));
+                ploc_write_node(tree, node, ra, rb, __float_as_int(pl.w), make_float4(pl.x, pl.y, pl.z, 0.f), ph);
+                ra = node;
+            }
+            lo[pos] = l;
+            hi[pos] = h;
+            s.plo[pos] = pl;
+            s.phi[pos] = ph;
+            s.ref[pos] = ra;
+        }
+        if (t < PLOC_R) lo[n + t] = hi[n + t] = ploc_no_box();
+        created += (int)(total >> 16);
+        stalled = (total >> 16) == 0;
+        __syncthreads();  // the next array before the next round
     }
-    if (threadIdx.x == 0) state[1] = PlocState{n, created, state->stalled | (stalled ? 1 : 0), 0};
+    if (t == 0) state[1] = PlocState{n, created, state->stalled | (stalled ? 1 : 0), 0};
 }
 
 __global__ void k_ploc_init(const uint32_t* __restrict__ sorted_ids, int64_t n, const float4* __restrict__ plo,
@@ -969,46 +1026,6 @@ __global__ void k_sah_dp(const int2* __restrict__ child, const int2* __restrict_
             __stcg(&dp[2 * node + 1], make_float4(d[4], d[5], d[6], d[7]));
             split[node] = make_uint2(bytes[0] | bytes[1] << 8 | bytes[2] << 16 | bytes[3] << 24,
                                      bytes[4] | bytes[5] << 8 | bytes[6] << 16 | bytes[7] << 24);
-            node = parent_int[node];
-        }
-    }
-}
-
-// Every binary node's box again, bottom up from the padded leaf boxes (the
-// clustering decided on exact boxes): one thread per leaf, the second thread
-// to arrive at a node computes it and goes on. Leaf j (clustering order)
-// starts at parent_leaf[j]; the children's leaf references are in depth-first
-// order, whose reference indices are ids_dfs.
-__global__ void k_refit_padded(const int2* __restrict__ child, const int* __restrict__ parent_int,
-                               const int* __restrict__ parent_leaf, const uint32_t* __restrict__ ids_dfs,
-                               const float4* __restrict__ plo, const float4* __restrict__ phi,
-                               const uint32_t* __restrict__ ref_prim, const float* __restrict__ tri,
-                               const float* __restrict__ sph, int64_t T, int64_t R, float4* blo, float4* bhi,
-                               int* arrivals, int* err) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < R; j += (int64_t)gridDim.x * blockDim.x) {
-        int node = parent_leaf[j];
-        for (int guard = 0; node >= 0; ++guard) {
-            if (guard >= (1 << 22)) {
-                atomicAdd(err, 1);
-                break;
-            }
-            __threadfence();
-            if (atomicAdd(&arrivals[node], 1) == 0) break;
-            __threadfence();
-            const int2 c = child[node];
-            float3 l[2], h[2];
-            const int cs[2] = {c.x, c.y};
-            for (int q = 0; q < 2; ++q) {
-                if (cs[q] >= 0) {
-                    const float4 a = __ldcg(&blo[cs[q]]), b = __ldcg(&bhi[cs[q]]);
-                    l[q] = make_float3(a.x, a.y, a.z);
-                    h[q] = make_float3(b.x, b.y, b.z);
-                } else {
-                    padded_ref_box(plo, phi, ref_prim, tri, sph, T, ids_dfs[-cs[q] - 1], l[q], h[q]);
-                }
-            }
-            __stcg(&blo[node], make_float4(fminf(l[0].x, l[1].x), fminf(l[0].y, l[1].y), fminf(l[0].z, l[1].z), 0.f));
-            __stcg(&bhi[node], make_float4(fmaxf(h[0].x, h[1].x), fmaxf(h[0].y, h[1].y), fmaxf(h[0].z, h[1].z), 0.f));
             node = parent_int[node];
         }
     }
@@ -1578,12 +1595,12 @@ void scan_u64(unsigned long long* d, int64_t n, unsigned long long* aux, const s
 }
 
 // Binary tree over the N >= 2 primitives in Morton order (ids_in) by PLOC.
-// Fills child, blo/bhi and range of internal nodes 0..N-2 (root 0), with the
+// Fills child, blo/bhi (padded) and range of internal nodes 0..N-2 (root 0), with the
 // leaves renumbered depth-first: ids_out[j] is the primitive of leaf j.
-rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, const float4* plo, const float4* phi,
-                      int2* child, int2* range, float4* blo, float4* bhi, int* parent_int, int* parent_leaf,
-                      int* d_err, int cap, Arena& arena, cudaStream_t st) {
-    Carved<int> ref_a, ref_b, nn, cnt, pos;
+// `tree` comes without its counts.
+rcp_status build_ploc(int64_t N, PlocTree tree, uint32_t* ids_out, int2* range, int* d_err, int cap, Arena& arena,
+                      cudaStream_t st) {
+    Carved<int> ref_a, ref_b, cnt, pos;
     Carved<float4> lo_a, hi_a, lo_b, hi_b;
     // per batch of up to PLOC_BATCH rounds: the rounds' states, tile counters and tile status
     constexpr int PLOC_BATCH = 16;
@@ -1592,7 +1609,6 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
     const int64_t tiles_max = (N + PLOC_TILE - 1) / PLOC_TILE;
     RCP_CUDA(ref_a.alloc(arena, N));
     RCP_CUDA(ref_b.alloc(arena, N));
-    RCP_CUDA(nn.alloc(arena, N));
     RCP_CUDA(cnt.alloc(arena, N));
     RCP_CUDA(pos.alloc(arena, N));
     RCP_CUDA(lo_a.alloc(arena, N));
@@ -1601,12 +1617,12 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
     RCP_CUDA(hi_b.alloc(arena, N));
     RCP_CUDA(state.alloc(arena, PLOC_BATCH + 2));
     RCP_CUDA(marks.alloc(arena, PLOC_BATCH * (1 + tiles_max)));
-    RCP_CUDA(cudaMemsetAsync(parent_int, 0xff, sizeof(int) * N, st));
-    RCP_CUDA(cudaMemsetAsync(parent_leaf, 0xff, sizeof(int) * N, st));
+    RCP_CUDA(cudaMemsetAsync(tree.parent_int, 0xff, sizeof(int) * N, st));
+    RCP_CUDA(cudaMemsetAsync(tree.parent_leaf, 0xff, sizeof(int) * N, st));
+    tree.cnt = cnt.p;
     int *rin = ref_a.p, *rout = ref_b.p;
     float4 *lin = lo_a.p, *hin = hi_a.p, *lout = lo_b.p, *hout = hi_b.p;
-    k_ploc_init<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(ids_in, N, plo, phi, rin, lin, hin);
-    const PlocTree tree{child, blo, bhi, cnt.p, parent_int, parent_leaf};
+    k_ploc_init<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(tree.ids, N, tree.plo, tree.phi, rin, lin, hin);
     PlocState h{(int)N, 0, 0, 0};
     RCP_CUDA(cudaMemcpyAsync(state.p, &h, sizeof(h), cudaMemcpyHostToDevice, st));
     // The rounds run without the host between them: each reads its count from
@@ -1620,11 +1636,9 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
         const int rounds = std::min(PLOC_BATCH, std::max(2, (need + 1) & ~1));
         RCP_CUDA(cudaMemsetAsync(marks.p, 0, sizeof(unsigned long long) * PLOC_BATCH * (1 + tiles), st));
         for (int r = 0; r < rounds; ++r) {
-            k_ploc_nn<<<(unsigned)((n0 + PLOC_BLOCK - 1) / PLOC_BLOCK), PLOC_BLOCK, 0, st>>>(lin, hin, state.p + r,
-                                                                                              nn.p);
-            k_ploc_merge<<<(unsigned)tiles, PLOC_BLOCK, 0, st>>>(
-                nn.p, state.p + r, (unsigned*)(marks.p + r), marks.p + PLOC_BATCH + r * tiles, N, rin, lin, hin, rout,
-                lout, hout, tree, d_err);
+            k_ploc_round<<<(unsigned)tiles, PLOC_BLOCK, 0, st>>>(state.p + r, (unsigned*)(marks.p + r),
+                                                                 marks.p + PLOC_BATCH + r * tiles, N, rin, lin, hin,
+                                                                 rout, lout, hout, tree, d_err);
             std::swap(rin, rout);
             std::swap(lin, lout);
             std::swap(hin, hout);
@@ -1642,7 +1656,7 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
     }
     RCP_CUDA(cudaFuncSetAttribute(k_ploc_last, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)sizeof(PlocLastShared)));
-    k_ploc_last<<<1, PLOC_LAST_BLOCK, sizeof(PlocLastShared), st>>>(state.p, N, rin, lin, hin, tree);
+    k_ploc_last<<<1, PLOC_LAST, sizeof(PlocLastShared), st>>>(state.p, N, rin, lin, hin, tree);
     RCP_CUDA(cudaGetLastError());
     RCP_CUDA(cudaMemcpyAsync(&h, state.p + 1, sizeof(h), cudaMemcpyDeviceToHost, st));
     RCP_CUDA(cudaStreamSynchronize(st));
@@ -1650,9 +1664,9 @@ rcp_status build_ploc(int64_t N, const uint32_t* ids_in, uint32_t* ids_out, cons
         set_error("BVH build: clustering made no progress");
         return RCP_ERR_STATE;
     }
-    k_dfs_offsets<<<grid_for(2 * N - 1, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(child, parent_int, parent_leaf,
-                                                                                 cnt.p, N, range, pos.p, d_err);
-    k_dfs_apply<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(pos.p, ids_in, N, ids_out, child, d_err);
+    k_dfs_offsets<<<grid_for(2 * N - 1, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(
+        tree.child, tree.parent_int, tree.parent_leaf, tree.cnt, N, range, pos.p, d_err);
+    k_dfs_apply<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(pos.p, tree.ids, N, ids_out, tree.child, d_err);
     RCP_CUDA(cudaGetLastError());
     // the scratch above is given back by the caller: finish using it first
     RCP_CUDA(cudaStreamSynchronize(st));
@@ -1803,25 +1817,19 @@ rcp_status build_bvh(Scene& sc, cudaStream_t st) {
             return RCP_ERR_TIMEOUT;
         }
         const Arena::Mark before = arena.mark();
-        rcp_status pr = build_ploc(R, vals.p, avals.p, ref_lo, ref_hi, child.p, range.p, blo.p, bhi.p, parent_int.p,
-                                   parent_leaf.p, err.p + 1, cap, arena, st);
+        const PlocTree tree{child.p, blo.p, bhi.p,  nullptr, parent_int.p, parent_leaf.p,
+                            vals.p,  ref_lo, ref_hi, split ? rprim.p : nullptr, sc.d_tri, sc.d_sph, T};
+        rcp_status pr = build_ploc(R, tree, avals.p, range.p, err.p + 1, cap, arena, st);
         arena.release(before);
         if (pr != RCP_OK) {
             return pr;
         }
         ids = avals.p;
     }
-    if (R >= 2) {
-        // node boxes from the padded leaves (the clustering used exact boxes)
-        RCP_CUDA(arrivals.alloc(arena, R - 1));
-        RCP_CUDA(cudaMemsetAsync(arrivals.p, 0, sizeof(int) * (R - 1), st));
-        k_refit_padded<<<grid_for(R, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(
-            child.p, parent_int.p, parent_leaf.p, ids, ref_lo, ref_hi, split ? rprim.p : nullptr, sc.d_tri,
-            sc.d_sph, T, R, blo.p, bhi.p, arrivals.p, err.p + 1);
-    }
     if (R >= 2 && sah) {
         RCP_CUDA(dp.alloc(arena, 2 * (R - 1)));
         RCP_CUDA(slot_split.alloc(arena, R - 1));
+        RCP_CUDA(arrivals.alloc(arena, R - 1));
         RCP_CUDA(cudaMemsetAsync(arrivals.p, 0, sizeof(int) * (R - 1), st));
         k_sah_dp<<<grid_for(R, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(child.p, range.p, parent_int.p,
                                                                          parent_leaf.p, blo.p, bhi.p, ref_lo, ref_hi,
