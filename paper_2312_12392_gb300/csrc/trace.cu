@@ -178,6 +178,8 @@ __device__ __forceinline__ void tiles_done(const ViewDev* v, int n, int lane) {
     }
 }
 
+constexpr int MS_MANY = 1, MS_FEW = 2;
+
 // MULTI: every view names its own scene (views of several scenes in one
 // launch); otherwise all views render the launch's scene S0.
 // CHAIN: one launch runs v.passes passes of each view v (v.in its first
@@ -186,13 +188,16 @@ __device__ __forceinline__ void tiles_done(const ViewDev* v, int n, int lane) {
 // pass's outputs. At one sample per pixel with a camera that reads only the
 // pixel's own previous value (every mapping but the image-space one), this
 // computes exactly what one launch per pass computes.
-// CHAIN and MS: 24 warps per SM (80 registers; what spills is the pixel's state
+// CHAIN and MS_MANY: 24 warps per SM (80 registers; what spills is the pixel's state
 // between passes, outside the walk). 20, 28 and 32 warps: 1.575, 1.574 and
 // 1.773 against 1.559 ms for a mid 1080p K = 6 frame, forest 1.810, 1.820 and
 // 1.983 against 1.785 ms; 4 samples at 720p K = 6 with 16, 20, 24 and 28 warps:
 // 3.069, 3.033, 2.964 and 3.002 ms.
-template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
-__global__ void __launch_bounds__(BLOCK, CHAIN || MS ? 768 / BLOCK : 0)
+// MS: 0 one sample per pixel, MS_MANY several samples, MS_FEW the same with 16
+// warps per SM (128 registers, nothing spilled) for a launch of few tiles, where
+// a tile's own chain of samples bounds it, not the warps in flight.
+template <int BLOCK, bool FUSED, bool COUNT, int MS, bool MULTI, bool CHAIN, bool SPILL>
+__global__ void __launch_bounds__(BLOCK, MS == MS_FEW ? 512 / BLOCK : CHAIN || MS ? 768 / BLOCK : 0)
     k_trace(SceneDev S0, const ViewDev* __restrict__ views, int n_views,
                                                  int64_t total_chunks, int chunk_tiles,
                                                  const float4* __restrict__ rays, unsigned* work, StackCfg stk,
@@ -585,7 +590,7 @@ int sm_count() {
     return sms;
 }
 
-template <int BLOCK, bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
+template <int BLOCK, bool FUSED, bool COUNT, int MS, bool MULTI, bool CHAIN, bool SPILL>
 rcp_status launch_trace_t(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                           int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
                           unsigned long long* d_counters, cudaStream_t st) {
@@ -626,7 +631,7 @@ rcp_status launch_trace_t(const SceneDev& S, const LaunchCfg& cfg, const ViewDev
 // a node: a mid 1080p K = 6 frame 1.548 -> 1.469 ms, of which 3 % are the
 // checks; forest 1.774 -> 1.699 ms). The counting and separate-camera kernels,
 // which no frame is timed on, always check.
-template <bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN, bool SPILL>
+template <bool FUSED, bool COUNT, int MS, bool MULTI, bool CHAIN, bool SPILL>
 rcp_status launch_trace_s(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                           int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
                           unsigned long long* d_counters, cudaStream_t st) {
@@ -643,7 +648,7 @@ rcp_status launch_trace_s(const SceneDev& S, const LaunchCfg& cfg, const ViewDev
     }
 }
 
-template <bool FUSED, bool COUNT, bool MS, bool MULTI, bool CHAIN = false>
+template <bool FUSED, bool COUNT, int MS, bool MULTI, bool CHAIN = false>
 rcp_status launch_trace_b(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                           int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
                           unsigned long long* d_counters, cudaStream_t st) {
@@ -663,9 +668,9 @@ rcp_status launch_trace_b(const SceneDev& S, const LaunchCfg& cfg, const ViewDev
 rcp_status launch_separate(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                            int64_t total_chunks, const float4* rays, unsigned* d_work, unsigned long long* d_rays,
                            unsigned long long* d_counters, cudaStream_t st) {
-    return cfg.count ? launch_trace_b<false, true, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+    return cfg.count ? launch_trace_b<false, true, 0, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                  d_rays, d_counters, st)
-                     : launch_trace_b<false, false, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                     : launch_trace_b<false, false, 0, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                   d_rays, d_counters, st);
 }
 
@@ -675,9 +680,9 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
                        int64_t total_pix, int64_t total_chunks, float4* rays, unsigned* d_work,
                        unsigned long long* d_rays, unsigned long long* d_counters, cudaStream_t st) {
     if (cfg.multi) {  // views of several scenes: fused camera, no counters
-        return cfg.ms ? launch_trace_b<true, false, true, true>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+        return cfg.ms ? launch_trace_b<true, false, MS_MANY, true>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                 d_rays, nullptr, st)
-                      : launch_trace_b<true, false, false, true>(S, cfg, d_views, n_views, total_chunks, rays,
+                      : launch_trace_b<true, false, 0, true>(S, cfg, d_views, n_views, total_chunks, rays,
                                                                  d_work, d_rays, nullptr, st);
     }
     if (!cfg.fused && !cfg.ms) {
@@ -691,14 +696,23 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
         return launch_separate(S, behind_camera, d_views, n_views, total_chunks, rays, d_work, d_rays, d_counters, st);
     }
     if (cfg.ms) {  // jittered samples: camera inside the trace kernel
-        return cfg.count ? launch_trace_b<true, true, true, false>(S, cfg, d_views, n_views, total_chunks, rays,
-                                                                   d_work, d_rays, d_counters, st)
-                         : launch_trace_b<true, false, true, false>(S, cfg, d_views, n_views, total_chunks, rays,
-                                                                    d_work, d_rays, d_counters, st);
-    }
-    return cfg.count ? launch_trace_b<true, true, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+        if (cfg.count)
+            return launch_trace_b<true, true, MS_MANY, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                              d_rays, d_counters, st);
+        // Up to four tiles per resident warp of MS_FEW its shorter chains win:
+        // of 20 frames below the line (terrain and forest, 1 to 6 passes, 1 to 4
+        // samples) it was 2 to 8 % faster on 17 and 1 to 3 % slower on 3 (5,600
+        // to 7,900 tiles); above it 24 warps win by 3 to 9 % from 14,000 tiles on.
+        const int64_t tiles = total_chunks * (cfg.chunk / 32);
+        return tiles <= 4 * 16 * (int64_t)sm_count()
+                   ? launch_trace_b<true, false, MS_FEW, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                 d_rays, d_counters, st)
-                     : launch_trace_b<true, false, false, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                   : launch_trace_b<true, false, MS_MANY, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                 d_rays, d_counters, st);
+    }
+    return cfg.count ? launch_trace_b<true, true, 0, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
+                                                                d_rays, d_counters, st)
+                     : launch_trace_b<true, false, 0, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                  d_rays, d_counters, st);
 }
 
@@ -709,9 +723,9 @@ rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* 
         return RCP_ERR_STATE;
     }
     if (cfg.multi)  // views of several scenes: no counters
-        return launch_trace_b<true, false, false, true, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
+        return launch_trace_b<true, false, 0, true, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
                                                               d_rays, nullptr, st);
-    return launch_trace_b<true, false, false, false, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
+    return launch_trace_b<true, false, 0, false, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
                                                            d_rays, nullptr, st);
 }
 
