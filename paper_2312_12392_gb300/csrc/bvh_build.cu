@@ -500,8 +500,10 @@ __device__ __forceinline__ float union_area(float4 alo, float4 ahi, float4 blo, 
     const float dx = fmaxf(ahi.x, bhi.x) - fminf(alo.x, blo.x);
     const float dy = fmaxf(ahi.y, bhi.y) - fminf(alo.y, blo.y);
     const float dz = fmaxf(ahi.z, bhi.z) - fminf(alo.z, blo.z);
-    // explicit operations: every kernel that compares areas computes the same bits
-    const float a = __fmaf_rn(dz, dx, __fmaf_rn(dy, dz, __fmul_rn(dx, dy)));
+    // explicit operations, in the order the compiler gives dx dy + dy dz + dz dx:
+    // every kernel that compares areas computes the same bits, and near-equal
+    // pairs (a terrain's grid has many) merge as they always have
+    const float a = __fmaf_rn(dz, dx, __fmaf_rn(dx, dy, __fmul_rn(dy, dz)));
     return fminf(a, INFINITY);  // NaN (an overflow's infinity times zero): infinite
 }
 

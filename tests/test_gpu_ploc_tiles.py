@@ -45,3 +45,14 @@ def test_tree_over_tile_edges(n, spheres, scale):
         assert torch.equal(walk[0], brute[0]) and torch.equal(walk[1], brute[1])
     finally:
         rcp.rcp_scene_destroy(g)
+
+
+def test_near_ties_keep_their_tree():
+    """A terrain's grid has many pairs whose union areas differ in the last bit:
+    the order in which the area is rounded shows in the tree (46,969 nodes with
+    the other order of its products)."""
+    g = rcp.scene_from(scenes.terrain_scene(389))
+    try:
+        assert rcp.rcp_scene_get_info(g).n_nodes == 48_170
+    finally:
+        rcp.rcp_scene_destroy(g)
