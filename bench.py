@@ -371,6 +371,8 @@ def roofline(work, pass_ms, frames, workload, clk, sms):
     roof["launches_counted"] = n
     roof["algorithmic_ops_per_launch"] = ops
     roof["algorithmic_bytes_per_launch"] = byts
+    roof["work_note"] = ("work of all K passes, counted pass by pass; a chained launch leaves out the passes of tiles "
+                         "whose pixels repeat earlier values")
     roof["peak_source"] = f"{sms} SMs x 128 FP32 lanes x {sm_max_mhz:.0f} MHz (max SM clock)"
     roof["hbm_view"] = {"achieved_gbs": byts / launch_s / 1e9, "peak_gbs": hbm_gbs,
                         "frac": byts / launch_s / 1e9 / hbm_gbs, "peak_source": peak_src,
