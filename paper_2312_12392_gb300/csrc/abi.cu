@@ -107,6 +107,7 @@ rcp_status cuda_fail(cudaError_t e, const char* what) {
 }
 
 RenderCtx::~RenderCtx() {
+    if (done) cudaEventSynchronize(done);  // before anything its work still uses goes
     if (graph) cudaGraphExecDestroy(graph);
     if (img[0]) cudaFree(img[0]);
     if (rays) cudaFree(rays);
@@ -117,10 +118,7 @@ RenderCtx::~RenderCtx() {
     if (io_prim) cudaFree(io_prim);
     if (base_img) cudaFree(base_img);
     if (repeat) cudaFree(repeat);
-    if (done) {
-        cudaEventSynchronize(done);
-        cudaEventDestroy(done);
-    }
+    if (done) cudaEventDestroy(done);
     if (staged) cudaEventDestroy(staged);
     for (auto e : pass_ev)
         if (e) cudaEventDestroy(e);
@@ -413,6 +411,36 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
     return RCP_OK;
 }
 
+// One call's work on a context. Its buffers (descriptors, counters, images,
+// hints) serve one frame at a time, and calls on several streams may share a
+// context, which is keyed by shape alone: before its first work the call's
+// stream waits for the context's latest work, unless that is on the same
+// stream. Streams are told apart by their ids, which, unlike handles, are never
+// used again. Whatever the call enqueued, also one that failed part-way, is the
+// context's latest work from then on.
+class CtxUse {
+  public:
+    CtxUse(RenderCtx& ctx, cudaStream_t st) : ctx_(ctx), st_(st) {}
+    CtxUse(const CtxUse&) = delete;
+    CtxUse& operator=(const CtxUse&) = delete;
+    ~CtxUse() {
+        if (begun_) cudaEventRecord(ctx_.done, st_);
+    }
+    rcp_status begin() {
+        unsigned long long id = 0;
+        RCP_CUDA(cudaStreamGetId(st_, &id));
+        if (id != ctx_.stream_id) RCP_CUDA(cudaStreamWaitEvent(st_, ctx_.done, 0));
+        ctx_.stream_id = id;
+        begun_ = true;
+        return RCP_OK;
+    }
+
+  private:
+    RenderCtx& ctx_;
+    cudaStream_t st_;
+    bool begun_ = false;
+};
+
 // Enqueue the K passes of ctx (views already staged in ctx->d_views).
 rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, unsigned long long* counters,
                           cudaStream_t st, bool capturing) {
@@ -468,22 +496,14 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
 // few launches of a frame that may be the only one of its shape. On a stream
 // that is itself being captured the graph is used from the start.
 rcp_status run_frame(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cudaStream_t st) {
-    if (ctx.direct) {
-        rcp_status r = enqueue_passes(sc, ctx, cfg, nullptr, st, false);
-        if (r != RCP_OK) return r;
-        RCP_CUDA(cudaEventRecord(ctx.done, st));
-        return RCP_OK;
-    }
+    if (ctx.direct) return enqueue_passes(sc, ctx, cfg, nullptr, st, false);
     const std::string key = cfg_key(cfg) + (ctx.image_mode ? "/image" : "/trace") + (ctx.chained ? "/chain" : "");
     if (!ctx.graph || ctx.graph_key != key) {
         cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
         if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
         if (capture == cudaStreamCaptureStatusNone && ctx.seen_key != key) {
             ctx.seen_key = key;
-            rcp_status r = enqueue_passes(sc, ctx, cfg, nullptr, st, false);
-            if (r != RCP_OK) return r;
-            RCP_CUDA(cudaEventRecord(ctx.done, st));
-            return RCP_OK;
+            return enqueue_passes(sc, ctx, cfg, nullptr, st, false);
         }
         if (ctx.graph) {
             cudaGraphExecDestroy(ctx.graph);
@@ -505,7 +525,6 @@ rcp_status run_frame(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cuda
         ctx.graph_key = key;
     }
     RCP_CUDA(cudaGraphLaunch(ctx.graph, st));
-    RCP_CUDA(cudaEventRecord(ctx.done, st));
     return RCP_OK;
 }
 
@@ -701,6 +720,9 @@ rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const in
     if (r != RCP_OK) return r;
     LaunchCfg cfg = cfg_override ? *cfg_override : cfg_of(sc);
     cfg.ms = p->spp > 0;
+    CtxUse use(*ctx, st);
+    r = use.begin();
+    if (r != RCP_OK) return r;
     r = stage_views(*ctx, base, ins, outs, prims, rgbs, st, cfg.chain, true);
     if (r != RCP_OK) return r;
     if (ctx->chained) cfg.fused = true;  // a chained launch makes its rays itself
@@ -1080,6 +1102,9 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
         if (r != RCP_OK) return r;
     }
     float4* outs[1] = {d_out ? (float4*)d_out : ctx->img[0]};
+    CtxUse use(*ctx, st);
+    r = use.begin();
+    if (r != RCP_OK) return r;
     r = stage_views(*ctx, base, ins, outs, nullptr, nullptr, st);
     if (r != RCP_OK) return r;
     DevBuf<unsigned long long> d_cnt;

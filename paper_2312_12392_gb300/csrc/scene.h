@@ -48,7 +48,8 @@ struct RenderCtx {
     int launches = 0;              // launches of the latest render: K, or 1 (image mode: 2) when chained
     cudaGraphExec_t graph = nullptr;
     std::string graph_key, seen_key;  // the captured configuration; the one last enqueued directly
-    cudaEvent_t done = nullptr;  // recorded after the context's latest launch
+    cudaEvent_t done = nullptr;  // recorded after the context's latest work
+    unsigned long long stream_id = ~0ull;  // of the stream that work is on (claim_ctx)
     uint64_t last_use = 0;
     int64_t bytes = 0;
     ~RenderCtx();

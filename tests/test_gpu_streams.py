@@ -1,0 +1,119 @@
+"""Renders of one shape on several streams and threads, which share the scene's
+buffers for that shape: every frame equals the one rendered alone, bit for bit."""
+import threading
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from paper_2312_12392_gb300 import rcp, scenes  # noqa: E402
+import gpu_util as U  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+JIT = np.array([[0.2, 0.6], [0.7, 0.1]], np.float32)
+W, H, N = 1280, 720, 8
+
+# mapping, K, samples, chained passes, views: one launch; two; one per pass (its
+# first run, then its graph); the same with repeats; many descriptors
+KINDS = {"chain": (rcp.RCP_MAP_EYE, 6, None, 1, 1), "image": (rcp.RCP_MAP_IMAGE, 4, None, 1, 1),
+         "passes": (rcp.RCP_MAP_TARGET, 3, None, 0, 1), "samples": (rcp.RCP_MAP_EYE, 4, JIT, 1, 1),
+         "batch": (rcp.RCP_MAP_NORMAL, 3, None, 1, 6)}
+
+
+@pytest.fixture(scope="module")
+def scene():
+    sc = scenes.terrain_scene(48, n_boxes=20)
+    g = U.gpu_scene(sc)
+    yield sc, g
+    rcp.rcp_scene_destroy(g)
+
+
+class Job:
+    def __init__(self, sc, g, kind):
+        mapping, self.K, jit, chain, self.views = KINDS[kind]
+        self.g, self.sc = g, sc
+        d = sc.diameter()
+        self.p = rcp.make_params(mapping, 8.0 if mapping == rcp.RCP_MAP_IMAGE else 0.02 * d, 0.1 * d, jitter=jit)
+        rcp.rcp_set_tuning(g, rcp.rcp_tuning(block=128, chunk=32, fused_camera=1, stack_entries=0, hints=3,
+                                             chain_passes=chain))
+
+    def cams(self, i):
+        return [rcp.camera_from(self.sc.poses[(5 * i + v) % len(self.sc.poses)]) for v in range(self.views)]
+
+    def outs(self):
+        return [torch.full((H, W, 4), -1.0, device="cuda") for _ in range(self.views)]
+
+    def render(self, i, outs, stream):
+        if self.views == 1:
+            rcp.rcp_render_device(self.g, self.cams(i)[0], W, H, self.K, self.p, None, outs[0], None, stream)
+        else:
+            rcp.rcp_render_batch_device(self.g, self.cams(i), [W] * self.views, [H] * self.views, self.K, self.p, outs,
+                                        stream)
+
+    def alone(self):
+        res = []
+        for i in range(N):
+            outs = self.outs()
+            self.render(i, outs, torch.cuda.current_stream())
+            torch.cuda.synchronize()
+            res.append(outs)
+        return res
+
+
+def _same(a, b):
+    return all(torch.equal(x.view(torch.int32), y.view(torch.int32)) for x, y in zip(a, b))
+
+
+@pytest.mark.parametrize("kind", KINDS)
+def test_streams_take_turns(scene, kind):
+    job = Job(*scene, kind)
+    got = [job.outs() for _ in range(N)]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for i in range(N):
+        job.render(i, got[i], streams[i % 2])
+    torch.cuda.synchronize()
+    ref = job.alone()
+    assert [_same(a, b) for a, b in zip(got, ref)] == [True] * N
+
+
+def test_host_render_behind_a_device_render(scene):
+    job = Job(*scene, "chain")
+    ref = job.alone()
+    out = job.outs()
+    torch.cuda.synchronize()
+    st = torch.cuda.Stream()
+    for i in range(0, N, 2):  # the second runs on the library's own stream
+        job.render(i, out, st)
+        host = rcp.rcp_render(job.g, job.cams(i + 1)[0], W, H, job.K, job.p)
+        st.synchronize()
+        assert _same(out, ref[i])
+        assert np.array_equal(host, ref[i + 1][0].cpu().numpy()[..., :3])
+
+
+@pytest.mark.parametrize("kind", ["chain", "passes"])
+def test_threads_share_a_shape(scene, kind):
+    job = Job(*scene, kind)
+    got = [job.outs() for _ in range(N)]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(t):
+        try:
+            st = torch.cuda.Stream()
+            for i in range(t, N, 2):
+                job.render(i, got[i], st)
+        except Exception as e:  # noqa: BLE001
+            failed.append(e)
+
+    threads = [threading.Thread(target=work, args=(t,)) for t in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not failed
+    ref = job.alone()
+    assert [_same(a, b) for a, b in zip(got, ref)] == [True] * N
