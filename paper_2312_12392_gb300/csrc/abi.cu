@@ -365,7 +365,10 @@ void layout_views(std::vector<ViewDev>& v, int64_t& total_pix, int64_t& total_ch
 constexpr size_t CTX_MAX = 64;
 constexpr int64_t CTX_BYTES = (int64_t)16 << 30;
 
-rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t total_chunks, RenderCtx** out) {
+// A new context's counters and hints are cleared on `st`, the stream of the
+// frame that it is made for.
+rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t total_chunks, cudaStream_t st,
+                   RenderCtx** out) {
     std::ostringstream key;
     key << n_views << ":" << K << ":" << total_pix << ":" << total_chunks;
     auto it = sc.ctx.find(key.str());
@@ -400,12 +403,14 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
     c->d_status = (int*)(c->block + head) - 4;
     c->d_views = (ViewDev*)(c->block + head);
     c->hints = (int2*)(c->block + head + views);
-    RCP_CUDA(cudaMemset(c->block, 0, head));
-    RCP_CUDA(cudaMemset(c->hints, 0xff, sizeof(int2) * total_pix));  // -1: no earlier hit
     c->views.resize((size_t)K * n_views);
     RCP_CUDA(cudaEventCreateWithFlags(&c->staged, cudaEventDisableTiming));
     RCP_CUDA(cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming));
     for (int n = 0; n <= K; ++n) RCP_CUDA(cudaEventCreate(&c->pass_ev[n]));
+    RCP_CUDA(cudaStreamGetId(st, &c->stream_id));
+    RCP_CUDA(cudaMemsetAsync(c->block, 0, head, st));
+    RCP_CUDA(cudaMemsetAsync(c->hints, 0xff, sizeof(int2) * total_pix, st));  // -1: no earlier hit
+    RCP_CUDA(cudaEventRecord(c->done, st));
     *out = c.get();
     sc.ctx[key.str()] = std::move(c);
     return RCP_OK;
@@ -716,7 +721,7 @@ rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const in
     int64_t total_pix, total_chunks;
     layout_views(base, total_pix, total_chunks);
     RenderCtx* ctx = nullptr;
-    rcp_status r = get_ctx(sc, n_views, K, total_pix, total_chunks, &ctx);
+    rcp_status r = get_ctx(sc, n_views, K, total_pix, total_chunks, st, &ctx);
     if (r != RCP_OK) return r;
     LaunchCfg cfg = cfg_override ? *cfg_override : cfg_of(sc);
     cfg.ms = p->spp > 0;
@@ -962,7 +967,7 @@ rcp_status rcp_render(const rcp_scene* csc, const rcp_camera* cam, int W, int H,
     cudaStream_t st = lib_stream();
     const int64_t P = (int64_t)W * H;
     RenderCtx* ctx = nullptr;
-    r = get_ctx(*sc, 1, K, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), &ctx);
+    r = get_ctx(*sc, 1, K, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
     if (r != RCP_OK) return r;
     const bool direct = p->mapping != RCP_MAP_IMAGE && use_direct_output(out_rgb, sizeof(float) * 3 * P);
     r = ensure_io(*ctx, !direct, false);
@@ -1009,7 +1014,7 @@ rcp_status rcp_render_pass(const rcp_scene* csc, const rcp_camera* cam, int W, i
     cudaStream_t st = lib_stream();
     const int64_t P = (int64_t)W * H;
     RenderCtx* ctx = nullptr;
-    r = get_ctx(*sc, 1, 1, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), &ctx);
+    r = get_ctx(*sc, 1, 1, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
     if (r != RCP_OK) return r;
     r = ensure_io(*ctx, false, out_prim != nullptr);
     if (r != RCP_OK) return r;
@@ -1090,7 +1095,7 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     cudaStream_t st = lib_stream();
     const int64_t P = (int64_t)W * H;
     RenderCtx* ctx = nullptr;
-    r = get_ctx(*sc, 1, 1, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), &ctx);
+    r = get_ctx(*sc, 1, 1, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
     if (r != RCP_OK) return r;
     std::vector<ViewDev> base(1);
     make_view(base[0], *cam, W, H, *p);

@@ -117,3 +117,26 @@ def test_threads_share_a_shape(scene, kind):
     assert not failed
     ref = job.alone()
     assert [_same(a, b) for a, b in zip(got, ref)] == [True] * N
+
+
+@pytest.mark.parametrize("kind", ["chain", "samples"])
+def test_first_render_of_a_shape_does_not_wait_for_the_legacy_stream(scene, kind):
+    """The buffers made for a shape are cleared on the frame's own stream: a clear
+    behind the legacy stream's work would land in or after the frame."""
+    job = Job(*scene, kind)
+    w, h = (611, 333) if kind == "chain" else (613, 335)  # shapes that nothing else here renders
+    st = torch.cuda.Stream()
+    img = torch.rand((h, w, 4), generator=torch.Generator().manual_seed(3)).cuda()
+    first = img.clone()
+    torch.cuda.synchronize()
+    torch.cuda._sleep(100_000_000)  # about 50 ms of the legacy stream
+    rcp.rcp_render_device(job.g, job.cams(0)[0], w, h, job.K, job.p, img, img, None, st)
+    st.synchronize()
+    rays = rcp.rcp_last_ray_counts(job.g)  # read behind the legacy stream's work
+    torch.cuda.synchronize()
+    assert rays[0] == w * h * job.K * max(job.p.spp, 1)
+    out = torch.empty_like(first)
+    rcp.rcp_render_device(job.g, job.cams(0)[0], w, h, job.K, job.p, first, out, None, st)
+    torch.cuda.synchronize()
+    assert rcp.rcp_last_ray_counts(job.g) == rays
+    assert torch.equal(img.view(torch.int32), out.view(torch.int32))
