@@ -847,7 +847,9 @@ rcp_status rcp_scene_create_ex(const float* tri, int64_t T, const float* sph, in
     r = validate_bvh(*sc, st);
     if (r != RCP_OK) return r;
     const SceneDev dv = sc->dev();
-    RCP_CUDA(cudaMemcpy(sc->d_dev, &dv, sizeof(SceneDev), cudaMemcpyHostToDevice));
+    // complete before any stream can read it
+    RCP_CUDA(cudaMemcpyAsync(sc->d_dev, &dv, sizeof(SceneDev), cudaMemcpyHostToDevice, st));
+    RCP_CUDA(cudaStreamSynchronize(st));
     *out = sc.release();
     return RCP_OK;
 }

@@ -477,7 +477,7 @@ rcp_status rcp_server_create(int64_t budget, int max_slots, rcp_server** out) {
     RCP_CUDA(cudaStreamCreateWithFlags(&s->st_main, cudaStreamNonBlocking));
     RCP_CUDA(cudaStreamCreateWithFlags(&s->st_copy, cudaStreamNonBlocking));
     RCP_CUDA(cudaMalloc((void**)&s->d_rays, sizeof(unsigned long long) * 2));
-    RCP_CUDA(cudaMemset(s->d_rays, 0, sizeof(unsigned long long) * 2));
+    RCP_CUDA(cudaMemsetAsync(s->d_rays, 0, sizeof(unsigned long long) * 2, s->st_main));  // the steps' stream
     // admitted, unfinished requests: at most max_slots in flight and as many
     // again waiting for copy-out (admission waits for a free word)
     const int n_status = 2 * max_slots + 16;

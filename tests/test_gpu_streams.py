@@ -1,6 +1,7 @@
 """Renders of one shape on several streams and threads, which share the scene's
 buffers for that shape: every frame equals the one rendered alone, bit for bit."""
 import threading
+import time
 
 import numpy as np
 import pytest
@@ -140,3 +141,21 @@ def test_first_render_of_a_shape_does_not_wait_for_the_legacy_stream(scene, kind
     torch.cuda.synchronize()
     assert rcp.rcp_last_ray_counts(job.g) == rays
     assert torch.equal(img.view(torch.int32), out.view(torch.int32))
+
+
+def test_a_new_servers_counts_do_not_wait_for_the_legacy_stream(scene):
+    sc, g = scene
+    d = sc.diameter()
+    p = rcp.make_params(rcp.RCP_MAP_EYE, 0.02 * d, 0.1 * d)
+    torch.cuda.synchronize()
+    torch.cuda._sleep(200_000_000)
+    srv = rcp.rcp_server_create(1 << 30, 2)
+    try:
+        out = np.zeros((90, 160, 3), np.float32)
+        t = rcp.rcp_server_submit(srv, g, rcp.camera_from(sc.poses[0]), 160, 90, 4, p, out)
+        rcp.rcp_server_wait(srv, t, 60.0)
+        time.sleep(0.1)  # the step's end, where its rays are added up
+        s = rcp.rcp_server_stats_get(srv)
+        assert s.mrays_per_s / s.frames_per_s * 1e6 >= 0.999 * 160 * 90 * 4
+    finally:
+        rcp.rcp_server_destroy(srv)
