@@ -107,7 +107,7 @@ rcp_status cuda_fail(cudaError_t e, const char* what) {
 }
 
 RenderCtx::~RenderCtx() {
-    if (done) cudaEventSynchronize(done);  // before anything its work still uses goes
+    if (work.done) cudaEventSynchronize(work.done);  // before anything its work still uses goes
     if (graph) cudaGraphExecDestroy(graph);
     if (img[0]) cudaFree(img[0]);
     if (rays) cudaFree(rays);
@@ -118,7 +118,7 @@ RenderCtx::~RenderCtx() {
     if (io_prim) cudaFree(io_prim);
     if (base_img) cudaFree(base_img);
     if (repeat) cudaFree(repeat);
-    if (done) cudaEventDestroy(done);
+    if (work.done) cudaEventDestroy(work.done);
     if (staged) cudaEventDestroy(staged);
     for (auto e : pass_ev)
         if (e) cudaEventDestroy(e);
@@ -126,6 +126,7 @@ RenderCtx::~RenderCtx() {
 
 Scene::~Scene() {
     ctx.clear();
+    if (spill_work.done) cudaEventDestroy(spill_work.done);
     for (void* p : {(void*)d_store, d_nodes, (void*)d_prims, (void*)d_refbox, (void*)d_part_uv, (void*)d_rbox,
                     (void*)d_spill})
         if (p) cudaFree(p);
@@ -302,11 +303,41 @@ LaunchCfg cfg_of(const Scene& sc) {
     return c;
 }
 
+// One call's work on buffers that serve one frame at a time but that calls on
+// several streams may share: a context's (descriptors, counters, images, hints;
+// keyed by shape alone) and a scene's spill region. Before its first work the
+// call's stream waits for the buffers' latest work, unless that is on the same
+// stream. Streams are told apart by their ids, which, unlike handles, are never
+// used again. Whatever the call enqueued, also one that failed part-way, is the
+// buffers' latest work from then on.
+class StreamUse {
+  public:
+    StreamUse() = default;
+    StreamUse(const StreamUse&) = delete;
+    StreamUse& operator=(const StreamUse&) = delete;
+    ~StreamUse() {
+        if (work_) cudaEventRecord(work_->done, st_);
+    }
+    rcp_status begin(LastWork& work, cudaStream_t st) {
+        unsigned long long id = 0;
+        RCP_CUDA(cudaStreamGetId(st, &id));
+        if (id != work.stream_id) RCP_CUDA(cudaStreamWaitEvent(st, work.done, 0));
+        work.stream_id = id;
+        work_ = &work;
+        st_ = st;
+        return RCP_OK;
+    }
+
+  private:
+    LastWork* work_ = nullptr;
+    cudaStream_t st_ = nullptr;
+};
+
 // The global-memory region of a short shared stack: spill_entries per thread
 // of the largest persistent grid a launch can have (the SMs' resident
 // threads, or the tuned blocks per SM). Grown before any capture, never during
 // one; the graph key names the region.
-rcp_status ensure_spill(Scene& sc, LaunchCfg& c) {
+rcp_status ensure_spill(Scene& sc, LaunchCfg& c, cudaStream_t st, StreamUse& use) {
     if (c.spill_entries <= 0) return RCP_OK;
     const int64_t per_sm = std::max<int64_t>(2048, (int64_t)c.blocks_per_sm * c.block);
     const int64_t need = (int64_t)device_sms() * per_sm * c.spill_entries;
@@ -326,7 +357,8 @@ rcp_status ensure_spill(Scene& sc, LaunchCfg& c) {
     }
     c.spill = sc.d_spill;
     c.spill_cap = sc.spill_cap;
-    return RCP_OK;
+    if (!sc.spill_work.done) RCP_CUDA(cudaEventCreateWithFlags(&sc.spill_work.done, cudaEventDisableTiming));
+    return use.begin(sc.spill_work, st);
 }
 
 // The separate camera kernel's ray buffer (2 float4 per pixel), allocated
@@ -405,46 +437,16 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
     c->hints = (int2*)(c->block + head + views);
     c->views.resize((size_t)K * n_views);
     RCP_CUDA(cudaEventCreateWithFlags(&c->staged, cudaEventDisableTiming));
-    RCP_CUDA(cudaEventCreateWithFlags(&c->done, cudaEventDisableTiming));
+    RCP_CUDA(cudaEventCreateWithFlags(&c->work.done, cudaEventDisableTiming));
     for (int n = 0; n <= K; ++n) RCP_CUDA(cudaEventCreate(&c->pass_ev[n]));
-    RCP_CUDA(cudaStreamGetId(st, &c->stream_id));
+    RCP_CUDA(cudaStreamGetId(st, &c->work.stream_id));
     RCP_CUDA(cudaMemsetAsync(c->block, 0, head, st));
     RCP_CUDA(cudaMemsetAsync(c->hints, 0xff, sizeof(int2) * total_pix, st));  // -1: no earlier hit
-    RCP_CUDA(cudaEventRecord(c->done, st));
+    RCP_CUDA(cudaEventRecord(c->work.done, st));
     *out = c.get();
     sc.ctx[key.str()] = std::move(c);
     return RCP_OK;
 }
-
-// One call's work on a context. Its buffers (descriptors, counters, images,
-// hints) serve one frame at a time, and calls on several streams may share a
-// context, which is keyed by shape alone: before its first work the call's
-// stream waits for the context's latest work, unless that is on the same
-// stream. Streams are told apart by their ids, which, unlike handles, are never
-// used again. Whatever the call enqueued, also one that failed part-way, is the
-// context's latest work from then on.
-class CtxUse {
-  public:
-    CtxUse(RenderCtx& ctx, cudaStream_t st) : ctx_(ctx), st_(st) {}
-    CtxUse(const CtxUse&) = delete;
-    CtxUse& operator=(const CtxUse&) = delete;
-    ~CtxUse() {
-        if (begun_) cudaEventRecord(ctx_.done, st_);
-    }
-    rcp_status begin() {
-        unsigned long long id = 0;
-        RCP_CUDA(cudaStreamGetId(st_, &id));
-        if (id != ctx_.stream_id) RCP_CUDA(cudaStreamWaitEvent(st_, ctx_.done, 0));
-        ctx_.stream_id = id;
-        begun_ = true;
-        return RCP_OK;
-    }
-
-  private:
-    RenderCtx& ctx_;
-    cudaStream_t st_;
-    bool begun_ = false;
-};
 
 // Enqueue the K passes of ctx (views already staged in ctx->d_views).
 rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, unsigned long long* counters,
@@ -560,7 +562,7 @@ RepeatLayout repeat_layout(const RenderCtx& ctx, bool ids) {
 rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
     if (ctx.repeat && (ctx.repeat_ids || !ids)) return RCP_OK;
     if (ctx.repeat) {
-        RCP_CUDA(cudaEventSynchronize(ctx.done));  // no launch may still use the smaller one
+        RCP_CUDA(cudaEventSynchronize(ctx.work.done));  // no launch may still use the smaller one
         cudaFree(ctx.repeat);
         ctx.bytes -= (int64_t)repeat_layout(ctx, ctx.repeat_ids).total;
         ctx.repeat = nullptr;
@@ -725,13 +727,13 @@ rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const in
     if (r != RCP_OK) return r;
     LaunchCfg cfg = cfg_override ? *cfg_override : cfg_of(sc);
     cfg.ms = p->spp > 0;
-    CtxUse use(*ctx, st);
-    r = use.begin();
+    StreamUse use, spill_use;
+    r = use.begin(ctx->work, st);
     if (r != RCP_OK) return r;
     r = stage_views(*ctx, base, ins, outs, prims, rgbs, st, cfg.chain, true);
     if (r != RCP_OK) return r;
     if (ctx->chained) cfg.fused = true;  // a chained launch makes its rays itself
-    r = ensure_spill(sc, cfg);
+    r = ensure_spill(sc, cfg, st, spill_use);
     if (r != RCP_OK) return r;
     r = ensure_rays(*ctx, cfg);
     if (r != RCP_OK) return r;
@@ -1109,8 +1111,8 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
         if (r != RCP_OK) return r;
     }
     float4* outs[1] = {d_out ? (float4*)d_out : ctx->img[0]};
-    CtxUse use(*ctx, st);
-    r = use.begin();
+    StreamUse use, spill_use;
+    r = use.begin(ctx->work, st);
     if (r != RCP_OK) return r;
     r = stage_views(*ctx, base, ins, outs, nullptr, nullptr, st);
     if (r != RCP_OK) return r;
@@ -1120,7 +1122,7 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     LaunchCfg cfg = cfg_of(*sc);
     cfg.count = true;
     cfg.ms = p->spp > 0;
-    r = ensure_spill(*sc, cfg);
+    r = ensure_spill(*sc, cfg, st, spill_use);
     if (r != RCP_OK) return r;
     r = ensure_rays(*ctx, cfg);
     if (r != RCP_OK) return r;

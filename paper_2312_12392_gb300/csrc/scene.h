@@ -14,6 +14,13 @@
 
 namespace rcp {
 
+// The latest work on buffers that calls on several streams share: its event and
+// the id of its stream.
+struct LastWork {
+    cudaEvent_t done = nullptr;
+    unsigned long long stream_id = ~0ull;
+};
+
 // Cached resources of one launch shape: ping-pong images, ray buffer, view
 // descriptors (device + pinned staging), work counters and the CUDA graph of
 // the K-pass sequence.
@@ -48,8 +55,7 @@ struct RenderCtx {
     int launches = 0;              // launches of the latest render: K, or 1 (image mode: 2) when chained
     cudaGraphExec_t graph = nullptr;
     std::string graph_key, seen_key;  // the captured configuration; the one last enqueued directly
-    cudaEvent_t done = nullptr;  // recorded after the context's latest work
-    unsigned long long stream_id = ~0ull;  // of the stream that work is on (claim_ctx)
+    LastWork work;
     uint64_t last_use = 0;
     int64_t bytes = 0;
     ~RenderCtx();
@@ -87,6 +93,7 @@ struct Scene {
     SceneDev* d_dev = nullptr;  // device copy of dev(), named by views of multi-scene launches
     uint2* d_spill = nullptr;   // global-memory traversal stack entries of a short shared stack
     int64_t spill_cap = 0;
+    LastWork spill_work;  // of the launches that use it, whatever their shape
     ~Scene();
     SceneDev dev() const;
     int64_t device_bytes() const;

@@ -159,3 +159,26 @@ def test_a_new_servers_counts_do_not_wait_for_the_legacy_stream(scene):
         assert s.mrays_per_s / s.frames_per_s * 1e6 >= 0.999 * 160 * 90 * 4
     finally:
         rcp.rcp_server_destroy(srv)
+
+
+@pytest.mark.parametrize("chain", [0, 1])
+def test_shapes_on_two_streams_share_the_stack_region(scene, chain):
+    """A shared stack of one entry spills to a region of the scene that launches of
+    every shape use."""
+    job = Job(*scene, "chain")
+    rcp.rcp_set_tuning(job.g, rcp.rcp_tuning(block=128, chunk=32, fused_camera=1, stack_entries=1, hints=3,
+                                             chain_passes=chain))
+    sizes = [(W, H), (W - 8, H)]
+    outs = [torch.empty((h, w, 4), device="cuda") for w, h in sizes for _ in range(4)]
+    refs = [torch.empty_like(o) for o in outs]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    for alone, res in ((False, outs), (True, refs)):
+        for i in range(4):
+            for v, (w, h) in enumerate(sizes):
+                rcp.rcp_render_device(job.g, job.cams(i + v)[0], w, h, job.K, job.p, None, res[4 * v + i], None,
+                                      streams[v])
+                if alone:
+                    torch.cuda.synchronize()
+        torch.cuda.synchronize()
+    assert [_same([a], [b]) for a, b in zip(outs, refs)] == [True] * 8
