@@ -22,8 +22,11 @@
  *  - Valid arguments: 1 <= width, height <= 8192; 1 <= K <= 16; k >= 0;
  *    focal_dist > 0; finite coordinates. Degenerate (zero-area) triangles are
  *    accepted and never hit.
- *  - A scene may be rendered from several threads at once; rcp_scene_update_*
- *    must not run concurrently with renders of the same scene.
+ *  - A scene may be rendered from several threads and on several streams at
+ *    once (renders of one shape run one after the other on the device);
+ *    rcp_scene_update_* must not run concurrently with renders of the same
+ *    scene. A render on a stream that is being captured is refused
+ *    (RCP_ERR_CUDA), and the capture goes on.
  */
 #ifndef RCP_H
 #define RCP_H

@@ -500,15 +500,12 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
 // chain of twelve rays). Others run through the context's CUDA graph, captured when a launch
 // configuration comes a second time: the first time its launches are enqueued
 // directly, since capturing and instantiating a graph takes longer than the
-// few launches of a frame that may be the only one of its shape. On a stream
-// that is itself being captured the graph is used from the start.
+// few launches of a frame that may be the only one of its shape.
 rcp_status run_frame(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cudaStream_t st) {
     if (ctx.direct) return enqueue_passes(sc, ctx, cfg, nullptr, st, false);
     const std::string key = cfg_key(cfg) + (ctx.image_mode ? "/image" : "/trace") + (ctx.chained ? "/chain" : "");
     if (!ctx.graph || ctx.graph_key != key) {
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
-        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
-        if (capture == cudaStreamCaptureStatusNone && ctx.seen_key != key) {
+        if (ctx.seen_key != key) {
             ctx.seen_key = key;
             return enqueue_passes(sc, ctx, cfg, nullptr, st, false);
         }
@@ -602,11 +599,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
     ctx.chained = chain && base[0].spp == 0 && K > 1;
     ctx.launches = ctx.chained ? (ctx.image_mode ? 2 : 1) : K;
     ctx.n_desc = ctx.chained ? nv * (ctx.image_mode ? 2 : 1) : nv * K;
-    // a stream that is being captured takes the copy and the graph
-    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusActive;
-    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
-    ctx.direct = allow_direct && (ctx.chained || K == 1) && ctx.n_desc <= STAGE_VIEWS &&
-                 capture == cudaStreamCaptureStatusNone;
+    ctx.direct = allow_direct && (ctx.chained || K == 1) && ctx.n_desc <= STAGE_VIEWS;
     if (ctx.image_mode && !ctx.base_img) RCP_CUDA(cudaMalloc((void**)&ctx.base_img, sizeof(float4) * ctx.total_pix));
     if (ctx.chained) {
         for (int i = 0; i < nv; ++i) {
@@ -719,6 +712,15 @@ rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const in
     if (sc.depth > MAX_STACK) {
         set_error("BVH deeper than the traversal stack");
         return RCP_ERR_STACK;
+    }
+    // A render orders itself against other streams and stages its descriptors on
+    // the host, once per call, so it cannot become part of the caller's graph.
+    // Refused before anything that would invalidate the caller's capture.
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    RCP_CUDA(cudaStreamIsCapturing(st, &capture));
+    if (capture != cudaStreamCaptureStatusNone) {
+        set_error("renders cannot be captured: the stream is being captured");
+        return RCP_ERR_CUDA;
     }
     int64_t total_pix, total_chunks;
     layout_views(base, total_pix, total_chunks);
