@@ -361,13 +361,45 @@ rcp_status ensure_spill(Scene& sc, LaunchCfg& c, cudaStream_t st, StreamUse& use
     return use.begin(sc.spill_work, st);
 }
 
+// Render contexts are cached per launch shape, least recently used first out
+// when the cache exceeds CTX_MAX entries or CTX_BYTES of device memory. A
+// context is freed only after its last launch has completed.
+constexpr size_t CTX_MAX = 64;
+constexpr int64_t CTX_BYTES = (int64_t)16 << 30;
+
+// Drop contexts other than `keep` until `more` bytes fit, and for a new context
+// (keep null) a further entry.
+void make_room(Scene& sc, const RenderCtx* keep, int64_t more) {
+    for (;;) {
+        int64_t held = 0;
+        auto victim = sc.ctx.end();
+        for (auto it = sc.ctx.begin(); it != sc.ctx.end(); ++it) {
+            held += it->second->bytes;
+            if (it->second.get() != keep &&
+                (victim == sc.ctx.end() || it->second->last_use < victim->second->last_use))
+                victim = it;
+        }
+        if (victim == sc.ctx.end() || (sc.ctx.size() < CTX_MAX + (keep ? 1 : 0) && held + more <= CTX_BYTES)) return;
+        if (sc.last == victim->second.get()) sc.last = nullptr;
+        sc.ctx.erase(victim);  // the destructor waits for the context's last launch
+    }
+}
+
+// n elements more for a context, counted against the cache's limit.
+template <class T>
+rcp_status ctx_alloc(Scene& sc, RenderCtx& ctx, T** p, int64_t n) {
+    const int64_t bytes = (int64_t)sizeof(T) * n;
+    make_room(sc, &ctx, bytes);
+    RCP_CUDA(cudaMalloc((void**)p, bytes));
+    ctx.bytes += bytes;
+    return RCP_OK;
+}
+
 // The separate camera kernel's ray buffer (2 float4 per pixel), allocated
 // before the first capture that needs it.
-rcp_status ensure_rays(RenderCtx& ctx, const LaunchCfg& c) {
+rcp_status ensure_rays(Scene& sc, RenderCtx& ctx, const LaunchCfg& c) {
     if (c.fused || c.ms || c.multi || ctx.rays) return RCP_OK;
-    RCP_CUDA(cudaMalloc((void**)&ctx.rays, sizeof(float4) * 2 * ctx.total_pix));
-    ctx.bytes += (int64_t)sizeof(float4) * 2 * ctx.total_pix;
-    return RCP_OK;
+    return ctx_alloc(sc, ctx, &ctx.rays, 2 * ctx.total_pix);
 }
 
 std::string cfg_key(const LaunchCfg& c) {
@@ -391,12 +423,6 @@ void layout_views(std::vector<ViewDev>& v, int64_t& total_pix, int64_t& total_ch
     }
 }
 
-// Render contexts are cached per launch shape, least recently used first out
-// when the cache exceeds CTX_MAX entries or CTX_BYTES of device memory. A
-// context is freed only after its last launch has completed.
-constexpr size_t CTX_MAX = 64;
-constexpr int64_t CTX_BYTES = (int64_t)16 << 30;
-
 // A new context's counters and hints are cleared on `st`, the stream of the
 // frame that it is made for.
 rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t total_chunks, cudaStream_t st,
@@ -410,16 +436,7 @@ rcp_status get_ctx(Scene& sc, int n_views, int K, int64_t total_pix, int64_t tot
         return RCP_OK;
     }
     const int64_t need = total_pix * (int64_t)sizeof(int2) + (int64_t)sizeof(ViewDev) * K * n_views;
-    for (;;) {
-        int64_t held = 0;
-        for (auto& kv : sc.ctx) held += kv.second->bytes;
-        if (sc.ctx.empty() || (sc.ctx.size() < CTX_MAX && held + need <= CTX_BYTES)) break;
-        auto victim = sc.ctx.begin();
-        for (auto jt = sc.ctx.begin(); jt != sc.ctx.end(); ++jt)
-            if (jt->second->last_use < victim->second->last_use) victim = jt;
-        if (sc.last == victim->second.get()) sc.last = nullptr;
-        sc.ctx.erase(victim);  // the destructor waits for the context's last launch
-    }
+    make_room(sc, nullptr, need);
     auto c = std::make_unique<RenderCtx>();
     c->n_views = n_views;
     c->K = K;
@@ -534,12 +551,11 @@ rcp_status run_frame(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg, cuda
 
 // The context's ping-pong images: renders of several launches, and inputs and
 // outputs that the caller leaves to the library. A chained render has none.
-rcp_status ensure_img(RenderCtx& ctx) {
+rcp_status ensure_img(Scene& sc, RenderCtx& ctx) {
     if (ctx.img[0]) return RCP_OK;
-    RCP_CUDA(cudaMalloc((void**)&ctx.img[0], sizeof(float4) * 2 * ctx.total_pix));
-    ctx.img[1] = ctx.img[0] + ctx.total_pix;
-    ctx.bytes += (int64_t)sizeof(float4) * 2 * ctx.total_pix;
-    return RCP_OK;
+    rcp_status r = ctx_alloc(sc, ctx, &ctx.img[0], 2 * ctx.total_pix);
+    if (r == RCP_OK) ctx.img[1] = ctx.img[0] + ctx.total_pix;
+    return r;
 }
 
 // The state of a multi-sample render that leaves out repeated tiles: two
@@ -556,7 +572,7 @@ RepeatLayout repeat_layout(const RenderCtx& ctx, bool ids) {
     return l;
 }
 
-rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
+rcp_status ensure_repeat(Scene& sc, RenderCtx& ctx, bool ids) {
     if (ctx.repeat && (ctx.repeat_ids || !ids)) return RCP_OK;
     if (ctx.repeat) {
         RCP_CUDA(cudaEventSynchronize(ctx.work.done));  // no launch may still use the smaller one
@@ -564,11 +580,8 @@ rcp_status ensure_repeat(RenderCtx& ctx, bool ids) {
         ctx.bytes -= (int64_t)repeat_layout(ctx, ctx.repeat_ids).total;
         ctx.repeat = nullptr;
     }
-    const RepeatLayout l = repeat_layout(ctx, ids);
-    RCP_CUDA(cudaMalloc((void**)&ctx.repeat, l.total));
     ctx.repeat_ids = ids;
-    ctx.bytes += (int64_t)l.total;
-    return RCP_OK;
+    return ctx_alloc(sc, ctx, &ctx.repeat, (int64_t)repeat_layout(ctx, ids).total);
 }
 
 // The staged descriptors to the device (a direct frame's go with its launch).
@@ -588,7 +601,7 @@ rcp_status upload_views(RenderCtx& ctx, cudaStream_t st) {
 // it and the render allows it), one per view that runs all K passes (an
 // image-space render: one per view that traces pass 1, then one per view that
 // gathers passes 2..K).
-rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const float4* const* ins,
+rcp_status stage_views(Scene& sc, RenderCtx& ctx, const std::vector<ViewDev>& base, const float4* const* ins,
                        float4* const* outs, int32_t* const* prims, float* const* rgbs, cudaStream_t st,
                        bool chain = false, bool allow_direct = false) {
     const int K = ctx.K, nv = ctx.n_views;
@@ -600,7 +613,10 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
     ctx.launches = ctx.chained ? (ctx.image_mode ? 2 : 1) : K;
     ctx.n_desc = ctx.chained ? nv * (ctx.image_mode ? 2 : 1) : nv * K;
     ctx.direct = allow_direct && (ctx.chained || K == 1) && ctx.n_desc <= STAGE_VIEWS;
-    if (ctx.image_mode && !ctx.base_img) RCP_CUDA(cudaMalloc((void**)&ctx.base_img, sizeof(float4) * ctx.total_pix));
+    if (ctx.image_mode && !ctx.base_img) {
+        rcp_status r = ctx_alloc(sc, ctx, &ctx.base_img, ctx.total_pix);
+        if (r != RCP_OK) return r;
+    }
     if (ctx.chained) {
         for (int i = 0; i < nv; ++i) {
             ViewDev v = base[i];
@@ -626,7 +642,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
         return upload_views(ctx, st);
     }
     if (K > 1) {
-        rcp_status r = ensure_img(ctx);
+        rcp_status r = ensure_img(sc, ctx);
         if (r != RCP_OK) return r;
     }
     bool want_ids = false;
@@ -634,7 +650,7 @@ rcp_status stage_views(RenderCtx& ctx, const std::vector<ViewDev>& base, const f
     const bool repeats = base[0].spp > 0 && K > 2;
     RepeatLayout lay{};
     if (repeats) {
-        rcp_status r = ensure_repeat(ctx, want_ids);
+        rcp_status r = ensure_repeat(sc, ctx, want_ids);
         if (r != RCP_OK) return r;
         lay = repeat_layout(ctx, ctx.repeat_ids);
     }
@@ -732,12 +748,12 @@ rcp_status render_views(Scene& sc, int n_views, const rcp_camera* cams, const in
     StreamUse use, spill_use;
     r = use.begin(ctx->work, st);
     if (r != RCP_OK) return r;
-    r = stage_views(*ctx, base, ins, outs, prims, rgbs, st, cfg.chain, true);
+    r = stage_views(sc, *ctx, base, ins, outs, prims, rgbs, st, cfg.chain, true);
     if (r != RCP_OK) return r;
     if (ctx->chained) cfg.fused = true;  // a chained launch makes its rays itself
     r = ensure_spill(sc, cfg, st, spill_use);
     if (r != RCP_OK) return r;
-    r = ensure_rays(*ctx, cfg);
+    r = ensure_rays(sc, *ctx, cfg);
     if (r != RCP_OK) return r;
     r = run_frame(sc, *ctx, cfg, st);
     sc.last = ctx;
@@ -948,12 +964,13 @@ rcp_status rcp_render_batch_device(const rcp_scene* csc, int n_views, const rcp_
                         d_prims, (cudaStream_t)stream);
 }
 
-static rcp_status ensure_io(RenderCtx& ctx, bool rgb, bool prim) {
+static rcp_status ensure_io(Scene& sc, RenderCtx& ctx, bool rgb, bool prim) {
     const int64_t P = ctx.total_pix;
-    if (!ctx.io) RCP_CUDA(cudaMalloc((void**)&ctx.io, sizeof(float4) * P));
-    if (rgb && !ctx.d_rgb) RCP_CUDA(cudaMalloc((void**)&ctx.d_rgb, sizeof(float) * 3 * P));
-    if (prim && !ctx.io_prim) RCP_CUDA(cudaMalloc((void**)&ctx.io_prim, sizeof(int32_t) * P));
-    return RCP_OK;
+    rcp_status r = RCP_OK;
+    if (!ctx.io) r = ctx_alloc(sc, ctx, &ctx.io, P);
+    if (r == RCP_OK && rgb && !ctx.d_rgb) r = ctx_alloc(sc, ctx, &ctx.d_rgb, 3 * P);
+    if (r == RCP_OK && prim && !ctx.io_prim) r = ctx_alloc(sc, ctx, &ctx.io_prim, P);
+    return r;
 }
 
 rcp_status rcp_render(const rcp_scene* csc, const rcp_camera* cam, int W, int H, int K, const rcp_params* p,
@@ -976,7 +993,7 @@ rcp_status rcp_render(const rcp_scene* csc, const rcp_camera* cam, int W, int H,
     r = get_ctx(*sc, 1, K, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
     if (r != RCP_OK) return r;
     const bool direct = p->mapping != RCP_MAP_IMAGE && use_direct_output(out_rgb, sizeof(float) * 3 * P);
-    r = ensure_io(*ctx, !direct, false);
+    r = ensure_io(*sc, *ctx, !direct, false);
     if (r != RCP_OK) return r;
     const float4* ins[1] = {nullptr};
     float4* outs[1] = {ctx->io};
@@ -1022,12 +1039,12 @@ rcp_status rcp_render_pass(const rcp_scene* csc, const rcp_camera* cam, int W, i
     RenderCtx* ctx = nullptr;
     r = get_ctx(*sc, 1, 1, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
     if (r != RCP_OK) return r;
-    r = ensure_io(*ctx, false, out_prim != nullptr);
+    r = ensure_io(*sc, *ctx, false, out_prim != nullptr);
     if (r != RCP_OK) return r;
     // I_{n-1} goes to ctx->img[1] (unused by a one-pass render) and I_n to
     // ctx->io: separate buffers, since jittered samples read neighbouring pixels
     if (in_rgbz) {
-        r = ensure_img(*ctx);
+        r = ensure_img(*sc, *ctx);
         if (r != RCP_OK) return r;
     }
     if (in_rgbz) RCP_CUDA(cudaMemcpyAsync(ctx->img[1], in_rgbz, sizeof(float4) * P, cudaMemcpyHostToDevice, st));
@@ -1109,14 +1126,14 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     layout_views(base, tp, tc);
     const float4* ins[1] = {(const float4*)d_in};
     if (!d_out) {
-        r = ensure_img(*ctx);
+        r = ensure_img(*sc, *ctx);
         if (r != RCP_OK) return r;
     }
     float4* outs[1] = {d_out ? (float4*)d_out : ctx->img[0]};
     StreamUse use, spill_use;
     r = use.begin(ctx->work, st);
     if (r != RCP_OK) return r;
-    r = stage_views(*ctx, base, ins, outs, nullptr, nullptr, st);
+    r = stage_views(*sc, *ctx, base, ins, outs, nullptr, nullptr, st);
     if (r != RCP_OK) return r;
     DevBuf<unsigned long long> d_cnt;
     RCP_CUDA(d_cnt.alloc(8));
@@ -1126,7 +1143,7 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     cfg.ms = p->spp > 0;
     r = ensure_spill(*sc, cfg, st, spill_use);
     if (r != RCP_OK) return r;
-    r = ensure_rays(*ctx, cfg);
+    r = ensure_rays(*sc, *ctx, cfg);
     if (r != RCP_OK) return r;
     r = enqueue_passes(*sc, *ctx, cfg, d_cnt.p, st, false);
     if (r != RCP_OK) return r;
