@@ -703,8 +703,8 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
         // of 20 frames below the line (terrain and forest, 1 to 6 passes, 1 to 4
         // samples) it was 2 to 8 % faster on 17 and 1 to 3 % slower on 3 (5,600
         // to 7,900 tiles); above it 24 warps win by 3 to 9 % from 14,000 tiles on.
-        const int64_t tiles = total_chunks * (cfg.chunk / 32);
-        return tiles <= 4 * 16 * (int64_t)sm_count()
+        // (total_chunks counts tiles, whatever number of them a warp claims at once.)
+        return total_chunks <= 4 * 16 * (int64_t)sm_count()
                    ? launch_trace_b<true, false, MS_FEW, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                 d_rays, d_counters, st)
                    : launch_trace_b<true, false, MS_MANY, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
