@@ -674,16 +674,30 @@ rcp_status launch_separate(const SceneDev& S, const LaunchCfg& cfg, const ViewDe
                                                                   d_rays, d_counters, st);
 }
 
+// Whether a multi-sample launch takes MS_FEW. Up to four tiles per resident
+// warp of it its shorter chains win: of 20 frames below the line (terrain and
+// forest, 1 to 6 passes, 1 to 4 samples) it was 2 to 8 % faster on 17 and 1 to
+// 3 % slower on 3 (5,600 to 7,900 tiles); above it 24 warps win by 3 to 9 %
+// from 14,000 tiles on. Served requests of 460 to 7,200 tiles, one at a time,
+// are answered 4 to 9 % sooner by MS_FEW (640x360 K = 6, 4 samples: terrain 1.48
+// -> 1.36 ms, forest 3.71 -> 3.46 ms), those above the line as before.
+// total_chunks counts tiles, whatever number of them a warp claims at once.
+bool few_tiles(int64_t total_chunks) { return total_chunks <= 4 * 16 * (int64_t)sm_count(); }
+
 }  // namespace
 
 rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
                        int64_t total_pix, int64_t total_chunks, float4* rays, unsigned* d_work,
                        unsigned long long* d_rays, unsigned long long* d_counters, cudaStream_t st) {
     if (cfg.multi) {  // views of several scenes: fused camera, no counters
-        return cfg.ms ? launch_trace_b<true, false, MS_MANY, true>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
-                                                                d_rays, nullptr, st)
-                      : launch_trace_b<true, false, 0, true>(S, cfg, d_views, n_views, total_chunks, rays,
-                                                                 d_work, d_rays, nullptr, st);
+        if (!cfg.ms)
+            return launch_trace_b<true, false, 0, true>(S, cfg, d_views, n_views, total_chunks, rays, d_work, d_rays,
+                                                        nullptr, st);
+        return few_tiles(total_chunks) ? launch_trace_b<true, false, MS_FEW, true>(S, cfg, d_views, n_views, total_chunks,
+                                                                                   rays, d_work, d_rays, nullptr, st)
+                                       : launch_trace_b<true, false, MS_MANY, true>(S, cfg, d_views, n_views,
+                                                                                    total_chunks, rays, d_work, d_rays,
+                                                                                    nullptr, st);
     }
     if (!cfg.fused && !cfg.ms) {
         int64_t g = (total_pix + 255) / 256;
@@ -699,12 +713,7 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
         if (cfg.count)
             return launch_trace_b<true, true, MS_MANY, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                               d_rays, d_counters, st);
-        // Up to four tiles per resident warp of MS_FEW its shorter chains win:
-        // of 20 frames below the line (terrain and forest, 1 to 6 passes, 1 to 4
-        // samples) it was 2 to 8 % faster on 17 and 1 to 3 % slower on 3 (5,600
-        // to 7,900 tiles); above it 24 warps win by 3 to 9 % from 14,000 tiles on.
-        // (total_chunks counts tiles, whatever number of them a warp claims at once.)
-        return total_chunks <= 4 * 16 * (int64_t)sm_count()
+        return few_tiles(total_chunks)
                    ? launch_trace_b<true, false, MS_FEW, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,
                                                                 d_rays, d_counters, st)
                    : launch_trace_b<true, false, MS_MANY, false>(S, cfg, d_views, n_views, total_chunks, rays, d_work,

@@ -1,5 +1,6 @@
-"""Which multi-sample kernel a launch takes: the one with fewer warps and nothing
-spilled up to 64 tiles per SM, the other above, whatever a warp claims at once."""
+"""Which multi-sample kernel a launch takes, served or not: the one with fewer
+warps and nothing spilled up to 64 tiles per SM, the other above, whatever a
+warp claims at once."""
 import re
 
 import numpy as np
@@ -55,3 +56,21 @@ def test_line_is_in_tiles(scene, chunk, rows, want):
     cam = rcp.camera_from(sc.poses[0])
     assert _variants(lambda: rcp.rcp_render_device(g, cam, W, H, 1, p, None, out, None,
                                                    torch.cuda.current_stream())) == [want]
+
+
+@pytest.mark.parametrize("rows,want", [(1, FEW), (0, FEW), (-1, MANY)])
+def test_served_launches_follow_the_line(scene, rows, want):
+    sc, g = scene
+    p = rcp.make_params(rcp.RCP_MAP_EYE, 0.05 * sc.diameter(), 6.0, jitter=JIT)
+    W, H = 64 * 8, 4 * (_line_rows() if rows == 0 else _line_rows() + 1 if rows < 0 else rows)
+    cam = rcp.camera_from(sc.poses[0])
+    out = np.empty((H, W, 3), np.float32)
+    srv = rcp.rcp_server_create(1 << 30, 2)
+    try:
+        def serve():
+            rcp.rcp_server_wait(srv, rcp.rcp_server_submit(srv, g, cam, W, H, 2, p, out), 60.0)
+
+        assert _variants(serve) == [want] * 2
+    finally:
+        rcp.rcp_server_destroy(srv)
+    assert np.array_equal(out, rcp.rcp_render(g, cam, W, H, 2, p))
