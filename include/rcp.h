@@ -337,12 +337,18 @@ int64_t rcp_render_h2d_bytes(int n_views, int K);
  *    the call returns RCP_ERR_STACK.
  *  rcp_debug_sort_pairs: stable LSD radix sort of n (key, value) pairs on the
  *    low `bits` bits of the keys, in place.
+ *  rcp_debug_sort_pairs_tiles: the same, all digit passes tried in one launch for
+ *    at most resident_tiles tiles of 7,168 pairs (0: never; negative: the
+ *    device's SMs, as rcp_debug_sort_pairs); one launch per pass otherwise, and
+ *    where the device refuses to run so many tiles at once.
  *  rcp_debug_morton: 30-bit Morton codes of n points (xyz[n*3]) in the cube
  *    with corner lo[3] and side max_a(hi[a] - lo[a]) (host arrays). */
 rcp_status rcp_debug_trace(const rcp_scene* scene, int64_t n, const float* orig_tmin,
                            const float* dir_tmax, int any_hit, int brute, float* t_out,
                            int32_t* prim_out, int stack_entries, void* stream);
 rcp_status rcp_debug_sort_pairs(uint32_t* keys, uint32_t* values, int64_t n, int bits, void* stream);
+rcp_status rcp_debug_sort_pairs_tiles(uint32_t* keys, uint32_t* values, int64_t n, int bits,
+                                      int64_t resident_tiles, void* stream);
 rcp_status rcp_debug_morton(const float* xyz, int64_t n, const float* lo, const float* hi,
                             uint32_t* codes, void* stream);
 /* Test of the radix sort's bounded wait: one block of a sort pass takes the

@@ -1232,7 +1232,6 @@ rcp_status rcp_last_pass_times(const rcp_scene* sc, float* ms, int max_passes, i
     return RCP_OK;
 }
 
-rcp_status rcp_debug_sort_pairs(uint32_t* keys, uint32_t* values, int64_t n, int bits, void* stream);
 rcp_status rcp_debug_morton(const float* xyz, int64_t n, const float* lo, const float* hi, uint32_t* codes,
                             void* stream) {
     if (n < 0 || (n > 0 && (!xyz || !lo || !hi || !codes))) {
@@ -1247,13 +1246,12 @@ rcp_status rcp_debug_morton(const float* xyz, int64_t n, const float* lo, const 
 
 }  // extern "C"
 
-namespace rcp {
-size_t radix_sort_scratch_bytes(int64_t n);
-rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n,
-                            int bits, void* scratch, int* d_error, cudaStream_t stream);
+extern "C" rcp_status rcp_debug_sort_pairs(uint32_t* keys, uint32_t* values, int64_t n, int bits, void* stream) {
+    return rcp_debug_sort_pairs_tiles(keys, values, n, bits, -1, stream);
 }
 
-extern "C" rcp_status rcp_debug_sort_pairs(uint32_t* keys, uint32_t* values, int64_t n, int bits, void* stream) {
+extern "C" rcp_status rcp_debug_sort_pairs_tiles(uint32_t* keys, uint32_t* values, int64_t n, int bits,
+                                                 int64_t resident_tiles, void* stream) {
     if (n < 0 || bits < 1 || bits > 32 || (n > 0 && (!keys || !values))) {
         set_error("rcp_debug_sort_pairs: bad argument");
         return RCP_ERR_ARG;
@@ -1270,7 +1268,7 @@ extern "C" rcp_status rcp_debug_sort_pairs(uint32_t* keys, uint32_t* values, int
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_err, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(d_err, 0, sizeof(int), st);
     if (e != cudaSuccess) r = cuda_fail(e, "rcp_debug_sort_pairs alloc");
-    if (r == RCP_OK) r = radix_sort_pairs(keys, values, ak, av, n, bits, scratch, d_err, st);
+    if (r == RCP_OK) r = radix_sort_pairs(keys, values, ak, av, n, bits, scratch, d_err, st, resident_tiles);
     int h = 0;
     if (r == RCP_OK) {
         e = cudaMemcpyAsync(&h, d_err, sizeof(int), cudaMemcpyDeviceToHost, st);

@@ -44,10 +44,6 @@
 
 namespace rcp {
 
-size_t radix_sort_scratch_bytes(int64_t n);
-rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals,
-                            int64_t n, int bits, void* scratch, int* d_error, cudaStream_t stream);
-
 namespace {
 
 constexpr int BUILD_BLOCK = 256;

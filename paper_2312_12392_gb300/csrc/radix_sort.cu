@@ -7,7 +7,8 @@
 // digit run are contiguous.
 //  * While the tiles fit the GPU at once (one per SM, 1.09 million pairs on
 //    152 SMs), one cooperative launch runs every pass (k_sort_resident).
-//  * Beyond that, onesweep: one histogram kernel counts all digit passes at
+//  * Beyond that, or where the device does not run that many blocks at once,
+//    onesweep: one histogram kernel counts all digit passes at
 //    once (its last block scans the counts), then one launch per digit finds a
 //    tile's place by decoupled look-back over earlier tiles (numbered in launch
 //    order by an atomic counter, so every earlier tile is already running).
@@ -23,7 +24,7 @@
 // status words, and programmatic launches, so that a pass's blocks are
 // resident when the pass before ends. 1,000,003 pairs on 30 bits, the whole
 // call with its last read-back: 170 us (four passes of 25 us and a histogram),
-// onesweep as here 102 us, resident 96 us (53 us in the kernel).
+// onesweep as here 99-101 us, resident 96-98 us (52 us in the kernel).
 //
 // Every wait on another tile's status is bounded: after spin_limit polls
 // (SPIN_LIMIT in a sort) the kernel records an error flag and proceeds, so a
@@ -397,10 +398,11 @@ rcp_status launch_onesweep(const uint32_t* ki, const uint32_t* vi, uint32_t* ko,
     return RCP_OK;
 }
 
-rcp_status launch_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n, int passes,
-                           uint32_t* counts, uint32_t* arrived, int64_t tiles, int* d_error, cudaStream_t stream) {
-    RCP_CUDA(cudaFuncSetAttribute(k_sort_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)sizeof(ResidentShared)));
+cudaError_t launch_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n, int passes,
+                            uint32_t* counts, uint32_t* arrived, int64_t tiles, int* d_error, cudaStream_t stream) {
+    cudaError_t e = cudaFuncSetAttribute(k_sort_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(ResidentShared));
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)tiles);
     cfg.blockDim = dim3(SORT_BLOCK);
@@ -411,9 +413,8 @@ rcp_status launch_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, u
     attr.val.cooperative = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    RCP_CUDA(cudaLaunchKernelEx(&cfg, k_sort_resident, keys, vals, alt_keys, alt_vals, n, passes, counts, arrived,
-                                d_error, SPIN_LIMIT));
-    return RCP_OK;
+    return cudaLaunchKernelEx(&cfg, k_sort_resident, keys, vals, alt_keys, alt_vals, n, passes, counts, arrived,
+                              d_error, SPIN_LIMIT);
 }
 
 // The sorted pairs, if they lie elsewhere, back to the caller's arrays.
@@ -427,15 +428,12 @@ rcp_status copy_back(uint32_t* keys, uint32_t* vals, const uint32_t* ki, const u
 
 }  // namespace
 
-// Sort n pairs in place on the low `bits` bits of the keys. alt_keys/alt_vals
-// are n-element scratch buffers; scratch holds the histogram, tile status and
-// counters (size from radix_sort_scratch_bytes).
 size_t radix_sort_scratch_bytes(int64_t n) {
     return sizeof(uint32_t) * scratch_words(std::max<int64_t>((n + TILE - 1) / TILE, 1), PASSES_MAX);
 }
 
-rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals,
-                            int64_t n, int bits, void* scratch, int* d_error, cudaStream_t stream) {
+rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n, int bits,
+                            void* scratch, int* d_error, cudaStream_t stream, int64_t resident_tiles) {
     if (n <= 1) return RCP_OK;
     if (n >= (int64_t)COUNT_MASK) {
         set_error("radix sort: too many keys (limit 2^30)");
@@ -451,16 +449,24 @@ rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
     RCP_CUDA(cudaGetDevice(&dev));
     RCP_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     uint32_t *ki = keys, *vi = vals, *ko = alt_keys, *vo = alt_vals;
-    // One tile per SM at most: one launch for all passes (1,000,003 pairs 96 us, onesweep 102 us)
-    if (tiles <= sms) {
-        rcp_status r = launch_resident(keys, vals, alt_keys, alt_vals, n, passes, status, counters, tiles, d_error,
-                                       stream);
-        if (r != RCP_OK) return r;
-        if (passes & 1) {
-            std::swap(ki, ko);
-            std::swap(vi, vo);
+    // One tile per SM at most: one launch for all passes. The call on 1,000,003
+    // pairs takes 96-98 us, onesweep 99-101; at 1,000 to 600,000 pairs the two
+    // are within 2 % of each other (the same chain of loads, ranks and barriers
+    // or look-backs, and the call's read-back).
+    if (tiles <= (resident_tiles < 0 ? sms : resident_tiles)) {
+        const cudaError_t e = launch_resident(keys, vals, alt_keys, alt_vals, n, passes, status, counters, tiles, d_error,
+                                              stream);
+        if (e == cudaSuccess) {
+            if (passes & 1) {
+                std::swap(ki, ko);
+                std::swap(vi, vo);
+            }
+            return copy_back(keys, vals, ki, vi, n, stream);
         }
-        return copy_back(keys, vals, ki, vi, n, stream);
+        // fewer SMs to be had at once than the device has (a partition of it):
+        // the passes one by one need no tiles to run together
+        if (e != cudaErrorCooperativeLaunchTooLarge) return cuda_fail(e, "cooperative sort launch");
+        cudaGetLastError();
     }
     int64_t hblocks = (n + HIST_BLOCK * HIST_KEYS - 1) / (HIST_BLOCK * HIST_KEYS);
     if (hblocks > sms) hblocks = sms;

@@ -220,4 +220,12 @@ struct EventPair {
         if (e_ != cudaSuccess) return rcp::cuda_fail(e_, #call); \
     } while (0)
 
+// The radix sort (radix_sort.cu): n pairs in place on the low `bits` bits of the
+// keys. alt_keys/alt_vals are n-element buffers, scratch has
+// radix_sort_scratch_bytes(n). resident_tiles: the most tiles that one launch
+// for all passes is tried with (negative: as many as the device has SMs).
+size_t radix_sort_scratch_bytes(int64_t n);
+rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n, int bits,
+                            void* scratch, int* d_error, cudaStream_t stream, int64_t resident_tiles = -1);
+
 }  // namespace rcp

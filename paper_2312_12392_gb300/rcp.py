@@ -108,6 +108,7 @@ _SIGS = {
     "rcp_render_h2d_bytes": [C.c_int, C.c_int],
     "rcp_debug_trace": [_vp, C.c_int64, _vp, _vp, C.c_int, C.c_int, _vp, _vp, C.c_int, _vp],
     "rcp_debug_sort_pairs": [_vp, _vp, C.c_int64, C.c_int, _vp],
+    "rcp_debug_sort_pairs_tiles": [_vp, _vp, C.c_int64, C.c_int, C.c_int64, _vp],
     "rcp_debug_morton": [_vp, C.c_int64, _vp, _vp, _vp, _vp],
     "rcp_debug_sort_lookback_timeout": [C.c_int64, _vp],
     "rcp_imagespace_pass_device": [_vp, _vp, _vp, C.c_int, C.c_int, C.c_float, _vp],
@@ -364,6 +365,11 @@ def rcp_debug_trace(scene, n, orig_tmin, dir_tmax, any_hit, brute, t_out, prim_o
 
 def rcp_debug_sort_pairs(keys, values, n, bits, stream=None):
     _check(lib().rcp_debug_sort_pairs(_ptr(keys), _ptr(values), n, bits, _stream(stream)), "rcp_debug_sort_pairs")
+
+
+def rcp_debug_sort_pairs_tiles(keys, values, n, bits, resident_tiles, stream=None):
+    _check(lib().rcp_debug_sort_pairs_tiles(_ptr(keys), _ptr(values), n, bits, int(resident_tiles), _stream(stream)),
+           "rcp_debug_sort_pairs_tiles")
 
 
 def rcp_debug_morton(xyz, n, lo, hi, codes, stream=None):
