@@ -358,6 +358,11 @@ rcp_status rcp_debug_morton(const float* xyz, int64_t n, const float* lo, const 
  * flag and the block finishes. Returns RCP_ERR_TIMEOUT when the flag was set,
  * as a sort whose wait ran out does. Synchronous; allocates its own buffers. */
 rcp_status rcp_debug_sort_lookback_timeout(int64_t spin_limit, void* stream);
+/* The same for the BVH build's clustering: its first round never runs its
+ * first tile, so the others' waits run out. They write nothing, the rounds
+ * behind it leave at once, and the call returns RCP_ERR_TIMEOUT as a scene build
+ * whose wait ran out does. */
+rcp_status rcp_debug_cluster_lookback_timeout(int64_t spin_limit, void* stream);
 
 /* Allocation-free sort. The paper has no counterpart: this is a library
  * facility. Some callers cannot allocate device memory at the point where they

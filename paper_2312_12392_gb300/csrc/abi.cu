@@ -1232,6 +1232,14 @@ rcp_status rcp_last_pass_times(const rcp_scene* sc, float* ms, int max_passes, i
     return RCP_OK;
 }
 
+rcp_status rcp_debug_cluster_lookback_timeout(int64_t spin_limit, void* stream) {
+    if (spin_limit < 1 || spin_limit > (1ll << 20)) {
+        set_error("rcp_debug_cluster_lookback_timeout: spin_limit outside [1, 2^20]");
+        return RCP_ERR_ARG;
+    }
+    return debug_cluster_timeout((int)spin_limit, (cudaStream_t)stream);
+}
+
 rcp_status rcp_debug_morton(const float* xyz, int64_t n, const float* lo, const float* hi, uint32_t* codes,
                             void* stream) {
     if (n < 0 || (n > 0 && (!xyz || !lo || !hi || !codes))) {

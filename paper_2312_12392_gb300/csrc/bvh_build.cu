@@ -29,9 +29,9 @@
 //     its part of the triangle, so that a refit after a vertex update bounds
 //     it by that part of the moved triangle.
 #include <cuda_runtime.h>
+#include <limits.h>
 #include <math.h>
 #include <stdint.h>
-
 #include <string.h>
 
 #include <algorithm>
@@ -629,7 +629,9 @@ __device__ __forceinline__ void box_union(float4 la, float4 ha, float4 lb, float
 // merges and the clusters it keeps, finds the counts before it by decoupled
 // look-back (tiles numbered by an atomic counter, so every earlier tile is
 // already running; each wait is bounded), and writes its nodes and its part of
-// the next array. The merge with m merges before it, over all rounds, becomes
+// the next array. A tile whose wait runs out writes neither; as its places then
+// hold no clusters, the rounds after it, which would follow them, leave at once.
+// The merge with m merges before it, over all rounds, becomes
 // node N - 2 - m: the last one is the root, node 0. A status word carries both
 // counts, 31 bits each, and its flag. From 24,000 clusters down, where launch,
 // look-back and the chain of 32 candidates bound it, a round takes 7 to 12 us
@@ -641,14 +643,18 @@ constexpr unsigned long long PLOC_AGG = 1ull << 62, PLOC_INC = 2ull << 62, PLOC_
 constexpr int PLOC_SPINS = 1 << 26;
 
 // Called by one whole warp of a block: publishes the tile's counts and returns
-// the sum of the earlier tiles', 32 of them per round of loads. Past
-// PLOC_SPINS polls it records an error and goes on.
+// the sum of the earlier tiles', 32 of them per round of loads. Past spin_limit
+// polls it records the round as failed, publishes what it has (no more than the
+// true counts, so later tiles write in range) and returns PLOC_NONE.
+constexpr unsigned long long PLOC_NONE = ~0ull;
 __device__ __forceinline__ unsigned long long counts_before(unsigned long long* status, int64_t tile,
-                                                            unsigned long long total, int* err) {
+                                                            unsigned long long total, int* failed, int round,
+                                                            int spin_limit) {
     const int lane = threadIdx.x & 31;
     volatile unsigned long long* st = status;
     if (lane == 0) st[tile] = (tile == 0 ? PLOC_INC : PLOC_AGG) | total;
     unsigned long long before = 0;
+    bool ran_out = false;
     int64_t t = tile - 1;
     for (int spins = 0; t >= 0;) {
         unsigned long long w = PLOC_INC;  // before the first tile: nothing more to add
@@ -659,8 +665,8 @@ __device__ __forceinline__ unsigned long long counts_before(unsigned long long* 
         const int last = inclusive ? __ffs(inclusive) - 1 : 31;
         const unsigned use = 0xffffffffu >> (31 - last);
         if (waiting & use) {
-            if (++spins > PLOC_SPINS) {
-                if (lane == 0) atomicAdd(err, 1);
+            if (++spins > spin_limit) {
+                ran_out = true;
                 break;
             }
             continue;
@@ -671,8 +677,9 @@ __device__ __forceinline__ unsigned long long counts_before(unsigned long long* 
         if (inclusive) break;
         t -= 32;
     }
+    if (lane == 0 && ran_out) atomicMin(failed, round);
     if (lane == 0 && tile > 0) st[tile] = PLOC_INC | (before + total);
-    return before;
+    return ran_out ? PLOC_NONE : before;
 }
 
 __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_round(PlocState* __restrict__ state, unsigned* ticket,
@@ -680,7 +687,7 @@ __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_round(PlocState* __restrict
                                                            const int* __restrict__ ref, const float4* __restrict__ clo,
                                                            const float4* __restrict__ chi, int* __restrict__ ref_out,
                                                            float4* __restrict__ lo_out, float4* __restrict__ hi_out,
-                                                           PlocTree tree, int* err) {
+                                                           PlocTree tree, int* failed, int round, int spin_limit) {
     constexpr int WARPS = PLOC_BLOCK / 32, HELD = PLOC_BLOCK + 2 * PLOC_R;
     static_assert(WARPS <= 32, "one warp scans the warps' counts");
     __shared__ float4 s_lo[HELD], s_hi[HELD];  // clusters first - PLOC_R ..
@@ -688,11 +695,11 @@ __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_round(PlocState* __restrict
     __shared__ unsigned long long s_row[WARPS];  // per warp: counts before it in the tile
     __shared__ unsigned long long s_before;
     __shared__ unsigned s_tile;
+    const int n = state->n, first_failed = *failed;  // both loads overlap the ticket
     if (threadIdx.x == 0) s_tile = atomicAdd(ticket, 1u);
     __syncthreads();
-    const int n = state->n;
     const int64_t tile = s_tile;
-    if (tile * PLOC_TILE >= n) return;
+    if (first_failed < round || tile * PLOC_TILE >= n) return;
     const int first = (int)(tile * PLOC_TILE) - PLOC_R;  // thread t's cluster is first + t
     for (int t = threadIdx.x; t < HELD; t += PLOC_BLOCK) {
         const int g = first - PLOC_R + t;
@@ -733,10 +740,10 @@ __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_round(PlocState* __restrict
         }
         if (lane < WARPS) s_row[lane] = x - row;
         const unsigned long long total = __shfl_sync(0xffffffffu, x, 31);
-        const unsigned long long before = counts_before(status, tile, total, err);
+        const unsigned long long before = counts_before(status, tile, total, failed, round, spin_limit);
         if (lane == 0) s_before = before;
         // the last tile's counts and those before it are the round's
-        if (lane == 0 && (tile + 1) * PLOC_TILE >= n) {
+        if (lane == 0 && before != PLOC_NONE && (tile + 1) * PLOC_TILE >= n) {
             const unsigned long long all = before + total;
             const int merged = (int)(all >> 31);
             state[1] = PlocState{(int)(all & 0x7fffffffull), state->created + merged,
@@ -745,7 +752,7 @@ __global__ void __launch_bounds__(PLOC_BLOCK) k_ploc_round(PlocState* __restrict
     }
     if ((merges >> lane) & 1u) ploc_pair(tree, s_ref[me], s_ref[other], pl, ph, leaves);
     __syncthreads();
-    if (!((stays >> lane) & 1u)) return;
+    if (s_before == PLOC_NONE || !((stays >> lane) & 1u)) return;
     const unsigned lt = (1u << lane) - 1u;
     const unsigned long long run = s_before + s_row[warp];
     const int64_t pos = (int64_t)(run & 0x7fffffffull) + __popc(stays & lt);
@@ -1596,12 +1603,15 @@ void scan_u64(unsigned long long* d, int64_t n, unsigned long long* aux, const s
 // Fills child, blo/bhi (padded) and range of internal nodes 0..N-2 (root 0), with the
 // leaves renumbered depth-first: ids_out[j] is the primitive of leaf j.
 // `tree` comes without its counts.
+// first_tile (a test's): the first tile that the first round runs; the ones
+// before it never do.
 rcp_status build_ploc(int64_t N, PlocTree tree, uint32_t* ids_out, int2* range, int* d_err, int cap, Arena& arena,
-                      cudaStream_t st) {
+                      cudaStream_t st, int spin_limit = PLOC_SPINS, unsigned first_tile = 0) {
     Carved<int> ref_a, ref_b, cnt, pos;
     Carved<float4> lo_a, hi_a, lo_b, hi_b;
     // per batch of up to PLOC_BATCH rounds: the rounds' states, tile counters and tile status
     constexpr int PLOC_BATCH = 16;
+    constexpr int FAILED = PLOC_BATCH + 1;  // the state whose n is the first round with a wait that ran out
     Carved<PlocState> state;
     Carved<unsigned long long> marks;
     const int64_t tiles_max = (N + PLOC_TILE - 1) / PLOC_TILE;
@@ -1613,7 +1623,7 @@ rcp_status build_ploc(int64_t N, PlocTree tree, uint32_t* ids_out, int2* range, 
     RCP_CUDA(hi_a.alloc(arena, N));
     RCP_CUDA(lo_b.alloc(arena, N));
     RCP_CUDA(hi_b.alloc(arena, N));
-    RCP_CUDA(state.alloc(arena, PLOC_BATCH + 2));
+    RCP_CUDA(state.alloc(arena, FAILED + 1));
     RCP_CUDA(marks.alloc(arena, PLOC_BATCH * (1 + tiles_max)));
     RCP_CUDA(cudaMemsetAsync(tree.parent_int, 0xff, sizeof(int) * N, st));
     RCP_CUDA(cudaMemsetAsync(tree.parent_leaf, 0xff, sizeof(int) * N, st));
@@ -1621,8 +1631,11 @@ rcp_status build_ploc(int64_t N, PlocTree tree, uint32_t* ids_out, int2* range, 
     int *rin = ref_a.p, *rout = ref_b.p;
     float4 *lin = lo_a.p, *hin = hi_a.p, *lout = lo_b.p, *hout = hi_b.p;
     k_ploc_init<<<grid_for(N, BUILD_BLOCK, cap), BUILD_BLOCK, 0, st>>>(tree.ids, N, tree.plo, tree.phi, rin, lin, hin);
-    PlocState h{(int)N, 0, 0, 0};
-    RCP_CUDA(cudaMemcpyAsync(state.p, &h, sizeof(h), cudaMemcpyHostToDevice, st));
+    PlocState hs[FAILED + 1] = {};
+    hs[0].n = (int)N;
+    hs[FAILED].n = INT_MAX;
+    RCP_CUDA(cudaMemcpyAsync(state.p, hs, sizeof(hs), cudaMemcpyHostToDevice, st));
+    PlocState h = hs[0];
     // The rounds run without the host between them: each reads its count from
     // the device, under a grid sized for the count at the batch's start, which
     // only shrinks. The host reads the count once per batch.
@@ -1633,18 +1646,26 @@ rcp_status build_ploc(int64_t N, PlocTree tree, uint32_t* ids_out, int2* range, 
         const int need = (int)std::ceil(std::log((double)n0 / PLOC_LAST) / std::log(4.0 / 3.0));
         const int rounds = std::min(PLOC_BATCH, std::max(2, (need + 1) & ~1));
         RCP_CUDA(cudaMemsetAsync(marks.p, 0, sizeof(unsigned long long) * PLOC_BATCH * (1 + tiles), st));
+        if (first_tile && h.created == 0)
+            RCP_CUDA(cudaMemcpyAsync(marks.p, &first_tile, sizeof(first_tile), cudaMemcpyHostToDevice, st));
         for (int r = 0; r < rounds; ++r) {
             k_ploc_round<<<(unsigned)tiles, PLOC_BLOCK, 0, st>>>(state.p + r, (unsigned*)(marks.p + r),
                                                                  marks.p + PLOC_BATCH + r * tiles, N, rin, lin, hin,
-                                                                 rout, lout, hout, tree, d_err);
+                                                                 rout, lout, hout, tree, &state.p[FAILED].n, r,
+                                                                 spin_limit);
             std::swap(rin, rout);
             std::swap(lin, lout);
             std::swap(hin, hout);
         }
         RCP_CUDA(cudaGetLastError());
+        RCP_CUDA(cudaMemcpyAsync(hs, state.p, sizeof(hs), cudaMemcpyDeviceToHost, st));
         RCP_CUDA(cudaMemcpyAsync(state.p, state.p + rounds, sizeof(h), cudaMemcpyDeviceToDevice, st));
-        RCP_CUDA(cudaMemcpyAsync(&h, state.p, sizeof(h), cudaMemcpyDeviceToHost, st));
         RCP_CUDA(cudaStreamSynchronize(st));
+        if (hs[FAILED].n != INT_MAX) {
+            set_error("BVH build: the clustering's look-back wait ran out");
+            return RCP_ERR_TIMEOUT;
+        }
+        h = hs[rounds];
         // the smallest pair is always mutual, so a round without a merge means
         // the device state is corrupt
         if (h.stalled || h.n < 1 || h.n >= n0 || h.n + h.created != N) {
@@ -2022,6 +2043,38 @@ rcp_status validate_bvh(const Scene& sc, cudaStream_t st) {
             return RCP_ERR_STATE;
         }
     return RCP_OK;
+}
+
+// A clustering whose first round never runs its first tile: 2,000 boxes, all
+// equal (nine tiles, of which eight wait for the first).
+rcp_status debug_cluster_timeout(int spin_limit, cudaStream_t st) {
+    const int64_t N = 2000;
+    Arena arena;
+    Carved<float4> lo, hi, blo, bhi;
+    Carved<uint32_t> ids, ids_out;
+    Carved<int2> child, range;
+    Carved<int> parent_int, parent_leaf, err;
+    RCP_CUDA(arena.reserve(N * 320 + (1 << 16)));
+    RCP_CUDA(lo.alloc(arena, N));
+    RCP_CUDA(hi.alloc(arena, N));
+    RCP_CUDA(blo.alloc(arena, N));
+    RCP_CUDA(bhi.alloc(arena, N));
+    RCP_CUDA(ids.alloc(arena, N));
+    RCP_CUDA(ids_out.alloc(arena, N));
+    RCP_CUDA(child.alloc(arena, N));
+    RCP_CUDA(range.alloc(arena, N));
+    RCP_CUDA(parent_int.alloc(arena, N));
+    RCP_CUDA(parent_leaf.alloc(arena, N));
+    RCP_CUDA(err.alloc(arena, 1));
+    RCP_CUDA(cudaMemsetAsync(lo.p, 0, sizeof(float4) * N, st));
+    RCP_CUDA(cudaMemsetAsync(hi.p, 0, sizeof(float4) * N, st));
+    RCP_CUDA(cudaMemsetAsync(ids.p, 0, sizeof(uint32_t) * N, st));  // every leaf is box 0
+    RCP_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
+    const PlocTree tree{child.p, blo.p, bhi.p, nullptr, parent_int.p, parent_leaf.p, ids.p,
+                        lo.p,    hi.p,  nullptr, nullptr, nullptr, 0};  // no triangles: no box is padded
+    const rcp_status r = build_ploc(N, tree, ids_out.p, range.p, err.p, 64, arena, st, spin_limit, 1);
+    RCP_CUDA(cudaStreamSynchronize(st));
+    return r;
 }
 
 rcp_status debug_morton(const float* xyz, int64_t n, const float* lo, const float* hi, uint32_t* codes,

@@ -106,6 +106,7 @@ rcp_status ingest_scene(Scene& sc, const float* albedo3, bool* bad_tri, bool* ba
 rcp_status build_bvh(Scene& sc, cudaStream_t st);
 rcp_status refit_bvh(Scene& sc, cudaStream_t st);
 rcp_status validate_bvh(const Scene& sc, cudaStream_t st);
+rcp_status debug_cluster_timeout(int spin_limit, cudaStream_t st);
 rcp_status debug_morton(const float* xyz, int64_t n, const float* lo, const float* hi, uint32_t* codes,
                         cudaStream_t st);
 
