@@ -358,6 +358,9 @@ rcp_status rcp_debug_morton(const float* xyz, int64_t n, const float* lo, const 
  * flag and the block finishes. Returns RCP_ERR_TIMEOUT when the flag was set,
  * as a sort whose wait ran out does. Synchronous; allocates its own buffers. */
 rcp_status rcp_debug_sort_lookback_timeout(int64_t spin_limit, void* stream);
+/* The same for the sort in one launch: its one block waits at the grid's
+ * barriers for an arrival that never comes. */
+rcp_status rcp_debug_sort_barrier_timeout(int64_t spin_limit, void* stream);
 /* The same for the BVH build's clustering: its first round never runs its
  * first tile, so the others' waits run out. They write nothing, the rounds
  * behind it leave at once, and the call returns RCP_ERR_TIMEOUT as a scene build

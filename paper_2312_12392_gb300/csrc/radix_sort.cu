@@ -292,7 +292,9 @@ __global__ void __launch_bounds__(SORT_BLOCK, 1) k_onesweep(const uint32_t* __re
 // adds up every tile's counts itself (all tiles' and the earlier tiles'), where
 // separate passes need a histogram beforehand and look back tile by tile; the
 // pairs go to the other buffer and a second barrier ends the pass. The launch is cooperative, so that every block
-// that a barrier waits for runs; each wait is bounded all the same.
+// that a barrier waits for runs; each wait is bounded all the same, and as the
+// counts are zero beforehand, one that runs out leaves sums too small: the pairs
+// still go to places in range.
 struct ResidentShared {
     SortShared t;
     uint32_t part[GROUPS][2][RADIX];  // per group: all tiles' counts, earlier tiles' counts
@@ -399,7 +401,8 @@ rcp_status launch_onesweep(const uint32_t* ki, const uint32_t* vi, uint32_t* ko,
 }
 
 cudaError_t launch_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, uint32_t* alt_vals, int64_t n, int passes,
-                            uint32_t* counts, uint32_t* arrived, int64_t tiles, int* d_error, cudaStream_t stream) {
+                            uint32_t* counts, uint32_t* arrived, int64_t tiles, int* d_error, long long spin_limit,
+                            cudaStream_t stream) {
     cudaError_t e = cudaFuncSetAttribute(k_sort_resident, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)sizeof(ResidentShared));
     if (e != cudaSuccess) return e;
@@ -414,7 +417,7 @@ cudaError_t launch_resident(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, k_sort_resident, keys, vals, alt_keys, alt_vals, n, passes, counts, arrived,
-                              d_error, SPIN_LIMIT);
+                              d_error, spin_limit);
 }
 
 // The sorted pairs, if they lie elsewhere, back to the caller's arrays.
@@ -455,7 +458,7 @@ rcp_status radix_sort_pairs(uint32_t* keys, uint32_t* vals, uint32_t* alt_keys, 
     // or look-backs, and the call's read-back).
     if (tiles <= (resident_tiles < 0 ? sms : resident_tiles)) {
         const cudaError_t e = launch_resident(keys, vals, alt_keys, alt_vals, n, passes, status, counters, tiles, d_error,
-                                              stream);
+                                              SPIN_LIMIT, stream);
         if (e == cudaSuccess) {
             if (passes & 1) {
                 std::swap(ki, ko);
@@ -618,6 +621,41 @@ extern "C" rcp_status rcp_debug_sort_lookback_timeout(int64_t spin_limit, void* 
     RCP_CUDA(cudaStreamSynchronize(st));
     if (h) {
         set_error("radix sort: look-back wait ran out");
+        return RCP_ERR_TIMEOUT;
+    }
+    return RCP_OK;
+}
+
+// rcp_debug_sort_barrier_timeout: one tile sorted in one launch, the barriers'
+// counter one short of what they expect, so each of the three of two digit passes
+// runs out.
+
+extern "C" rcp_status rcp_debug_sort_barrier_timeout(int64_t spin_limit, void* stream) {
+    using namespace rcp;
+    if (spin_limit < 1 || spin_limit > (1ll << 20)) {
+        set_error("rcp_debug_sort_barrier_timeout: spin_limit outside [1, 2^20]");
+        return RCP_ERR_ARG;
+    }
+    cudaStream_t st = (cudaStream_t)stream;
+    const int64_t n = TILE;
+    DevBuf<uint32_t> pairs, scratch;  // keys, values and their alternates
+    DevBuf<int> err;
+    RCP_CUDA(pairs.alloc(4 * n));
+    RCP_CUDA(scratch.alloc(scratch_words(1, 2)));
+    RCP_CUDA(err.alloc(1));
+    uint32_t* counter = scratch.p + PASSES_MAX * RADIX;
+    RCP_CUDA(cudaMemsetAsync(pairs.p, 0, sizeof(uint32_t) * 4 * n, st));
+    RCP_CUDA(cudaMemsetAsync(scratch.p, 0, sizeof(uint32_t) * scratch_words(1, 2), st));
+    RCP_CUDA(cudaMemsetAsync(counter, 0xff, sizeof(uint32_t), st));  // -1
+    RCP_CUDA(cudaMemsetAsync(err.p, 0, sizeof(int), st));
+    const cudaError_t e = launch_resident(pairs.p, pairs.p + n, pairs.p + 2 * n, pairs.p + 3 * n, n, 2, counter + COUNTERS,
+                                          counter, 1, err.p, (long long)spin_limit, st);
+    if (e != cudaSuccess) return cuda_fail(e, "rcp_debug_sort_barrier_timeout");
+    int h = 0;
+    RCP_CUDA(cudaMemcpyAsync(&h, err.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+    RCP_CUDA(cudaStreamSynchronize(st));
+    if (h) {
+        set_error("radix sort: barrier wait ran out");
         return RCP_ERR_TIMEOUT;
     }
     return RCP_OK;

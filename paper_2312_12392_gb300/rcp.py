@@ -111,6 +111,7 @@ _SIGS = {
     "rcp_debug_sort_pairs_tiles": [_vp, _vp, C.c_int64, C.c_int, C.c_int64, _vp],
     "rcp_debug_morton": [_vp, C.c_int64, _vp, _vp, _vp, _vp],
     "rcp_debug_sort_lookback_timeout": [C.c_int64, _vp],
+    "rcp_debug_sort_barrier_timeout": [C.c_int64, _vp],
     "rcp_debug_cluster_lookback_timeout": [C.c_int64, _vp],
     "rcp_imagespace_pass_device": [_vp, _vp, _vp, C.c_int, C.c_int, C.c_float, _vp],
     "rcp_sort_pairs_static": [_vp, _vp, C.c_int64, C.c_int, _vp],
@@ -382,6 +383,10 @@ def rcp_debug_morton(xyz, n, lo, hi, codes, stream=None):
 
 def rcp_debug_sort_lookback_timeout(spin_limit, stream=None):
     _check(lib().rcp_debug_sort_lookback_timeout(int(spin_limit), _stream(stream)), "rcp_debug_sort_lookback_timeout")
+
+
+def rcp_debug_sort_barrier_timeout(spin_limit, stream=None):
+    _check(lib().rcp_debug_sort_barrier_timeout(int(spin_limit), _stream(stream)), "rcp_debug_sort_barrier_timeout")
 
 
 def rcp_debug_cluster_lookback_timeout(spin_limit, stream=None):

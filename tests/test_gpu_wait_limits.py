@@ -1,4 +1,4 @@
-"""Bounded waits of the build that run out: a status comes back, nothing is
+"""Bounded waits of the sort and the build that run out: a status comes back, nothing is
 followed that was not written, and the device stays usable."""
 import pytest
 
@@ -35,8 +35,17 @@ def test_clustering_wait(limit):
     _build_and_walk()
 
 
-def test_limits_are_checked():
-    for bad in (0, (1 << 20) + 1):
-        with pytest.raises(rcp.RcpError) as e:
-            rcp.rcp_debug_cluster_lookback_timeout(bad)
-        assert e.value.status == rcp.RCP_ERR_ARG
+@pytest.mark.parametrize("limit", [1, 1000, 100_000])
+def test_barrier_wait(limit):
+    with pytest.raises(rcp.RcpError) as e:
+        rcp.rcp_debug_sort_barrier_timeout(limit)
+    assert e.value.status == rcp.RCP_ERR_TIMEOUT and "ran out" in str(e.value)
+    _build_and_walk()
+
+
+@pytest.mark.parametrize("entry", [rcp.rcp_debug_cluster_lookback_timeout, rcp.rcp_debug_sort_barrier_timeout])
+@pytest.mark.parametrize("limit", [0, (1 << 20) + 1])
+def test_limits_are_checked(entry, limit):
+    with pytest.raises(rcp.RcpError) as e:
+        entry(limit)
+    assert e.value.status == rcp.RCP_ERR_ARG
