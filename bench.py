@@ -315,29 +315,30 @@ def time_frames(g, cams, W, H, K, params, stream, flush):
 
 
 def count_work(g, cams, W, H, K, params, sizes=None, frames=None):
-    """The algorithmic work of the timed frames: an instrumented copy of the
-    trace kernel run over the same cameras, K passes each, each reading the
-    previous one's image. sizes: one (W, H) per camera (else W x H for all);
-    frames: how many timed frames the cameras make up (default one each)."""
+    """The work of the timed frames, the operations they execute: an
+    instrumented copy of the trace kernels run over the same cameras, K passes
+    each, which leaves out the passes whose values repeat as the timed kernels do.
+    rays_all: the rays of all K passes, left out or not (rcp_last_ray_counts).
+    sizes: one (W, H) per camera (else W x H for all); frames: how many timed
+    frames the cameras make up (default one each)."""
     import torch
 
     from paper_2312_12392_gb300 import rcp
-    tot = dict(box=0, tri=0, sph=0, nodes=0, prim_rays=0, rays=0, frames=len(cams) if frames is None else frames)
+    tot = dict(box=0, tri=0, sph=0, nodes=0, prim_rays=0, rays=0, rays_all=0,
+               frames=len(cams) if frames is None else frames)
     sizes = sizes or [(W, H)] * len(cams)
     for c, (W, H) in zip(cams, sizes):
-        a = torch.empty((H, W, 4), dtype=torch.float32, device="cuda")
-        b = torch.empty_like(a)
-        prev = None
-        for n in range(K):
-            dst = a if n % 2 == 0 else b
-            cnt = rcp.rcp_count_pass(g, c, W, H, params, prev, dst)
-            tot["box"] += cnt.box_tests
-            tot["tri"] += cnt.tri_tests
-            tot["sph"] += cnt.sphere_tests
-            tot["nodes"] += cnt.nodes
-            tot["prim_rays"] += cnt.primary_rays
-            tot["rays"] += cnt.rays
-            prev = dst
+        out = torch.empty((H, W, 4), dtype=torch.float32, device="cuda")
+        rcp.rcp_render_device(g, c, W, H, K, params, None, out, None, torch.cuda.current_stream())
+        torch.cuda.synchronize()
+        tot["rays_all"] += sum(rcp.rcp_last_ray_counts(g))
+        cnt = rcp.rcp_count_frame(g, c, W, H, K, params, None, out)
+        tot["box"] += cnt.box_tests
+        tot["tri"] += cnt.tri_tests
+        tot["sph"] += cnt.sphere_tests
+        tot["nodes"] += cnt.nodes
+        tot["prim_rays"] += cnt.primary_rays
+        tot["rays"] += cnt.rays
     return tot
 
 
@@ -371,8 +372,9 @@ def roofline(work, pass_ms, frames, workload, clk, sms):
     roof["launches_counted"] = n
     roof["algorithmic_ops_per_launch"] = ops
     roof["algorithmic_bytes_per_launch"] = byts
-    roof["work_note"] = ("work of all K passes, counted pass by pass; a chained launch leaves out the passes of tiles "
-                         "whose pixels repeat earlier values")
+    roof["work_note"] = ("operations executed; passes whose values repeat are left out of the launch and of this count "
+                         "(rays_left_out_frac of the rays of all K passes, which mrays_per_s counts)")
+    roof["rays_left_out_frac"] = 1.0 - work["rays"] / max(work.get("rays_all", work["rays"]), 1)
     roof["peak_source"] = f"{sms} SMs x 128 FP32 lanes x {sm_max_mhz:.0f} MHz (max SM clock)"
     roof["hbm_view"] = {"achieved_gbs": byts / launch_s / 1e9, "peak_gbs": hbm_gbs,
                         "frac": byts / launch_s / 1e9 / hbm_gbs, "peak_source": peak_src,

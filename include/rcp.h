@@ -312,6 +312,13 @@ rcp_status rcp_last_ray_counts(const rcp_scene* scene, int64_t* primary, int64_t
 rcp_status rcp_count_pass(const rcp_scene* scene, const rcp_camera* cam, int width, int height,
                           const rcp_params* params, const float* d_in, float* d_out, rcp_counters* out);
 
+/* The same for a K-pass frame as rcp_render_device runs it: the passes that a
+ * chained render or a repeated tile leaves out (rcp_last_ray_counts) are not
+ * counted, so these are the operations executed. d_in, d_out as there (d_out
+ * nullable). The gathers of an RCP_MAP_IMAGE render have no counters. */
+rcp_status rcp_count_frame(const rcp_scene* scene, const rcp_camera* cam, int width, int height, int K,
+                           const rcp_params* params, const float* d_in, float* d_out, rcp_counters* out);
+
 /* Device time (ms) of each launch of the scene's most recent render, from CUDA
  * events recorded on the render's stream between the launches (inside the
  * captured graph): one per pass, or one for all K passes when they ran

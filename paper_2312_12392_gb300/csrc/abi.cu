@@ -487,9 +487,9 @@ rcp_status enqueue_passes(const Scene& sc, RenderCtx& ctx, const LaunchCfg& cfg,
     if (ctx.chained) {  // one descriptor per view, all K passes (image mode: pass 1, then the gathers' descriptors)
         rcp_status r = ctx.image_mode
                            ? launch_pass(S, first, ctx.d_views, ctx.n_views, ctx.total_pix, ctx.total_chunks, nullptr,
-                                         ctx.d_work, ctx.d_rays, nullptr, st)
+                                         ctx.d_work, ctx.d_rays, counters, st)
                            : launch_chain(S, first, ctx.d_views, ctx.n_views, ctx.total_chunks, ctx.d_work, ctx.d_rays,
-                                          st);
+                                          counters, st);
         if (r != RCP_OK) return r;
         RCP_CUDA(record(ctx.pass_ev[1]));
         if (ctx.image_mode) {
@@ -1105,20 +1105,21 @@ rcp_status rcp_set_tuning(rcp_scene* sc, const rcp_tuning* t) {
     return RCP_OK;
 }
 
-rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, int H, const rcp_params* p,
-                          const float* d_in, float* d_out, rcp_counters* out) {
-    if (!csc || !out) {
-        set_error("rcp_count_pass: NULL argument");
-        return RCP_ERR_ARG;
-    }
-    rcp_scene* sc = const_cast<rcp_scene*>(csc);
+// K passes with work counters, chained where `chain` asks for it and the render
+// allows it.
+static rcp_status count_frame(rcp_scene* sc, const rcp_camera* cam, int W, int H, int K, const rcp_params* p,
+                              const float* d_in, float* d_out, bool chain, rcp_counters* out) {
     std::lock_guard<std::mutex> lk(sc->mu);
     rcp_status r = check_view(cam, W, H, p);
     if (r != RCP_OK) return r;
+    if (K < 1 || K > 16) {
+        set_error("K must be in [1, 16]");
+        return RCP_ERR_ARG;
+    }
     cudaStream_t st = lib_stream();
     const int64_t P = (int64_t)W * H;
     RenderCtx* ctx = nullptr;
-    r = get_ctx(*sc, 1, 1, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
+    r = get_ctx(*sc, 1, K, P, (int64_t)((W + 7) / 8) * ((H + 3) / 4), st, &ctx);
     if (r != RCP_OK) return r;
     std::vector<ViewDev> base(1);
     make_view(base[0], *cam, W, H, *p);
@@ -1126,14 +1127,14 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     layout_views(base, tp, tc);
     const float4* ins[1] = {(const float4*)d_in};
     if (!d_out) {
-        r = ensure_img(*sc, *ctx);
+        r = ensure_io(*sc, *ctx, false, false);
         if (r != RCP_OK) return r;
     }
-    float4* outs[1] = {d_out ? (float4*)d_out : ctx->img[0]};
+    float4* outs[1] = {d_out ? (float4*)d_out : ctx->io};
     StreamUse use, spill_use;
     r = use.begin(ctx->work, st);
     if (r != RCP_OK) return r;
-    r = stage_views(*sc, *ctx, base, ins, outs, nullptr, nullptr, st);
+    r = stage_views(*sc, *ctx, base, ins, outs, nullptr, nullptr, st, chain);
     if (r != RCP_OK) return r;
     DevBuf<unsigned long long> d_cnt;
     RCP_CUDA(d_cnt.alloc(8));
@@ -1141,6 +1142,7 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     LaunchCfg cfg = cfg_of(*sc);
     cfg.count = true;
     cfg.ms = p->spp > 0;
+    if (ctx->chained) cfg.fused = true;
     r = ensure_spill(*sc, cfg, st, spill_use);
     if (r != RCP_OK) return r;
     r = ensure_rays(*sc, *ctx, cfg);
@@ -1158,6 +1160,28 @@ rcp_status rcp_count_pass(const rcp_scene* csc, const rcp_camera* cam, int W, in
     out->tri_tests = (int64_t)h[5];
     out->sphere_tests = (int64_t)h[6];
     return check_status(*ctx, st);
+}
+
+rcp_status rcp_count_pass(const rcp_scene* sc, const rcp_camera* cam, int W, int H, const rcp_params* p,
+                          const float* d_in, float* d_out, rcp_counters* out) {
+    if (!sc || !out) {
+        set_error("rcp_count_pass: NULL argument");
+        return RCP_ERR_ARG;
+    }
+    return count_frame(const_cast<rcp_scene*>(sc), cam, W, H, 1, p, d_in, d_out, false, out);
+}
+
+rcp_status rcp_count_frame(const rcp_scene* sc, const rcp_camera* cam, int W, int H, int K, const rcp_params* p,
+                           const float* d_in, float* d_out, rcp_counters* out) {
+    if (!sc || !out) {
+        set_error("rcp_count_frame: NULL argument");
+        return RCP_ERR_ARG;
+    }
+    if (p && ((p->mapping == RCP_MAP_IMAGE && d_in) || (p->spp > 0 && K == 1 && d_in && d_in == d_out))) {
+        set_error("rcp_count_frame: d_in as for rcp_render_device");
+        return RCP_ERR_ARG;
+    }
+    return count_frame(const_cast<rcp_scene*>(sc), cam, W, H, K, p, d_in, d_out, sc->tuning.chain_passes != 0, out);
 }
 
 rcp_status rcp_debug_trace(const rcp_scene* sc, int64_t n, const float* orig_tmin, const float* dir_tmax, int any,

@@ -142,7 +142,8 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
 // camera (cfg.fused is not read), and a mapping that reads only the pixel's
 // own previous value; cfg.multi: the views name their scenes.
 rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
-                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays, cudaStream_t st);
+                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays,
+                        unsigned long long* d_counters, cudaStream_t st);
 // n descriptors (at most STAGE_VIEWS) to d_views, and n_zero words at `zero`
 // to 0, in one launch.
 constexpr int STAGE_VIEWS = 4;

@@ -276,7 +276,7 @@ rcp_status rcp_server::enqueue_step(std::vector<Request*>& batch, StepSlot& slot
     r = ms ? launch_pass((*scenes.begin())->dev(), cfg, slot.d_views, (int)batch.size(), total_pix, total_chunks,
                          nullptr, slot.d_work, d_rays, nullptr, st_main)
            : launch_chain((*scenes.begin())->dev(), cfg, slot.d_views, (int)batch.size(), total_chunks, slot.d_work,
-                          d_rays, st_main);
+                          d_rays, nullptr, st_main);
     if (r != RCP_OK) return r;
     for (Request* q : batch)  // after the step, whatever the done words say
         if (q->passes_done + q->step_passes == q->K) RCP_CUDA(cudaEventRecord(q->ready, st_main));

@@ -117,9 +117,10 @@ __device__ __forceinline__ bool same_bits(const float4& a, const float4& b) {
 // I_n is I_{n-2}, which its ping-pong buffer still holds; where all nine had
 // I_{n-1} = I_{n-2}, it is I_{n-1}, the same bits again. The last pass copies
 // them to its output. Called by the whole warp. Ray counts are those of the
-// pass repeated. On the mid terrain (720p, 4 samples, K = 6, TARGET) about a
+// pass repeated (COUNT: none, the work done is counted). On the mid terrain (720p, 4 samples, K = 6, TARGET) about a
 // quarter of all tile passes repeat, the cheaper ones, whose rays stay within a
 // triangle: a frame 3.17 -> 2.96 ms with the 24 warps per SM above.
+template <bool COUNT>
 __device__ __forceinline__ bool repeat_tile(const ViewDev& v, int tile, int lane, uint32_t& n_primary,
                                             uint32_t& n_shadow) {
     const MsRepeat& m = v.repeat;
@@ -148,7 +149,7 @@ __device__ __forceinline__ bool repeat_tile(const ViewDev& v, int tile, int lane
             const int32_t* ids = two ? m.ids_two_ago : m.ids_before;
             if (v.prim != ids) v.prim[p] = ids[p];
         }
-        n_primary += v.spp > 0 ? v.spp : 1;
+        if (!COUNT) n_primary += v.spp > 0 ? v.spp : 1;
     }
     __syncwarp();
     if (lane == 0) {
@@ -156,7 +157,7 @@ __device__ __forceinline__ bool repeat_tile(const ViewDev& v, int tile, int lane
         m.flags_out[tile] = (uint8_t)(2u | (two ? own & 1u : 1u));
         const unsigned sh = two ? m.shadow[tile] : m.shadow_before[tile];
         m.shadow[tile] = sh;
-        n_shadow += sh;
+        if (!COUNT) n_shadow += sh;
     }
     return true;
 }
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(BLOCK, MS == MS_FEW ? 512 / BLOCK : CHAIN || M
                 __syncwarp();
             }
             const SceneDev& S = MULTI ? s_scene[threadIdx.x >> 5] : S0;
-            if (MS && !MULTI && v.repeat.flags_out && repeat_tile(v, (int)(chunk - v.chunk_begin), lane, n_primary, n_shadow))
+            if (MS && !MULTI && v.repeat.flags_out && repeat_tile<COUNT>(v, (int)(chunk - v.chunk_begin), lane, n_primary, n_shadow))
                 continue;
             bool same1 = true, same2 = true;  // MS: this pixel equals the pass before, and the one before that
             const uint32_t shadow_before = n_shadow;
@@ -334,8 +335,10 @@ __global__ void __launch_bounds__(BLOCK, MS == MS_FEW ? 512 / BLOCK : CHAIN || M
                             // the orbit has closed: I_{n+1} is I_n, or I_{n+1}, I_{n+2}, ... alternate
                             // between I_{n-1} and I_n
                             const uint32_t odd = fixed ? 0u : (left + 1) / 2;
-                            n_primary += left;
-                            n_shadow += odd * prev_shadow + (left - odd) * shadow;
+                            if (!COUNT) {  // the work done is counted, the rays of all passes are
+                                n_primary += left;
+                                n_shadow += odd * prev_shadow + (left - odd) * shadow;
+                            }
                             if (fixed || !(left & 1u)) {
                                 out = cur;
                                 prim = id;
@@ -726,11 +729,15 @@ rcp_status launch_pass(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d
 }
 
 rcp_status launch_chain(const SceneDev& S, const LaunchCfg& cfg, const ViewDev* d_views, int n_views,
-                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays, cudaStream_t st) {
-    if (cfg.ms || cfg.count) {
-        set_error("launch_chain: a chained launch is single-sample and keeps no work counters");
+                        int64_t total_chunks, unsigned* d_work, unsigned long long* d_rays,
+                        unsigned long long* d_counters, cudaStream_t st) {
+    if (cfg.ms || (cfg.multi && cfg.count)) {
+        set_error("launch_chain: a chained launch is single-sample, and one of several scenes keeps no work counters");
         return RCP_ERR_STATE;
     }
+    if (cfg.count)
+        return launch_trace_b<true, true, 0, false, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
+                                                          d_rays, d_counters, st);
     if (cfg.multi)  // views of several scenes: no counters
         return launch_trace_b<true, false, 0, true, true>(S, cfg, d_views, n_views, total_chunks, nullptr, d_work,
                                                               d_rays, nullptr, st);

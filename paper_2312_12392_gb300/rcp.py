@@ -104,6 +104,8 @@ _SIGS = {
     "rcp_last_ray_counts": [_vp, C.POINTER(C.c_int64), C.POINTER(C.c_int64)],
     "rcp_count_pass": [_vp, C.POINTER(rcp_camera), C.c_int, C.c_int, C.POINTER(rcp_params), _vp, _vp,
                        C.POINTER(rcp_counters)],
+    "rcp_count_frame": [_vp, C.POINTER(rcp_camera), C.c_int, C.c_int, C.c_int, C.POINTER(rcp_params), _vp, _vp,
+                        C.POINTER(rcp_counters)],
     "rcp_last_pass_times": [_vp, C.POINTER(C.c_float), C.c_int, C.POINTER(C.c_int)],
     "rcp_render_h2d_bytes": [C.c_int, C.c_int],
     "rcp_debug_trace": [_vp, C.c_int64, _vp, _vp, C.c_int, C.c_int, _vp, _vp, C.c_int, _vp],
@@ -345,6 +347,14 @@ def rcp_count_pass(scene, cam: rcp_camera, width, height, params: rcp_params, d_
     c = rcp_counters()
     _check(lib().rcp_count_pass(scene, C.byref(cam), width, height, C.byref(params), _ptr(d_in), _ptr(d_out),
                                 C.byref(c)), "rcp_count_pass")
+    return c
+
+
+def rcp_count_frame(scene, cam: rcp_camera, width, height, K, params: rcp_params, d_in=None,
+                    d_out=None) -> rcp_counters:
+    c = rcp_counters()
+    _check(lib().rcp_count_frame(scene, C.byref(cam), width, height, K, C.byref(params), _ptr(d_in), _ptr(d_out),
+                                 C.byref(c)), "rcp_count_frame")
     return c
 
 
