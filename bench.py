@@ -285,13 +285,13 @@ def tuning_dict(t):
 def time_frames(g, cams, W, H, K, params, stream, flush):
     """Render one frame per camera (K passes each) through the device path,
     L2 flushed before each (outside the events). Returns per-frame ms, per-
-    launch ms and the rays traced. A frame's time is its captured graph's
+    launch ms and the rays of all K passes. A frame's time is its launches'
     device time, from the CUDA events the library records on the launching
-    stream around the graph's launches (rcp_last_pass_times, summed): events
+    stream around them (rcp_last_pass_times, summed): events
     recorded by this loop around the call would also count any wait of the
     idle GPU for this host thread between the two records. The per-frame
     outer events are kept in time_frames.outer_ms (their excess over the
-    graph's time: the descriptor upload and such waits)."""
+    launches' time: such waits)."""
     import torch
 
     from paper_2312_12392_gb300 import rcp
@@ -343,8 +343,8 @@ def count_work(g, cams, W, H, K, params, sizes=None, frames=None):
 
 
 def roofline(work, pass_ms, frames, workload, clk, sms):
-    """The trace kernel's roofline: algorithmic FP32 lane-operations per launch
-    over the mean launch time, against SMs x 128 lanes x the maximum SM clock
+    """The trace kernel's roofline: the FP32 lane-operations a launch executes
+    (box, triangle, sphere and camera arithmetic, no bookkeeping) over the mean launch time, against SMs x 128 lanes x the maximum SM clock
     (the kernel is bound by instruction issue and the ALU pipe, ncu); the byte
     view charges every node, primitive and image fetch at the measured HBM
     peak; the ncu view (issue, pipes, L1) comes from the committed profile when
@@ -497,12 +497,11 @@ def run_ours(args):
         "steps": args.steps,
         "warmup": args.warmup,
         "ms_per_step": tmax / args.steps,
-        "step_timing": {"source": "CUDA events the library records on the launching stream around the graph's "
-                                  "launches, summed per frame",
+        "step_timing": {"source": "CUDA events the library records on the launching stream around the "
+                                  "frame's launches, summed per frame",
                         "call_bracket_ms_per_step": statistics.mean(outer_ms),
                         "call_bracket_note": "events recorded by the bench before and after each rcp_render_device "
-                                             "call: also the descriptor upload and any wait of the GPU for the "
-                                             "host between them"},
+                                             "call: also any wait of the GPU for the host between them"},
         "higher_is_better": True,
         "scaling": "weak",
         "vs_baseline": None,

@@ -225,7 +225,9 @@ rcp_status rcp_render_pass(const rcp_scene* scene, const rcp_camera* cam, int wi
  * last pass's hit ids to d_prim (device, nullable). Enqueued on `stream`
  * (cudaStream_t, NULL = legacy default); the call returns once enqueued. A
  * K-pass sequence of several launches is captured per (scene, shape, K) in a
- * CUDA graph and replayed. Intermediate images live in library-owned device memory. */
+ * CUDA graph when its configuration comes a second time, and replayed from then
+ * on; one of one or two launches is enqueued as it is. Intermediate images live
+ * in library-owned device memory, kept per shape up to 16 GiB a scene. */
 rcp_status rcp_render_device(const rcp_scene* scene, const rcp_camera* cam, int width, int height,
                              int K, const rcp_params* params, const float* d_in, float* d_out,
                              int32_t* d_prim, void* stream);
@@ -246,8 +248,8 @@ rcp_status rcp_imagespace_pass_device(const float* d_base, const float* d_prev, 
  * aliasing rule as rcp_render_device. d_outs: host array of n_views device
  * pointers (rgbz, width*height*4 floats each). d_prims: NULL or a host array of
  * n_views device pointers (width*height int32 each, or NULL) receiving the
- * last pass's hit ids. All views run K passes; the K-pass recursion is
- * captured in a CUDA graph keyed by the view shapes. Enqueued on `stream`. */
+ * last pass's hit ids. All views run K passes, in the launches that
+ * rcp_render_device describes. Enqueued on `stream`. */
 rcp_status rcp_render_batch_device(const rcp_scene* scene, int n_views, const rcp_camera* cams,
                                    const int* widths, const int* heights, int K,
                                    const rcp_params* params, const float* const* d_ins,
@@ -320,19 +322,20 @@ rcp_status rcp_count_frame(const rcp_scene* scene, const rcp_camera* cam, int wi
                            const rcp_params* params, const float* d_in, float* d_out, rcp_counters* out);
 
 /* Device time (ms) of each launch of the scene's most recent render, from CUDA
- * events recorded on the render's stream between the launches (inside the
- * captured graph): one per pass, or one for all K passes when they ran
- * chained (an RCP_MAP_IMAGE render of K >= 2: the traced pass, then all
- * gathers). Read after the render has completed. */
+ * events recorded on the render's stream between the launches. *n_passes
+ * receives the number of times, which is not always K: one per pass, or one for
+ * all K passes when they ran chained, or two for a chained RCP_MAP_IMAGE render
+ * of K >= 2 (the traced pass, then all gathers). With chain_passes = 0 in the
+ * tuning there is one per pass. Read after the render has completed. */
 rcp_status rcp_last_pass_times(const rcp_scene* scene, float* ms, int max_passes, int* n_passes);
 
-/* Bytes that one rcp_render call of K passes over n_views views copies from
- * host to device: the views' per-pass descriptors (camera terms, image
- * pointers), uploaded once per call. The library's own bookkeeping, not part of
- * the method. A render whose passes run chained uploads one descriptor per
- * view, rcp_render_h2d_bytes(n_views, 1), or two (RCP_MAP_IMAGE, K >= 2).
- * Returns -1 when K or n_views is out
- * of range. */
+/* Bytes that one rcp_render call of K passes over n_views views sends from host
+ * to device: the views' per-pass descriptors (camera terms, image pointers),
+ * once per call. The library's own bookkeeping, not part of the method. A
+ * render of one or two launches and at most four descriptors passes them as a
+ * launch's parameters, others copy them. A render whose passes run chained has
+ * one descriptor per view, rcp_render_h2d_bytes(n_views, 1), or two
+ * (RCP_MAP_IMAGE, K >= 2). Returns -1 when K or n_views is out of range. */
 int64_t rcp_render_h2d_bytes(int n_views, int K);
 
 /* Diagnostics used by the tests (all device pointers, enqueued on `stream`):

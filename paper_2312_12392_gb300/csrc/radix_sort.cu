@@ -291,8 +291,8 @@ __global__ void __launch_bounds__(SORT_BLOCK, 1) k_onesweep(const uint32_t* __re
 // ranks its keys, publishes its 256 digit counts, and after a grid-wide barrier
 // adds up every tile's counts itself (all tiles' and the earlier tiles'), where
 // separate passes need a histogram beforehand and look back tile by tile; the
-// pairs go to the other buffer and a second barrier ends the pass. The launch is cooperative, so that every block
-// that a barrier waits for runs; each wait is bounded all the same, and as the
+// pairs go to the other buffer and a second barrier ends the pass. The launch is
+// cooperative, so that every block that a barrier waits for runs; each wait is bounded all the same, and as the
 // counts are zero beforehand, one that runs out leaves sums too small: the pairs
 // still go to places in range.
 struct ResidentShared {

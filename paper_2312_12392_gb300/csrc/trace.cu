@@ -117,9 +117,10 @@ __device__ __forceinline__ bool same_bits(const float4& a, const float4& b) {
 // I_n is I_{n-2}, which its ping-pong buffer still holds; where all nine had
 // I_{n-1} = I_{n-2}, it is I_{n-1}, the same bits again. The last pass copies
 // them to its output. Called by the whole warp. Ray counts are those of the
-// pass repeated (COUNT: none, the work done is counted). On the mid terrain (720p, 4 samples, K = 6, TARGET) about a
-// quarter of all tile passes repeat, the cheaper ones, whose rays stay within a
-// triangle: a frame 3.17 -> 2.96 ms with the 24 warps per SM above.
+// pass repeated (COUNT: none, the work done is counted). On the mid terrain
+// (720p, 4 samples, K = 6, TARGET) about a quarter of all tile passes repeat, the
+// cheaper ones, whose rays stay within a triangle: a frame 3.17 -> 2.96 ms with
+// the 24 warps per SM of MS_MANY (below).
 template <bool COUNT>
 __device__ __forceinline__ bool repeat_tile(const ViewDev& v, int tile, int lane, uint32_t& n_primary,
                                             uint32_t& n_shadow) {
